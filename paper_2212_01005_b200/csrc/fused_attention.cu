@@ -30,8 +30,8 @@
 //       maximum of the row's first 32 scores. Softmax does not depend on the reference value; the true row maximum
 //       only keeps the exponentials in range: when the last chunk is in registers, the partial row sum (it bounds every
 //       exponential so far) and the last chunk's maximum tell whether it did; if not, the warp keeps the score half,
-//       takes the true row maximum from it and repeats the pass. Three exponentials in four run on the
-//       special-function unit, the fourth as a cubic on the FMA pipe)
+//       takes the true row maximum from it and repeats the pass. Five exponentials in eight run on the
+//       special-function unit, the others as a cubic on the FMA pipe, in packed pairs)
 //   P5  tcgen05.mma: O_h[128 x 64] = P_h V_h        (V is the N-major B operand, as it lies in HBM)
 //   P6  four epilogue warps (a query row per thread): TMEM -> registers as soon as a half's product is complete (its
 //       accumulator is released at once), (f_0 O_0 + f_1 O_1) / sum, bf16 -> per warp, pieces of 16 columns x 32 rows
@@ -90,6 +90,10 @@ struct AttnParams {
   int p_half_bytes;
 };
 
+// Which of a chunk's 16 column pairs take their exponentials on the FMA pipe: three in eight (none 34.0, one in eight 33.5,
+// one in four 32.8, three in eight 32.1, one in two 34.5 us at 32 x 12 heads x 384 keys: both pipes are then about evenly full).
+__device__ constexpr bool poly_pair(int j) { return (j & 7) == 2 || (j & 7) == 4 || (j & 7) == 7; }
+
 // 2^x on the special-function unit (arguments here are <= 0; results below 2^-126 flush to 0).
 __device__ __forceinline__ float ex2_approx(float x) {
   float y;
@@ -97,18 +101,47 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
-// 2^x on the FMA pipe, for a share of the exponentials (the special-function unit delivers 16 results per cycle and SM,
-// which bounds the probability pass): x is split with the magic-number addition into an integer n, which goes straight
-// into the exponent field, and a fraction f in [-0.5, 0.5], on which a cubic (fitted to 2^f, relative error < 8e-5, well
-// below the bf16 rounding of the result) is evaluated. Results below 2^-125 are clamped there instead of flushed to 0.
-__device__ __forceinline__ float ex2_poly(float x) {
-  x = fmaxf(x, -125.0f);
-  const float t = x + 12582912.0f;              // 1.5 * 2^23: round(x) appears in the low mantissa bits
-  const float f = x - (t - 12582912.0f);
-  float q = fmaf(f, 0.05517092f, 0.24260956f);
-  q = fmaf(q, f, 0.69326097f);
-  q = fmaf(q, f, 0.9999282f);
-  return __uint_as_float(__float_as_uint(q) + (__float_as_uint(t) << 23));
+// Packed pairs of fp32: one instruction for two elements (half the issue slots; the FMA pipe's rate is the same).
+__device__ __forceinline__ uint64_t pair2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpair2(uint64_t v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// 2^x of a pair on the FMA pipe, for a share of the exponentials (the special-function unit delivers 16 results per cycle
+// and SM, which bounds the probability pass): x is split with the magic-number addition into an integer n, which goes
+// straight into the exponent field, and a fraction f in [-0.5, 0.5], on which a cubic (fitted to 2^f, relative error
+// < 8e-5, well below the bf16 rounding of the result) is evaluated. Results below 2^-125 are clamped there instead of
+// flushed to 0.
+__device__ __forceinline__ void ex2_poly2(float& x0, float& x1) {
+  const uint64_t x = pair2(fmaxf(x0, -125.0f), fmaxf(x1, -125.0f));
+  const uint64_t magic = pair2(12582912.0f, 12582912.0f);   // 1.5 * 2^23: round(x) appears in the low mantissa bits
+  const uint64_t t = add2(x, magic);
+  const uint64_t f = sub2(x, sub2(t, magic));
+  uint64_t q = fma2(f, pair2(0.05517092f, 0.05517092f), pair2(0.24260956f, 0.24260956f));
+  q = fma2(q, f, pair2(0.69326097f, 0.69326097f));
+  q = fma2(q, f, pair2(0.9999282f, 0.9999282f));
+  float t0, t1, q0, q1;
+  unpair2(t, t0, t1);
+  unpair2(q, q0, q1);
+  x0 = __uint_as_float(__float_as_uint(q0) + (__float_as_uint(t0) << 23));
+  x1 = __uint_as_float(__float_as_uint(q1) + (__float_as_uint(t1) << 23));
 }
 
 // Orders the compiler only: no use of these registers moves above this point, no later write to them above their last use.
@@ -332,30 +365,34 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
       for (int j = 0; j < 32; ++j) if (j < nreal) m = fmaxf(m, __uint_as_float(v[j]));
       return m;
     };
-    // 32 columns of real keys -> four 16-byte chunks of the probability row; s4 collects the row sum. All 32 exponentials
+    // 32 columns of real keys -> four 16-byte chunks of the probability row; s2 collects the row sum. All 32 exponentials
     // are issued back to back, in place, before anything consumes one: the special-function unit takes a warp's
-    // instruction every eight cycles, and only independent ones in flight keep it busy from a single warp.
-    auto exp32 = [&](uint32_t (&v)[32], uint8_t* blk, uint32_t ch0, float mc, float (&s4)[4]) {
+    // instruction every eight cycles, and only independent ones in flight keep it busy from a single warp. Scaling, the
+    // cubic and the row sum work on packed pairs and the bf16 pairs replace the values in place (32.8 -> 31.3 us at
+    // 32 x 12 heads x 384 keys; spreading the conversions between the exponentials made it 32.3).
+    auto exp32 = [&](uint32_t (&v)[32], uint8_t* blk, uint32_t ch0, uint64_t c2, uint64_t nmc2, uint64_t (&s2)[4]) {
 #pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        const float x = fmaf(__uint_as_float(v[j]), c, -mc);
-        v[j] = __float_as_uint((j & 3) == 3 ? ex2_poly(x) : ex2_approx(x));   // one in four on the FMA pipe
+      for (int j = 0; j < 16; ++j) {
+        float x0, x1;
+        unpair2(fma2(pair2(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1])), c2, nmc2), x0, x1);
+        if (poly_pair(j)) {
+          ex2_poly2(x0, x1);
+        } else {
+          x0 = ex2_approx(x0); x1 = ex2_approx(x1);
+        }
+        v[2 * j] = __float_as_uint(x0); v[2 * j + 1] = __float_as_uint(x1);
       }
 #pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        uint32_t w[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float e0 = __uint_as_float(v[g * 8 + 2 * j]), e1 = __uint_as_float(v[g * 8 + 2 * j + 1]);
-          s4[j] += e0 + e1;
-          w[j] = pack_p(e0, e1);
-        }
-        *reinterpret_cast<uint4*>(blk + (((ch0 + g) ^ sw) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+      for (int j = 0; j < 16; ++j) {
+        const float e0 = __uint_as_float(v[2 * j]), e1 = __uint_as_float(v[2 * j + 1]);
+        s2[j & 3] = add2(s2[j & 3], pair2(e0, e1));
+        v[j] = pack_p(e0, e1);
+        if ((j & 3) == 3) *reinterpret_cast<uint4*>(blk + (((ch0 + (j >> 2)) ^ sw) << 4)) = make_uint4(v[j - 3], v[j - 2], v[j - 1], v[j]);
       }
     };
     // The last chunk of a half: ncols (16 or 32) columns belong to the half, the first nreal of them are keys; the
     // probabilities of the padding columns are zeros (their V rows are zeros too, but must not meet a NaN).
-    auto exp_tail = [&](uint32_t (&v)[32], uint8_t* blk, uint32_t ch0, int ncols, int nreal, float mc, float (&s4)[4]) {
+    auto exp_tail = [&](uint32_t (&v)[32], uint8_t* blk, uint32_t ch0, int ncols, int nreal, float mc, uint64_t (&s2)[4]) {
 #pragma unroll
       for (int g = 0; g < 4; ++g) {
         if (g * 8 < ncols) {
@@ -367,7 +404,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
             float e1 = ex2_approx(fmaf(__uint_as_float(v[e + 1]), c, -mc));
             if (e >= nreal) e0 = 0.0f;
             if (e + 1 >= nreal) e1 = 0.0f;
-            s4[j] += e0 + e1;
+            s2[j] = add2(s2[j], pair2(e0, e1));
             w[j] = pack_p(e0, e1);
           }
           *reinterpret_cast<uint4*>(blk + (((ch0 + g) ^ sw) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
@@ -407,7 +444,13 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         bool exact = false;
         if (nch == 1) exact = last_chunk_landed(attempt, 0.0f, m);
         const float mc = m * c;
-        float s4[4] = {0.f, 0.f, 0.f, 0.f};
+        const uint64_t c2 = pair2(c, c), nmc2 = pair2(-mc, -mc);
+        uint64_t s2[4] = {0ull, 0ull, 0ull, 0ull};   // the row sum in eight parts
+        auto row_sum = [&]() -> float {
+          float lo, hi;
+          unpair2(add2(add2(s2[0], s2[1]), add2(s2[2], s2[3])), lo, hi);
+          return lo + hi;
+        };
         uint8_t* blk = prow;
 #pragma unroll 1
         for (int ch = 0; ch < nch; ch += 2, blk += kBlockM * 128) {
@@ -415,22 +458,22 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
             if (lane == 0) mbar_wait(bar_pfree + grp * 3 + (ch >> 1), ph ^ 1u, abort_flag, p.status, 0x211);
             __syncwarp();
           }
-          if (kv - ch * 32 >= 32) exp32(va, blk, 0u, mc, s4); else exp_tail(va, blk, 0u, hw - ch * 32, kv - ch * 32, mc, s4);
+          if (kv - ch * 32 >= 32) exp32(va, blk, 0u, c2, nmc2, s2); else exp_tail(va, blk, 0u, hw - ch * 32, kv - ch * 32, mc, s2);
           if (ch + 1 < nch) {
             wait32(vb);
             if (ch + 2 < nch) tmem_ld_x32(s_addr + (uint32_t)((ch + 2) * 32), va);
-            else exact = last_chunk_landed(attempt, (s4[0] + s4[1]) + (s4[2] + s4[3]),
+            else exact = last_chunk_landed(attempt, row_sum(),
                                            kv - ch * 32 >= 64 ? max32(vb) : max_tail(vb, kv - ch * 32 - 32));
-            if (kv - ch * 32 >= 64) exp32(vb, blk, 4u, mc, s4); else exp_tail(vb, blk, 4u, hw - ch * 32 - 32, kv - ch * 32 - 32, mc, s4);
+            if (kv - ch * 32 >= 64) exp32(vb, blk, 4u, c2, nmc2, s2); else exp_tail(vb, blk, 4u, hw - ch * 32 - 32, kv - ch * 32 - 32, mc, s2);
             if (ch + 2 < nch) {
               wait32(va);
               if (ch + 3 < nch) tmem_ld_x32(s_addr + (uint32_t)((ch + 3) * 32), vb);
-              else exact = last_chunk_landed(attempt, (s4[0] + s4[1]) + (s4[2] + s4[3]),
+              else exact = last_chunk_landed(attempt, row_sum(),
                                              kv - ch * 32 >= 96 ? max32(va) : max_tail(va, kv - ch * 32 - 64));
             }
           }
         }
-        sum = (s4[0] + s4[1]) + (s4[2] + s4[3]);
+        sum = row_sum();
         if (!exact) break;
         // ---------------- exact path: the row maximum over all chunks first ----------------
         m = -INFINITY;
