@@ -3,8 +3,8 @@
 Every function of ``include/ago.h`` is exposed under its C name
 (``ago_subgraph_create`` ...). ``Subgraph`` is a convenience wrapper that builds
 the descriptor from a neutral operator list and passes torch tensors' device
-pointers and the current CUDA stream; all computation happens inside the
-library's kernels. There is no CPU or PyTorch fallback: if the library cannot
+pointers and the current CUDA stream (in native code, pyext/ago_call.cpp); all
+computation happens inside the library's kernels. There is no CPU or PyTorch fallback: if the library cannot
 be loaded, or a call fails, an exception is raised.
 """
 from __future__ import annotations
@@ -320,7 +320,9 @@ class Subgraph:
             raise AgoError(*ago_last_error())
         self.mode = mode
         self.dtype = dtype
+        self._num_inputs = len(input_shapes)
         self._ws = None
+        self._runner = None
         rank = self.query(AGO_Q_OUTPUT_RANK)
         self.output_shape = tuple(self.query(AGO_Q_OUTPUT_DIM, i) for i in range(rank))
         self.num_weights = self.query(AGO_Q_NUM_WEIGHTS)
@@ -350,21 +352,27 @@ class Subgraph:
         dt = torch.float32 if self.dtype == AGO_FP32 else torch.bfloat16
         return torch.empty(self.output_shape, dtype=dt, device=device)
 
+    def _make_runner(self):
+        """The native caller of this handle (created at the first run: it needs torch)."""
+        if not getattr(self, "_h", None):
+            raise AgoError(AGO_ERR_INVALID_ARG, "handle is NULL")
+        import torch  # noqa: F401  (its libraries have to be loaded before the extension's)
+        from . import _ago_call
+        lib = load()
+        addr = lambda f: ctypes.cast(f, ctypes.c_void_p).value
+        self._runner = _ago_call.make_runner(addr(lib.ago_subgraph_run), addr(lib.ago_last_error), AgoError, self._h, self.output_shape,
+                                             self.dtype == AGO_FP32, self.workspace_bytes, self._num_inputs, self.num_weights)
+        return self._runner
+
     def run(self, inputs, weights, out=None, stream=None):
         """inputs / weights: torch CUDA tensors (contiguous). Enqueues on the
         current torch stream (or ``stream``) and returns the output tensor."""
-        import torch
-        dev = inputs[0].device
-        if dev.type != "cuda":
-            raise AgoError(AGO_ERR_CUDA, "inputs must be CUDA tensors: this library has no CPU path")
-        if out is None:
-            out = self.empty_output(dev)
-        self.ensure_workspace(dev)
-        s = stream if stream is not None else torch.cuda.current_stream(dev).cuda_stream
-        st = ago_subgraph_run(self._h, [t.data_ptr() for t in inputs], [t.data_ptr() for t in weights],
-                              [out.data_ptr()], s)
-        self._check(st)
-        return out
+        runner = self._runner or self._make_runner()
+        res = runner(inputs, weights, out, stream, self._ws)
+        if res is None:                        # the handle needs a workspace on this device
+            self.ensure_workspace(inputs[0].device)
+            res = runner(inputs, weights, out, stream, self._ws)
+        return res
 
     def run_host(self, host_inputs, weights, host_out, dev_inputs, dev_out, stream=None):
         """Pinned host tensors in and out, device staging tensors supplied by the caller."""
@@ -382,6 +390,7 @@ class Subgraph:
 
     def close(self):
         if getattr(self, "_h", None):
+            self._runner = None
             ago_subgraph_destroy(self._h)
             self._h = None
 

@@ -1,4 +1,5 @@
-"""Builds libago.so (the C-ABI library) in-tree with nvcc for sm_100a."""
+"""Builds libago.so (the C-ABI library) in-tree with nvcc for sm_100a, and _ago_call.so (the native host path of
+Subgraph.run: CPython and torch headers only) with g++."""
 from __future__ import annotations
 
 import glob
@@ -11,6 +12,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "libago.so")
+EXT_SRC = os.path.join(HERE, "pyext", "ago_call.cpp")
+EXT = os.path.join(HERE, "_ago_call.so")
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -37,6 +40,7 @@ def _deps_mtime() -> float:
 
 def build(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OBJ, exist_ok=True)
+    build_ext(force)
     hdr_m = _deps_mtime()
     nvcc = _nvcc()
     todo, objs = [], []
@@ -68,6 +72,24 @@ def build(force: bool = False, verbose: bool = False) -> str:
                                "-cudart", "static"])
         os.replace(tmp, LIB)
     return LIB
+
+
+def build_ext(force: bool = False) -> str:
+    if not force and os.path.exists(EXT) and os.path.getmtime(EXT) >= os.path.getmtime(EXT_SRC):
+        return EXT
+    import sysconfig
+    import torch
+    root = os.path.dirname(torch.__file__)
+    tmp = EXT + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+           "-I" + os.path.join(root, "include"), "-I" + os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           "-I" + sysconfig.get_paths()["include"], "-I/usr/local/cuda/include", EXT_SRC, "-o", tmp,
+           "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed for {EXT_SRC}:\n{r.stderr[-4000:]}")
+    os.replace(tmp, EXT)
+    return EXT
 
 
 if __name__ == "__main__":
