@@ -72,7 +72,7 @@ struct Mbv2Params {
   int Coutp, NC;
   // 2^32 / d + 1 for the run-time divisors of the index arithmetic: x / d == __umulhi(x, recip) for x, d < 65536
   uint32_t coutp_recip, w_recip, strips_recip, per_row_recip, cexp8_recip;   // cexp8: Cexp / 8 (>= 2)
-  int per_row, nseg, step_r, step_c, col_slots;   // depthwise item geometry (see the kernel), fixed per shape
+  int per_row, nseg, segw, step_r, step_c, col_slots;   // depthwise item geometry (see the kernel), fixed per shape
   int tmem_cols, ecol0, pcol0;
   int e_plane, d_plane;         // byte distance between the two 8-channel planes of an E / D chunk
   // shared-memory byte offsets (from the 1024-aligned base)
@@ -423,9 +423,9 @@ mbv2_fused_kernel(const Mbv2Params p) {
     const bool has_item = slot < dw_items;
     uint32_t it_e, it_d; int it_a, it_b;
     if (p.stride == 1) {
-      const int wo = item0_c * kSegCols;
+      const int wo = item0_c * p.segw;
       it_e = (uint32_t)(2 * item0_r) * e_pitch + wo * 16; it_d = (uint32_t)(2 * item0_r) * d_pitch + wo * 16;
-      it_a = min(kSegCols, p.Wo - wo); it_b = min(2, rows_valid - 2 * item0_r);
+      it_a = min(p.segw, p.Wo - wo); it_b = min(2, rows_valid - 2 * item0_r);
     } else {
       it_e = item0_c * 32; it_d = item0_c * 16;
       it_a = item0_r * rows_per_group; it_b = min(rows_valid, it_a + rows_per_group);
@@ -490,24 +490,26 @@ mbv2_fused_kernel(const Mbv2Params p) {
         const float2 bias = make_float2(__uint_as_float(lds32<0>(bd_addr)), __uint_as_float(lds32<4>(bd_addr)));
         wd_addr += (uint32_t)NG * 9u * kChunkRowBytes; bd_addr += (uint32_t)NG * kChunk * 4u;   // the group's next chunk is c + NG
         const uint32_t e_plane = e_plane0 + (EXPAND ? 0u : (uint32_t)((it & 1) * e_bytes));
-        if (has_item) {   // the thread's first item: geometry fixed before the chunk loop
-          if (p.stride == 1) depthwise_block(e_plane + it_e, d_plane + it_d, e_pitch, d_pitch, it_a, it_b, wgt, bias);
-          else if (it_a < it_b) depthwise_column_s2(e_plane + it_e, d_plane + it_d, it_a, it_b, p.IW, p.Wo, wgt, bias);
-        }
-        if (dw_items > kSlots) {   // shapes with more items than slots
-          int r = item0_r + step_r, col = item0_c + step_c;
-          if (col >= per_row) { col -= per_row; ++r; }
-          for (int item = slot + kSlots; item < dw_items; item += kSlots) {
-            if (p.stride == 1) {
-              const int wo = col * kSegCols;
-              depthwise_block(e_plane + (uint32_t)(2 * r) * e_pitch + wo * 16, d_plane + (uint32_t)(2 * r) * d_pitch + wo * 16, e_pitch,
-                              d_pitch, min(kSegCols, p.Wo - wo), min(2, rows_valid - 2 * r), wgt, bias);
-            } else {
-              const int r0 = r * rows_per_group, r1 = min(rows_valid, r0 + rows_per_group);
-              if (r0 < r1) depthwise_column_s2(e_plane + col * 32, d_plane + col * 16, r0, r1, p.IW, p.Wo, wgt, bias);
-            }
+        if (has_item) {
+          // the geometry of the thread's first item was fixed before the chunk loop; shapes with more items than slots
+          // go around with that of the next ones (one copy of the unrolled block: the code of a chunk stays small)
+          uint32_t e = e_plane + it_e, d = d_plane + it_d;
+          int ia = it_a, ib = it_b, r = item0_r, col = item0_c;
+#pragma unroll 1
+          for (int item = slot;;) {
+            if (p.stride == 1) depthwise_block(e, d, e_pitch, d_pitch, p.segw, ia, ib, wgt, bias);
+            else if (ia < ib) depthwise_column_s2(e, d, ia, ib, p.IW, p.Wo, wgt, bias);
+            if ((item += kSlots) >= dw_items) break;
             r += step_r; col += step_c;
             if (col >= per_row) { col -= per_row; ++r; }
+            if (p.stride == 1) {
+              const int wo = col * p.segw;
+              e = e_plane + (uint32_t)(2 * r) * e_pitch + wo * 16; d = d_plane + (uint32_t)(2 * r) * d_pitch + wo * 16;
+              ia = min(p.segw, p.Wo - wo); ib = min(2, rows_valid - 2 * r);
+            } else {
+              ia = r * rows_per_group; ib = min(rows_valid, ia + rows_per_group);
+              e = e_plane + col * 32; d = d_plane + col * 16;
+            }
           }
         }
       }
@@ -665,7 +667,8 @@ ago_status_t mbv2_plan(Plan* plan, FusedState* st, std::string* err) {
   q.coutp_recip = recip(q.Coutp);
   q.w_recip = recip(q.W);
   q.cexp8_recip = recip(q.Cexp / 8);
-  q.nseg = (q.Wo + kSegCols - 1) / kSegCols;
+  q.segw = seg_width(q.Wo);
+  q.nseg = (q.Wo + q.segw - 1) / q.segw;
   q.per_row = q.stride == 1 ? q.nseg : q.Wo;
   q.per_row_recip = recip(q.per_row);
   auto set_groups = [&](Mbv2Params& t, int ng) {   // depthwise item geometry of a group of 32 / ng warps
