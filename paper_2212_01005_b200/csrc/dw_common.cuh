@@ -100,10 +100,11 @@ __device__ __forceinline__ void depthwise_column_s2(uint32_t e_col, uint32_t d_c
 // output pixel. The loads of a block with fewer valid rows or columns run past the valid pixels, inside shared memory.
 constexpr int kSegCols = 7;       // the widest block
 constexpr int kMinSegCols = 3;    // the narrowest one the early ends below know
-// width of the blocks a row of `wo` outputs is cut into: the narrowest that keeps the number of blocks
+// Width of the blocks a row of `wo` outputs is cut into: the narrowest that keeps the number of blocks, made odd -- a warp
+// works on four neighbouring blocks, whose 16-byte pixels then lie in different banks.
 inline int seg_width(int wo) {
   const int n = (wo + kSegCols - 1) / kSegCols, w = (wo + n - 1) / n;
-  return w < kMinSegCols ? kMinSegCols : w;
+  return w < kMinSegCols ? kMinSegCols : (w | 1);
 }
 
 template <int J>

@@ -193,8 +193,9 @@ ago_status_t dwdw_plan(Plan* plan, FusedState* st, std::string* err) {
   if (best == 0) return bad("image too large");
   st->impl = host;
   st->impl_free = [](void* p) { delete static_cast<DwDwHost*>(p); };
-  st->tile_rows = q.R; st->grid = (q.items + kThreads - 1) / kThreads * q.N; st->smem_bytes = 0;
-  plan->tile_rows = q.R; plan->smem_bytes = 0;
+  st->tile_rows = q.R; st->grid = (q.items + kThreads - 1) / kThreads * q.N;
+  st->smem_bytes = 1024;       // nothing but the 1 KB that is reserved for every CTA
+  plan->tile_rows = q.R; plan->smem_bytes = st->smem_bytes;
   return AGO_OK;
 }
 

@@ -9,15 +9,21 @@
 // output rows of one image per CTA), so nothing is recomputed except the
 // expand convolution on the strip's one-row halo.
 //
-// Per CTA (one image, R output rows, full width):
-//   P1  the compute warps copy the NHWC input strip (with its row halo; rows
-//       outside the image -> 0, channels padded to the MMA K granularity), W1
-//       and W3 into swizzled K-major tiles with coalesced 16-byte loads -- all
-//       loads of a thread are issued before its first store, so the prologue
-//       is one round trip to device memory. (A pixel is Cin * 2 bytes there,
+// Wide blocks and small batches: the expanded channels of a strip are split over
+// a cluster of CS CTAs (the chunks of a CTA are what its time grows with, and a
+// handful of strips leaves most SMs idle). Each runs the steps below on its share;
+// the partial output sums are exchanged through distributed shared memory.
+// 25 images of 15 x 15, 96 -> 576 -> 96: 34 us as three launches (the weights of
+// so wide a block do not fit one SM), 16.5 us on clusters of four.
+//
+// Per CTA (one image, R output rows, full width, its share of the channels):
+//   P1  16-byte asynchronous copies bring the NHWC input strip (with its row
+//       halo; rows outside the image -> 0, channels padded to the MMA K
+//       granularity), W1 and W3 into swizzled K-major tiles; descriptors and work
+//       mapping are computed while they travel. (A pixel is Cin * 2 bytes there,
 //       e.g. 48: one TMA box row per pixel was several times slower.)
 //   for each 16-channel chunk c of the expanded tensor:
-//     P2  tcgen05.mma: expand[pixels x 16] = X[pixels x Cin] * W1[c]^T   (TMEM, fp32)
+//     P2  tcgen05.mma: expand[pixels x 16] = X[pixels x Cin] * W1[c]^T   (TMEM, fp32; Cin > 64: K blocks of 64)
 //     P3  TMEM -> registers: + b1, ReLU6, zero outside the image (the depthwise
 //         conv pads the post-activation tensor), bf16 -> shared memory; the
 //         padding columns of the E chunk are written once
@@ -25,13 +31,13 @@
 //         mixed-precision FMAs (bf16 activations and weights as stored, fp32
 //         accumulate), result written as the K-major A operand of the project GEMM
 //     P5  tcgen05.mma: out[pixels x Cout] += DW[pixels x 16] * W3[:, c]^T  (TMEM)
-//   P6  TMEM -> registers: + b3 (+ x), bf16, 16-byte stores.
+//   P6  TMEM -> registers: [sum over the cluster] + b3 (+ x), bf16, 16-byte stores.
 // The expand MMA of chunk c+1 is issued before the CUDA-core work of chunk c.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
-#include <cstdlib>
+#include <cmath>
 
 #include "dw_common.cuh"
 #include "fused.h"
@@ -44,12 +50,15 @@ namespace {
 using namespace tc;
 using namespace dw;
 
-constexpr int kWarps = 32;                         // every warp computes; MMAs are issued inline by some of them
+// Sixteen warps with 128 registers a thread; every warp computes, MMAs are issued inline by some of them. (With 32 warps the
+// cap of 64 registers left the depthwise block no room to have its loads in flight: it took twice the cycles it takes alone.
+// One 14 x 14 image of 32 -> 192 -> 32 channels 9.8 -> 6.5 us, 12 images of 16 x 16 10.9 -> 7.3 us; 56 x 56 strips the same.)
+constexpr int kWarps = 16;
 constexpr int kThreads = kWarps * 32;
-// The warps form NG groups (2 or 4) that own the chunks c = g, g + NG, ...: two groups of 16 warps for strips whose
-// chunk is real work (their phases overlap), four groups of 8 warps for small strips, where a chunk is a chain of
-// latencies (MMA hand-off, tensor-memory round trip, two barriers) and more chains in flight is all that helps.
-constexpr int kTilesPerWarp = 2;                   // expand-epilogue tiles per warp: at most 8 tiles over the 4 warps of a lane quarter
+// The warps form NG groups (2 or 4) that own the chunks c = g, g + NG, ...: two groups of eight warps for strips whose
+// chunk is real work (their phases overlap), four groups of four warps for small strips, where a chunk is a chain of
+// latencies (MMA hand-off, tensor-memory round trip, two barriers) and more chains in flight is what helps.
+constexpr int kTilesPerWarp = 4;                   // expand-epilogue tiles per warp
 constexpr int kExpandIssuers = 2;                  // the last two warps of a group issue its expand GEMMs
 constexpr int kChunk = 16;      // expanded channels per chunk = one MMA K step of the project GEMM
 constexpr int kChunkRowBytes = 32;
@@ -64,7 +73,12 @@ struct Mbv2Params {
   const float* b3;
   __nv_bfloat16* out;
   unsigned int* status;
-  int N, H, W, Cin, Cexp, Cout, stride, Ho, Wo, residual;
+  int N, H, W, Cin, Cexp, Cout, stride, Ho, Wo, residual;   // Cexp: expanded channels of one CTA
+  int CS, Cfull;                // the expanded channels are split over CS CTAs; Cfull = CS * Cexp
+  int PP;                       // CS > 1: output pixels of a strip that one CTA of the cluster sums up and stores (odd)
+  int off_send, off_recv, recv_shared;   // CS > 1: blocks of partial sums for / from the other CTAs; recv_shared: over dead operands
+  int kblocks, ksteps, cpr;     // reduction of the expand GEMM: 128-byte-row blocks, MMA steps, 16-byte chunks per row (kblocks > 1)
+  uint32_t pp_recip, cpr_recip, cout8_recip;
   int groups;                   // warp groups: 2 or 4 (the kernel template's NG)
   int fold_b1;                  // the expand bias rides in two spare reduction channels of the expand GEMM (Cin < Kp)
   int R, strips, IH, IW, P_x, P_in, M1, M2;   // P_x = IH * W pixels in the input tile, P_in = IH * IW in an E chunk
@@ -89,6 +103,11 @@ __device__ __forceinline__ float4 lds128f(uint32_t saddr) {
 __device__ __forceinline__ void sts128(uint32_t saddr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(saddr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
+
+// The two halves of a cluster barrier (all threads). The arrival publishes nothing -- barriers are made visible by
+// fence_mbar_init, data by the bulk copies' own completion -- so it is relaxed: a release at cluster scope takes 1200 cycles.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // FOLD: the expand bias rides in the expand GEMM (see the prologue). EXPAND / PROJECT select the pairs of the
 // block: <true, true> the whole block, <true, false> pointwise -> depthwise
@@ -115,11 +134,17 @@ mbv2_fused_kernel(const Mbv2Params p) {
   uint64_t* bar_d = bars + 8;       // [NG] project MMA has consumed D[g] (MMA commit)
   uint64_t* bar_first = bars + 16;  // project GEMM of chunk 0 complete (it overwrites the output accumulators: the other groups issue after it)
   uint64_t* bar_done = bars + 17;   // every project MMA complete (the groups do not follow each other's bar_d phases)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 18);
-  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 19);
+  uint64_t* bar_chain = bars + 18;  // two groups: group 0's first expand GEMM complete. One phase only: a waiter on bar_e could
+                                    // fall behind its next phase and then wait for a parity that has come and gone
+  uint64_t* bar_red = bars + 19;    // the partial sums of the other CTAs of the cluster have arrived
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 20);
+  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 21);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n = (int)fast_div(blockIdx.x, (uint32_t)p.strips, p.strips_recip), strip = (int)blockIdx.x - n * p.strips;
+  // CS CTAs (a cluster when their partial products are to be added) work on one strip, each on its share of the channels
+  const int unit = p.CS == 1 ? (int)blockIdx.x : (int)(blockIdx.x / (unsigned)p.CS), rank = (int)blockIdx.x - unit * p.CS;
+  const int n = (int)fast_div((uint32_t)unit, (uint32_t)p.strips, p.strips_recip), strip = unit - n * p.strips;
+  const int ch0 = rank * p.Cexp;        // first expanded channel of this CTA
   const int ho0 = strip * p.R;
   const int rows_valid = min(p.R, p.Ho - ho0);
   const int gh0 = ho0 * p.stride - 1;   // image row of tile row 0
@@ -132,68 +157,81 @@ mbv2_fused_kernel(const Mbv2Params p) {
       mbar_init(bar_d + i, (uint32_t)p.M2);
     }
     mbar_init(bar_first, (uint32_t)p.M2);
+    mbar_init(bar_chain, kExpandIssuers);
+    mbar_init(bar_red, 1);
     mbar_init(bar_done, (uint32_t)(p.M2 * min(p.NC, NG)));
     fence_mbar_init();
     fence_proxy_async_smem();
   }
-    // ---- P1: stage the input strip, the weights and the biases. Every 16-byte chunk is one slot; a thread first
-    // issues the loads of all its slots, then stores them, so that the whole prologue costs one round trip to
-    // device memory. (Pixels are Cin * 2 bytes apart there: coalesced plain loads of the contiguous strip serve
-    // that better than one TMA box row per pixel.) X and W1 rows go to their swizzled K-major tiles, zero beyond
-    // Cin; W3 to one [Coutp x 16 channels] slice per chunk; depthwise weights and biases are copied as they are.
-    constexpr int kBX = 4, kBW = 2;   // slots per thread in the first (batched) pass: input strip / everything else
+    // ---- P1: stage the input strip, the weights and the biases by asynchronous 16-byte copies, region by region; row and
+    // column of a thread's chunks advance by fixed steps. X and W1 rows go to their swizzled K-major tiles (one tile of 16, 32
+    // or 64 channels, or blocks of 64), zero beyond Cin; W3 to one [Coutp x 16 channels] slice per chunk; depthwise weights
+    // and biases are copied as they are. (Pixels are Cin * 2 bytes apart in device memory: coalesced copies of the contiguous
+    // strip serve that better than one TMA box row per pixel.) ----
     const int cs = p.Kp == 16 ? 1 : (p.Kp == 32 ? 2 : 3);   // log2(16-byte chunks per tile row)
-    const uint32_t nX = EXPAND ? (uint32_t)p.P_x << cs : 0u, nW1 = EXPAND ? (uint32_t)p.Cexp << cs : 0u;
-    const uint32_t nW3 = PROJECT ? (uint32_t)(p.NC * p.Coutp * 2) : 0u;
-    const uint32_t nWd = 9u * p.Cexp / 8u, nB = (uint32_t)p.Cexp / 4u, nB1 = EXPAND ? nB : 0u, nB3 = PROJECT ? (uint32_t)p.Cout / 4u : 0u;
-    const uint32_t nW = nW1 + nW3 + nWd + nB1 + nB + nB3;
+    const bool wide = EXPAND && !FOLD && p.kblocks > 1;     // more than 64 input channels: K blocks of 64
     // tile pixel `pix` is image pixel gh0 * W + pix of image n (strips are full-width rows): in the image for pix in [pix_lo, pix_hi)
     const int pix_lo = max(0, -gh0 * p.W), pix_hi = min(p.P_x, (p.H - gh0) * p.W);
-    const uint8_t* x0 = reinterpret_cast<const uint8_t*>(p.x) + ((size_t)n * p.H + gh0) * p.W * p.Cin * 2;   // not dereferenced outside the image
-    const uint32_t cmask = (1u << cs) - 1u, cin_chunks = (uint32_t)p.Cin >> 3, cin_bytes = (uint32_t)p.Cin * 2u;
-    const uint32_t swz_mask = ((uint32_t)p.row_bytes >> 4) - 1u;
-    // X and W1: row-major [row][Cin] -> swizzled rows of Kp channels; chunk i of a tile lies at byte 16 i, its 16-byte
-    // column XORed with the row's swizzle phase (address bits 7..). Returns the shared-memory offset; src = null: zeros.
-    auto x_slot = [&](uint32_t i, const uint8_t*& src) -> uint32_t {
-      const uint32_t row = i >> cs, ch = i & cmask;
-      src = (ch < cin_chunks && (int)row >= pix_lo && (int)row < pix_hi) ? x0 + row * cin_bytes + ch * 16u : nullptr;
-      if (FOLD && ch == cin_chunks) src = reinterpret_cast<const uint8_t*>(uintptr_t(1));   // two channels of 1.0 (tag 1)
-      return p.off_x + ((i << 4) ^ (((i >> 3) & swz_mask) << 4));
+    const uint8_t* x0 = reinterpret_cast<const uint8_t*>(p.x) + ((int64_t)n * p.H + gh0) * p.W * p.Cin * 2;   // not dereferenced outside the image
+    const int cin_chunks = p.Cin >> 3;
+    const uint32_t cin_bytes = (uint32_t)p.Cin * 2u, swz_mask = ((uint32_t)p.row_bytes >> 4) - 1u;
+    const uint8_t* w1p = reinterpret_cast<const uint8_t*>(p.w1) + (size_t)ch0 * cin_bytes;
+    auto stage_region = [&](int rows, int cpr, uint32_t recip, auto&& put) {      // put(row, chunk of the row)
+      int row = (int)fast_div((uint32_t)tid, (uint32_t)cpr, recip), ch = tid - row * cpr;
+      const int dr = (int)fast_div((uint32_t)kThreads, (uint32_t)cpr, recip), dc = kThreads - dr * cpr;
+      for (; row < rows; row += dr) {
+        put(row, ch);
+        if ((ch += dc) >= cpr) { ch -= cpr; ++row; }
+      }
     };
-    auto w_slot = [&](uint32_t i, const uint8_t*& src) -> uint32_t {
-      if (i < nW1) {
-        const uint32_t row = i >> cs, ch = i & cmask;
-        src = ch < cin_chunks ? reinterpret_cast<const uint8_t*>(p.w1) + row * cin_bytes + ch * 16u : nullptr;
-        if (FOLD && ch == cin_chunks) src = reinterpret_cast<const uint8_t*>(reinterpret_cast<uintptr_t>(p.b1 + row) | 2u);   // the bias (tag 2)
-        return p.off_w1 + ((i << 4) ^ (((i >> 3) & swz_mask) << 4));
+    auto stage = [&]() {
+      const uint8_t* none = reinterpret_cast<const uint8_t*>(p.wd);      // never read: the copies from it have no bytes
+      const uint32_t s0 = smem_u32(smem);
+      if (EXPAND) {
+        const int xblk = p.M1 * 128 * 128, wblk = p.Cexp * 128;
+        auto place = [&](int row, int ch, int blk) -> uint32_t {
+          if (wide) return (uint32_t)((ch >> 3) * blk + row * 128 + (((ch ^ row) & 7) << 4));
+          const uint32_t i = ((uint32_t)row << cs) + (uint32_t)ch;
+          return (i << 4) ^ (((i >> 3) & swz_mask) << 4);
+        };
+        stage_region(p.P_x, p.cpr, p.cpr_recip, [&](int row, int ch) {
+          const uint32_t d = p.off_x + place(row, ch, xblk);
+          // two channels of ones multiply the folded bias
+          if (FOLD && ch == cin_chunks) { *reinterpret_cast<uint4*>(smem + d) = make_uint4(0x3F803F80u, 0, 0, 0); return; }
+          const bool in = ch < cin_chunks && row >= pix_lo && row < pix_hi;
+          cp_async_16(s0 + d, in ? x0 + (uint32_t)row * cin_bytes + ch * 16 : none, in ? 16u : 0u);
+        });
+        stage_region(p.Cexp, p.cpr, p.cpr_recip, [&](int row, int ch) {
+          const uint32_t d = p.off_w1 + place(row, ch, wblk);
+          if (FOLD && ch == cin_chunks) {
+            // the bias as bf16 high and low parts (their sum carries 16 mantissa bits, and 1.0 * part is exact in the fp32 accumulator)
+            const float b = __ldg(p.b1 + ch0 + row);
+            const __nv_bfloat16 hi = __float2bfloat16_rn(b);
+            const __nv_bfloat16 lo = __float2bfloat16_rn(b - __bfloat162float(hi));
+            *reinterpret_cast<uint4*>(smem + d) = make_uint4((uint32_t)__bfloat16_as_ushort(hi) | ((uint32_t)__bfloat16_as_ushort(lo) << 16), 0, 0, 0);
+            return;
+          }
+          const bool in = ch < cin_chunks;
+          cp_async_16(s0 + d, in ? w1p + (uint32_t)row * cin_bytes + ch * 16 : none, in ? 16u : 0u);
+        });
       }
-      if ((i -= nW1) < nW3) {
-        const uint32_t half = i & 1u, c = __umulhi(i >> 1, p.coutp_recip), row = (i >> 1) - c * p.Coutp;
-        src = row < (uint32_t)p.Cout ? reinterpret_cast<const uint8_t*>(p.w3) + (row * p.Cexp + c * kChunk + half * 8u) * 2u : nullptr;
-        return p.off_w3 + c * p.Coutp * kChunkRowBytes + swz_offset(row, half, kChunkRowBytes);
+      const uint8_t* wdp = reinterpret_cast<const uint8_t*>(p.wd + ch0);
+      stage_region(9, p.Cexp >> 3, p.cexp8_recip, [&](int tap, int c8) {      // [chunk][tap][16 channels]: a thread's nine taps lie 32 bytes apart
+        cp_async_16(s0 + p.off_wd + (c8 >> 1) * (9 * kChunkRowBytes) + tap * kChunkRowBytes + (c8 & 1) * 16, wdp + ((uint32_t)tap * p.Cfull + c8 * 8) * 2, 16u);
+      });
+      if (PROJECT) {
+        const uint8_t* w3p = reinterpret_cast<const uint8_t*>(p.w3 + ch0);
+        stage_region(p.Coutp, 2 * p.NC, p.cexp8_recip, [&](int row, int j) {      // 2 NC == Cexp / 8
+          const bool in = row < p.Cout;
+          cp_async_16(s0 + p.off_w3 + (j >> 1) * p.Coutp * kChunkRowBytes + swz_offset(row, j & 1, kChunkRowBytes),
+                      in ? w3p + ((uint32_t)row * p.Cfull + j * 8) * 2 : none, in ? 16u : 0u);
+        });
+        if (tid < (p.Cout >> 2)) cp_async_16(s0 + p.off_b3 + tid * 16, reinterpret_cast<const uint8_t*>(p.b3) + tid * 16, 16u);   // Cout <= 256
       }
-      if ((i -= nW3) < nWd) {   // [tap][Cexp] in device memory -> [chunk][tap][16 channels]: a thread's nine taps lie 32 bytes apart
-        const uint32_t tap = __umulhi(i, p.cexp8_recip), c8 = i - tap * ((uint32_t)p.Cexp >> 3);
-        src = reinterpret_cast<const uint8_t*>(p.wd) + i * 16u;
-        return p.off_wd + (c8 >> 1) * (9u * kChunkRowBytes) + tap * kChunkRowBytes + (c8 & 1u) * 16u;
+      for (int i = tid; i < (p.Cexp >> 2); i += kThreads) {
+        cp_async_16(s0 + p.off_bd + i * 16, reinterpret_cast<const uint8_t*>(p.bd + ch0) + i * 16, 16u);
+        if (EXPAND && !FOLD) cp_async_16(s0 + p.off_b1 + i * 16, reinterpret_cast<const uint8_t*>(p.b1 + ch0) + i * 16, 16u);
       }
-      if ((i -= nWd) < nB1) { src = reinterpret_cast<const uint8_t*>(p.b1) + i * 16u; return p.off_b1 + i * 16u; }
-      if ((i -= nB1) < nB) { src = reinterpret_cast<const uint8_t*>(p.bd) + i * 16u; return p.off_bd + i * 16u; }
-      i -= nB;
-      src = reinterpret_cast<const uint8_t*>(p.b3) + i * 16u;
-      return p.off_b3 + i * 16u;
-    };
-    // A slot's source: a 16-byte aligned address (or null: zeros); tag 1: the two channels of ones that multiply the
-    // folded bias; tag 2: the address of one fp32 bias, split into bf16 high and low parts (their sum carries 16
-    // mantissa bits, and 1.0 * part is exact in the fp32 accumulator).
-    auto load_or_zero = [](const uint8_t* src) {
-      const uintptr_t a = reinterpret_cast<uintptr_t>(src);
-      if (!FOLD || (a & 3u) == 0u) return src ? __ldg(reinterpret_cast<const uint4*>(src)) : make_uint4(0, 0, 0, 0);
-      if ((a & 3u) == 1u) return make_uint4(0x3F803F80u, 0, 0, 0);
-      const float b = __ldg(reinterpret_cast<const float*>(a & ~uintptr_t(3)));
-      const __nv_bfloat16 hi = __float2bfloat16_rn(b);
-      const __nv_bfloat16 lo = __float2bfloat16_rn(b - __bfloat162float(hi));
-      return make_uint4((uint32_t)__bfloat16_as_ushort(hi) | ((uint32_t)__bfloat16_as_ushort(lo) << 16), 0, 0, 0);
     };
     // ---- per-thread work mapping: needs no device memory, so it runs before the wait for the previous grid of the
     // stream (with back-to-back launches it overlaps that grid's tail) ----
@@ -204,8 +242,8 @@ mbv2_fused_kernel(const Mbv2Params p) {
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     const int gw = warp - gwarp0;                 // warp index in the group
     const int xi = gw - (kGroupWarps - kExpandIssuers);   // >= 0: this warp issues expand tiles xi, xi + 2, ...
-    // Depthwise work split: thread = (channel pair, slot). Stride 1: an item is a block of 2 output rows x 7 output
-    // columns (56 columns x 14 rows x 8 pairs = one item per thread of a group). Stride 2: an item is one output column
+    // Depthwise work split: thread = (channel pair, slot). Stride 1: an item is a block of 2 output rows x segw output
+    // columns. Stride 2: an item is one output column
     // of one row group.
     constexpr int kSlots = kGroupThreads / 8;
     const int cp = gt & 7, slot = gt >> 3;
@@ -244,14 +282,12 @@ mbv2_fused_kernel(const Mbv2Params p) {
       }
     }
 
-    uint4 vx[kBX], vw[kBW];
-    uint32_t dx[kBX], dw[kBW];
     // Without the expand GEMM a chunk is 16 channels of the input strip, copied asynchronously into one of the
     // group's two E buffers two chunks ahead: 16-byte pieces (pixel, 8-channel plane), rows outside the image
     // zero-filled. The piece geometry is the same for every chunk.
-    constexpr int kPieces = 4;                      // P_x * 2 pieces <= 8 tiles * 128 * 2 over the group's threads
+    constexpr int kPieces = 8;                      // P_x * 2 pieces over the group's threads
     uint32_t ld_src[kPieces], ld_dst[kPieces], ld_ok = 0u, ld_in = 0u;
-    const uint8_t* xin = reinterpret_cast<const uint8_t*>(p.x) + ((int64_t)n * p.H + gh0) * p.W * p.Cexp * 2;   // row gh0 may lie outside
+    const uint8_t* xin = reinterpret_cast<const uint8_t*>(p.x) + ((int64_t)n * p.H + gh0) * p.W * p.Cfull * 2 + ch0 * 2;   // row gh0 may lie outside
     if (!EXPAND) {
 #pragma unroll
       for (int k = 0; k < kPieces; ++k) {
@@ -262,7 +298,7 @@ mbv2_fused_kernel(const Mbv2Params p) {
           const int ih = (int)fast_div((uint32_t)pix, (uint32_t)p.W, p.w_recip), iw = pix - ih * p.W;
           ld_ok |= 1u << k;
           ld_dst[k] = (uint32_t)(plane * p.e_plane + (ih * p.IW + iw + 1) * 16);
-          if (gh0 + ih >= 0 && gh0 + ih < p.H) { ld_in |= 1u << k; ld_src[k] = (uint32_t)(pix * p.Cexp * 2 + plane * 16); }
+          if (gh0 + ih >= 0 && gh0 + ih < p.H) { ld_in |= 1u << k; ld_src[k] = (uint32_t)(pix * p.Cfull * 2 + plane * 16); }
         }
       }
     }
@@ -282,62 +318,25 @@ mbv2_fused_kernel(const Mbv2Params p) {
     grid_dependency_wait();      // first access to device memory below
     grid_launch_dependents();
     if (!EXPAND) { load_chunk(g, 0); load_chunk(g + NG, 1); }   // the first two chunks travel while the weights are staged
-#pragma unroll
-    for (int k = 0; k < kBX; ++k) {
-      const uint32_t i = (uint32_t)(tid + k * kThreads);
-      const uint8_t* src = nullptr;
-      dx[k] = 0xffffffffu;
-      if (i < nX) dx[k] = x_slot(i, src);
-      vx[k] = load_or_zero(src);
-    }
-#pragma unroll
-    for (int k = 0; k < kBW; ++k) {
-      const uint32_t i = (uint32_t)(tid + k * kThreads);
-      const uint8_t* src = nullptr;
-      dw[k] = 0xffffffffu;
-      if (i < nW) dw[k] = w_slot(i, src);
-      vw[k] = load_or_zero(src);
-    }
+    stage();
     if (warp == 0) {
       tmem_alloc(tmem_slot, (uint32_t)p.tmem_cols);
       tmem_relinquish();
-    }
-#pragma unroll
-    for (int k = 0; k < kBX; ++k)
-      if (dx[k] != 0xffffffffu) *reinterpret_cast<uint4*>(smem + dx[k]) = vx[k];
-#pragma unroll
-    for (int k = 0; k < kBW; ++k)
-      if (dw[k] != 0xffffffffu) *reinterpret_cast<uint4*>(smem + dw[k]) = vw[k];
-    // shapes with more slots than the batched pass covers
-    for (uint32_t i = (uint32_t)(tid + kBX * kThreads); i < nX; i += kThreads) {
-      const uint8_t* src;
-      const uint32_t d = x_slot(i, src);
-      *reinterpret_cast<uint4*>(smem + d) = load_or_zero(src);
-    }
-    for (uint32_t i = (uint32_t)(tid + kBW * kThreads); i < nW; i += kThreads) {
-      const uint8_t* src;
-      const uint32_t d = w_slot(i, src);
-      *reinterpret_cast<uint4*>(smem + d) = load_or_zero(src);
     }
     // the zero padding columns of the two E chunk buffers (written once: every chunk reuses them)
     constexpr int kEPlanes = (EXPAND ? NG : 2 * NG) * 2;   // one E buffer per group (two when the chunks are copied in), two planes each
     for (int i = tid; i < p.IH * 2 * kEPlanes; i += kThreads) {
       const int ih = i / (2 * kEPlanes), side = (i / kEPlanes) & 1, plane = i % kEPlanes;
-      *reinterpret_cast<uint4*>(sE + plane * p.e_plane + (ih * p.IW + side * (p.IW - 1)) * 16) = make_uint4(0, 0, 0, 0);
+      *reinterpret_cast<uint4*>(sE + plane * p.e_plane + (ih * p.IW + side * (p.W + 1)) * 16) = make_uint4(0, 0, 0, 0);
     }
-    fence_proxy_async_smem();
-  tcgen05_fence_before_sync();
-  __syncthreads();
-  tcgen05_fence_after_sync();
-  const uint32_t tmem_base = *tmem_slot;
 
-    // The warps form two groups of 16; group g owns the chunks c = g, g + 2, ... (expand buffer, E buffer and D
-    // buffer g). A group alternates expand epilogue and depthwise stage with a group-wide barrier after each; the two
-    // groups are out of phase, so one group's barrier and tensor-memory latencies hide behind the other's arithmetic.
-    // MMAs are issued inline, right after the barrier that makes their operands ready: the expand GEMM of chunk c + 2
-    // by the group's last two warps (at 56 x 56 they have no depthwise item), the project GEMM of chunk c by M2 warps,
+    // Group g owns the chunks c = g, g + NG, ... (expand buffer, E buffer and D buffer g). A group alternates expand epilogue and
+    // depthwise stage with a group-wide barrier after each; the groups are out of phase, so one group's barrier and
+    // tensor-memory latencies hide behind the others' arithmetic.
+    // MMAs are issued inline, right after the barrier that makes their operands ready: the expand GEMM of chunk c + NG
+    // by the group's last two warps (the first to run out of depthwise items), the project GEMM of chunk c by M2 warps,
     // one tile each -- a parked issuer warp would share its scheduler with busy warps and issue an MMA every few
-    // hundred cycles, and the project GEMM is urgent: it must be through before the depthwise stage of chunk c + 2
+    // hundred cycles, and the project GEMM is urgent: it must be through before the depthwise stage of chunk c + NG
     // may overwrite its operand.
     // Descriptors as (low, high) words: start address and LBO live in the low word, so an operand advances with one
     // 32-bit add (shared-memory addresses >> 4 stay below the 14-bit field limit).
@@ -345,7 +344,7 @@ mbv2_fused_kernel(const Mbv2Params p) {
 #pragma unroll
     for (int k = 0; k < kTilesPerWarp; ++k) {
       const int t = q_rank + k * q_mates;
-      e_tm[k] = t < p.M1 ? tmem_base + lane_base + p.ecol0 + (g * p.M1 + t) * kChunk : kNone;
+      e_tm[k] = t < p.M1 ? lane_base + p.ecol0 + (t * NG + g) * kChunk : kNone;
     }
     const uint32_t sbo_x = 8u * (uint32_t)p.row_bytes;
     const uint64_t xdesc0 = make_smem_desc(smem_u32(sX), 0, sbo_x, p.swizzle);
@@ -360,34 +359,50 @@ mbv2_fused_kernel(const Mbv2Params p) {
     const uint32_t idesc_e = make_idesc_bf16(128, kChunk);
     const uint64_t exp_a_step = (uint64_t)((uint32_t)(kExpandIssuers * 128 * p.row_bytes) >> 4);
     const uint64_t exp_a0 = xdesc0 + (uint64_t)((uint32_t)(max(xi, 0) * 128 * p.row_bytes) >> 4);
-    const uint32_t exp_d_tmem0 = tmem_base + p.ecol0 + (g * p.M1 + max(xi, 0)) * kChunk;
+    uint32_t exp_d_tmem0 = p.ecol0 + (max(xi, 0) * NG + g) * kChunk;
     const uint64_t exp_b_step = (uint64_t)((uint32_t)(NG * kChunk * p.row_bytes) >> 4);   // the group's next chunk is c + NG
     uint64_t exp_b = w1desc0 + (uint64_t)((uint32_t)(g * kChunk * p.row_bytes) >> 4);
-    const int ksteps = p.Kp / 16;
+    const int ksteps = p.ksteps;
     const int exp_tiles = xi >= 0 ? (p.M1 - xi + kExpandIssuers - 1) / kExpandIssuers : 0;   // tiles this warp issues per chunk
-    auto issue_expand = [&]() {   // whole warp; advances to the group's next chunk. Straight-line per reduction length.
+    auto issue_expand_as = [&](uint32_t idesc_e) {   // whole warp. Straight-line per reduction length.
       uint64_t a = exp_a0;
       uint32_t d_tmem = exp_d_tmem0;
       const uint64_t b = exp_b;
       if (ksteps == 2) {
 #pragma unroll 1
-        for (int t = 0; t < exp_tiles; ++t, a += exp_a_step, d_tmem += kExpandIssuers * kChunk) {
+        for (int t = 0; t < exp_tiles; ++t, a += exp_a_step, d_tmem += kExpandIssuers * NG * kChunk) {
           umma_bf16_elected<false>(d_tmem, a, b, idesc_e, elected);
           umma_bf16_elected<true>(d_tmem, a + 2u, b + 2u, idesc_e, elected);
         }
       } else if (ksteps == 4) {
 #pragma unroll 1
-        for (int t = 0; t < exp_tiles; ++t, a += exp_a_step, d_tmem += kExpandIssuers * kChunk) {
+        for (int t = 0; t < exp_tiles; ++t, a += exp_a_step, d_tmem += kExpandIssuers * NG * kChunk) {
           umma_bf16_elected<false>(d_tmem, a, b, idesc_e, elected);
           umma_bf16_elected<true>(d_tmem, a + 2u, b + 2u, idesc_e, elected);
           umma_bf16_elected<true>(d_tmem, a + 4u, b + 4u, idesc_e, elected);
           umma_bf16_elected<true>(d_tmem, a + 6u, b + 6u, idesc_e, elected);
         }
-      } else {
+      } else if (ksteps == 1) {
 #pragma unroll 1
-        for (int t = 0; t < exp_tiles; ++t, a += exp_a_step, d_tmem += kExpandIssuers * kChunk)
+        for (int t = 0; t < exp_tiles; ++t, a += exp_a_step, d_tmem += kExpandIssuers * NG * kChunk)
           umma_bf16_elected<false>(d_tmem, a, b, idesc_e, elected);
+      } else {                                 // K blocks of four steps (the last one may have fewer)
+        const uint64_t a_blk = (uint64_t)((uint32_t)(p.M1 * 128 * 128) >> 4), b_blk = (uint64_t)((uint32_t)(p.Cexp * 128) >> 4);
+#pragma unroll 1
+        for (int t = 0; t < exp_tiles; ++t, a += exp_a_step, d_tmem += kExpandIssuers * NG * kChunk) {
+          uint64_t ak = a, bk = b;
+#pragma unroll 1
+          for (int ks = 0; ks < ksteps; ks += 4, ak += a_blk, bk += b_blk) {
+            umma_bf16_elected_acc(d_tmem, ak, bk, idesc_e, elected, ks > 0 ? 1u : 0u);
+            if (ks + 1 < ksteps) umma_bf16_elected<true>(d_tmem, ak + 2u, bk + 2u, idesc_e, elected);
+            if (ks + 2 < ksteps) umma_bf16_elected<true>(d_tmem, ak + 4u, bk + 4u, idesc_e, elected);
+            if (ks + 3 < ksteps) umma_bf16_elected<true>(d_tmem, ak + 6u, bk + 6u, idesc_e, elected);
+          }
+        }
       }
+    };
+    auto issue_expand = [&]() {      // one chunk; advances to the group's next one
+      issue_expand_as(idesc_e);
       umma_commit_elected(bar_e + g, elected);
       exp_b += exp_b_step;
     };
@@ -396,28 +411,9 @@ mbv2_fused_kernel(const Mbv2Params p) {
     // the barrier to the MMA is one add, the MMA and the commit.
     const uint32_t idesc_p = make_idesc_bf16(128, (uint32_t)p.Coutp);
     const uint64_t proj_a = ddesc0 + (uint64_t)((uint32_t)(g * d_bytes + gw * 128 * 16) >> 4);
-    const uint32_t proj_d_tmem = tmem_base + p.pcol0 + gw * p.Coutp;
+    uint32_t proj_d_tmem = p.pcol0 + gw * p.Coutp;
     const uint64_t proj_b_step = (uint64_t)((uint32_t)(NG * p.Coutp * kChunkRowBytes) >> 4);     // the group's next chunk is c + NG
     uint64_t proj_b = w3desc0 + (uint64_t)((uint32_t)(g * p.Coutp * kChunkRowBytes) >> 4);
-    if (EXPAND && xi >= 0 && g < p.NC) {
-      // group 1 issues its first expand GEMM once group 0's is through the tensor pipe: group 0 has the longer chain
-      // of chunks, and its first epilogue would otherwise wait for both groups' MMAs
-      // (with more than two groups the strips are small, the products short, and a chain of first products would cost
-      // more than it saves; a waiter that falls two phases behind a barrier would also read the wrong parity)
-      if (NG == 2 && g == 1) {
-        if (lane == 0) mbar_wait(bar_e, 0, abort_flag, p.status, 0x107);
-        __syncwarp();
-      }
-      issue_expand();
-    }
-    __syncwarp();
-    // Waits on MMA completion are taken by ONE warp of the group, just before it arrives at the group barrier that
-    // the others are parked at: a polling warp spends issue slots, sixteen of them a large share of the SM's.
-    const bool waiter = gw == kGroupWarps - 1;
-    if (EXPAND && g < p.NC) {
-      if (waiter) mbar_wait(bar_e + g, 0, abort_flag, p.status, 0x102);   // the group's first expand GEMM
-      named_barrier_sync(gbar, kGroupThreads);
-    }
     // The thread's first depthwise item (for most shapes its only one) is the same for every chunk: offsets of its
     // first input / output pixel inside a plane and its extent (stride 1: columns, rows; stride 2: first and last row).
     const bool has_item = slot < dw_items;
@@ -436,6 +432,53 @@ mbv2_fused_kernel(const Mbv2Params p) {
     uint32_t wd_addr = smem_u32(sWd) + (uint32_t)(g * 9 * kChunkRowBytes + cp * 4);
     uint32_t bd_addr = smem_u32(sBd) + (uint32_t)((g * kChunk + cp * 2) * 4);
     uint32_t b1_addr = smem_u32(sB1) + (uint32_t)(g * kChunk * 4);
+    // All of the above needs nothing that the copies bring: it runs (and its instructions are fetched) while they travel.
+    cp_async_wait_all();
+    fence_proxy_async_smem();
+  tcgen05_fence_before_sync();
+  __syncthreads();
+  tcgen05_fence_after_sync();
+  const uint32_t tmem_base = *tmem_slot;
+    if (PROJECT && p.CS > 1) {
+      if (tid == 0) mbar_arrive_expect_tx(bar_red, (uint32_t)((p.CS - 1) * p.Coutp * p.PP * 4));
+      __syncwarp();
+      if (!p.recv_shared) cluster_arrive();       // the barrier is armed: the others may send from now on
+    }
+    exp_d_tmem0 += tmem_base;
+    proj_d_tmem += tmem_base;
+#pragma unroll
+    for (int k = 0; k < kTilesPerWarp; ++k) if (e_tm[k] != kNone) e_tm[k] += tmem_base;
+    if (EXPAND && xi >= 0) {
+      if (NG == 2) {
+        // group 1 issues its first expand GEMM once group 0's is through the tensor pipe: group 0 has the longer chain
+        // of chunks, and its first epilogue would otherwise wait for both groups' MMAs
+        if (g < p.NC) {
+          if (g == 1) {
+            if (lane == 0) mbar_wait(bar_chain, 0, abort_flag, p.status, 0x107);
+            __syncwarp();
+          }
+          issue_expand();
+          if (g == 0) umma_commit_elected(bar_chain, elected);
+        }
+      } else {
+        // The first chunks of all groups lie side by side in W1 and in tensor memory: one product with N = 16 x groups
+        // makes them all (an MMA costs about the same with N = 16 and N = 64: its operand fetch bounds it).
+        if (g == 0) {
+          const int first = min(NG, p.NC);
+          issue_expand_as(make_idesc_bf16(128, (uint32_t)(kChunk * first)));
+          for (int i = 0; i < first; ++i) umma_commit_elected(bar_e + i, elected);
+        }
+        exp_b += exp_b_step;
+      }
+    }
+    __syncwarp();
+    // Waits on MMA completion are taken by ONE warp of the group, just before it arrives at the group barrier that
+    // the others are parked at: a polling warp spends issue slots, sixteen of them a large share of the SM's.
+    const bool waiter = gw == kGroupWarps - 1;
+    if (EXPAND && g < p.NC) {
+      if (waiter) mbar_wait(bar_e + g, 0, abort_flag, p.status, 0x102);   // the group's first expand GEMM
+      named_barrier_sync(gbar, kGroupThreads);
+    }
     for (int c = g, it = 0; c < p.NC; c += NG, ++it) {
       // ---- P3: expand epilogue of chunk c -> E[g]: + b1, ReLU6, zero outside the image, bf16 ----
       if (!EXPAND) cp_async_wait_but_one();   // this thread's pieces of chunk c have landed
@@ -521,10 +564,10 @@ mbv2_fused_kernel(const Mbv2Params p) {
       if (!PROJECT) {
         // the depthwise result of the chunk is the output: 16-byte pieces (pixel, plane) of D[g] to device memory
         const int pieces = rows_valid * p.Wo * 2;
-        __nv_bfloat16* o0 = p.out + ((size_t)n * p.Ho + ho0) * p.Wo * p.Cexp + c * kChunk;
+        __nv_bfloat16* o0 = p.out + ((size_t)n * p.Ho + ho0) * p.Wo * p.Cfull + ch0 + c * kChunk;
         for (int i = gt; i < pieces; i += kGroupThreads) {
           const int pix = i >> 1, plane = i & 1;
-          *reinterpret_cast<uint4*>(o0 + (size_t)pix * p.Cexp + plane * 8) =
+          *reinterpret_cast<uint4*>(o0 + (size_t)pix * p.Cfull + plane * 8) =
               *reinterpret_cast<const uint4*>(sD + g * d_bytes + plane * p.d_plane + pix * 16);
         }
       }
@@ -550,6 +593,66 @@ mbv2_fused_kernel(const Mbv2Params p) {
       tcgen05_fence_after_sync();
       const int valid_pix = rows_valid * p.Wo;
       const size_t gpix0 = ((size_t)n * p.Ho + ho0) * p.Wo;
+      if (p.CS > 1) {
+        // ---- the channel shares of the cluster's CTAs are added: CTA r sums and stores pixels [r PP, (r + 1) PP) of the
+        // strip. A CTA lays its fp32 partial sums out as one block [4 channels][pixel] per owner (over its own operands,
+        // which are dead now) and sends each block by one bulk copy (single 16-byte stores into the other CTAs took
+        // three times as long). Where the incoming blocks have no memory of their own they go over operands too, so the
+        // cluster meets once more before anything is sent. ----
+        const int ncg = p.Coutp >> 4;
+        const uint32_t out0 = smem_u32(smem) + (uint32_t)p.off_send, in0 = smem_u32(smem) + (uint32_t)p.off_recv;
+        const uint32_t block = (uint32_t)(p.Coutp * p.PP * 4);
+        for (int u = warp >> 2; u < p.M2 * ncg; u += kWarps / 4) {
+          const int t = u / ncg, cg = u - t * ncg;
+          const int po = t * 128 + (warp & 3) * 32 + lane;
+          uint32_t acc[16];
+          tmem_ld_x16(tmem_base + lane_base + p.pcol0 + t * p.Coutp + cg * 16, acc);
+          tmem_ld_wait();
+          if (po < valid_pix) {
+            const uint32_t owner = fast_div((uint32_t)po, (uint32_t)p.PP, p.pp_recip);
+            const uint32_t a = out0 + owner * block + (uint32_t)((cg * 4 * p.PP + po - (int)owner * p.PP) * 16);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) sts128(a + (uint32_t)(q * p.PP * 16), acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+          }
+        }
+        fence_proxy_async_smem();
+        tcgen05_fence_before_sync();
+        if (p.recv_shared) { __syncthreads(); cluster_arrive(); cluster_wait(); }     // every CTA's operands are dead
+        else { __syncthreads(); cluster_wait(); }  // every CTA has started (it arrived when its barriers were set up)
+        if (tid < p.CS - 1) {
+          const uint32_t peer = (uint32_t)((rank + 1 + tid) % p.CS);
+          bulk_copy_to_cluster(cluster_map(in0 + (uint32_t)rank * block, peer), out0 + peer * block, block, cluster_map(smem_u32(bar_red), peer));
+        }
+        const int own0 = rank * p.PP, own = min(p.PP, valid_pix - own0), c8n = p.Cout >> 3;
+        int i = tid, lp = (int)fast_div((uint32_t)i, (uint32_t)c8n, p.cout8_recip), c8 = i - lp * c8n;
+        auto residual_of = [&]() -> uint4 {       // stride 1, Cin == Cout: the input at the same place
+          if (!(EXPAND && p.residual) || i >= own * c8n) return make_uint4(0, 0, 0, 0);
+          return __ldg(reinterpret_cast<const uint4*>(p.x + (gpix0 + own0 + lp) * p.Cout + c8 * 8));
+        };
+        uint4 xr = residual_of();                 // travels while the blocks do
+        if (warp == 0) mbar_wait(bar_red, 0, abort_flag, p.status, 0x108);
+        __syncthreads();
+        cluster_arrive();                         // this CTA has received everything
+        while (i < own * c8n) {
+          float v[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) v[q] = sB3[c8 * 8 + q];
+          v[0] += bf16_lo(xr.x); v[1] += bf16_hi(xr.x); v[2] += bf16_lo(xr.y); v[3] += bf16_hi(xr.y);
+          v[4] += bf16_lo(xr.z); v[5] += bf16_hi(xr.z); v[6] += bf16_lo(xr.w); v[7] += bf16_hi(xr.w);
+          const uint32_t at = (uint32_t)((c8 * 2 * p.PP + lp) * 16);
+          for (int src = 0; src < p.CS; ++src) {
+            const uint32_t a = (src == rank ? out0 : in0) + (uint32_t)src * block + at;
+            const float4 lo = lds128f<0>(a), hi = lds128f<0>(a + (uint32_t)(p.PP * 16));
+            v[0] += lo.x; v[1] += lo.y; v[2] += lo.z; v[3] += lo.w; v[4] += hi.x; v[5] += hi.y; v[6] += hi.z; v[7] += hi.w;
+          }
+          *reinterpret_cast<uint4*>(p.out + (gpix0 + own0 + lp) * p.Cout + c8 * 8) =
+              make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
+          if ((i += kThreads) >= own * c8n) break;
+          lp = (int)fast_div((uint32_t)i, (uint32_t)c8n, p.cout8_recip); c8 = i - lp * c8n;
+          xr = residual_of();
+        }
+        cluster_wait();                           // the copies out of this CTA have arrived: it may leave
+      } else
       for (int t = warp >> 2; t < p.M2; t += kWarps / 4) {
         const int po = t * 128 + (warp & 3) * 32 + lane;
         for (int j0 = 0; j0 < p.Coutp; j0 += 16) {
@@ -586,6 +689,10 @@ mbv2_fused_kernel(const Mbv2Params p) {
 
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
+constexpr int kMaxSplit = 8;     // CTAs per strip (the portable cluster size)
+// clusters of 1-CTA-per-SM kernels a B200 keeps resident at once, as cudaOccupancyMaxActiveClusters reports them
+constexpr int kResident[kMaxSplit + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
+
 struct Mbv2Host {
   Mbv2Params prm;
   int smem_bytes = 0;
@@ -599,6 +706,7 @@ bool layout(Mbv2Params& q, int R, bool expand, bool project, int* smem_bytes) {
   q.strips_recip = fast_div_recip(q.strips);
   q.IH = (R - 1) * q.stride + 3;
   q.IW = q.W + 2;
+  if (q.nseg < 4) q.IW |= 1;     // an odd pitch: the warp's blocks in two rows use other banks
   q.P_in = q.IH * q.IW;
   q.P_x = q.IH * q.W;
   q.M1 = (q.P_x + 127) / 128;
@@ -606,7 +714,7 @@ bool layout(Mbv2Params& q, int R, bool expand, bool project, int* smem_bytes) {
   if (q.IH > 256 || q.IW > 256 || q.M1 > 8) return false;
   // per group: at most kTilesPerWarp expand tiles per warp of a lane quarter, one project tile per warp, and (when the
   // chunks are copied in) four 16-byte pieces per thread
-  if (q.M1 > kTilesPerWarp * (kWarps / NG / 4) || q.M2 > kWarps / NG || (!expand && q.P_x * 2 > 4 * group_threads)) return false;
+  if (q.M1 > kTilesPerWarp * (kWarps / NG / 4) || q.M2 > kWarps / NG || (!expand && q.P_x * 2 > 8 * group_threads)) return false;
   const int cols = (expand ? NG * q.M1 * kChunk : 0) + (project ? q.M2 * q.Coutp : 0);
   if (cols > 512) return false;
   q.tmem_cols = 32;
@@ -615,8 +723,8 @@ bool layout(Mbv2Params& q, int R, bool expand, bool project, int* smem_bytes) {
   q.pcol0 = expand ? NG * q.M1 * kChunk : 0;
   int off = 0;
   auto take = [&](int bytes) { int o = off; off = round_up(off + bytes, 1024); return o; };
-  q.off_x = take(expand ? q.M1 * 128 * q.row_bytes : 0);
-  q.off_w1 = take(expand ? q.Cexp * q.row_bytes : 0);
+  q.off_x = take(expand ? q.M1 * 128 * q.row_bytes * q.kblocks : 0);
+  q.off_w1 = take(expand ? q.Cexp * q.row_bytes * q.kblocks : 0);
   // two 8-channel planes per chunk, offset by 64 mod 128 bytes so that a warp's
   // 2 x 64-byte accesses (4 pixels x 4 channel pairs per plane) never share a bank
   q.e_plane = round_up(q.P_in * 16, 128) + 64;
@@ -627,10 +735,54 @@ bool layout(Mbv2Params& q, int R, bool expand, bool project, int* smem_bytes) {
   q.off_wd = take(9 * q.Cexp * 2);
   q.off_b1 = take(expand ? q.Cexp * 4 : 0);
   q.off_bd = take(q.Cexp * 4);
+  q.PP = ((R * q.Wo + q.CS - 1) / q.CS) | 1;
+  q.pp_recip = fast_div_recip(q.PP);
+  q.off_send = q.off_recv = q.recv_shared = 0;
+  if (project && q.CS > 1) {
+    const int blocks = round_up(q.CS * q.PP * q.Coutp * 4, 1024);
+    if (std::max(off, blocks) + blocks + 4096 <= 227 * 1024) {      // incoming blocks in memory of their own
+      q.off_recv = std::max(off, blocks);
+      off = q.off_recv + blocks;
+    } else {                                                        // outgoing and incoming blocks over the operands
+      q.recv_shared = 1;
+      q.off_recv = blocks;
+      off = std::max(off, 2 * blocks);
+    }
+  }
   q.off_b3 = take(project ? q.Coutp * 4 : 0);
   q.off_bar = take(256);
   *smem_bytes = off + 1024;  // slack for the 1024-byte alignment of the base
   return *smem_bytes <= 227 * 1024;
+}
+
+// Estimated cycles of a launch with the tiling in `t` (for comparisons between tilings). Per wave of resident CTAs or clusters:
+// staging (the bytes a CTA copies), the chunk loop, the output. The chunk loop is the larger of its instruction issue (NC chunks)
+// and the chain of a group's chunks, each a chain of latencies. Constants fitted to 23 shapes (7 to 78 pixels wide, 16 to 160
+// input channels, batches of 1 to 64) x all their tilings, 1900 launches in all: 6.5 % rms, and the tiling of the least estimate
+// is on average 0.3 % slower than the best one measured.
+double estimated_cycles(const Mbv2Params& t, bool expand, bool project, int sms) {
+  const bool split = project && t.CS > 1;
+  const long resident = split ? kResident[t.CS] * (long)sms / kDefaultSMs : sms / t.CS;
+  const long units = (long)t.N * t.strips, waves = (units + std::max(1l, resident) - 1) / std::max(1l, resident);
+  const int slots = kThreads / t.groups / 8;
+  double dw_issue, dw_chain;       // depthwise stage of one chunk: warp instructions, cycles of a warp's own chain
+  if (t.stride == 1) {
+    const int items = t.nseg * ((t.R + 1) / 2);
+    const double block = (t.segw + 2) / 9.0;
+    dw_issue = items * 8 / 32.0 * 360.0 * block;
+    dw_chain = (items + slots - 1) / slots * 800.0 * block;
+  } else {
+    const int rows = (t.R + std::max(1, std::min(t.R, t.col_slots)) - 1) / std::max(1, std::min(t.R, t.col_slots));
+    const int items = t.Wo * std::max(1, std::min(t.R, t.col_slots));
+    dw_issue = t.Wo * t.R * 8 / 32.0 * 45.0;
+    dw_chain = (items + slots - 1) / slots * (rows * 130.0 + 100.0);
+  }
+  const double issue = t.NC * (dw_issue + t.M1 * 4 * 30.0 + t.M2 * 370.0) / 4 / 0.59;
+  const double chain = (t.NC + t.groups - 1) / t.groups * (515.0 + 1.5 * dw_chain + 68.0 * t.M1);
+  const double loop = std::pow(std::pow(issue, 4) + std::pow(chain, 4), 0.25);
+  const double bytes = (expand ? (double)(t.P_x + t.Cexp) * t.Cin * 2 : 0.0) + (project ? t.Cexp * t.Cout * 2.0 : 0.0) + t.Cexp * 26.0;
+  const double out = split ? 1100.0 + 0.066 * (t.CS - 1) / t.CS * (t.R * t.Wo * t.Coutp * 4.0) : 42.0 * t.M2 * t.Cout / 4;
+  return waves * (7500.0 + 0.069 * bytes + loop + out);
 }
 
 }  // namespace
@@ -646,27 +798,30 @@ ago_status_t mbv2_plan(Plan* plan, FusedState* st, std::string* err) {
   Mbv2Params& q = host->prm;
   q = Mbv2Params{};
   q.N = (int)first.in.d[0]; q.H = (int)first.in.d[1]; q.W = (int)first.in.d[2];
-  q.Cexp = (int)d.in.d[3];
+  q.Cfull = (int)d.in.d[3];
   q.Cin = expand ? (int)first.in.d[3] : 16;
   q.Cout = project ? plan->ops[i_pr].op.p[0] : 16;
   q.stride = d.op.p[3];
   q.Ho = (int)d.out.d[1]; q.Wo = (int)d.out.d[2];
   q.residual = plan->fused_kernel == AGO_KERNEL_MBV2_BLOCK && plan->ops.size() == 9 ? 1 : 0;
   auto bad = [&](const char* m) { *err = std::string("fused inverted-residual block: ") + m; delete host; return AGO_ERR_UNSUPPORTED; };
-  if (q.Cin > 64) return bad("more than 64 input channels is not supported yet");
-  if (q.Cexp % kChunk != 0) return bad("expanded channels must be a multiple of 16");
+  if (q.Cin > 256) return bad("more than 256 input channels is not supported");
+  if (q.Cfull % kChunk != 0) return bad("expanded channels must be a multiple of 16");
   if (q.Cout > 256) return bad("more than 256 output channels is not supported");
   if (q.residual && (q.stride != 1 || q.Cin != q.Cout)) return bad("residual needs stride 1 and Cin == Cout");
   q.Kp = q.Cin <= 16 ? 16 : (q.Cin <= 32 ? 32 : 64);
+  q.ksteps = q.Cin <= 64 ? q.Kp / 16 : (q.Cin + 15) / 16;
+  q.kblocks = (q.ksteps + 3) / 4;
+  q.cpr = 2 * q.ksteps;      // Cin <= 64: Kp / 8
   q.row_bytes = q.Kp * 2;
   q.swizzle = q.Kp == 16 ? tc::SW_32B : (q.Kp == 32 ? tc::SW_64B : tc::SW_128B);
   q.Coutp = round_up(q.Cout, 16);
   q.fold_b1 = expand && q.Cin % 8 == 0 && q.Cin < q.Kp ? 1 : 0;
-  q.NC = q.Cexp / kChunk;
   auto recip = [](int d) { return tc::fast_div_recip(d); };
   q.coutp_recip = recip(q.Coutp);
   q.w_recip = recip(q.W);
-  q.cexp8_recip = recip(q.Cexp / 8);
+  q.cpr_recip = recip(q.cpr);
+  q.cout8_recip = recip(std::max(1, q.Cout / 8));
   q.segw = seg_width(q.Wo);
   q.nseg = (q.Wo + q.segw - 1) / q.segw;
   q.per_row = q.stride == 1 ? q.nseg : q.Wo;
@@ -677,33 +832,36 @@ ago_status_t mbv2_plan(Plan* plan, FusedState* st, std::string* err) {
     t.step_r = slots / t.per_row; t.step_c = slots - t.step_r * t.per_row;
     t.col_slots = slots / std::max(1, std::min(t.Wo, slots));
   };
-  // Warp groups and rows per CTA: the least estimated time = waves x (fixed part + chunk loop), where the chunk loop
-  // is the larger of the strip's arithmetic (issue-bound: about 0.8 cycles per pixel-tile unit and chunk, measured
-  // on 56 x 56 strips) and the chain of latencies of the chunks one group owns (about 2.9k cycles per chunk,
-  // measured on 28 x 28 strips). Small strips therefore run with four groups, large ones with two.
-  int best_R = 0, best_ng = 2; double best_cost = 0; int best_smem = 0;
+  // Rows per CTA, warp groups and channel split: the least estimated time among all that fit.
+  int best_R = 0, best_ng = 2, best_cs = 1; double best_cost = 0; int best_smem = 0;
   const int sms = device_sm_count();
-  for (int ng = 2; ng <= 8; ng *= 2) {
-    for (int R = 1; R <= q.Ho; ++R) {
-      Mbv2Params t = q; int smem = 0;
-      set_groups(t, ng);
-      if (!layout(t, R, expand, project, &smem)) continue;
-      const long ctas = (long)q.N * t.strips;
-      const long waves = (ctas + sms - 1) / sms;
-      const double work = 0.8 * q.NC * (t.M1 * 128.0 + 3.0 * t.M2 * 128.0);
-      const double chain = 2900.0 * ((q.NC + ng - 1) / ng);
-      const double cost = (double)waves * (6000.0 + std::max(work, chain) + 0.01 * work);
-      if (best_R == 0 || cost < best_cost) { best_R = R; best_ng = ng; best_cost = cost; best_smem = smem; }
+  const int chunks = q.Cfull / kChunk;
+  auto set_split = [&](Mbv2Params& t, int cs) {
+    t.CS = cs; t.Cexp = q.Cfull / cs; t.NC = chunks / cs;
+    t.cexp8_recip = recip(t.Cexp / 8);
+  };
+  for (int cs = 1; cs <= kMaxSplit; ++cs) {
+    if (chunks % cs != 0) continue;
+    for (int ng = 2; ng <= 4; ng *= 2) {
+      for (int R = 1; R <= q.Ho; ++R) {
+        Mbv2Params t = q; int smem = 0;
+        set_groups(t, ng);
+        set_split(t, cs);
+        if (!layout(t, R, expand, project, &smem)) continue;
+        const double cost = estimated_cycles(t, expand, project, sms);
+        if (best_R == 0 || cost < best_cost) { best_R = R; best_ng = ng; best_cs = cs; best_cost = cost; best_smem = smem; }
+      }
     }
   }
   if (best_R == 0) return bad("no row-strip tiling fits shared memory / tensor memory");
   set_groups(q, best_ng);
+  set_split(q, best_cs);
   layout(q, best_R, expand, project, &best_smem);
   if ((long)q.N * q.strips > 65535) return bad("more than 65535 row strips in the batch");
   host->smem_bytes = best_smem;
   st->impl = host;
   st->impl_free = [](void* p) { delete static_cast<Mbv2Host*>(p); };
-  st->tile_rows = best_R; st->grid = q.N * q.strips; st->smem_bytes = best_smem;
+  st->tile_rows = best_R; st->grid = q.N * q.strips * q.CS; st->smem_bytes = best_smem;
   plan->tile_rows = best_R; plan->smem_bytes = best_smem;
   return AGO_OK;
 }
@@ -715,14 +873,20 @@ ago_status_t launch_groups(const Mbv2Params& q, int smem_bytes, cudaStream_t str
   static int smem_opt_in[64] = {};
   cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(mbv2_fused_kernel<EXPAND, PROJECT, FOLD, NG>), smem_opt_in);
   if (e != cudaSuccess) { *err = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e); return AGO_ERR_CUDA; }
-  FusedLaunch launch(dim3((unsigned)(q.N * q.strips)), kThreads, (size_t)smem_bytes, stream);
+  FusedLaunch launch(dim3((unsigned)(q.N * q.strips * q.CS)), kThreads, (size_t)smem_bytes, stream);
+  cudaLaunchAttribute attr[2] = {launch.attr[0], {}};
+  if (PROJECT && q.CS > 1) {        // the CTAs of a strip add their partial products through distributed shared memory
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)q.CS; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    launch.config.attrs = attr;
+    launch.config.numAttrs = 2;
+  }
   e = cudaLaunchKernelEx(&launch.config, mbv2_fused_kernel<EXPAND, PROJECT, FOLD, NG>, q);
   if (e != cudaSuccess) { *err = std::string("fused inverted-residual launch: ") + cudaGetErrorString(e); return AGO_ERR_CUDA; }
   return AGO_OK;
 }
 template <bool EXPAND, bool PROJECT, bool FOLD>
 ago_status_t launch_variant(const Mbv2Params& q, int smem_bytes, cudaStream_t stream, std::string* err) {
-  if (q.groups == 8) return launch_groups<EXPAND, PROJECT, FOLD, 8>(q, smem_bytes, stream, err);
   return q.groups == 4 ? launch_groups<EXPAND, PROJECT, FOLD, 4>(q, smem_bytes, stream, err)
                        : launch_groups<EXPAND, PROJECT, FOLD, 2>(q, smem_bytes, stream, err);
 }

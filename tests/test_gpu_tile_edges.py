@@ -23,3 +23,36 @@ def check(ago, wl, mode="fused"):
 def test_depthwise_pair_segments_and_strips(ago, shape):
     c = shape[3]
     check(ago, WL.Workload("dw_dw_edges", [201, *shape], [shape], WL.dw_dw("x", [0], 1, 8, c).ops, samples=shape[0], input_dist=["relu_normal"]))
+
+
+@pytest.mark.parametrize("shape", [
+    # n, h, c_in, c_exp, c_out, stride, residual: channels split over clusters of 2 to 8 CTAs
+    (1, 14, 32, 192, 32, 1, True), (1, 1, 16, 96, 16, 1, True), (2, 5, 24, 144, 24, 1, True), (3, 9, 64, 384, 64, 1, True),
+    (1, 8, 64, 384, 160, 1, False), (5, 7, 40, 240, 8, 2, False), (1, 18, 40, 240, 32, 2, False),
+    # more than 64 input channels: two and three K blocks, whole and with a remainder of one or more steps, padded last step
+    (2, 15, 96, 576, 96, 1, True), (1, 8, 72, 432, 40, 1, False), (2, 9, 72, 432, 72, 2, False), (1, 13, 160, 960, 160, 1, True),
+    (3, 12, 160, 960, 96, 2, False), (1, 20, 128, 768, 128, 1, True), (1, 4, 256, 512, 256, 1, True),
+    # widths that cut into one, two, three odd segments with and without a remainder; rows that leave half a block
+    (2, 8, 16, 96, 24, 1, False), (1, 10, 24, 144, 24, 1, True), (1, 16, 32, 192, 16, 1, False), (9, 22, 16, 96, 16, 1, True),
+])
+def test_inverted_residual_channel_splits_and_k_blocks(ago, shape):
+    n, h, c_in, c_exp, c_out, stride, residual = shape
+    check(ago, WL.mbv2_block("mbv2_edges", [202, *map(int, shape)], n, h, c_in, c_exp, c_out, stride, residual))
+
+
+def test_split_channels_repeat_within_the_order_of_the_groups(ago):
+    # many launches in flight on clusters that share SMs with the next grid's: every result stays that of the first one, up to
+    # the order in which the groups add their chunks (one bf16 step)
+    import torch
+    from helpers import to_device
+    wl = WL.mbv2_block("mbv2_repeat", [203], 25, 15, 96, 576, 96, 1, True)
+    data = WL.generate(wl)
+    sg = ago.Subgraph(wl.ops, wl.input_shapes, mode="fused")
+    ins, ws = to_device(wl, data)
+    outs = [sg.run(ins, ws) for _ in range(40)]
+    torch.cuda.synchronize()
+    assert sg.status() == ago.AGO_OK, ago.ago_last_error()
+    scale = float(outs[0].float().abs().max())
+    for o in outs[1:]:
+        assert float((o.float() - outs[0].float()).abs().max()) <= 2.0 ** -7 * scale
+    sg.close()
