@@ -623,8 +623,8 @@ cudaError_t launch_conv3x3_tc(const void* x, const void* w, const float* bias, c
     cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(conv3x3_pair_kernel<true>), smem_opt_in);
     if (e != cudaSuccess) return e;
   }
-  conv3x3_pair_kernel<true><<<q.N * q.strips, kThreads, entry.smem_bytes, stream>>>(entry.mx, entry.mxt, entry.mw, entry.mw, entry.mo, q);
-  return cudaGetLastError();
+  FusedLaunch launch(dim3((unsigned)(q.N * q.strips)), kThreads, (size_t)entry.smem_bytes, stream);
+  return cudaLaunchKernelEx(&launch.config, conv3x3_pair_kernel<true>, entry.mx, entry.mxt, entry.mw, entry.mw, entry.mo, q);
 }
 
 }  // namespace ago

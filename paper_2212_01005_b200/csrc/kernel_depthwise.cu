@@ -10,7 +10,9 @@
 // shapes take one output pixel per thread and leave the overlap to L1 / L2.
 #include <cuda_bf16.h>
 
+#include "fused.h"
 #include "kernels.h"
+#include "tc_common.cuh"
 
 namespace ago {
 
@@ -57,6 +59,7 @@ __device__ __forceinline__ float gelu_tanh_f(float v) {
 template <typename T>
 __global__ void __launch_bounds__(256) depthwise_vec_kernel(const DepthwiseArgs a, int64_t total_vec) {
   constexpr int V = Vec<T>::N;
+  tc::grid_dependency_wait();
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (gid >= total_vec) return;
   const int cv = a.C / V;
@@ -187,6 +190,7 @@ constexpr int kRowBlock = 8;   // output rows per thread of the sliding-window k
 template <typename T, int STRIDE>
 __global__ void __launch_bounds__(256, 3) depthwise3x3_rows_kernel(const DepthwiseArgs a, int64_t total_items) {
   constexpr int V = Vec<T>::N;
+  tc::grid_dependency_wait();
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (gid >= total_items) return;
   const int cv = a.C / V;
@@ -253,24 +257,15 @@ cudaError_t launch_depthwise_fused(const DepthwiseArgs& a, cudaStream_t stream) 
     const int64_t items = (int64_t)a.N * ((a.Ho + kRowBlock - 1) / kRowBlock) * a.Wo * (a.C / V);
     // small tensors keep one output pixel per thread: row blocks would leave most of the device without threads
     if (items >= 100000) {
-    const unsigned blocks = (unsigned)((items + 255) / 256);
-    if (a.dtype == AGO_FP32) {
-      if (a.stride == 1) depthwise3x3_rows_kernel<float, 1><<<blocks, 256, 0, stream>>>(a, items);
-      else depthwise3x3_rows_kernel<float, 2><<<blocks, 256, 0, stream>>>(a, items);
-    } else {
-      if (a.stride == 1) depthwise3x3_rows_kernel<__nv_bfloat16, 1><<<blocks, 256, 0, stream>>>(a, items);
-      else depthwise3x3_rows_kernel<__nv_bfloat16, 2><<<blocks, 256, 0, stream>>>(a, items);
-    }
-    return cudaGetLastError();
+      FusedLaunch launch(dim3((unsigned)((items + 255) / 256)), 256, 0, stream);
+      if (a.dtype == AGO_FP32)
+        return cudaLaunchKernelEx(&launch.config, a.stride == 1 ? depthwise3x3_rows_kernel<float, 1> : depthwise3x3_rows_kernel<float, 2>, a, items);
+      return cudaLaunchKernelEx(&launch.config, a.stride == 1 ? depthwise3x3_rows_kernel<__nv_bfloat16, 1> : depthwise3x3_rows_kernel<__nv_bfloat16, 2>, a, items);
     }
   }
   const int64_t total = (int64_t)a.N * a.Ho * a.Wo * (a.C / V);
-  const unsigned blocks = (unsigned)((total + 255) / 256);
-  if (a.dtype == AGO_FP32)
-    depthwise_vec_kernel<float><<<blocks, 256, 0, stream>>>(a, total);
-  else
-    depthwise_vec_kernel<__nv_bfloat16><<<blocks, 256, 0, stream>>>(a, total);
-  return cudaGetLastError();
+  FusedLaunch launch(dim3((unsigned)((total + 255) / 256)), 256, 0, stream);
+  return cudaLaunchKernelEx(&launch.config, a.dtype == AGO_FP32 ? depthwise_vec_kernel<float> : depthwise_vec_kernel<__nv_bfloat16>, a, total);
 }
 
 }  // namespace ago

@@ -109,6 +109,10 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
   __syncthreads();
   cluster_sync_all();                // the peer's barriers exist before anything signals them
   tcgen05_fence_after_sync();
+  // The set-up above overlaps the previous grid's tail. The next grid may be scheduled from here on: it can only take SMs
+  // that this grid does not need (one CTA per SM).
+  grid_dependency_wait();
+  grid_launch_dependents();
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == kPEpiWarps) {
@@ -403,8 +407,8 @@ cudaError_t launch_gemm_pair(const GemmArgs& a, cudaStream_t stream) {
     resident = g_pair_resident[dev];
   }
   p.pairs = std::min(resident, p.tiles_m * p.tiles_n);
-  gemm_pair_kernel<<<dim3(2 * p.pairs), kPThreads, kPSmemBytes, stream>>>(ma, mb, mc, p);
-  return cudaGetLastError();
+  FusedLaunch launch(dim3((unsigned)(2 * p.pairs)), kPThreads, kPSmemBytes, stream);     // the cluster of two is the kernel's own attribute
+  return cudaLaunchKernelEx(&launch.config, gemm_pair_kernel, ma, mb, mc, p);
 }
 
 }  // namespace ago

@@ -95,6 +95,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   __syncthreads();
   tcgen05_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
+  grid_dependency_wait();      // the set-up above overlaps the previous grid's tail
 
   if (warp == kEpiThreads / 32) {
     // ================================ TMA producer ================================
@@ -315,8 +316,8 @@ cudaError_t launch_gemm_tc(const GemmArgs& a, int add_dtype, cudaStream_t stream
   if (dev >= 0 && dev < 64)
     std::call_once(once[dev], [&] { cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max); });
   dim3 grid((a.M + kBM - 1) / kBM, (a.N + kBN - 1) / kBN, heads * nb);
-  gemm_tc_kernel<<<grid, kThreads, smem, stream>>>(ma, mb, p);
-  return cudaGetLastError();
+  FusedLaunch launch(grid, kThreads, (size_t)smem, stream);
+  return cudaLaunchKernelEx(&launch.config, gemm_tc_kernel, ma, mb, p);
 }
 
 }  // namespace ago
