@@ -470,6 +470,7 @@ ago_status_t ago_subgraph_status(ago_subgraph_t h) {
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy(status word)");
   if (w != 0) {
     cudaMemset(h->status_word, 0, sizeof(w));
+    ++h->fused.workspace_epoch;   // a run that gave up may have left sums and counters behind in the workspace
     char buf[96];
     std::snprintf(buf, sizeof(buf), "a bounded device-side wait expired (code 0x%x)", w);
     return fail(AGO_ERR_TIMEOUT, buf);

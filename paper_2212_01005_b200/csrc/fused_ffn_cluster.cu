@@ -39,15 +39,16 @@ namespace {
 using namespace tc;
 
 constexpr int kBM = 128;        // rows per cluster
-constexpr int kBH = 128;        // hidden units per tile
 constexpr int kBK = 64;         // reduction elements per ring stage
 constexpr int kMaxCS = 4;       // CTAs per cluster
-constexpr int kBlocks = 7;      // 32 KB blocks of shared memory: CS slots for H tiles + ring stages
-constexpr int kMaxStages = 5;
-constexpr int kStageBytes = 32 * 1024;
-constexpr int kEpiWarps = 8;    // two per tensor-memory lane quarter: each takes 64 of a tile's 128 columns
+constexpr int kMaxStages = 8;
+constexpr int kSmemMax = 227 * 1024 - 1024 - 256;   // ring + slots (alignment slack and barriers apart)
+constexpr int kEpiWarps = 16;   // four per tensor-memory lane quarter: each takes a quarter of a tile's columns
 constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kThreads = kEpiThreads + 64;   // + TMA warp + MMA warp
+#ifndef FFN_BH64_MAX
+#define FFN_BH64_MAX 2
+#endif
 constexpr uint32_t kOutCol = 256;            // tensor memory: [0, 256) two first-GEMM accumulators, [256, 256 + NC) the output
 
 struct FfnClusterParams {
@@ -58,10 +59,14 @@ struct FfnClusterParams {
   int M, K, Hid, N2;
   int CS, NC;              // CTAs per cluster, output columns per CTA (N2 / CS, a multiple of 64, <= 256)
   int T;                   // steps per row block = Hid / 128 / CS
+  int BH;                  // hidden units per tile: 128, or 64 where 128 would leave SMs without a tile
+  int RP;                  // rows kept in shared memory: min(128, M rounded up to 16). The MMAs span 128 rows all the same: rows
+                           // past RP are read from whatever follows in shared memory and land in accumulator rows nobody reads
+  int stage_bytes, slot_bytes, slots_off, bars_off;
   int J, Tp;               // a row block is split over J clusters, each with Tp = T / J of its steps (J = 1: no split)
   float* acc;              // J > 1: fp32 [M x N2] partial sums, zero between launches
   int kblocks;             // K / 64
-  int stages;              // ring stages = 7 - CS (at most 5)
+  int stages;              // ring stages
 };
 
 __device__ __forceinline__ float gelu_tanh_fast(float v) {
@@ -82,9 +87,10 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
   // the same offset in every CTA of the cluster: peers address each other's slots and barriers by it
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int CS = p.CS, stages = p.stages;
-  uint8_t* sRing = smem;                                   // stages x 32 KB
-  uint8_t* sH = smem + stages * kStageBytes;               // CS slots x (2 x [128 x 64] bf16, 128-byte-swizzled)
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sH + CS * kStageBytes);
+  const int BH = p.BH, RP = p.RP, halves = BH >> 6, stage_bytes = p.stage_bytes, slot_bytes = p.slot_bytes;
+  uint8_t* sRing = smem;                                   // stages x stage_bytes
+  uint8_t* sH = smem + p.slots_off;                        // CS slots x ([RP x 64] bf16 per 64 hidden units, 128-byte-swizzled)
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.bars_off);
   uint64_t* bar_full = bars;                       // [kMaxStages] ring stage landed
   uint64_t* bar_empty = bars + kMaxStages;         // [kMaxStages] ring stage consumed
   uint64_t* bar_hacc = bars + 2 * kMaxStages;      // [2] first GEMM complete in accumulator b
@@ -130,7 +136,10 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
   }
   tcgen05_fence_before_sync();
   __syncthreads();
-  cluster_sync_all();          // every CTA's barriers exist before a peer signals them
+  // Every CTA's barriers exist before a peer signals them: the arrival is here (relaxed: fence_mbar_init published them), each
+  // role waits before it first touches another CTA.
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  auto cluster_started = [] { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); };
   tcgen05_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
   const int n0 = r * p.NC;     // first output column of this CTA
@@ -142,19 +151,19 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
       tma_prefetch_desc(&tmap_w1);
       tma_prefetch_desc(&tmap_w2);
       int s = 0, round = 0;
-      auto next_stage = [&]() -> uint8_t* {
+      auto next_stage = [&](uint32_t bytes) -> uint8_t* {
         if (round > 0) mbar_wait(bar_empty + s, (uint32_t)(round - 1) & 1u, abort_flag, p.status, 0x701);
-        mbar_arrive_expect_tx(bar_full + s, kStageBytes);
-        return sRing + s * kStageBytes;
+        mbar_arrive_expect_tx(bar_full + s, bytes);
+        return sRing + s * stage_bytes;
       };
       auto advance = [&]() { if (++s == stages) { s = 0; ++round; } };
       auto load_g1 = [&](int step) {       // first GEMM of this CTA's hidden tile of that step
-        const int hid0 = (tile0_of(step) + r) * kBH, row0 = row0_of(step);
+        const int hid0 = (tile0_of(step) + r) * BH, row0 = row0_of(step);
         for (int kb = 0; kb < p.kblocks; ++kb) {
-          uint8_t* st = next_stage();
-          tma_load_2d(st, &tmap_x, bar_full + s, kb * kBK, row0);                          // X [128 rows x 64 k]
-          tma_load_2d(st + 16384, &tmap_w1, bar_full + s, hid0, kb * kBK);                 // W1 [64 k x 64 n] twice
-          tma_load_2d(st + 16384 + 8192, &tmap_w1, bar_full + s, hid0 + 64, kb * kBK);
+          uint8_t* st = next_stage((uint32_t)(RP * 128 + BH * 128));
+          tma_load_2d(st, &tmap_x, bar_full + s, kb * kBK, row0);                          // X [RP rows x 64 k]
+          for (int h = 0; h < halves; ++h)                                                 // W1 [64 k x 64 n] blocks
+            tma_load_2d(st + RP * 128 + h * 8192, &tmap_w1, bar_full + s, hid0 + h * 64, kb * kBK);
           advance();
         }
       };
@@ -163,23 +172,24 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         if (step + 1 < steps) load_g1(step + 1);
         for (int i = 0; i < CS; ++i) {      // second GEMM over hidden tile t CS + k: two stages of 64 hidden units
           const int k = (int)((r + CS - i) % CS);   // in the order the MMA warp consumes the slots: own tile first
-          const int hid0 = (tile0_of(step) + k) * kBH;
-          for (int h = 0; h < 2; ++h) {
-            uint8_t* st = next_stage();
-            for (int nb = 0; nb < 4; ++nb)   // W2 [64 k x 64 n] per block; blocks past NC read as zero and are not multiplied
-              tma_load_2d(st + nb * 8192, &tmap_w2, bar_full + s, nb * 64 < p.NC ? n0 + nb * 64 : p.N2, hid0 + h * 64);
+          const int hid0 = (tile0_of(step) + k) * BH;
+          for (int h = 0; h < halves; ++h) {
+            uint8_t* st = next_stage((uint32_t)(p.NC * 128));
+            for (int nb = 0; nb < p.NC; nb += 64)   // W2 [64 k x 64 n] per block
+              tma_load_2d(st + nb * 128, &tmap_w2, bar_full + s, n0 + nb, hid0 + h * 64);
             advance();
           }
         }
       }
     }
     __syncwarp();
+    cluster_started();
   } else if (warp == kEpiWarps + 1) {
     // ================================ MMA issuer ================================
     // the whole warp, converged; MMAs and commits predicated on one elected lane (see tc_common.cuh)
     {
       const uint32_t elected = elect_one();
-      const uint32_t idesc1 = make_idesc_bf16(128, kBH, 0, 1);              // A K-major, B N-major (weights as they lie in memory)
+      const uint32_t idesc1 = make_idesc_bf16(128, (uint32_t)BH, 0, 1);     // A K-major, B N-major (weights as they lie in memory)
       const uint32_t idesc2 = make_idesc_bf16(128, (uint32_t)p.NC, 0, 1);
       int s = 0, round = 0;
       auto advance = [&]() { if (++s == stages) { s = 0; ++round; } };
@@ -192,18 +202,19 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         for (int kb = 0; kb < p.kblocks; ++kb) {
           mbar_wait(bar_full + s, (uint32_t)round & 1u, abort_flag, p.status, 0x703);
           tcgen05_fence_after_sync();
-          const uint32_t st = smem_u32(sRing + s * kStageBytes);
+          const uint32_t st = smem_u32(sRing + s * stage_bytes);
           const uint64_t ad = make_smem_desc(st, 0, 1024, SW_128B);
-          const uint64_t bd = make_smem_desc(st + 16384, 8192, 1024, SW_128B);
+          const uint64_t bd = make_smem_desc(st + (uint32_t)(RP * 128), 8192, 1024, SW_128B);
 #pragma unroll
           for (int ks = 0; ks < kBK / 16; ++ks)
-            umma_bf16_elected_acc(tmem_base + b * kBH, ad + 2u * ks, bd + (uint64_t)((ks * 2048) >> 4), idesc1, elected, (kb | ks) != 0);
+            umma_bf16_elected_acc(tmem_base + b * BH, ad + 2u * ks, bd + (uint64_t)((ks * 2048) >> 4), idesc1, elected, (kb | ks) != 0);
           umma_commit_elected(bar_empty + s, elected);
           advance();
         }
         umma_commit_elected(bar_hacc + b, elected);
       };
       if (steps > 0) g1(0);
+      cluster_started();
       for (int step = 0; step < steps; ++step) {
         if (step + 1 < steps) g1(step + 1);
         const int t = step % T, bi = step / T;
@@ -216,11 +227,11 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         for (int i = 0; i < CS; ++i) {
           const int k = (int)((r + CS - i) % CS);
           mbar_wait(bar_hfull + k, (uint32_t)step & 1u, abort_flag, p.status, 0x704);   // H tile t CS + k is in slot k
-          for (int h = 0; h < 2; ++h) {
+          for (int h = 0; h < halves; ++h) {
             mbar_wait(bar_full + s, (uint32_t)round & 1u, abort_flag, p.status, 0x705);
             tcgen05_fence_after_sync();
-            const uint64_t hd = make_smem_desc(smem_u32(sH + k * kStageBytes + h * (kBM * 128)), 0, 1024, SW_128B);
-            const uint64_t bd = make_smem_desc(smem_u32(sRing + s * kStageBytes), 8192, 1024, SW_128B);
+            const uint64_t hd = make_smem_desc(smem_u32(sH + k * slot_bytes + h * (RP * 128)), 0, 1024, SW_128B);
+            const uint64_t bd = make_smem_desc(smem_u32(sRing + s * stage_bytes), 8192, 1024, SW_128B);
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
               umma_bf16_elected_acc(tmem_base + kOutCol, hd + 2u * ks, bd + (uint64_t)((ks * 2048) >> 4), idesc2, elected, (t | i | h | ks) != 0);
@@ -235,11 +246,15 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     }
     __syncwarp();
   } else {
-    // ================ epilogue warps: thread = (row, half of a tile's 128 columns) ================
+    // ================ epilogue warps: thread = (row, quarter of a tile's columns) ================
     const int row = (warp & 3) * 32 + lane;
-    const int half = warp >> 2;
+    const int part = warp >> 2;
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-    uint8_t* slot = sH + r * kStageBytes;          // this CTA produces into slot r everywhere
+    const bool warp_rows = (warp & 3) * 32 < RP;   // some row of this warp exists
+    uint8_t* slot = sH + r * slot_bytes;           // this CTA produces into slot r everywhere
+    constexpr int kParts = kEpiWarps / 4;
+    const int pc = BH / kParts;                        // columns per thread: 16 or 32
+    cluster_started();
 
     for (int step = 0; step < steps; ++step) {
       const int b = step & 1, t = step % T;
@@ -247,26 +262,31 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
       tcgen05_fence_after_sync();
       // every CTA has multiplied the previous content of slot r (and the copies that delivered it are complete)
       if (step >= 1) mbar_wait(bar_hdone, (uint32_t)(step - 1) & 1u, abort_flag, p.status, 0x707);
-      uint8_t* tile = slot + half * (kBM * 128);
-      const float* bb = p.b1 + (size_t)(tile0_of(step) + r) * kBH + half * 64;
+      const int col0 = part * pc;
+      uint8_t* tile = slot + (col0 >> 6) * (RP * 128);
+      const float* bb = p.b1 + (size_t)(tile0_of(step) + r) * BH + col0;
+      if (warp_rows) {
+        for (int c0 = 0; c0 < pc; c0 += 16) {
+          uint32_t v[16];
+          tmem_ld_x16(tmem_base + lane_base + b * BH + col0 + c0, v);
+          float4 bv4[4];
 #pragma unroll
-      for (int c0 = 0; c0 < 64; c0 += 32) {
-        uint32_t v[32];
-        tmem_ld_x32(tmem_base + lane_base + b * kBH + half * 64 + c0, v);
-        tmem_ld_wait();
+          for (int q = 0; q < 4; ++q) bv4[q] = __ldg(reinterpret_cast<const float4*>(bb + c0) + q);
+          tmem_ld_wait();
+          if (row < RP) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const float4 b0 = __ldg(reinterpret_cast<const float4*>(bb + c0 + q * 8));
-          const float4 b1v = __ldg(reinterpret_cast<const float4*>(bb + c0 + q * 8 + 4));
-          const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1v.x, b1v.y, b1v.z, b1v.w};
-          uint32_t w[4];
+            for (int q = 0; q < 2; ++q) {
+              const float bv[8] = {bv4[2 * q].x, bv4[2 * q].y, bv4[2 * q].z, bv4[2 * q].w, bv4[2 * q + 1].x, bv4[2 * q + 1].y, bv4[2 * q + 1].z, bv4[2 * q + 1].w};
+              uint32_t w[4];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int e = q * 8 + j * 2;
-            w[j] = pack_bf16x2(gelu_tanh_fast(__uint_as_float(v[e]) + bv[2 * j]),
-                               gelu_tanh_fast(__uint_as_float(v[e + 1]) + bv[2 * j + 1]));
+              for (int j = 0; j < 4; ++j) {
+                const int e = q * 8 + j * 2;
+                w[j] = pack_bf16x2(gelu_tanh_fast(__uint_as_float(v[e]) + bv[2 * j]),
+                                   gelu_tanh_fast(__uint_as_float(v[e + 1]) + bv[2 * j + 1]));
+              }
+              *reinterpret_cast<uint4*>(tile + swz_offset(row, (((col0 & 63) + c0) >> 3) + q, 128)) = make_uint4(w[0], w[1], w[2], w[3]);
+            }
           }
-          *reinterpret_cast<uint4*>(tile + swz_offset(row, (c0 >> 3) + q, 128)) = make_uint4(w[0], w[1], w[2], w[3]);
         }
       }
       fence_proxy_async_smem();      // the MMA and the bulk copies read the tile through the async proxy
@@ -279,31 +299,62 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         for (int q = 1; q < CS; ++q) {                                // the peers, starting with the next rank
           const uint32_t peer = (uint32_t)((r + q) % CS);
           const uint32_t rbar = cluster_map(bar, peer);
-          mbar_remote_arrive_expect_tx(rbar, kStageBytes);
-          bulk_copy_to_cluster(cluster_map(src, peer), src, kStageBytes, rbar);
+          mbar_remote_arrive_expect_tx(rbar, (uint32_t)slot_bytes);
+          bulk_copy_to_cluster(cluster_map(src, peer), src, (uint32_t)slot_bytes, rbar);
         }
       }
       if (t == T - 1) {
-        // ---- output of the row block: out (TMEM) -> + b2 -> bf16 -> device memory; thread = (row, half of the CTA's columns) ----
+        // ---- output of the row block: out (TMEM) -> + b2 -> bf16 -> device memory; thread = (row, quarter of the CTA's columns) ----
         const int bi = step / T, row0 = row0_of(step);
         const bool row_ok = row0 + row < p.M;
         mbar_wait(bar_out, (uint32_t)bi & 1u, abort_flag, p.status, 0x708);
         tcgen05_fence_after_sync();
-        const int hc = p.NC >> 1;                                          // columns per half: 32, 64, 96 or 128
+        const int hc = p.NC / kParts;                                          // columns per thread: 16, 32, 48 or 64
         if (J > 1) {
-          // ---- split row block: add this cluster's share into the fp32 buffer; a second, small kernel turns the buffer
-          // into the output (+ b2, bf16) with every SM of the device and leaves it zeroed. (A last-arriver sweep inside
-          // this kernel -- one CTA per column slice reading 96 KB back -- took 8 us on the critical path.) ----
-          float* arow = p.acc + (size_t)(row0 + row) * p.N2 + n0 + half * hc;
-          for (int c0 = 0; c0 < hc; c0 += 32) {
-            uint32_t v[32];
-            tmem_ld_x32(tmem_base + lane_base + kOutCol + half * hc + c0, v);
-            tmem_ld_wait();
-            if (row_ok) {
+          // ---- split row block: this cluster's share is added into the fp32 buffer; the second launch turns the buffer
+          // into the output (+ b2, bf16) and zeroes it. ----
+          if (RP < 64) {
+            // few rows: every thread adds from its registers (one barrier less than below: 10.9 against 12.0 us for one row)
+            float* arow = p.acc + (size_t)(row0 + row) * p.N2 + n0 + part * hc;
+            if (warp_rows) {
+              for (int c0 = 0; c0 < hc; c0 += 16) {
+                uint32_t v[16];
+                tmem_ld_x16(tmem_base + lane_base + kOutCol + part * hc + c0, v);
+                tmem_ld_wait();
+                if (row_ok) {
 #pragma unroll
-              for (int q = 0; q < 8; ++q)
-                red_add_v4(arow + c0 + q * 4, __uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
-                           __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
+                  for (int q = 0; q < 4; ++q)
+                    red_add_v4(arow + c0 + q * 4, __uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
+                               __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
+                }
+              }
+            }
+          } else {
+            // Blocks of 64 columns go through shared memory (two buffers over the ring, which this cluster's one unit has
+            // used up), so that a half-warp adds 256 contiguous bytes of a row: additions of 16 bytes per row took the L2 twice
+            // as long. The clusters of a row block start with different blocks, not to meet on the same addresses.
+            const int blocks = p.NC >> 6, first = (unit_of(step) % J) % blocks, rows_here = min(RP, p.M - row0);
+            for (int k = 0; k < blocks; ++k) {
+              int cb = first + k;
+              if (cb >= blocks) cb -= blocks;
+              uint8_t* buf = sRing + (k & 1) * (RP * 256);
+              if (warp_rows) {
+                uint32_t v[16];
+                tmem_ld_x16(tmem_base + lane_base + kOutCol + cb * 64 + part * 16, v);
+                tmem_ld_wait();
+                if (row < RP) {
+  #pragma unroll
+                  for (int q = 0; q < 4; ++q)
+                    *reinterpret_cast<uint4*>(buf + row * 256 + ((((part * 4 + q) ^ row) & 15) << 4)) = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                }
+              }
+              named_barrier_sync(1, kEpiThreads);
+              float* ablk = p.acc + (size_t)row0 * p.N2 + n0 + cb * 64;
+              for (int i = tid; i < rows_here * 16; i += kEpiThreads) {
+                const int rr = i >> 4, c = i & 15;
+                const float4 f = *reinterpret_cast<const float4*>(buf + rr * 256 + (((c ^ rr) & 15) << 4));
+                red_add_v4(ablk + (size_t)rr * p.N2 + c * 4, f.x, f.y, f.z, f.w);
+              }
             }
           }
           tcgen05_fence_before_sync();
@@ -311,22 +362,24 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
           if (tid == 0) mbar_arrive(bar_outfree);
           continue;
         }
-        __nv_bfloat16* orow = p.out + (size_t)(row0 + row) * p.N2 + n0 + half * hc;
-        const float* b2 = p.b2 + n0 + half * hc;
-        for (int c0 = 0; c0 < hc; c0 += 32) {
-          uint32_t v[32];
-          tmem_ld_x32(tmem_base + lane_base + kOutCol + half * hc + c0, v);
-          tmem_ld_wait();
-          if (row_ok) {
+        __nv_bfloat16* orow = p.out + (size_t)(row0 + row) * p.N2 + n0 + part * hc;
+        const float* b2 = p.b2 + n0 + part * hc;
+        if (warp_rows) {
+          for (int c0 = 0; c0 < hc; c0 += 16) {
+            uint32_t v[16];
+            tmem_ld_x16(tmem_base + lane_base + kOutCol + part * hc + c0, v);
+            tmem_ld_wait();
+            if (row_ok) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const float4 b0 = __ldg(reinterpret_cast<const float4*>(b2 + c0 + q * 8));
-              const float4 b1v = __ldg(reinterpret_cast<const float4*>(b2 + c0 + q * 8 + 4));
-              *reinterpret_cast<uint4*>(orow + c0 + q * 8) =
-                  make_uint4(pack_bf16x2(__uint_as_float(v[q * 8]) + b0.x, __uint_as_float(v[q * 8 + 1]) + b0.y),
-                             pack_bf16x2(__uint_as_float(v[q * 8 + 2]) + b0.z, __uint_as_float(v[q * 8 + 3]) + b0.w),
-                             pack_bf16x2(__uint_as_float(v[q * 8 + 4]) + b1v.x, __uint_as_float(v[q * 8 + 5]) + b1v.y),
-                             pack_bf16x2(__uint_as_float(v[q * 8 + 6]) + b1v.z, __uint_as_float(v[q * 8 + 7]) + b1v.w));
+              for (int q = 0; q < 2; ++q) {
+                const float4 b0 = __ldg(reinterpret_cast<const float4*>(b2 + c0 + q * 8));
+                const float4 b1v = __ldg(reinterpret_cast<const float4*>(b2 + c0 + q * 8 + 4));
+                *reinterpret_cast<uint4*>(orow + c0 + q * 8) =
+                    make_uint4(pack_bf16x2(__uint_as_float(v[q * 8]) + b0.x, __uint_as_float(v[q * 8 + 1]) + b0.y),
+                               pack_bf16x2(__uint_as_float(v[q * 8 + 2]) + b0.z, __uint_as_float(v[q * 8 + 3]) + b0.w),
+                               pack_bf16x2(__uint_as_float(v[q * 8 + 4]) + b1v.x, __uint_as_float(v[q * 8 + 5]) + b1v.y),
+                               pack_bf16x2(__uint_as_float(v[q * 8 + 6]) + b1v.z, __uint_as_float(v[q * 8 + 7]) + b1v.w));
+              }
             }
           }
         }
@@ -342,7 +395,9 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
   if (warp == 0) tmem_dealloc(tmem_base, 512);
 }
 
-// Second launch of a split run: out = bf16(acc + b2), acc = 0. One float4 per thread and iteration, coalesced.
+// Second launch of a split run: out = bf16(acc + b2), acc = 0. One float4 per thread and iteration, coalesced. (A sweep that
+// follows per-slice arrival counters instead of the end of the first grid was slower at every size: 16.6 against 16.3 us at 256
+// rows, 56 against 53 at 2048; the counters' fences wait for the additions, which keep the L2 busy.)
 __global__ void __launch_bounds__(256) ffn_cluster_finalize_kernel(float* acc, const float* b2, __nv_bfloat16* out, long long total4, int n2) {
   grid_dependency_wait();      // the additions of the first launch are complete and visible
   grid_launch_dependents();
@@ -353,6 +408,52 @@ __global__ void __launch_bounds__(256) ffn_cluster_finalize_kernel(float* acc, c
     reinterpret_cast<float4*>(acc)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     reinterpret_cast<uint2*>(out)[i] = make_uint2(pack_bf16x2(a.x + bb.x, a.y + bb.y), pack_bf16x2(a.z + bb.z, a.w + bb.w));
   }
+}
+
+// Ring, slots and barriers: as many stages as fit. Behind ring and slots lies at least one 128-row operand (the MMAs read 128
+// rows from the start of the last tile whatever RP is).
+int layout(FfnClusterParams* q) {
+  q->slot_bytes = q->RP * q->BH * 2;
+  q->stage_bytes = (std::max(q->RP * 128 + q->BH * 128, q->NC * 128) + 1023) & ~1023;
+  const int slots = q->CS * q->slot_bytes, slack = kBM * 128 - q->RP * 128;
+  q->stages = std::min(kMaxStages, (kSmemMax - slots - slack) / q->stage_bytes);
+  q->slots_off = q->stages * q->stage_bytes;
+  q->bars_off = q->slots_off + slots + slack;
+  return q->bars_off + 256 + 1024;
+}
+
+// Cluster size, hidden tile and split of the row blocks' hidden tiles over clusters.
+bool choose_split(FfnClusterParams* q, int row_blocks, const int* resident) {
+  // Whole row blocks: among the cluster sizes whose column share fits tensor memory, the least estimated time = rounds of
+  // resident clusters x steps per row block x ring stages per step.
+  q->CS = 0; q->BH = 128; q->J = 1;
+  long best = 0;
+  const int htiles = q->Hid / 128;
+  for (int cs = 2; cs <= kMaxCS; ++cs) {
+    if (q->N2 % cs != 0 || htiles % cs != 0) continue;
+    const int nc = q->N2 / cs;
+    if (nc % 64 != 0 || nc > 256) continue;
+    const long rounds = (row_blocks + resident[cs] - 1) / resident[cs];
+    const long cost = rounds * (htiles / cs) * (q->K / kBK + 2 * cs);
+    if (q->CS == 0 || cost < best) { q->CS = cs; q->NC = nc; best = cost; }
+  }
+  if (q->CS == 0) return false;
+  q->T = htiles / q->CS;
+  if ((long)row_blocks * q->CS < 120) {
+    // Few row blocks: one cluster per block of 128 rows leaves most SMs idle, and the hidden dimension is what can fill
+    // them. A row block is split over J clusters (J divides its T steps); their outputs meet in an fp32 buffer in device
+    // memory, J additions per element instead of one per hidden tile. J = as many parts as still fit one round of
+    // resident clusters, each with at least one step. With one or two row blocks even that leaves SMs idle: tiles of 64.
+    const int bh_small = FFN_BH64_MAX >= row_blocks ? 64 : 128;
+    for (int bh = bh_small; bh <= 128; bh += 64) {
+      const int T = q->Hid / bh / q->CS;
+      for (int j = T; j >= 2; --j)
+        if (T % j == 0 && (long)row_blocks * j <= resident[q->CS]) { q->BH = bh; q->T = T; q->J = j; break; }
+      if (q->J > 1) break;
+    }
+  }
+  q->Tp = q->T / q->J;
+  return true;
 }
 
 struct FfnClusterHost {
@@ -393,42 +494,15 @@ ago_status_t ffn_cluster_plan(Plan* plan, FusedState* st, std::string* err) {
   q.M = (int)(plan->inputs[0].numel() / q.K);
   q.Hid = plan->ops[0].op.p[0];
   q.N2 = plan->ops[3].op.p[0];
-  if (q.K % kBK != 0 || q.Hid % kBH != 0) return AGO_ERR_UNSUPPORTED;
-  const int htiles = q.Hid / kBH;
-  // Cluster size: among the sizes whose column share fits tensor memory, the one with the least estimated time =
-  // rounds of resident clusters x steps per row block x ring stages per step. Resident clusters of 1-CTA-per-SM
-  // kernels on a B200 (148 SMs in GPCs of unequal size), as cudaOccupancyMaxActiveClusters reports them: 74 / 45 / 33
-  // for sizes 2 / 3 / 4; the launch asks the device again and sizes its grid by the answer.
+  if (q.K % kBK != 0 || q.Hid % 128 != 0) return AGO_ERR_UNSUPPORTED;
+  const int resident[kMaxCS + 1] = {0, 0, 74, 45, 33};   // clusters of 1-CTA-per-SM kernels a B200 keeps resident at once
   const int row_blocks_plan = (q.M + kBM - 1) / kBM;
-  const int resident[kMaxCS + 1] = {0, 0, 74, 45, 33};
-  q.CS = 0;
-  long best = 0;
-  for (int cs = 2; cs <= kMaxCS; ++cs) {
-    if (q.N2 % cs != 0 || htiles % cs != 0) continue;
-    const int nc = q.N2 / cs;
-    if (nc % 64 != 0 || nc > 256) continue;
-    const long rounds = (row_blocks_plan + resident[cs] - 1) / resident[cs];
-    const long cost = rounds * (htiles / cs) * (q.K / kBK + 2 * cs);
-    if (q.CS == 0 || cost < best) { q.CS = cs; q.NC = nc; best = cost; }
-  }
-  if (q.CS == 0) return AGO_ERR_UNSUPPORTED;
-  q.T = htiles / q.CS;
-  q.J = 1;
-  if ((long)row_blocks_plan * q.CS < 120) {
-    // Few row blocks: one cluster per block of 128 rows leaves most SMs idle, and the hidden dimension is what can fill
-    // them. A row block is split over J clusters (J divides its T steps); their outputs meet in an fp32 buffer in device
-    // memory, J additions per element instead of one per hidden tile. J = as many parts as still fit one round of
-    // resident clusters, each with at least one step.
-    for (int j = q.T; j >= 1; --j)
-      if (q.T % j == 0 && (long)row_blocks_plan * j <= resident[q.CS]) { q.J = j; break; }
-    if (q.J == 1 || q.N2 % 4 != 0 || (q.NC / 2) % 32 != 0) return AGO_ERR_UNSUPPORTED;   // nothing to split: the other kernel
-  }
-  q.Tp = q.T / q.J;
+  q.RP = std::min(kBM, (q.M + 15) / 16 * 16);
+  if (!choose_split(&q, row_blocks_plan, resident)) return AGO_ERR_UNSUPPORTED;
   q.kblocks = q.K / kBK;
-  q.stages = std::min(kMaxStages, kBlocks - q.CS);
   auto* host = new FfnClusterHost();
+  host->smem_bytes = layout(&q);
   host->prm = q;
-  host->smem_bytes = (q.stages + q.CS) * kStageBytes + 256 + 1024;
   st->impl = host;
   st->impl_free = [](void* p) { delete static_cast<FfnClusterHost*>(p); };
   st->variant = 1;
@@ -479,7 +553,7 @@ ago_status_t ffn_cluster_run(const Plan& plan, FusedState* st, const void* const
     if (it == host->maps.end()) {
       CUtensorMap m;
       uint64_t dims[2]; uint64_t strides[1]; uint32_t box[2];
-      if (which == 0) { dims[0] = q.K; dims[1] = q.M; strides[0] = (uint64_t)q.K * 2; box[0] = kBK; box[1] = kBM; }
+      if (which == 0) { dims[0] = q.K; dims[1] = q.M; strides[0] = (uint64_t)q.K * 2; box[0] = kBK; box[1] = (uint32_t)q.RP; }
       else if (which == 1) { dims[0] = q.Hid; dims[1] = q.K; strides[0] = (uint64_t)q.Hid * 2; box[0] = 64; box[1] = kBK; }
       else { dims[0] = q.N2; dims[1] = q.Hid; strides[0] = (uint64_t)q.N2 * 2; box[0] = 64; box[1] = 64; }
       if (!encode_tmap_bf16(&m, base, 2, dims, strides, box, 128, err)) return false;
