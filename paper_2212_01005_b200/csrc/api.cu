@@ -308,10 +308,12 @@ namespace {
 // costs less than about a third of the contractions' tensor-core time: both modes are then bound by the contractions
 // (Section VI-B reports the same for pointwise -> pointwise chains). Data-sheet-class constants; only the ratio matters.
 bool fusion_pays(const Plan& p) {
-  // Exception: a feed-forward chain on so few rows that the fused kernel splits each row block's hidden tiles over
-  // several clusters. The two GEMM launches of the unfused mode have a handful of row tiles each and leave most SMs
-  // idle; the fused kernel fills them through the hidden dimension (config 1: 24 against 45 us).
-  if (p.fused_kernel == AGO_KERNEL_FFN && p.fused_variant == 2) return true;
+  // Feed-forward chains: both ways are estimated (768 -> 3072: fused 17.4 against 26 us at 512 rows, 26 against 30 at 1000, but 40
+  // against 32 at 1500 and 137 against 102 at 12288).
+  if (p.fused_kernel == AGO_KERNEL_FFN) {
+    const double fused = p.fused_variant == 3 ? ffn_pair_estimate(p) : p.fused_variant == 0 ? -1.0 : ffn_cluster_estimate(p);
+    return fused >= 0.0 && fused <= ffn_unfused_estimate(p);
+  }
   const double t_intermediates = (double)p.intermediate_bytes / 6.5e12;
   const double t_tensor = (double)p.flops_tensor / 1.6e15;
   return !(t_tensor > 0.0 && t_intermediates < 0.35 * t_tensor);

@@ -54,9 +54,13 @@ ago_status_t fused_plan(Plan* plan, FusedState* st, std::string* err) {
     case AGO_KERNEL_ATTENTION:
       return attention_plan(plan, st, err);
     case AGO_KERNEL_FFN: {
-      // many rows: the cluster of two CTA pairs (256 rows per weight tile); else the cluster kernel where the shape
-      // splits over 2..4 CTAs; else the kernel that tiles the reduction
-      ago_status_t s = ffn_pair_plan(plan, st, err);
+      // The cluster of two CTA pairs (256 rows per weight tile) where its 256-row blocks fill most of the device or where it is
+      // estimated to be the faster one (768 -> 3072: 2500 rows 50 against 67 us, 6144 rows 82 against 127, but 5120 rows 83 against
+      // 67); else the cluster kernel where the shape splits over 2..4 CTAs; else the kernel that tiles the reduction.
+      const double pair = ffn_pair_estimate(*plan), cluster = ffn_cluster_estimate(*plan);
+      const int64_t rows = plan->inputs[0].numel() / plan->inputs[0].last();
+      const bool fills = (rows + 255) / 256 * 4 >= (int64_t)device_sm_count() * 3 / 4;
+      ago_status_t s = fills || cluster < 0 || (pair >= 0 && pair < cluster) ? ffn_pair_plan(plan, st, err) : AGO_ERR_UNSUPPORTED;
       if (s == AGO_ERR_UNSUPPORTED) s = ffn_cluster_plan(plan, st, err);
       return s == AGO_ERR_UNSUPPORTED ? ffn_plan(plan, st, err) : s;
     }

@@ -1,24 +1,26 @@
 // Fused feed-forward chain on a thread-block cluster: Y = GELU(X W1 + b1) W2 + b2; the hidden activations H never leave
 // the SMs. With enough row blocks to fill the device nothing is reduced through device memory and the run is one kernel;
-// with few row blocks (config 1: 512 rows) each row block's hidden tiles are split over J clusters, whose output shares
-// meet in an fp32 buffer (J additions per element), and a second, small launch turns the buffer into the output.
+// with few row blocks each row block's hidden tiles are split over J clusters, whose output shares meet in an fp32 buffer
+// (J additions per element), and a second, small launch turns the buffer into the output. There the run is a chain of
+// latencies, so a cluster of one step requests everything it needs at once, keeps only the rows that exist and takes hidden
+// tiles of 64 where they put more clusters to work: 768 -> 3072 -> 768 with 1 row 14.6 -> 8.1 us, 128 rows 18.1 -> 11.9,
+// 256 rows 18.7 -> 12.6, 512 rows 19.9 -> 17.4 (of which 3.8 us are the 9.4 MB of additions at the rate of the L2).
 //
 // Tile choice (Section III-B, "downstream pointwise / matmul"): the second GEMM reuses H only along its output
 // columns, so the downstream tile keeps ALL output columns of a block of 128 rows. Those (768 fp32 columns for
 // BERT-base) do not fit the tensor memory of one SM next to the first GEMM's accumulator -- but they fit the tensor
 // memory of a CLUSTER: CS CTAs (CS = 2..4) work on the same 128 rows, CTA r owns output columns
-// [r N2/CS, (r+1) N2/CS) and computes every CS-th tile of 128 hidden units. A finished H tile (bias, GELU, bf16,
+// [r N2/CS, (r+1) N2/CS) and computes every CS-th tile of 128 (or 64) hidden units. A finished H tile (bias, GELU, bf16,
 // 32 KB as a swizzled K-major operand) is copied to the same shared-memory slot of every peer with one bulk
 // shared-to-shared copy per peer (distributed shared memory), so every H tile is computed once and multiplied
 // into all N2 output columns without recomputation and without reductions outside the SM.
 //
 // Per CTA (rank r), T = hidden tiles / CS steps:
-//   ring   TMA producer warp: 32 KB stages -- X [128 x 64] + W1 [64 x 128] for the first GEMM, W2 [64 x N2/CS]
-//          for the second
-//   MMA    one thread: G1(t+1): Hacc[(t+1) & 1] = X W1[:, tile (t+1) CS + r]; then for k = 0..CS-1
+//   ring   TMA producer warp: stages of X [RP x 64] + W1 [64 x BH] for the first GEMM, W2 [64 x N2/CS] for the second
+//   MMA    one warp: G1(t+1): Hacc[(t+1) & 1] = X W1[:, tile (t+1) CS + r]; then for k = 0..CS-1
 //          G2(k): out += H slot k * W2[tile t CS + k, own columns]; its completion is committed onto CTA k's
 //          "slot consumed" barrier
-//   epi    8 warps: Hacc[t & 1] -> + b1, GELU, bf16 -> own slot r (after every CTA has consumed its previous
+//   epi    8 or 16 warps: Hacc[t & 1] -> + b1, GELU, bf16 -> own slot r (after every CTA has consumed its previous
 //          content) -> announce locally, bulk-copy to the peers' slot r with completion on their "slot full" barrier
 //   end    out (TMEM) -> + b2 -> bf16 -> device memory
 // Every wait is bounded; a CTA leaves only after a cluster barrier, so no peer copies into an exited CTA.
@@ -26,6 +28,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cmath>
 #include <unordered_map>
 
 #include "fused.h"
@@ -41,14 +44,12 @@ using namespace tc;
 constexpr int kBM = 128;        // rows per cluster
 constexpr int kBK = 64;         // reduction elements per ring stage
 constexpr int kMaxCS = 4;       // CTAs per cluster
-constexpr int kMaxStages = 8;
-constexpr int kSmemMax = 227 * 1024 - 1024 - 256;   // ring + slots (alignment slack and barriers apart)
-constexpr int kEpiWarps = 16;   // four per tensor-memory lane quarter: each takes a quarter of a tile's columns
-constexpr int kEpiThreads = kEpiWarps * 32;
-constexpr int kThreads = kEpiThreads + 64;   // + TMA warp + MMA warp
-#ifndef FFN_BH64_MAX
-#define FFN_BH64_MAX 2
-#endif
+constexpr int kMaxStages = 16;
+constexpr int kSmemMax = 227 * 1024 - 1024 - 512;   // ring + slots (alignment slack and barriers apart)
+// Epilogue warps: four per tensor-memory lane quarter, each with a quarter of a tile's columns; two where the epilogue hides
+// behind the next step's products (whole row blocks in several steps).
+constexpr int epi_warps_of(int bh, bool full) { return full && bh == 128 ? 8 : 16; }
+constexpr int threads_of(int bh, bool full) { return epi_warps_of(bh, full) * 32 + 64; }   // + TMA warp + MMA warp
 constexpr uint32_t kOutCol = 256;            // tensor memory: [0, 256) two first-GEMM accumulators, [256, 256 + NC) the output
 
 struct FfnClusterParams {
@@ -67,6 +68,7 @@ struct FfnClusterParams {
   float* acc;              // J > 1: fp32 [M x N2] partial sums, zero between launches
   int kblocks;             // K / 64
   int stages;              // ring stages
+  int w2_off;              // > 0: one step per cluster and everything fits: the step's W2 tiles have stages of their own there
 };
 
 __device__ __forceinline__ float gelu_tanh_fast(float v) {
@@ -80,17 +82,23 @@ __device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float 
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
-__global__ void __launch_bounds__(kThreads, 1)
+// BH: hidden units per tile; FULL: all 128 rows of a block are kept (RP == 128).
+template <int BH, bool FULL>
+__global__ void __launch_bounds__(threads_of(BH, FULL), 1)
 ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w1,
                    const __grid_constant__ CUtensorMap tmap_w2, const FfnClusterParams p) {
   extern __shared__ uint8_t smem_raw[];
   // the same offset in every CTA of the cluster: peers address each other's slots and barriers by it
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int CS = p.CS, stages = p.stages;
-  const int BH = p.BH, RP = p.RP, halves = BH >> 6, stage_bytes = p.stage_bytes, slot_bytes = p.slot_bytes;
+  constexpr int kEpiWarps = epi_warps_of(BH, FULL), kEpiThreads = kEpiWarps * 32;
+  constexpr int halves = BH / 64;
+  constexpr bool kWhole = FULL && BH == 128;       // then a stage is 32 KB and the slots leave no room for own_w2
+  const int RP = FULL ? kBM : p.RP, stage_bytes = kWhole ? 32768 : p.stage_bytes, slot_bytes = RP * BH * 2;
   uint8_t* sRing = smem;                                   // stages x stage_bytes
   uint8_t* sH = smem + p.slots_off;                        // CS slots x ([RP x 64] bf16 per 64 hidden units, 128-byte-swizzled)
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.bars_off);
+  const bool own_w2 = !kWhole && p.w2_off > 0;
   uint64_t* bar_full = bars;                       // [kMaxStages] ring stage landed
   uint64_t* bar_empty = bars + kMaxStages;         // [kMaxStages] ring stage consumed
   uint64_t* bar_hacc = bars + 2 * kMaxStages;      // [2] first GEMM complete in accumulator b
@@ -99,8 +107,9 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
   uint64_t* bar_hdone = bar_hfull + kMaxCS;        // own slot consumed by every CTA of the cluster (count CS)
   uint64_t* bar_out = bar_hdone + 1;               // second GEMM of a row block complete
   uint64_t* bar_outfree = bar_out + 1;             // output accumulators drained: the next row block may overwrite them
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_outfree + 1);
-  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bar_outfree + 2);
+  uint64_t* bar_w2 = bar_outfree + 1;              // [kMaxCS * 2] a W2 stage of its own has landed
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_w2 + 2 * kMaxCS);
+  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bar_w2 + 2 * kMaxCS + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int r = (int)cluster_ctarank();
@@ -113,6 +122,9 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
   const int units = row_blocks * J;
   const int my_units = ((int)blockIdx.y < units) ? (units - 1 - (int)blockIdx.y) / (int)gridDim.y + 1 : 0;
   const int steps = my_units * T;
+  // A cluster of one step expects the tiles of the others right away; with more steps the sender announces each tile on the
+  // receiver's barrier (0.4 us each for its thread: 9.2 against 8.5 us for 16 rows, where nothing hides it).
+  const bool one_step = steps == 1;
   auto unit_of = [&](int step) { return (int)blockIdx.y + (step / T) * (int)gridDim.y; };
   auto row0_of = [&](int step) { return (unit_of(step) / J) * kBM; };
   auto tile0_of = [&](int step) { return ((unit_of(step) % J) * T + step % T) * CS; };   // first of the step's CS hidden tiles
@@ -127,7 +139,11 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     mbar_init(bar_hdone, (uint32_t)CS);
     mbar_init(bar_out, 1);
     mbar_init(bar_outfree, 1);
+    for (int i = 0; i < 2 * kMaxCS; ++i) mbar_init(bar_w2 + i, 1);
     fence_mbar_init();
+    if (one_step)
+      for (int i = 0; i < CS; ++i)
+        if (i != r) mbar_arrive_expect_tx(bar_hfull + i, (uint32_t)slot_bytes);
     fence_proxy_async_smem();
   }
   if (warp == 0) {
@@ -157,9 +173,9 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         return sRing + s * stage_bytes;
       };
       auto advance = [&]() { if (++s == stages) { s = 0; ++round; } };
-      auto load_g1 = [&](int step) {       // first GEMM of this CTA's hidden tile of that step
+      auto load_g1 = [&](int step, int from, int to) {       // first GEMM of this CTA's hidden tile of that step
         const int hid0 = (tile0_of(step) + r) * BH, row0 = row0_of(step);
-        for (int kb = 0; kb < p.kblocks; ++kb) {
+        for (int kb = from; kb < to; ++kb) {
           uint8_t* st = next_stage((uint32_t)(RP * 128 + BH * 128));
           tma_load_2d(st, &tmap_x, bar_full + s, kb * kBK, row0);                          // X [RP rows x 64 k]
           for (int h = 0; h < halves; ++h)                                                 // W1 [64 k x 64 n] blocks
@@ -167,16 +183,30 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
           advance();
         }
       };
-      if (steps > 0) load_g1(0);
-      for (int step = 0; step < steps; ++step) {
-        if (step + 1 < steps) load_g1(step + 1);
+      const int ahead = min(stages, p.kblocks);
+      if (steps > 0) load_g1(0, 0, ahead);
+      if (own_w2 && steps > 0) {             // the whole second GEMM's operand is on its way before the ring comes round
+        for (int i = 0; i < CS; ++i) {
+          const int hid0 = (tile0_of(0) + (int)((r + CS - i) % CS)) * BH;
+          for (int h = 0; h < halves; ++h) {
+            uint64_t* bar = bar_w2 + i * halves + h;
+            uint8_t* st = smem + p.w2_off + (i * halves + h) * p.NC * 128;
+            mbar_arrive_expect_tx(bar, (uint32_t)(p.NC * 128));
+            for (int nb = 0; nb < p.NC; nb += 64) tma_load_2d(st + nb * 128, &tmap_w2, bar, n0 + nb, hid0 + h * 64);
+          }
+        }
+      }
+      if (steps > 0) load_g1(0, ahead, p.kblocks);
+      for (int step = 0; step < steps && !own_w2; ++step) {
+        if (step + 1 < steps) load_g1(step + 1, 0, p.kblocks);
         for (int i = 0; i < CS; ++i) {      // second GEMM over hidden tile t CS + k: two stages of 64 hidden units
           const int k = (int)((r + CS - i) % CS);   // in the order the MMA warp consumes the slots: own tile first
           const int hid0 = (tile0_of(step) + k) * BH;
           for (int h = 0; h < halves; ++h) {
             uint8_t* st = next_stage((uint32_t)(p.NC * 128));
-            for (int nb = 0; nb < p.NC; nb += 64)   // W2 [64 k x 64 n] per block
-              tma_load_2d(st + nb * 128, &tmap_w2, bar_full + s, n0 + nb, hid0 + h * 64);
+#pragma unroll
+            for (int nb = 0; nb < 4; ++nb)          // W2 [64 k x 64 n] per block
+              if (nb * 64 < p.NC) tma_load_2d(st + nb * 8192, &tmap_w2, bar_full + s, n0 + nb * 64, hid0 + h * 64);
             advance();
           }
         }
@@ -228,15 +258,19 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
           const int k = (int)((r + CS - i) % CS);
           mbar_wait(bar_hfull + k, (uint32_t)step & 1u, abort_flag, p.status, 0x704);   // H tile t CS + k is in slot k
           for (int h = 0; h < halves; ++h) {
-            mbar_wait(bar_full + s, (uint32_t)round & 1u, abort_flag, p.status, 0x705);
+            if (own_w2) mbar_wait(bar_w2 + i * halves + h, 0, abort_flag, p.status, 0x70a);
+            else mbar_wait(bar_full + s, (uint32_t)round & 1u, abort_flag, p.status, 0x705);
             tcgen05_fence_after_sync();
             const uint64_t hd = make_smem_desc(smem_u32(sH + k * slot_bytes + h * (RP * 128)), 0, 1024, SW_128B);
-            const uint64_t bd = make_smem_desc(smem_u32(sRing + s * stage_bytes), 8192, 1024, SW_128B);
+            const uint64_t bd = make_smem_desc(own_w2 ? smem_u32(smem) + (uint32_t)(p.w2_off + (i * halves + h) * p.NC * 128) : smem_u32(sRing + s * stage_bytes),
+                                               8192, 1024, SW_128B);
 #pragma unroll
             for (int ks = 0; ks < 4; ++ks)
               umma_bf16_elected_acc(tmem_base + kOutCol, hd + 2u * ks, bd + (uint64_t)((ks * 2048) >> 4), idesc2, elected, (t | i | h | ks) != 0);
-            umma_commit_elected(bar_empty + s, elected);
-            advance();
+            if (!own_w2) {
+              umma_commit_elected(bar_empty + s, elected);
+              advance();
+            }
           }
           // slot k of this CTA has been read: tell its producer (CTA k)
           umma_commit_cluster_elected(cluster_map(smem_u32(bar_hdone), (uint32_t)k), elected);
@@ -253,30 +287,34 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     const bool warp_rows = (warp & 3) * 32 < RP;   // some row of this warp exists
     uint8_t* slot = sH + r * slot_bytes;           // this CTA produces into slot r everywhere
     constexpr int kParts = kEpiWarps / 4;
-    const int pc = BH / kParts;                        // columns per thread: 16 or 32
+    constexpr int pc = BH / kParts;                        // columns per thread: 16 or 32
     cluster_started();
 
     for (int step = 0; step < steps; ++step) {
       const int b = step & 1, t = step % T;
+      const int col0 = part * pc;
+      const float* bb = p.b1 + (size_t)(tile0_of(step) + r) * BH + col0;
+      float4 bv4[pc / 4];                          // the tile's biases travel while its product is made
+#pragma unroll
+      for (int q = 0; q < pc / 4; ++q) bv4[q] = __ldg(reinterpret_cast<const float4*>(bb) + q);
       mbar_wait(bar_hacc + b, (uint32_t)(step >> 1) & 1u, abort_flag, p.status, 0x706);
       tcgen05_fence_after_sync();
       // every CTA has multiplied the previous content of slot r (and the copies that delivered it are complete)
       if (step >= 1) mbar_wait(bar_hdone, (uint32_t)(step - 1) & 1u, abort_flag, p.status, 0x707);
-      const int col0 = part * pc;
       uint8_t* tile = slot + (col0 >> 6) * (RP * 128);
-      const float* bb = p.b1 + (size_t)(tile0_of(step) + r) * BH + col0;
       if (warp_rows) {
-        for (int c0 = 0; c0 < pc; c0 += 16) {
-          uint32_t v[16];
-          tmem_ld_x16(tmem_base + lane_base + b * BH + col0 + c0, v);
-          float4 bv4[4];
+        constexpr int kLd = pc >= 32 ? 32 : 16;    // columns per tensor-memory load
 #pragma unroll
-          for (int q = 0; q < 4; ++q) bv4[q] = __ldg(reinterpret_cast<const float4*>(bb + c0) + q);
+        for (int c0 = 0; c0 < pc; c0 += kLd) {
+          uint32_t v[kLd];
+          if constexpr (kLd == 32) tmem_ld_x32(tmem_base + lane_base + b * BH + col0 + c0, v);
+          else tmem_ld_x16(tmem_base + lane_base + b * BH + col0 + c0, v);
           tmem_ld_wait();
           if (row < RP) {
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
-              const float bv[8] = {bv4[2 * q].x, bv4[2 * q].y, bv4[2 * q].z, bv4[2 * q].w, bv4[2 * q + 1].x, bv4[2 * q + 1].y, bv4[2 * q + 1].z, bv4[2 * q + 1].w};
+            for (int q = 0; q < kLd / 8; ++q) {
+              const float4 lo = bv4[c0 / 4 + 2 * q], hi = bv4[c0 / 4 + 2 * q + 1];
+              const float bv[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
               uint32_t w[4];
 #pragma unroll
               for (int j = 0; j < 4; ++j) {
@@ -299,7 +337,7 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         for (int q = 1; q < CS; ++q) {                                // the peers, starting with the next rank
           const uint32_t peer = (uint32_t)((r + q) % CS);
           const uint32_t rbar = cluster_map(bar, peer);
-          mbar_remote_arrive_expect_tx(rbar, (uint32_t)slot_bytes);
+          if (!one_step) mbar_remote_arrive_expect_tx(rbar, (uint32_t)slot_bytes);
           bulk_copy_to_cluster(cluster_map(src, peer), src, (uint32_t)slot_bytes, rbar);
         }
       }
@@ -339,13 +377,15 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
               if (cb >= blocks) cb -= blocks;
               uint8_t* buf = sRing + (k & 1) * (RP * 256);
               if (warp_rows) {
-                uint32_t v[16];
-                tmem_ld_x16(tmem_base + lane_base + kOutCol + cb * 64 + part * 16, v);
-                tmem_ld_wait();
-                if (row < RP) {
-  #pragma unroll
-                  for (int q = 0; q < 4; ++q)
-                    *reinterpret_cast<uint4*>(buf + row * 256 + ((((part * 4 + q) ^ row) & 15) << 4)) = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                for (int c0 = part * (64 / kParts); c0 < (part + 1) * (64 / kParts); c0 += 16) {
+                  uint32_t v[16];
+                  tmem_ld_x16(tmem_base + lane_base + kOutCol + cb * 64 + c0, v);
+                  tmem_ld_wait();
+                  if (row < RP) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                      *reinterpret_cast<uint4*>(buf + row * 256 + ((((c0 / 4 + q) ^ row) & 15) << 4)) = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                  }
                 }
               }
               named_barrier_sync(1, kEpiThreads);
@@ -414,12 +454,24 @@ __global__ void __launch_bounds__(256) ffn_cluster_finalize_kernel(float* acc, c
 // rows from the start of the last tile whatever RP is).
 int layout(FfnClusterParams* q) {
   q->slot_bytes = q->RP * q->BH * 2;
-  q->stage_bytes = (std::max(q->RP * 128 + q->BH * 128, q->NC * 128) + 1023) & ~1023;
-  const int slots = q->CS * q->slot_bytes, slack = kBM * 128 - q->RP * 128;
+  const int slots = q->CS * q->slot_bytes, g1 = q->RP * 128 + q->BH * 128, w2 = q->CS * (q->BH / 64) * q->NC * 128;
+  q->w2_off = 0;
+  // One step per cluster: where the step's W2 tiles fit beside half of the first GEMM's stages, they get memory of their own and
+  // are requested at once instead of behind the ring.
+  if (q->J > 1 && q->Tp == 1 && w2 >= kBM * 128 && (kSmemMax - slots - w2) / g1 >= (q->kblocks + 1) / 2) {
+    q->stage_bytes = g1;
+    q->stages = std::min(std::min(kMaxStages, q->kblocks), (kSmemMax - slots - w2) / g1);
+    q->slots_off = q->stages * g1;
+    q->w2_off = q->slots_off + slots;            // behind the slots: what the MMAs read past the rows lies in it
+    q->bars_off = q->w2_off + w2;
+    return q->bars_off + 512 + 1024;
+  }
+  const int slack = kBM * 128 - q->RP * 128;
+  q->stage_bytes = (std::max(g1, q->NC * 128) + 1023) & ~1023;      // 32 KB for whole row blocks and tiles of 128 (NC <= 256)
   q->stages = std::min(kMaxStages, (kSmemMax - slots - slack) / q->stage_bytes);
   q->slots_off = q->stages * q->stage_bytes;
   q->bars_off = q->slots_off + slots + slack;
-  return q->bars_off + 256 + 1024;
+  return q->bars_off + 512 + 1024;
 }
 
 // Cluster size, hidden tile and split of the row blocks' hidden tiles over clusters.
@@ -443,13 +495,12 @@ bool choose_split(FfnClusterParams* q, int row_blocks, const int* resident) {
     // Few row blocks: one cluster per block of 128 rows leaves most SMs idle, and the hidden dimension is what can fill
     // them. A row block is split over J clusters (J divides its T steps); their outputs meet in an fp32 buffer in device
     // memory, J additions per element instead of one per hidden tile. J = as many parts as still fit one round of
-    // resident clusters, each with at least one step. With one or two row blocks even that leaves SMs idle: tiles of 64.
-    const int bh_small = FFN_BH64_MAX >= row_blocks ? 64 : 128;
-    for (int bh = bh_small; bh <= 128; bh += 64) {
+    // resident clusters, each with at least one step. Tiles of 64 hidden units where they put more clusters to work (256 rows of
+    // 768 -> 3072: 24 instead of 12, 17.4 -> 13.2 us); otherwise they only stream X twice (512 rows: 18.6 -> 21 us).
+    for (int bh = 128; bh >= 64; bh -= 64) {
       const int T = q->Hid / bh / q->CS;
-      for (int j = T; j >= 2; --j)
+      for (int j = T; j > q->J; --j)
         if (T % j == 0 && (long)row_blocks * j <= resident[q->CS]) { q->BH = bh; q->T = T; q->J = j; break; }
-      if (q->J > 1) break;
     }
   }
   q->Tp = q->T / q->J;
@@ -468,11 +519,17 @@ struct FfnClusterHost {
   std::unordered_map<Key, CUtensorMap, KeyHash> maps;
 };
 
+using ClusterKernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, FfnClusterParams);
+ClusterKernel kernel_of(int bh, bool full) {
+  if (bh == 64) return full ? ffn_cluster_kernel<64, true> : ffn_cluster_kernel<64, false>;
+  return full ? ffn_cluster_kernel<128, true> : ffn_cluster_kernel<128, false>;
+}
+
 void fill_launch(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, const FfnClusterParams& q, int clusters, int smem_bytes,
                  cudaStream_t stream) {
   *cfg = cudaLaunchConfig_t{};
   cfg->gridDim = dim3((unsigned)q.CS, (unsigned)clusters, 1);
-  cfg->blockDim = dim3(kThreads, 1, 1);
+  cfg->blockDim = dim3((unsigned)threads_of(q.BH, q.RP == kBM), 1, 1);
   cfg->dynamicSmemBytes = (size_t)smem_bytes;
   cfg->stream = stream;
   attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -485,21 +542,39 @@ void fill_launch(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* attr, const FfnCl
 
 }  // namespace
 
+namespace {
+constexpr int kResident[kMaxCS + 1] = {0, 0, 74, 45, 33};   // clusters of 1-CTA-per-SM kernels a B200 keeps resident at once
+bool cluster_shape(const Plan& plan, FfnClusterParams* q) {
+  q->K = (int)plan.inputs[0].last();
+  q->M = (int)(plan.inputs[0].numel() / q->K);
+  q->Hid = plan.ops[0].op.p[0];
+  q->N2 = plan.ops[3].op.p[0];
+  if (q->K % kBK != 0 || q->Hid % 128 != 0) return false;
+  q->kblocks = q->K / kBK;
+  q->RP = std::min(kBM, (q->M + 15) / 16 * 16);
+  return choose_split(q, (q->M + kBM - 1) / kBM, kResident);
+}
+}  // namespace
+
+// Steps of the longest cluster x ring stages per step (0.52 us for 32 KB; where the W2 tiles have stages of their own, the bytes
+// count) + set-up and end; split row blocks: the second launch and the additions (3 T bytes/s). Within 12 % of the measured
+// times from 1 to 7000 rows at widths of 256 to 1024.
+double ffn_cluster_estimate(const Plan& plan) {
+  FfnClusterParams q{};
+  if (!cluster_shape(plan, &q)) return -1.0;
+  layout(&q);
+  const double units = (double)((q.M + kBM - 1) / kBM) * q.J, rounds = std::ceil(units / kResident[q.CS]);
+  const double w2_stages = q.CS * (q.BH / 64);
+  const double bytes = q.w2_off > 0 ? q.kblocks * (double)q.stage_bytes + w2_stages * q.NC * 128.0 : (q.kblocks + w2_stages) * q.stage_bytes;
+  return rounds * q.Tp * bytes / 32768.0 * 0.52 + (q.J > 1 ? 5.0 + (double)q.J * q.M * q.N2 * 4 / 3.0e6 : 4.0);
+}
+
 // AGO_ERR_UNSUPPORTED (without touching *err) when the shape has no cluster split: the caller falls back to the
 // kernel that tiles the second GEMM's reduction across independent CTAs.
 ago_status_t ffn_cluster_plan(Plan* plan, FusedState* st, std::string* err) {
   (void)err;
   FfnClusterParams q{};
-  q.K = (int)plan->inputs[0].last();
-  q.M = (int)(plan->inputs[0].numel() / q.K);
-  q.Hid = plan->ops[0].op.p[0];
-  q.N2 = plan->ops[3].op.p[0];
-  if (q.K % kBK != 0 || q.Hid % 128 != 0) return AGO_ERR_UNSUPPORTED;
-  const int resident[kMaxCS + 1] = {0, 0, 74, 45, 33};   // clusters of 1-CTA-per-SM kernels a B200 keeps resident at once
-  const int row_blocks_plan = (q.M + kBM - 1) / kBM;
-  q.RP = std::min(kBM, (q.M + 15) / 16 * 16);
-  if (!choose_split(&q, row_blocks_plan, resident)) return AGO_ERR_UNSUPPORTED;
-  q.kblocks = q.K / kBK;
+  if (!cluster_shape(*plan, &q)) return AGO_ERR_UNSUPPORTED;
   auto* host = new FfnClusterHost();
   host->smem_bytes = layout(&q);
   host->prm = q;
@@ -566,17 +641,19 @@ ago_status_t ffn_cluster_run(const Plan& plan, FusedState* st, const void* const
   CUtensorMap mx, mw1, mw2;
   if (!get_map(inputs[0], 0, &mx) || !get_map(weights[0], 1, &mw1) || !get_map(weights[2], 2, &mw2)) return AGO_ERR_CUDA;
   {
-    static int smem_opt_in[64] = {};
-    cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(ffn_cluster_kernel), smem_opt_in);
+    static int smem_opt_in[4][64] = {};
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(kernel_of(i & 1 ? 128 : 64, (i & 2) != 0)), smem_opt_in[i]);
     if (e != cudaSuccess) { *err = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e); return AGO_ERR_CUDA; }
   }
+  const auto kernel = kernel_of(q.BH, q.RP == kBM);
   cudaLaunchConfig_t cfg; cudaLaunchAttribute attr[2];
   const int row_blocks = (q.M + kBM - 1) / kBM;
   if (host->clusters == 0) {
     // persistent clusters: as many as the device keeps resident at once (one CTA per SM, CS SMs of one GPC each)
     fill_launch(&cfg, attr, q, row_blocks * q.J, host->smem_bytes, stream);
     int resident = 0;
-    cudaError_t e = cudaOccupancyMaxActiveClusters(&resident, ffn_cluster_kernel, &cfg);
+    cudaError_t e = cudaOccupancyMaxActiveClusters(&resident, kernel, &cfg);
     if (e != cudaSuccess || resident < 1) {
       *err = std::string("fused feed-forward (cluster): no cluster of this size is schedulable: ") + cudaGetErrorString(e);
       return AGO_ERR_CUDA;
@@ -584,7 +661,7 @@ ago_status_t ffn_cluster_run(const Plan& plan, FusedState* st, const void* const
     host->clusters = std::min(row_blocks * q.J, resident);
   }
   fill_launch(&cfg, attr, q, host->clusters, host->smem_bytes, stream);
-  cudaError_t e = cudaLaunchKernelEx(&cfg, ffn_cluster_kernel, mx, mw1, mw2, q);
+  cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, mx, mw1, mw2, q);
   if (e != cudaSuccess) { *err = std::string("fused feed-forward (cluster) launch: ") + cudaGetErrorString(e); return AGO_ERR_CUDA; }
   if (q.J > 1) {
     const long long total4 = (long long)q.M * q.N2 / 4;

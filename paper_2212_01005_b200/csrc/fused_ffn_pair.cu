@@ -431,12 +431,13 @@ __global__ void __launch_bounds__(256) ffn_pair_finalize_kernel(const float* acc
 }
 
 // How the blocks of 256 rows are dealt to the resident clusters: the whole rounds as they are; the blocks of a last,
-// partial round are split into the largest J (a divisor of the S steps) whose parts still fit one round.
+// partial round -- all of them, when there is no whole one -- are split into the largest J (a divisor of the S steps) whose
+// parts still fit one round.
 void pair_split(int units, int S, int* units_whole, int* J) {
   const int resident = device_sm_count() >= 148 ? 33 : std::max(1, device_sm_count() / 4 - 4);   // clusters of 4 (1 CTA per SM): 33 on a B200
   *units_whole = units; *J = 1;
   const int full = units / resident, rest = units % resident;
-  if (full < 1 || rest == 0) return;
+  if (rest == 0) return;
   for (int j = S; j >= 2; --j)
     if (S % j == 0 && rest * j <= resident) { *units_whole = full * resident; *J = j; return; }
 }
@@ -478,27 +479,42 @@ size_t ffn_pair_workspace_bytes(const Plan& plan) {
   return ((size_t)J * (size_t)(M - (int64_t)whole * 2 * kFM) * N2 * 4 + 255) & ~size_t(255);   // J planes over the rows of the split blocks
 }
 
+namespace {
+bool pair_shape(const Plan& plan, FfnPairParams* q) {
+  q->K = (int)plan.inputs[0].last();
+  q->M = (int)(plan.inputs[0].numel() / q->K);
+  q->Hid = plan.ops[0].op.p[0];
+  q->N2 = plan.ops[3].op.p[0];
+  if (q->K % kFK != 0 || q->Hid % (2 * kFH) != 0 || q->N2 % 256 != 0 || q->N2 > 768) return false;
+  q->NC = q->N2 / 2;
+  q->S = q->Hid / (2 * kFH);
+  q->kblocks = q->K / kFK;
+  q->units = (q->M + 2 * kFM - 1) / (2 * kFM);
+  pair_split(q->units, q->S, &q->units_whole, &q->J);
+  q->split_rows = q->M - q->units_whole * 2 * kFM;
+  return true;
+}
+}  // namespace
+
+// Steps of the longest cluster x the bytes a CTA streams per step (24 KB in 0.42 us) + set-up and end; split blocks: the second
+// launch and the fp32 planes, written and read at 3 TB/s. Within 8 % of the measured times from 2048 to 12288 rows.
+double ffn_pair_estimate(const Plan& plan) {
+  FfnPairParams q{};
+  if (!pair_shape(plan, &q)) return -1.0;
+  const int resident = device_sm_count() >= 148 ? 33 : std::max(1, device_sm_count() / 4 - 4);
+  const double steps = (double)((q.units_whole + resident - 1) / resident) * q.S + (q.J > 1 || q.units_whole < q.units ? q.S / q.J : 0);
+  const double bytes = q.kblocks * 24576.0 + 4.0 * q.N2 / 4 * 128;
+  return steps * bytes / 24576.0 * 0.42 + 5.0 + (q.J > 1 ? 3.0 + 2.0 * q.J * q.split_rows * (double)q.N2 * 4 / 3.0e6 : 0.0);
+}
+
 ago_status_t ffn_pair_plan(Plan* plan, FusedState* st, std::string* err) {
   (void)err;
   FfnPairParams q{};
-  q.K = (int)plan->inputs[0].last();
-  q.M = (int)(plan->inputs[0].numel() / q.K);
-  q.Hid = plan->ops[0].op.p[0];
-  q.N2 = plan->ops[3].op.p[0];
-  if (q.K % kFK != 0 || q.Hid % (2 * kFH) != 0 || q.N2 % 256 != 0 || q.N2 > 768) return AGO_ERR_UNSUPPORTED;
-  q.NC = q.N2 / 2;
-  q.S = q.Hid / (2 * kFH);
-  q.kblocks = q.K / kFK;
-  q.units = (q.M + 2 * kFM - 1) / (2 * kFM);
-  // worth it only when the clusters (four SMs each) fill most of the device
-  if ((long)q.units * 4 < (long)device_sm_count() * 3 / 4) return AGO_ERR_UNSUPPORTED;
+  if (!pair_shape(*plan, &q)) return AGO_ERR_UNSUPPORTED;
   auto* host = new FfnPairHost();
   host->prm = q;
   st->impl = host;
   st->impl_free = [](void* p) { delete static_cast<FfnPairHost*>(p); };
-  pair_split(q.units, q.S, &q.units_whole, &q.J);
-  q.split_rows = q.M - q.units_whole * 2 * kFM;
-  host->prm = q;
   st->variant = 3;
   plan->fused_variant = 3;
   if (q.J > 1) {
@@ -559,7 +575,7 @@ ago_status_t ffn_pair_run(const Plan& plan, FusedState* st, const void* const* i
       *err = std::string("fused feed-forward (paired cluster): no cluster of four is schedulable: ") + cudaGetErrorString(e);
       return AGO_ERR_CUDA;
     }
-    host->clusters = std::min(q.units, resident);
+    host->clusters = std::min(q.units_whole + (q.units - q.units_whole) * q.J, resident);
   }
   fill_pair_launch(&cfg, attr, host->clusters, stream);
   cudaError_t e = cudaLaunchKernelEx(&cfg, ffn_pair_kernel, mx, mw1, mw2, q);

@@ -343,6 +343,16 @@ bool pair_epilogue(const EpiProgram& e, GemmPairParams* p) {
 
 }  // namespace
 
+static long pair_tiles(const GemmArgs& a, int bn) { return (long)((a.M + 255) / 256) * ((a.N + bn - 1) / bn); }
+// Columns per tile: 256 (128 flop per byte that crosses L2 -> SM), or 128 where tiles of 256 would leave half of the pairs idle or
+// fill a last round by less than a third (rounds x bytes per K block: 64 against 48 KB).
+static int pair_columns(const GemmArgs& a) {
+  if (a.N <= 128) return 128;
+  const long pairs = device_sm_count() / 2;
+  const long wide = (pair_tiles(a, 256) + pairs - 1) / pairs * 64, narrow = (pair_tiles(a, 128) + pairs - 1) / pairs * 48;
+  return narrow < wide ? 128 : 256;
+}
+
 // Unbatched products with enough rows to fill the SM pairs (wide or narrow, long or short reductions: the narrow,
 // short ones -- 1x1 convolutions of a few tens of channels -- are bound by the output stream, which the persistent
 // pairs overlap with the next tile's loads and products); everything else stays on the small-tile kernel.
@@ -355,16 +365,43 @@ bool gemm_pair_supported(const GemmArgs& a) {
   if (!a.a_im2col && a.lda % 8 != 0) return false;
   if (probe.add && a.c_dtype != AGO_BF16) return false;   // the added tensor has the I/O dtype of a bf16 subgraph
   if (a.M < 512) return false;
-  // worth it once the 256-row tiles fill most of the SM pairs
-  const long tiles = (long)((a.M + 255) / 256) * ((a.N + 255) / 256);
-  return tiles * 2 >= device_sm_count() / 2;
+  // worth it once the 256-row tiles (of 256 or 128 columns) fill most of the SM pairs
+  return pair_tiles(a, pair_columns(a)) * 2 >= device_sm_count() / 2;
+}
+
+// The chain as two GEMM launches. Per launch 5.5 us + rounds x K blocks x the time of a block: 0.5 / 0.375 us for a pair of CTAs
+// (tiles of 256 / 128 columns), 0.33 / 0.25 us for one CTA (128 / 64 columns). Within 10 % of the measured times from 512 to 12288
+// rows at widths of 256 to 1024.
+double ffn_unfused_estimate(const Plan& plan) {
+  GemmArgs a{};
+  a.a_dtype = a.c_dtype = AGO_BF16;
+  a.batches = 1;
+  double us = 0.0;
+  int K = (int)plan.inputs[0].last();
+  a.M = (int)(plan.inputs[0].numel() / K);
+  for (int i : {0, 3}) {
+    a.K = K; a.N = plan.ops[i].op.p[0];
+    a.lda = K; a.ldb = a.ldc = a.N;
+    const int kblocks = (K + 63) / 64;
+    if (gemm_pair_supported(a)) {
+      const int bn = pair_columns(a);
+      const long pairs = device_sm_count() / 2, rounds = (pair_tiles(a, bn) + pairs - 1) / pairs;
+      us += 5.5 + rounds * kblocks * (bn == 256 ? 0.5 : 0.375);
+    } else {
+      const int bn = gemm_tc_columns(a);
+      const long ctas = (long)((a.M + 127) / 128) * ((a.N + bn - 1) / bn), sms = device_sm_count();
+      us += 5.5 + (ctas + sms - 1) / sms * kblocks * (bn == 128 ? 0.33 : 0.25);
+    }
+    K = a.N;
+  }
+  return us;
 }
 
 cudaError_t launch_gemm_pair(const GemmArgs& a, cudaStream_t stream) {
   GemmPairParams p{};
   pair_epilogue(a.epi, &p);
   p.M = a.M; p.N = a.N; p.K = a.K;
-  p.BN = a.N > 128 ? 256 : 128;
+  p.BN = pair_columns(a);
   p.b_kmajor = a.b_kmajor;
   p.c_fp32 = a.c_dtype == AGO_FP32 ? 1 : 0;
   p.kblocks = (a.K + kPK - 1) / kPK;

@@ -26,10 +26,12 @@ namespace {
 
 using namespace tc;
 
-constexpr int kBM = 128, kBN = 128, kBK = 64;
-constexpr int kMaxStages = 4;   // ring stages: 3 when the grid exceeds one CTA per SM (two CTAs then share an SM and one CTA's epilogue
-                                // overlaps the other's products), else 4; never more than the K blocks
-constexpr int kStageBytes = 32 * 1024;
+constexpr int kBM = 128, kBK = 64;
+// Ring stages: 3 when the grid exceeds one CTA per SM (two CTAs then share an SM and one CTA's epilogue overlaps the other's
+// products), else as many as fit -- a lone CTA's stream is its bytes in flight over the latency, and with four stages a product
+// with 48 K blocks took 0.5 us per block -- but never more than the K blocks.
+constexpr int kMaxStages = 9;
+constexpr int kSmemMax = 227 * 1024;
 constexpr int kEpiThreads = 128;
 constexpr int kThreads = kEpiThreads + 64;   // + TMA warp + MMA warp
 
@@ -38,6 +40,7 @@ struct GemmTcParams {
   int M, N, K;
   int64_t ldc;
   int b_kmajor;
+  int BN;                  // columns per tile: 128, or 64 where 128 would leave half of the SMs without a tile
   int c_dtype, add_dtype;
   int kblocks, stages;
   int heads;               // blockIdx.z = batch * heads + head
@@ -67,7 +70,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sRing = smem;
-  const int kStages = p.stages;
+  const int kStages = p.stages, kBN = p.BN, kStageBytes = 16384 + kBN * 128;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.bar_off);
   uint64_t* bar_full = bars;
   uint64_t* bar_empty = bars + kMaxStages;
@@ -112,7 +115,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
           tma_load_4d(st + 16384, &tmap_b, bar_full + s, i * kBK, n0, zh, zb);  // B [128 n x 64 k]
         } else {
           tma_load_4d(st + 16384, &tmap_b, bar_full + s, n0, i * kBK, zh, zb);  // B [64 k x 64 n], twice
-          tma_load_4d(st + 16384 + 8192, &tmap_b, bar_full + s, n0 + 64, i * kBK, zh, zb);
+          if (kBN > 64) tma_load_4d(st + 16384 + 8192, &tmap_b, bar_full + s, n0 + 64, i * kBK, zh, zb);
         }
       }
     }
@@ -283,6 +286,12 @@ bool gemm_tc_supported(const GemmArgs& a) {
   return true;
 }
 
+// 128 x 64 tiles where 128 x 128 tiles would use less than half of the SMs: twice the CTAs, 24 instead of 32 KB per K block each.
+int gemm_tc_columns(const GemmArgs& a) {
+  const long tiles = (long)((a.M + kBM - 1) / kBM) * std::max(a.batches, 1) * ((a.N + 127) / 128);
+  return a.N > 64 && tiles * 2 > device_sm_count() ? 128 : 64;
+}
+
 cudaError_t launch_gemm_tc(const GemmArgs& a, int add_dtype, cudaStream_t stream) {
   CUtensorMap ma, mb;
   const int heads = a.batches > 1 ? std::max(a.heads, 1) : 1, nb = std::max(a.batches, 1) / heads;
@@ -291,6 +300,7 @@ cudaError_t launch_gemm_tc(const GemmArgs& a, int add_dtype, cudaStream_t stream
   const int64_t a_sh = a.batches > 1 ? a.a_sh : lda * a.M, a_sb = a.batches > 1 ? a.a_sb : lda * a.M;
   const int64_t b_rows = a.b_kmajor ? a.N : a.K;
   const int64_t b_sh = a.batches > 1 ? a.b_sh : a.ldb * b_rows, b_sb = a.batches > 1 ? a.b_sb : a.ldb * b_rows;
+  const int kBN = gemm_tc_columns(a);
   if (!get_map(a.A, a.K, a.M, heads, nb, lda, a_sh, a_sb, kBK, kBM, &ma)) return cudaErrorInvalidValue;
   if (a.b_kmajor ? !get_map(a.B, a.K, a.N, heads, nb, a.ldb, b_sh, b_sb, kBK, kBN, &mb)
                  : !get_map(a.B, a.N, a.K, heads, nb, a.ldb, b_sh, b_sb, 64, kBK, &mb)) return cudaErrorInvalidValue;
@@ -302,19 +312,18 @@ cudaError_t launch_gemm_tc(const GemmArgs& a, int add_dtype, cudaStream_t stream
   canonical_epilogue(a.epi, &p);
   p.status = a.status;
   const long ctas = (long)((a.M + kBM - 1) / kBM) * ((a.N + kBN - 1) / kBN) * heads * nb;
-  p.stages = std::min(ctas > device_sm_count() ? 3 : kMaxStages, p.kblocks);
+  const int stage_bytes = 16384 + kBN * 128;
+  p.BN = kBN;
+  p.stages = std::min(ctas > device_sm_count() ? 3 : std::min(kMaxStages, (kSmemMax - 1280) / stage_bytes), p.kblocks);
   // the epilogue stages the output tile (128 rows x (columns x element size + 16) bytes) over the idle ring
   const int tile_cols = std::min(kBN, (a.N + 15) & ~15);
   const int staging = kBM * (tile_cols * (a.c_dtype == AGO_FP32 ? 4 : 2) + 16);
-  p.bar_off = (std::max(p.stages * kStageBytes, staging) + 1023) & ~1023;
+  p.bar_off = (std::max(p.stages * stage_bytes, staging) + 1023) & ~1023;
   const int smem = p.bar_off + 256 + 1024;
-  const int smem_max = kMaxStages * kStageBytes + 256 + 1024;
-  static std::once_flag once[64];
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+
+  static int smem_opt_in[64] = {};
+  const cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(gemm_tc_kernel), smem_opt_in);
   if (e != cudaSuccess) return e;
-  if (dev >= 0 && dev < 64)
-    std::call_once(once[dev], [&] { cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max); });
   dim3 grid((a.M + kBM - 1) / kBM, (a.N + kBN - 1) / kBN, heads * nb);
   FusedLaunch launch(grid, kThreads, (size_t)smem, stream);
   return cudaLaunchKernelEx(&launch.config, gemm_tc_kernel, ma, mb, p);

@@ -56,3 +56,48 @@ def test_split_channels_repeat_within_the_order_of_the_groups(ago):
     for o in outs[1:]:
         assert float((o.float() - outs[0].float()).abs().max()) <= 2.0 ** -7 * scale
     sg.close()
+
+
+@pytest.mark.parametrize("rows", [1, 15, 16, 17, 63, 64, 65, 127, 128, 129, 256, 257, 513])
+def test_feed_forward_few_rows(ago, rows):
+    # rows kept in shared memory (16 .. 128), direct and staged additions (64 rows), one to five row blocks; hidden tiles of 64
+    check(ago, WL.ffn("ffn_rows", [204, rows], rows, 192, 1024, 1, d_out=512))
+
+
+@pytest.mark.parametrize("shape", [
+    # rows, d, hidden, d_out: the second GEMM's tiles behind the ring and in stages of their own, clusters of 2, 3 and 4, one and
+    # more steps per cluster, tiles of 64 and of 128; whole row blocks without a split (24 blocks); paired clusters all split
+    (40, 64, 256, 128), (100, 256, 768, 192), (100, 1024, 4096, 1024), (200, 128, 384, 768), (300, 64, 2048, 256),
+    (700, 320, 1536, 384), (1500, 128, 768, 512), (3001, 128, 512, 256), (2500, 192, 3072, 768),
+])
+def test_feed_forward_splits(ago, shape):
+    rows, d, hidden, d_out = shape
+    check(ago, WL.ffn("ffn_splits", [205, *shape], rows, d, hidden, 1, d_out=d_out))
+
+
+def test_feed_forward_few_rows_leave_the_sums_clean(ago):
+    # the fp32 buffer of the split row blocks is zeroed by the run itself: many runs in flight agree with the first one
+    import torch
+    from helpers import to_device
+    wl = WL.ffn("ffn_clean", [206], 40, 256, 1024, 1)
+    data = WL.generate(wl)
+    sg = ago.Subgraph(wl.ops, wl.input_shapes, mode="fused")
+    ins, ws = to_device(wl, data)
+    outs = [sg.run(ins, ws) for _ in range(20)]
+    torch.cuda.synchronize()
+    assert sg.status() == ago.AGO_OK, ago.ago_last_error()
+    scale = float(outs[0].float().abs().max())
+    for o in outs[1:]:
+        assert float((o.float() - outs[0].float()).abs().max()) <= 2.0 ** -7 * scale     # one bf16 step: the order of the additions
+    sg.close()
+
+
+@pytest.mark.parametrize("shape", [
+    # rows, K, N of one GEMM + bias + GELU: tiles of 128 x 64 (few tiles; N a remainder of 64), 128 x 128, pairs with tiles of 256
+    # and of 128 columns (N a remainder of either), more K blocks than ring stages and fewer
+    (70, 72, 40), (130, 1024, 72), (500, 640, 136), (600, 64, 2056), (2100, 768, 200), (3001, 200, 776), (4097, 64, 1032), (19000, 96, 264),
+])
+def test_unfused_gemm_tiles(ago, shape):
+    rows, k, n = shape
+    ops = [("gemm", dict(N=n)), ("bias_add", {}), ("gelu_tanh", {})]
+    check(ago, WL.Workload("gemm_tiles", [207, *shape], [(rows, k)], ops, samples=1), mode="per_mini_subgraph")
