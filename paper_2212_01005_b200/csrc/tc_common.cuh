@@ -200,9 +200,13 @@ __device__ __forceinline__ void umma_commit_cluster(uint32_t bar_cluster_addr) {
 __device__ __forceinline__ void cp_async_16(uint32_t dst_saddr, const void* src, uint32_t src_bytes) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst_saddr), "l"(src), "r"(src_bytes) : "memory");
 }
+// ... through L1: for what the CTAs of an SM all read (whole 128-byte lines are requested, once per SM)
+__device__ __forceinline__ void cp_async_16_l1(uint32_t dst_saddr, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst_saddr), "l"(src) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-// all of this thread's commit groups but the most recent one are complete
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+// all of this thread's commit groups but the most recent one are complete
 __device__ __forceinline__ void cp_async_wait_but_one() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 
 // ---- TMA (cp.async.bulk.tensor), every load into the issuing CTA only ---------------------

@@ -101,3 +101,38 @@ def test_unfused_gemm_tiles(ago, shape):
     rows, k, n = shape
     ops = [("gemm", dict(N=n)), ("bias_add", {}), ("gelu_tanh", {})]
     check(ago, WL.Workload("gemm_tiles", [207, *shape], [(rows, k)], ops, samples=1), mode="per_mini_subgraph")
+
+
+@pytest.mark.parametrize("shape", [
+    # pixels, c_in, c_mid, c_out: one tile of 32 rows per SM and around it, of 128 rows, two CTAs per SM, two rounds
+    (1, 64, 32, 64), (32, 96, 24, 96), (33, 8, 8, 8), (4736, 64, 32, 64), (4737, 64, 24, 72), (18944, 64, 32, 64), (18945, 72, 24, 64),
+    (37889, 48, 16, 48),
+    # two rounds with one CTA per SM; with two CTAs per SM whose products share their columns; padding in every operand
+    (18945, 256, 64, 256), (37889, 64, 64, 256), (40000, 24, 40, 88),
+])
+def test_pointwise_pair_tiles(ago, shape):
+    m, c0, c1, c2 = shape
+    check(ago, WL.pw_pw("pw_pw_edges", [207, *shape], m, 1, c0, c1, c2, act1=True))
+
+
+@pytest.mark.parametrize("shape", [(5, 9, 421, 96, 192), (3, 4, 3200, 64, 256), (1, 9, 2113, 40, 24)])
+def test_unfold_chain_rounds(ago, shape):
+    check(ago, WL.unfold_chain("unfold_edges", [208, *shape], *shape))
+
+
+def test_pointwise_pair_output_between_sectors(ago):
+    # an output 16 but not 32 bytes aligned: rows are stored in halves
+    import torch
+    from helpers import to_device
+    wl = WL.pw_pw("pw_pw_offset", [209], 3, 20, 64, 32, 64)
+    data = WL.generate(wl)
+    sg = ago.Subgraph(wl.ops, wl.input_shapes, mode="fused")
+    ins, ws = to_device(wl, data)
+    ref = sg.run(ins, ws)
+    flat = torch.zeros(ref.numel() + 16, dtype=ref.dtype, device=ref.device)
+    out = flat[8:8 + ref.numel()].view(ref.shape)
+    sg.run(ins, ws, out=out)
+    torch.cuda.synchronize()
+    assert sg.status() == ago.AGO_OK and torch.equal(out, ref)
+    assert not flat[:8].any() and not flat[-8:].any()
+    sg.close()
