@@ -136,3 +136,34 @@ def test_pointwise_pair_output_between_sectors(ago):
     assert sg.status() == ago.AGO_OK and torch.equal(out, ref)
     assert not flat[:8].any() and not flat[-8:].any()
     sg.close()
+
+
+@pytest.mark.parametrize("fp32", [True, False])
+@pytest.mark.parametrize("shape", [
+    # n, h, w, c, stride: one pixel, one row, one column, fewer pixels than a piece; even and odd sizes at stride 2
+    (1, 1, 1, 8, 1), (1, 1, 9, 16, 2), (3, 7, 1, 8, 1), (1, 3, 2, 24, 2), (2, 6, 5, 8, 1),
+    # two rows by two and by four columns, four rows by four and by eight, each with ragged last pieces
+    (5, 27, 13, 56, 1), (19, 23, 23, 64, 1), (23, 29, 21, 88, 1), (21, 45, 37, 144, 1),
+    (19, 29, 27, 96, 2), (9, 53, 51, 128, 2), (13, 73, 67, 144, 2), (15, 93, 91, 176, 2),
+])
+def test_depthwise_strips(ago, shape, fp32):
+    n, h, w, c, stride = shape
+    ops = [("conv2d", dict(O=c, R=3, S=3, stride=stride, pad=1, groups=c)), ("bias_add", {}), ("relu6", {})]
+    wl = WL.Workload("dw_edges", [210, *shape], [(n, h, w, c)], ops, samples=n, input_dist=["normal"])
+    data = WL.generate(wl)
+    ref = O.run_chain(wl.ops, data["inputs"], data["weights"])
+    out = run_gpu(ago, wl, data, "auto", fp32=fp32)
+    if fp32:   # nine products and a bias, each sum rounded: 10 x 2^-24 of the sum of the magnitudes, itself below 9 x 5 max
+        assert abs(out - ref).max() <= 1e-5 * max(1.0, abs(ref).max())
+    else:
+        assert_close(out, ref, what=f"depthwise {shape}")
+
+
+@pytest.mark.parametrize("ops", [
+    [], [("relu", {})], [("bias_add", {})], [("bias_add", {}), ("relu", {})], [("bias_add", {}), ("gelu_tanh", {})],
+    [("scale", dict(f=0.5)), ("bias_add", {}), ("relu6", {})], [("bias_add", {}), ("add_input", dict(input=0)), ("relu", {})],
+])
+def test_depthwise_strips_epilogues(ago, ops):
+    wl = WL.Workload("dw_epilogues", [211], [(3, 22, 19, 40)], [("conv2d", dict(O=40, R=3, S=3, stride=1, pad=1, groups=40))] + ops,
+                     samples=3, input_dist=["normal"])
+    check(ago, wl, "auto")
