@@ -62,6 +62,7 @@ constexpr int kTilesPerWarp = 4;                   // expand-epilogue tiles per 
 constexpr int kExpandIssuers = 2;                  // the last two warps of a group issue its expand GEMMs
 constexpr int kChunk = 16;      // expanded channels per chunk = one MMA K step of the project GEMM
 constexpr int kChunkRowBytes = 32;
+constexpr int kMaxPieces = 2;   // of the partial sums that the CTAs of a cluster exchange
 
 struct Mbv2Params {
   const __nv_bfloat16* x;
@@ -78,7 +79,8 @@ struct Mbv2Params {
   int PP;                       // CS > 1: output pixels of a strip that one CTA of the cluster sums up and stores (odd)
   int off_send, off_recv, recv_shared;   // CS > 1: blocks of partial sums for / from the other CTAs; recv_shared: over dead operands
   int kblocks, ksteps, cpr;     // reduction of the expand GEMM: 128-byte-row blocks, MMA steps, 16-byte chunks per row (kblocks > 1)
-  uint32_t pp_recip, cpr_recip, cout8_recip;
+  int piece_cgs;                // ... sent by pieces of piece_cgs x 16 output channels
+  uint32_t pp_recip, cpr_recip, c8s_recip, c8s_last_recip;
   int groups;                   // warp groups: 2 or 4 (the kernel template's NG)
   int fold_b1;                  // the expand bias rides in two spare reduction channels of the expand GEMM (Cin < Kp)
   int R, strips, IH, IW, P_x, P_in, M1, M2;   // P_x = IH * W pixels in the input tile, P_in = IH * IW in an E chunk
@@ -136,7 +138,7 @@ mbv2_fused_kernel(const Mbv2Params p) {
   uint64_t* bar_done = bars + 17;   // every project MMA complete (the groups do not follow each other's bar_d phases)
   uint64_t* bar_chain = bars + 18;  // two groups: group 0's first expand GEMM complete. One phase only: a waiter on bar_e could
                                     // fall behind its next phase and then wait for a parity that has come and gone
-  uint64_t* bar_red = bars + 19;    // the partial sums of the other CTAs of the cluster have arrived
+  uint64_t* bar_red = bars + 12;    // [kMaxPieces] a piece of the partial sums of the other CTAs of the cluster has arrived
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 20);
   volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 21);
 
@@ -158,7 +160,7 @@ mbv2_fused_kernel(const Mbv2Params p) {
     }
     mbar_init(bar_first, (uint32_t)p.M2);
     mbar_init(bar_chain, kExpandIssuers);
-    mbar_init(bar_red, 1);
+    for (int k = 0; k < kMaxPieces; ++k) mbar_init(bar_red + k, 1);
     mbar_init(bar_done, (uint32_t)(p.M2 * min(p.NC, NG)));
     fence_mbar_init();
     fence_proxy_async_smem();
@@ -226,12 +228,15 @@ mbv2_fused_kernel(const Mbv2Params p) {
           cp_async_16(s0 + p.off_w3 + (j >> 1) * p.Coutp * kChunkRowBytes + swz_offset(row, j & 1, kChunkRowBytes),
                       in ? w3p + ((uint32_t)row * p.Cfull + j * 8) * 2 : none, in ? 16u : 0u);
         });
-        if (tid < (p.Cout >> 2)) cp_async_16(s0 + p.off_b3 + tid * 16, reinterpret_cast<const uint8_t*>(p.b3) + tid * 16, 16u);   // Cout <= 256
       }
-      for (int i = tid; i < (p.Cexp >> 2); i += kThreads) {
-        cp_async_16(s0 + p.off_bd + i * 16, reinterpret_cast<const uint8_t*>(p.bd + ch0) + i * 16, 16u);
-        if (EXPAND && !FOLD) cp_async_16(s0 + p.off_b1 + i * 16, reinterpret_cast<const uint8_t*>(p.b1 + ch0) + i * 16, 16u);
-      }
+      // the biases, each by warps of its own: what a few warps run alone they also fetch the instructions for alone
+      auto stage_bias = [&](int first_warp, int off, const float* b, int count) {
+        const int i = (tid - first_warp * 32) & (kThreads - 1);
+        for (int j = i; j < (count >> 2); j += kThreads) cp_async_16(s0 + off + j * 16, reinterpret_cast<const uint8_t*>(b) + j * 16, 16u);
+      };
+      stage_bias(4, p.off_bd, p.bd + ch0, p.Cexp);
+      if (PROJECT) stage_bias(8, p.off_b3, p.b3, p.Cout);
+      if (EXPAND && !FOLD) stage_bias(12, p.off_b1, p.b1 + ch0, p.Cexp);
     };
     // ---- per-thread work mapping: needs no device memory, so it runs before the wait for the previous grid of the
     // stream (with back-to-back launches it overlaps that grid's tail) ----
@@ -315,14 +320,14 @@ mbv2_fused_kernel(const Mbv2Params p) {
       }
       cp_async_commit();
     };
+    if (warp == kWarps - 2) {      // before the wait: an allocation takes 400 cycles
+      tmem_alloc(tmem_slot, (uint32_t)p.tmem_cols);
+      tmem_relinquish();
+    }
     grid_dependency_wait();      // first access to device memory below
     grid_launch_dependents();
     if (!EXPAND) { load_chunk(g, 0); load_chunk(g + NG, 1); }   // the first two chunks travel while the weights are staged
     stage();
-    if (warp == 0) {
-      tmem_alloc(tmem_slot, (uint32_t)p.tmem_cols);
-      tmem_relinquish();
-    }
     // the zero padding columns of the two E chunk buffers (written once: every chunk reuses them)
     constexpr int kEPlanes = (EXPAND ? NG : 2 * NG) * 2;   // one E buffer per group (two when the chunks are copied in), two planes each
     for (int i = tid; i < p.IH * 2 * kEPlanes; i += kThreads) {
@@ -440,7 +445,9 @@ mbv2_fused_kernel(const Mbv2Params p) {
   tcgen05_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
     if (PROJECT && p.CS > 1) {
-      if (tid == 0) mbar_arrive_expect_tx(bar_red, (uint32_t)((p.CS - 1) * p.Coutp * p.PP * 4));
+      if (tid == 0)
+        for (int k = 0, cg = 0; cg < (p.Coutp >> 4); ++k, cg += p.piece_cgs)
+          mbar_arrive_expect_tx(bar_red + k, (uint32_t)((p.CS - 1) * min(p.piece_cgs, (p.Coutp >> 4) - cg) * 64 * p.PP));
       __syncwarp();
       if (!p.recv_shared) cluster_arrive();       // the barrier is armed: the others may send from now on
     }
@@ -596,60 +603,70 @@ mbv2_fused_kernel(const Mbv2Params p) {
       if (p.CS > 1) {
         // ---- the channel shares of the cluster's CTAs are added: CTA r sums and stores pixels [r PP, (r + 1) PP) of the
         // strip. A CTA lays its fp32 partial sums out as one block [4 channels][pixel] per owner (over its own operands,
-        // which are dead now) and sends each block by one bulk copy (single 16-byte stores into the other CTAs took
-        // three times as long). Where the incoming blocks have no memory of their own they go over operands too, so the
+        // which are dead now) and sends each block by bulk copies (single 16-byte stores into the other CTAs took
+        // three times as long), a piece of some output channels at a time: a piece travels while the next is laid out and the
+        // previous one summed up. Where the incoming blocks have no memory of their own they go over operands too, so the
         // cluster meets once more before anything is sent. ----
         const int ncg = p.Coutp >> 4;
         const uint32_t out0 = smem_u32(smem) + (uint32_t)p.off_send, in0 = smem_u32(smem) + (uint32_t)p.off_recv;
         const uint32_t block = (uint32_t)(p.Coutp * p.PP * 4);
-        for (int u = warp >> 2; u < p.M2 * ncg; u += kWarps / 4) {
-          const int t = u / ncg, cg = u - t * ncg;
-          const int po = t * 128 + (warp & 3) * 32 + lane;
-          uint32_t acc[16];
-          tmem_ld_x16(tmem_base + lane_base + p.pcol0 + t * p.Coutp + cg * 16, acc);
-          tmem_ld_wait();
-          if (po < valid_pix) {
-            const uint32_t owner = fast_div((uint32_t)po, (uint32_t)p.PP, p.pp_recip);
-            const uint32_t a = out0 + owner * block + (uint32_t)((cg * 4 * p.PP + po - (int)owner * p.PP) * 16);
+        for (int k = 0, cg0 = 0; cg0 < ncg; ++k, cg0 += p.piece_cgs) {
+          const int cgs = min(p.piece_cgs, ncg - cg0);
+          for (int u = warp >> 2; u < p.M2 * cgs; u += kWarps / 4) {
+            const int t = u / cgs, cg = cg0 + u - t * cgs;
+            const int po = t * 128 + (warp & 3) * 32 + lane;
+            uint32_t acc[16];
+            tmem_ld_x16(tmem_base + lane_base + p.pcol0 + t * p.Coutp + cg * 16, acc);
+            tmem_ld_wait();
+            if (po < valid_pix) {
+              const uint32_t owner = fast_div((uint32_t)po, (uint32_t)p.PP, p.pp_recip);
+              const uint32_t a = out0 + owner * block + (uint32_t)((cg * 4 * p.PP + po - (int)owner * p.PP) * 16);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) sts128(a + (uint32_t)(q * p.PP * 16), acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+              for (int q = 0; q < 4; ++q) sts128(a + (uint32_t)(q * p.PP * 16), acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+            }
           }
-        }
-        fence_proxy_async_smem();
-        tcgen05_fence_before_sync();
-        if (p.recv_shared) { __syncthreads(); cluster_arrive(); cluster_wait(); }     // every CTA's operands are dead
-        else { __syncthreads(); cluster_wait(); }  // every CTA has started (it arrived when its barriers were set up)
-        if (tid < p.CS - 1) {
-          const uint32_t peer = (uint32_t)((rank + 1 + tid) % p.CS);
-          bulk_copy_to_cluster(cluster_map(in0 + (uint32_t)rank * block, peer), out0 + peer * block, block, cluster_map(smem_u32(bar_red), peer));
+          fence_proxy_async_smem();
+          __syncthreads();
+          if (k == 0) {
+            if (p.recv_shared) cluster_arrive();   // this CTA's operands are dead
+            cluster_wait();                        // ... every CTA's, or: every CTA has started (it arrived when its barriers were set up)
+          }
+          if (tid < p.CS - 1) {
+            const uint32_t peer = (uint32_t)((rank + 1 + tid) % p.CS), at = (uint32_t)(cg0 * 64 * p.PP);
+            bulk_copy_to_cluster(cluster_map(in0 + (uint32_t)rank * block + at, peer), out0 + peer * block + at, (uint32_t)(cgs * 64 * p.PP),
+                                 cluster_map(smem_u32(bar_red + k), peer));
+          }
         }
         const int own0 = rank * p.PP, own = min(p.PP, valid_pix - own0), c8n = p.Cout >> 3;
-        int i = tid, lp = (int)fast_div((uint32_t)i, (uint32_t)c8n, p.cout8_recip), c8 = i - lp * c8n;
-        auto residual_of = [&]() -> uint4 {       // stride 1, Cin == Cout: the input at the same place
-          if (!(EXPAND && p.residual) || i >= own * c8n) return make_uint4(0, 0, 0, 0);
-          return __ldg(reinterpret_cast<const uint4*>(p.x + (gpix0 + own0 + lp) * p.Cout + c8 * 8));
-        };
-        uint4 xr = residual_of();                 // travels while the blocks do
-        if (warp == 0) mbar_wait(bar_red, 0, abort_flag, p.status, 0x108);
-        __syncthreads();
-        cluster_arrive();                         // this CTA has received everything
-        while (i < own * c8n) {
-          float v[8];
+        for (int k = 0, cg0 = 0; cg0 < ncg; ++k, cg0 += p.piece_cgs) {
+          const int c80 = cg0 * 2, c8s = min(2 * p.piece_cgs, c8n - c80);      // 16-byte pieces of a pixel
+          const uint32_t recip = c8s == 2 * p.piece_cgs ? p.c8s_recip : p.c8s_last_recip;
+          int i = tid, lp = (int)fast_div((uint32_t)i, (uint32_t)c8s, recip), c8 = c80 + i - lp * c8s;
+          auto residual_of = [&]() -> uint4 {       // stride 1, Cin == Cout: the input at the same place
+            if (!(EXPAND && p.residual) || i >= own * c8s) return make_uint4(0, 0, 0, 0);
+            return __ldg(reinterpret_cast<const uint4*>(p.x + (gpix0 + own0 + lp) * p.Cout + c8 * 8));
+          };
+          uint4 xr = residual_of();                 // travels while the blocks do
+          mbar_wait(bar_red + k, 0, abort_flag, p.status, 0x108);
+          if (cg0 + p.piece_cgs >= ncg) { __syncwarp(); cluster_arrive(); }      // this thread has seen everything arrive
+          while (i < own * c8s) {
+            float v[8];
 #pragma unroll
-          for (int q = 0; q < 8; ++q) v[q] = sB3[c8 * 8 + q];
-          v[0] += bf16_lo(xr.x); v[1] += bf16_hi(xr.x); v[2] += bf16_lo(xr.y); v[3] += bf16_hi(xr.y);
-          v[4] += bf16_lo(xr.z); v[5] += bf16_hi(xr.z); v[6] += bf16_lo(xr.w); v[7] += bf16_hi(xr.w);
-          const uint32_t at = (uint32_t)((c8 * 2 * p.PP + lp) * 16);
-          for (int src = 0; src < p.CS; ++src) {
-            const uint32_t a = (src == rank ? out0 : in0) + (uint32_t)src * block + at;
-            const float4 lo = lds128f<0>(a), hi = lds128f<0>(a + (uint32_t)(p.PP * 16));
-            v[0] += lo.x; v[1] += lo.y; v[2] += lo.z; v[3] += lo.w; v[4] += hi.x; v[5] += hi.y; v[6] += hi.z; v[7] += hi.w;
+            for (int q = 0; q < 8; ++q) v[q] = sB3[c8 * 8 + q];
+            v[0] += bf16_lo(xr.x); v[1] += bf16_hi(xr.x); v[2] += bf16_lo(xr.y); v[3] += bf16_hi(xr.y);
+            v[4] += bf16_lo(xr.z); v[5] += bf16_hi(xr.z); v[6] += bf16_lo(xr.w); v[7] += bf16_hi(xr.w);
+            const uint32_t at = (uint32_t)((c8 * 2 * p.PP + lp) * 16);
+            for (int src = 0; src < p.CS; ++src) {
+              const uint32_t a = (src == rank ? out0 : in0) + (uint32_t)src * block + at;
+              const float4 lo = lds128f<0>(a), hi = lds128f<0>(a + (uint32_t)(p.PP * 16));
+              v[0] += lo.x; v[1] += lo.y; v[2] += lo.z; v[3] += lo.w; v[4] += hi.x; v[5] += hi.y; v[6] += hi.z; v[7] += hi.w;
+            }
+            *reinterpret_cast<uint4*>(p.out + (gpix0 + own0 + lp) * p.Cout + c8 * 8) =
+                make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
+            if ((i += kThreads) >= own * c8s) break;
+            lp = (int)fast_div((uint32_t)i, (uint32_t)c8s, recip); c8 = c80 + i - lp * c8s;
+            xr = residual_of();
           }
-          *reinterpret_cast<uint4*>(p.out + (gpix0 + own0 + lp) * p.Cout + c8 * 8) =
-              make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
-          if ((i += kThreads) >= own * c8n) break;
-          lp = (int)fast_div((uint32_t)i, (uint32_t)c8n, p.cout8_recip); c8 = i - lp * c8n;
-          xr = residual_of();
         }
         cluster_wait();                           // the copies out of this CTA have arrived: it may leave
       } else
@@ -737,6 +754,15 @@ bool layout(Mbv2Params& q, int R, bool expand, bool project, int* smem_bytes) {
   q.off_bd = take(q.Cexp * 4);
   q.PP = ((R * q.Wo + q.CS - 1) / q.CS) | 1;
   q.pp_recip = fast_div_recip(q.PP);
+  {
+    // A second piece costs 0.1 to 0.9 us of hand-over and hides a layout and a summation: worth it from some 56 KB on (65 KB of
+    // 25 images 15 x 15 x 96: one piece 16.3, two 15.5, three 15.6 us; 45 KB of 39 images 11 x 11 x 96: 15.17, 15.16, 15.7;
+    // 38 KB of 32 images 14 x 14 x 64: 9.7, 9.9, 9.9; 5 KB of one image 14 x 14 x 32: 5.9, 6.8).
+    const int ncg = q.Coutp / 16, pieces = (q.CS - 1) * q.PP * q.Coutp * 4 >= 56 * 1024 ? 2 : 1;
+    q.piece_cgs = (ncg + pieces - 1) / pieces;
+    const int last = q.Cout / 8 - (ncg - 1) / q.piece_cgs * q.piece_cgs * 2;
+    q.c8s_recip = fast_div_recip(2 * q.piece_cgs); q.c8s_last_recip = fast_div_recip(std::max(1, last));
+  }
   q.off_send = q.off_recv = q.recv_shared = 0;
   if (project && q.CS > 1) {
     const int blocks = round_up(q.CS * q.PP * q.Coutp * 4, 1024);
@@ -821,7 +847,6 @@ ago_status_t mbv2_plan(Plan* plan, FusedState* st, std::string* err) {
   q.coutp_recip = recip(q.Coutp);
   q.w_recip = recip(q.W);
   q.cpr_recip = recip(q.cpr);
-  q.cout8_recip = recip(std::max(1, q.Cout / 8));
   q.segw = seg_width(q.Wo);
   q.nseg = (q.Wo + q.segw - 1) / q.segw;
   q.per_row = q.stride == 1 ? q.nseg : q.Wo;

@@ -32,6 +32,8 @@ def test_depthwise_pair_segments_and_strips(ago, shape):
     # more than 64 input channels: two and three K blocks, whole and with a remainder of one or more steps, padded last step
     (2, 15, 96, 576, 96, 1, True), (1, 8, 72, 432, 40, 1, False), (2, 9, 72, 432, 72, 2, False), (1, 13, 160, 960, 160, 1, True),
     (3, 12, 160, 960, 96, 2, False), (1, 20, 128, 768, 128, 1, True), (1, 4, 256, 512, 256, 1, True),
+    # partial sums exchanged in two pieces, the second one as wide as the first and narrower
+    (25, 15, 96, 576, 96, 1, True), (25, 15, 96, 576, 88, 1, False),
     # widths that cut into one, two, three odd segments with and without a remainder; rows that leave half a block
     (2, 8, 16, 96, 24, 1, False), (1, 10, 24, 144, 24, 1, True), (1, 16, 32, 192, 16, 1, False), (9, 22, 16, 96, 16, 1, True),
 ])
