@@ -8,40 +8,36 @@
 // computes R + 2 rows of the first convolution (2 of them recomputed by the
 // neighbouring strips) from R + 4 input rows.
 //
-// Both convolutions are implicit GEMMs on tcgen05. The three taps of a filter row
-// share their A operand: one MMA with N = 3 C multiplies a 128-pixel tile by
-// [W(dr,0) | W(dr,1) | W(dr,2)] and accumulates three partial sums
-// D_dc[q] = sum_dr x[q + dr rows] W(dr,dc) side by side in tensor memory (12 MMAs
-// of N = 192 per tile for 64 channels instead of 36 of N = 64: with N = 64 the
-// tensor pipe waits for its shared-memory operands, 6 KB per 32 cycles of
-// arithmetic; with N = 192 it is 10 KB per 96). The output is
-// out[q + 1] = D_0[q] + D_1[q + 1] + D_2[q + 2]; tcgen05.shift moves D_1 one row
-// and D_2 two rows towards row 0 so that the three terms of an output sit in the
-// same TMEM lane and the epilogue only adds them. The shift works inside each
-// block of 32 lanes (a block's last row keeps its value), which fixes the layout:
+// Both convolutions are implicit GEMMs on tcgen05. A product's operands come from shared memory, 128 bytes a cycle: 4 KB for
+// 128 pixels and 16 channels, 32 N bytes for the filters (measured: 58 cycles with N = 64, 100 with N = 192). So pixels are read
+// once for several taps: they are dealt out by column to PH phases, u = column + halo = PH q + phase, a phase's pixels one after
+// the other as rows [image row][q] of a swizzled K-major matrix (TMA loads of every PH-th column; zero outside the image).
+// Output column PH q + o needs the input columns PH q + j, j = o + dc, of three image rows, so the plane of phase j % PH, from
+// position j / PH on, serves the outputs o = j - 2, j - 1 and j of 128 positions at once: one MMA with N of up to 3 C that
+// multiplies it by [W(dr,2) | W(dr,1) | W(dr,0)] into neighbouring accumulators. PH + 2 products per filter row and 16
+// channels make 128 PH outputs; the taps meet in the accumulators, whatever the image's width.
+// PH = 4 or 2 for large images; with one phase a tile is 128 pixels and its chain the shortest, for small ones.
 //
-//   * the image width is cut into segments of 28 output columns; a segment's
-//     activations are [row][32 pixels][channels] in shared memory (swizzled
-//     K-major rows, one TMA box per segment, zero outside the image): 32 input
-//     columns -> 30 columns of the intermediate -> 28 output columns, the two
-//     columns lost per convolution being the ones a 32-lane block cannot shift in;
-//   * a 128-row MMA tile is four image rows of one segment, one row per 32-lane
-//     block; the operand of filter row dr is the same matrix 32 pixels further;
-//   * the intermediate value of (row, pixel j) is produced in the TMEM lane of
-//     pixel j and written over the input at the same place (every later tile
-//     reads rows further down), so the second convolution runs on the same
-//     addresses.
+// A tile is 128 consecutive positions (row * Q + q) of all phases. The intermediate value of (row, PH q + o) is written over
+// the input at position (row, q) of phase o: every later tile reads from its own first position on, and the second
+// convolution runs on the same addresses.
+//
+// Before, the taps of a filter row had an accumulator each (N = 3 C) that tcgen05.shift aligned, in segments of 28 columns, and
+// outputs were staged for TMA stores: the epilogue read three accumulators and took 2200 cycles per 112 pixels x 64
+// channels, twice the time of the products. 32 x 56 x 56 x 64 23.5 -> 21.6 us, 43 x 64 x 61 x 32 40.6 -> 17.3, 6 x 79 x 78 x 16
+// 11.4 -> 5.8, 14 x 14 x 64 (one image) 6.3 -> 5.3. Bound now by the products (13.8 us of the first, 8.9 at the dense rate), then by
+// the residual and the outputs, all of which move during the second convolution.
 //
 // All nine taps of one convolution stay resident (three slots of one filter row
 // each); the second convolution's rows replace the first's slot by slot as the
 // last tile of the first convolution releases them.
 //
-//   P1  TMA: input strip with halo -> swizzled [pixel][channel] rows, zero outside the image
-//   P2  tcgen05.mma: 3 filter rows x (I / 16) K-steps per tile, N = 3 C; tcgen05.shift   (TMEM, two tiles in flight)
-//   P3  TMEM -> registers: sum of the three aligned terms, + b1, ReLU, zero outside the image (the second
-//       convolution pads the post-activation tensor), bf16 -> swizzled rows in shared memory
-//   P5  tcgen05.mma: second convolution over the resident rows                           (TMEM)
-//   P6  TMEM -> registers: sum, + b2 + x, ReLU, bf16, 16-byte stores
+//   P1  TMA: input strip with halo -> phase planes of swizzled [position][channel] rows
+//   P2  tcgen05.mma: 3 filter rows x (C / 16) K steps x (PH + 2) products per tile   (TMEM, two tiles in flight)
+//   P3  TMEM -> registers: + b1, ReLU, zero outside the image (the second convolution pads the post-activation tensor),
+//       bf16 -> swizzled rows in shared memory
+//   P5  tcgen05.mma: second convolution over the resident rows                (TMEM)
+//   P6  TMEM -> registers: + b2 + x, ReLU, bf16 -> device memory, a 32-byte sector per store
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -59,13 +55,14 @@ namespace {
 
 using namespace tc;
 
-constexpr int kEpiWarps = 16;                // four per TMEM lane quarter: each takes 16 channels
+constexpr int kEpiWarps = 16;                // four per TMEM lane quarter
 constexpr int kEpiThreads = kEpiWarps * 32;
-constexpr int kShiftWarps = 3;
-constexpr int kThreads = kEpiThreads + 64 + 32 * kShiftWarps;   // + TMA warp + MMA warp + shift warps
-constexpr int kSegCols = 28;                 // output columns per segment (32 input columns, 30 of the intermediate)
+constexpr int kThreads = kEpiThreads + 64;   // + TMA warp + MMA warp
+constexpr int kTile = 128;                   // positions per tile (as many pixels each as there are phases)
 constexpr int kMaxTiles1 = 32;               // tiles of the first convolution (one "rows written" barrier each)
-constexpr int kMaxChunks = 32;               // row chunks of the input strip over all segments (one "landed" barrier each)
+constexpr int kChunkRows = 8;                // the strip arrives in chunks of image rows (whole swizzle groups of 8 positions)
+constexpr int kMaxChunks = 32;               // one "landed" barrier each
+constexpr int kMaxBoxCols = 256;             // columns of a row that one TMA box spans
 
 struct ConvParams {
   const __nv_bfloat16* x;
@@ -75,95 +72,121 @@ struct ConvParams {
   unsigned int* status;
   int N, H, W, C;          // C = input = middle = output channels
   int R, strips, IH;       // output rows per strip, strips per image, input rows per strip (R + 4; R + 2 for one convolution)
-  int NS, T1, T2, M1, M2;  // segments; tile rows (4 image rows each) and tiles (NS per tile row) of either convolution
-  int CH, NCH;             // the strip arrives in chunks of CH input rows (a multiple of 4) per segment, NCH chunks each
-  int nact;                // epilogue warps that own channels: 4 * min(4, C / 16)
-  int stage_mode;          // output staging: 0 none (direct stores), 1 in the input rows that no valid output reads, 2 own area
+  int PH;                  // column phases: 4, 2 or 1
+  int Q, T1, T2;           // positions per image row and phase; tiles of either convolution
+  int NCH, split_rows;     // chunks of kChunkRows input rows; rows wider than one TMA box: boxes of 32 positions of one row
+  int cg_shift;            // log2(C / 16)
+  int wide_store;          // the output starts at a multiple of 32 bytes
+  int plane_bytes;
+  uint32_t q_recip;
   // single-convolution variant (a stage of the unfused mode): out = [relu](conv(x) + b2 [+ res])
   const __nv_bfloat16* res; // residual tensor (the pair kernel adds its own input)
   int residual, relu;
   int w_row_bytes, w_swizzle, w_tap_bytes;
-  int off_x, off_w, off_bias, off_stage, off_bar;
+  int off_x, off_w, off_bias, off_bar;
 };
+
+// bf16x2(max(lo, 0), max(hi, 0)): the conversion clamps.
+__device__ __forceinline__ uint32_t pack_relu_bf16x2(float lo, float hi) {
+  uint32_t r;
+  asm("cvt.rn.relu.bf16x2.f32 %0, %2, %1;" : "=r"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+// a += low half of x, b += high half (mixed-precision FMAs with 1: the conversion costs nothing)
+__device__ __forceinline__ void add_bf16x2(float& a, float& b, uint32_t x) {
+  asm("{\n\t.reg .b16 xl, xh, one, z;\n\tmov.b32 {xl, xh}, %2;\n\tmov.b32 {one, z}, %3;\n\t"
+      "fma.rn.f32.bf16 %0, xl, one, %0;\n\tfma.rn.f32.bf16 %1, xh, one, %1;\n\t}"
+      : "+f"(a), "+f"(b) : "r"(x), "r"(0x00003F80u));
+}
 
 // SINGLE = false: the fused pair. SINGLE = true: one convolution with its simple operators (second-convolution
 // tiles only, reading the input rows directly), the tensor-core stage kernel of the unfused mode.
-template <bool SINGLE>
+template <bool SINGLE, int PH>
 __global__ void __launch_bounds__(kThreads, 1)
 conv3x3_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_xtail,
-                    const __grid_constant__ CUtensorMap tmap_w1,
-                    const __grid_constant__ CUtensorMap tmap_w2, const __grid_constant__ CUtensorMap tmap_out,
-                    const ConvParams p) {
+                    const __grid_constant__ CUtensorMap tmap_w1, const __grid_constant__ CUtensorMap tmap_w2, const ConvParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* sX = smem + p.off_x;   // [segment][row][32 pixels][C]; the intermediate overwrites it in place
-  uint8_t* sW = smem + p.off_w;   // [3 filter rows][3 taps][C rows]
+  uint8_t* sX = smem + p.off_x;   // [phase][row][q][C]; the intermediate overwrites it in place
+  uint8_t* sW = smem + p.off_w;   // [3 filter rows][taps 2, 1, 0][C rows]
   float* sBias = reinterpret_cast<float*>(smem + p.off_bias);   // b1[C], b2[C]
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.off_bar);
-  uint64_t* bar_wfull = bars + 1;         // [3] filter row landed (phase 0: first convolution, phase 1: second)
-  uint64_t* bar_wfree = bars + 4;         // [3] filter row of the first convolution no longer read
-  uint64_t* bar_acc = bars + 7;           // [2] accumulator of a tile complete (products and shifts)
-  uint64_t* bar_mma = bars + 13 + kMaxTiles1;   // [2] products of a tile complete
-  uint64_t* bar_shq = bars + 15 + kMaxTiles1;   // [2] shifts of a tile issued
-  uint64_t* bar_xc = bars + 17 + kMaxTiles1;    // [NCH][NS] chunk of input rows landed
-  uint64_t* bar_accfree = bars + 9;       // [2] accumulator read out by every epilogue warp
-  uint64_t* bar_y = bars + 11;            // [kMaxTiles1] intermediate rows of a tile written
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 11 + kMaxTiles1);
-  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 12 + kMaxTiles1);
+  uint64_t* bar_wfull = bars;             // [3] filter row landed (phase 0: first convolution, phase 1: second)
+  uint64_t* bar_wfree = bars + 3;         // [3] filter row of the first convolution no longer read
+  uint64_t* bar_acc = bars + 6;           // [2] accumulators of a tile complete
+  uint64_t* bar_accfree = bars + 8;       // [2] accumulators read out by every epilogue warp
+  uint64_t* bar_y = bars + 10;            // [kMaxTiles1] intermediate of a tile written
+  uint64_t* bar_xc = bar_y + kMaxTiles1;  // [kMaxChunks] chunk of input rows landed
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_xc + kMaxChunks);
+  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bar_xc + kMaxChunks + 1);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n = blockIdx.x / p.strips, strip = blockIdx.x % p.strips;
   const int h0 = strip * p.R;
   const int rows_valid = min(p.R, p.H - h0);
   const int ksteps = p.C / 16;
-  const int ntiles = p.M1 + p.M2;          // tile sequence: first convolution's tiles, then the second's
-  const uint32_t nacc = 3u * (uint32_t)p.C;   // accumulator columns of a tile
-  const uint32_t seg_bytes = (uint32_t)(p.IH * 32 * p.w_row_bytes);
+  const int ntiles = p.T1 + p.T2;          // tile sequence: first convolution's tiles, then the second's
+  const uint32_t nacc = (uint32_t)(PH * p.C);   // accumulator columns of a tile
 
-  grid_dependency_wait();      // the previous grid of the stream has completed; device memory may be touched
-  grid_launch_dependents();
   if (tid == kEpiThreads) {
     *abort_flag = 0u;
-    for (int i = 0; i < p.NCH * p.NS; ++i) mbar_init(bar_xc + i, 1);
     for (int i = 0; i < 3; ++i) { mbar_init(bar_wfull + i, 1); mbar_init(bar_wfree + i, 1); }
-    for (int i = 0; i < 2; ++i) { mbar_init(bar_acc + i, kShiftWarps); mbar_init(bar_mma + i, 1); mbar_init(bar_shq + i, kShiftWarps); mbar_init(bar_accfree + i, (uint32_t)p.nact); }
-    for (int i = 0; i < kMaxTiles1; ++i) mbar_init(bar_y + i, (uint32_t)p.nact);
+    for (int i = 0; i < 2; ++i) { mbar_init(bar_acc + i, 1); mbar_init(bar_accfree + i, kEpiWarps); }
+    for (int i = 0; i < p.T1; ++i) mbar_init(bar_y + i, kEpiWarps);
+    for (int i = 0; i < p.NCH; ++i) mbar_init(bar_xc + i, 1);
     fence_mbar_init();
     fence_proxy_async_smem();
     tma_prefetch_desc(&tmap_x);
-    // segment s: 32 columns from 28 s - 2 (one convolution: 28 s - 1), rows from h0 - 2 (h0 - 1); zero outside the
-    // image. The rows arrive in chunks, in the order the tiles need them, so that the first tile starts after the
-    // first chunks and the rest of the strip streams in behind the products.
-    for (int c = 0; c < p.NCH; ++c) {
-      const int rows = min(p.CH, p.IH - c * p.CH);
-      for (int s = 0; s < p.NS; ++s) {
-        uint64_t* bar = bar_xc + c * p.NS + s;
-        mbar_arrive_expect_tx(bar, (uint32_t)(rows * 32 * p.w_row_bytes));
-        tma_load_4d(sX + (size_t)s * seg_bytes + (size_t)(c * p.CH * 32) * p.w_row_bytes, rows == p.CH ? &tmap_x : &tmap_xtail, bar, 0,
-                    s * kSegCols - (SINGLE ? 1 : 2), (SINGLE ? h0 - 1 : h0 - 2) + c * p.CH, n);
-      }
-    }
+    tma_prefetch_desc(SINGLE ? &tmap_w2 : &tmap_w1);
   }
-  if (warp == 0) {
+  if (warp == kEpiWarps + 1) {
     tmem_alloc(tmem_slot, 512);
     tmem_relinquish();
   }
-  if (tid < 2 * p.C) sBias[tid] = SINGLE ? (tid >= p.C && p.b2 ? p.b2[tid - p.C] : 0.0f) : (tid < p.C ? p.b1[tid] : p.b2[tid - p.C]);
   tcgen05_fence_before_sync();
   __syncthreads();
   tcgen05_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
+  grid_dependency_wait();      // the previous grid of the stream has completed; device memory may be touched
+  grid_launch_dependents();
+  // Filter rows are taken in an order that starts at another one in neighbouring CTAs: all of them read the same lines, and
+  // the L2 slice of a line serves them one after the other.
+  const int rot = (int)(blockIdx.x % 3u);
+  auto filter_row = [&](int i) { const int f = rot + i; return f >= 3 ? f - 3 : f; };
 
   if (warp == kEpiWarps) {
-    // ================================ TMA producer: filter rows ================================
+    // ================================ TMA producer ================================
     if (lane == 0) {
-      tma_prefetch_desc(&tmap_w1); tma_prefetch_desc(&tmap_w2);
-      for (int conv = SINGLE ? 1 : 0; conv < 2; ++conv) {
-        for (int frow = 0; frow < 3; ++frow) {
-          if (!SINGLE && conv == 1) mbar_wait(bar_wfree + frow, 0, abort_flag, p.status, 0x401);
-          mbar_arrive_expect_tx(bar_wfull + frow, (uint32_t)(3 * p.w_tap_bytes));
-          for (int t3 = 0; t3 < 3; ++t3)
-            tma_load_3d(sW + (frow * 3 + t3) * p.w_tap_bytes, conv == 0 ? &tmap_w1 : &tmap_w2, bar_wfull + frow, 0, frow * 3 + t3, 0);
+      auto load_filter_row = [&](int conv, int f) {
+        mbar_arrive_expect_tx(bar_wfull + f, (uint32_t)(3 * p.w_tap_bytes));
+        for (int k = 0; k < 3; ++k)      // taps 2, 1, 0
+          tma_load_3d(sW + (f * 3 + k) * p.w_tap_bytes, conv == 0 ? &tmap_w1 : &tmap_w2, bar_wfull + f, 0, f * 3 + 2 - k, 0);
+      };
+      // phase f: columns PH q + f - 2 (one convolution: - 1) of the rows from h0 - 2 (h0 - 1) on; zero outside the image. The rows
+      // arrive in chunks, in the order the tiles need them, so that the first tile starts after the first chunks and the
+      // rest of the strip streams in behind the products.
+      constexpr int kHalo = SINGLE ? 1 : 2;
+      for (int c = 0; c < p.NCH; ++c) {
+        const int r0 = c * kChunkRows, rows = min(kChunkRows, p.IH - r0);
+        mbar_arrive_expect_tx(bar_xc + c, (uint32_t)(rows * PH * p.Q * p.w_row_bytes));
+        for (int f = 0; f < PH; ++f) {
+          uint8_t* dst = sX + (size_t)f * p.plane_bytes + (size_t)(r0 * p.Q) * p.w_row_bytes;
+          if (!p.split_rows) {
+            tma_load_4d(dst, rows == kChunkRows ? &tmap_x : &tmap_xtail, bar_xc + c, 0, f - kHalo, h0 - kHalo + r0, n);
+          } else {
+            for (int r = 0; r < rows; ++r)
+              for (int q = 0; q < p.Q; q += 32)
+                tma_load_4d(dst + (size_t)(r * p.Q + q) * p.w_row_bytes, &tmap_x, bar_xc + c, 0, PH * q + f - kHalo, h0 - kHalo + r0 + r, n);
+          }
+        }
+        if (c == 0)
+          for (int i = 0; i < 3; ++i) load_filter_row(SINGLE ? 1 : 0, filter_row(i));
+      }
+      if (!SINGLE) {
+        tma_prefetch_desc(&tmap_w2);
+        for (int i = 0; i < 3; ++i) {
+          mbar_wait(bar_wfree + filter_row(i), 0, abort_flag, p.status, 0x401);
+          load_filter_row(1, filter_row(i));
         }
       }
     }
@@ -172,222 +195,160 @@ conv3x3_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     // ================================ MMA issuer ================================
     // The warp runs its loop converged; MMAs and commits are predicated on one elected lane and take ready 64-bit
     // descriptors (several times the issue rate of a lane-0 branch next to busy warps, see tc_common.cuh).
-    // One issuer, tiles in sequence into alternating accumulators; the shift warps align a tile once its products are complete.
     const uint32_t elected = elect_one();
-    const uint32_t idesc = make_idesc_bf16(128, nacc);
-    const uint32_t rowu = (uint32_t)(32 * p.w_row_bytes) >> 4;   // one image row of a segment in 16-byte units
+    const uint32_t idesc[3] = {make_idesc_bf16(128, (uint32_t)p.C), make_idesc_bf16(128, (uint32_t)(2 * p.C)), make_idesc_bf16(128, (uint32_t)(3 * p.C))};
+    const uint32_t posu = (uint32_t)p.w_row_bytes >> 4;          // one position in 16-byte units
+    const uint32_t planeu = (uint32_t)p.plane_bytes >> 4, tapu = (uint32_t)p.w_tap_bytes >> 4;
     const uint64_t wdesc0 = make_smem_desc(smem_u32(sW), 0, 8u * p.w_row_bytes, p.w_swizzle);
     const uint64_t xdesc0 = make_smem_desc(smem_u32(sX), 0, 8u * p.w_row_bytes, p.w_swizzle);
-    const uint32_t frow_step = (uint32_t)(3 * p.w_tap_bytes) >> 4;
     int w_conv = -1;                       // convolution whose filter rows have been waited for
-    int t = 0, s = 0;                      // tile row and segment of the tile
+    int chunks = 0, written = 0;           // chunks landed, tiles of the intermediate written, as far as waited for
     for (int seq = 0; seq < ntiles; ++seq) {
-      if (seq == p.M1) { t = 0; s = 0; }
-      const int conv = seq >= p.M1 ? 1 : 0, buf = seq & 1;
+      const int conv = seq >= p.T1 ? 1 : 0, buf = seq & 1, t = conv ? seq - p.T1 : seq;
+      const int last_pos = t * kTile + kTile + 2 * p.Q;          // last position the tile's products read
       if (seq >= 2) mbar_wait(bar_accfree + buf, (uint32_t)((seq >> 1) - 1) & 1u, abort_flag, p.status, 0x403);
       if (SINGLE || conv == 0) {
-        // input rows 4 t .. 4 t + 5 of the segment: the chunks that hold them (waiting again for a landed chunk is free)
-        const int c_lo = (4 * t) / p.CH, c_hi = min(4 * t + 5, p.IH - 1) / p.CH;
-        for (int c = c_lo; c <= min(c_hi, p.NCH - 1); ++c) mbar_wait(bar_xc + c * p.NS + s, 0, abort_flag, p.status, 0x402);
-      }
-      if (!SINGLE && conv == 1) {
-        // rows 4 t .. 4 t + 5 of the segment's intermediate: its tiles of tile rows t and t + 1
-        mbar_wait(bar_y + t * p.NS + s, 0, abort_flag, p.status, 0x404);
-        if (t + 1 < p.T1) mbar_wait(bar_y + (t + 1) * p.NS + s, 0, abort_flag, p.status, 0x404);
+        const int need = min(p.NCH, (int)fast_div((uint32_t)last_pos, (uint32_t)p.Q, p.q_recip) / kChunkRows + 1);
+        for (; chunks < need; ++chunks) mbar_wait(bar_xc + chunks, 0, abort_flag, p.status, 0x402);
+      } else {
+        const int need = min(p.T1, last_pos / kTile + 1);
+        for (; written < need; ++written) mbar_wait(bar_y + written, 0, abort_flag, p.status, 0x404);
       }
       tcgen05_fence_after_sync();
-      const uint32_t d_tmem = tmem_base + (uint32_t)buf * nacc;
-      const uint64_t a0 = xdesc0 + (uint64_t)((uint32_t)(s * p.IH + 4 * t) * rowu);
-      for (int frow = 0; frow < 3; ++frow) {
+      const uint32_t d = tmem_base + (uint32_t)buf * nacc;
+      const uint64_t a0 = xdesc0 + (uint64_t)((uint32_t)(t * kTile) * posu);
+      for (int i = 0; i < 3; ++i) {
+        const int frow = filter_row(i);
         if (w_conv != conv) {
           mbar_wait(bar_wfull + frow, SINGLE ? 0u : (uint32_t)conv, abort_flag, p.status, 0x405);
           tcgen05_fence_after_sync();
         }
-        const uint64_t a = a0 + (uint64_t)((uint32_t)frow * rowu);
-        const uint64_t b = wdesc0 + (uint64_t)(frow_step * (uint32_t)frow);
-        if (ksteps == 4) {
-          umma_bf16_elected_acc(d_tmem, a, b, idesc, elected, frow != 0);
-          umma_bf16_elected<true>(d_tmem, a + 2u, b + 2u, idesc, elected);
-          umma_bf16_elected<true>(d_tmem, a + 4u, b + 4u, idesc, elected);
-          umma_bf16_elected<true>(d_tmem, a + 6u, b + 6u, idesc, elected);
-        } else {
-          for (int ks = 0; ks < ksteps; ++ks)
-            umma_bf16_elected_acc(d_tmem, a + 2u * ks, b + 2u * ks, idesc, elected, (ks | frow) != 0);
+        uint64_t a = a0 + (uint64_t)((uint32_t)(frow * p.Q) * posu), b = wdesc0 + (uint64_t)(3u * tapu * (uint32_t)frow);
+#pragma unroll 1
+        for (int ks = 0; ks < ksteps; ++ks, a += 2u, b += 2u) {
+          const uint32_t acc = (i | ks) != 0 ? 1u : 0u;
+          // input column j: outputs o = max(0, j - 2) .. min(PH - 1, j), from tap j - o of the first one on; the first
+          // products cover every output once and overwrite
+          if constexpr (PH == 4) {
+            umma_bf16_elected_acc(d, a + 2u * planeu, b, idesc[2], elected, acc);                       // j = 2
+            umma_bf16_elected_acc(d + 3u * p.C, a + planeu + posu, b, idesc[0], elected, acc);          // j = 5
+            umma_bf16_elected<true>(d, a, b + 2u * tapu, idesc[0], elected);                            // j = 0
+            umma_bf16_elected<true>(d, a + planeu, b + tapu, idesc[1], elected);                        // j = 1
+            umma_bf16_elected<true>(d + p.C, a + 3u * planeu, b, idesc[2], elected);                    // j = 3
+            umma_bf16_elected<true>(d + 2u * p.C, a + posu, b, idesc[1], elected);                      // j = 4
+          } else if constexpr (PH == 1) {
+            umma_bf16_elected_acc(d, a, b + 2u * tapu, idesc[0], elected, acc);                         // j = 0
+            umma_bf16_elected<true>(d, a + posu, b + tapu, idesc[0], elected);                          // j = 1
+            umma_bf16_elected<true>(d, a + 2u * posu, b, idesc[0], elected);                            // j = 2
+          } else {
+            umma_bf16_elected_acc(d, a + posu, b, idesc[1], elected, acc);                              // j = 2
+            umma_bf16_elected<true>(d, a, b + 2u * tapu, idesc[0], elected);                            // j = 0
+            umma_bf16_elected<true>(d, a + planeu, b + tapu, idesc[1], elected);                        // j = 1
+            umma_bf16_elected<true>(d + p.C, a + planeu + posu, b, idesc[0], elected);                  // j = 3
+          }
         }
-        if (!SINGLE && seq == p.M1 - 1) umma_commit_elected(bar_wfree + frow, elected);
-        // The shifts of the previous tile go into the tensor pipe's queue here, behind this tile's first filter row
-        // (which keeps the pipe busy while the shift warps learn that the previous tile's products are complete)
-        // and ahead of the rest: behind a whole tile they would hold the epilogue back by a tile.
-        if (frow == 0 && seq > 0) mbar_wait(bar_shq + (buf ^ 1), (uint32_t)((seq - 1) >> 1) & 1u, abort_flag, p.status, 0x408);
+        if (!SINGLE && seq == p.T1 - 1) umma_commit_elected(bar_wfree + frow, elected);
       }
       w_conv = conv;
-      umma_commit_elected(bar_mma + buf, elected);
-      if (++s == p.NS) { s = 0; ++t; }
-    }
-    __syncwarp();
-  } else if (warp > kEpiWarps + 1) {
-    // ================================ shift warps: align the accumulators ================================
-    // tcgen05.shift is not ordered behind the MMAs issued before it (their last accumulator updates are still in
-    // flight), so the shifts of a tile are issued here, after the tile's products have completed, while the MMA warp
-    // is already issuing the next tile into the other accumulator. D_1 moves one row, D_2 two rows towards row 0,
-    // 8 columns per instruction; issuing costs a warp ~40 cycles per instruction next to the busy epilogue warps,
-    // so three warps share the 3 C / 8 instructions of a tile (both shifts of a column block stay in one thread).
-    const int sw = warp - kEpiWarps - 2;
-    const uint32_t elected = elect_one();
-    const int units = p.C / 8;      // warp 0: D_1; warps 1 and 2: a half of D_2 each, both shifts of a column block in one thread
-    for (int seq = 0; seq < ntiles; ++seq) {
-      const int buf = seq & 1;
-      mbar_wait(bar_mma + buf, (uint32_t)(seq >> 1) & 1u, abort_flag, p.status, 0x407);
-      tcgen05_fence_after_sync();
-      const uint32_t d_tmem = tmem_base + (uint32_t)buf * nacc;
-      if (sw == 0) {
-        for (int u = 0; u < units; ++u) tmem_shift_down_elected(d_tmem + (uint32_t)(p.C + 8 * u), elected);
-      } else {
-        for (int u = (sw - 1) * units / 2; u < sw * units / 2; ++u) {
-          tmem_shift_down_elected(d_tmem + (uint32_t)(2 * p.C + 8 * u), elected);
-          tmem_shift_down_elected(d_tmem + (uint32_t)(2 * p.C + 8 * u), elected);
-        }
-      }
       umma_commit_elected(bar_acc + buf, elected);
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar_shq + buf);
     }
     __syncwarp();
-  } else if ((warp >> 2) * 16 < p.C) {
-    // ================ epilogue warps: thread = (image row of the tile, pixel of the segment, 16 channels) ================
+  } else {
+    // ====== epilogue warps: thread = position of the tile; a warp takes every fourth (phase, 16 channels) pair ======
     const int wq = warp & 3, cg = warp >> 2;
-    const int col0 = cg * 16;
     const uint32_t lane_base = (uint32_t)(wq * 32) << 16;
     const uint32_t x_addr = smem_u32(sX);
     const uint32_t swz_mask = ((uint32_t)p.w_row_bytes >> 4) - 1u;
-    // Output (P6): the 32 pixels x C channels of an image row of the tile are staged as swizzled rows by the warps
-    // that share the row (one per 16 channels) and leave with one TMA store of 28 pixels, clipped at the image's
-    // right edge. From the second tile row on, the staging block is the row four above in the same segment: every
-    // product that read it has completed, and no later tile writes it, so nothing waits for a store to drain. The
-    // first tile row stages in the input rows R + 2 and R + 3 of the segments, which only the rows past the strip
-    // read once the first convolution is complete, or in its own space (or stores directly if there is neither).
-    const uint32_t qbytes = 32u * (uint32_t)p.w_row_bytes;
-    uint8_t* stg0_ptr = sX;
-    if (p.stage_mode == 1) stg0_ptr = sX + (size_t)(wq >> 1) * seg_bytes + (size_t)(p.R + 2) * qbytes + (size_t)(wq & 1) * qbytes;
-    else if (p.stage_mode == 2) stg0_ptr = smem + p.off_stage + (size_t)wq * qbytes;
-    const uint32_t row_threads = (uint32_t)(p.nact / 4) * 32u;   // threads that share an image row of the tile
-    const bool storer = cg == 0 && lane == 0;
-    const bool do_res = SINGLE ? p.residual != 0 : true, do_relu = SINGLE ? p.relu != 0 : true;
-
-    // The residual of an output tile is fetched one tile ahead (its latency is a tile's worth of cycles when the
-    // input comes from device memory).
-    uint4 xn0 = make_uint4(0u, 0u, 0u, 0u), xn1 = xn0;
-    auto fetch_residual = [&](int t_, int s_) {
-      const int a_ = 4 * t_ + wq, c_ = s_ * kSegCols + lane;
-      xn0 = make_uint4(0u, 0u, 0u, 0u); xn1 = xn0;
-      if (do_res && lane < kSegCols && c_ < p.W && a_ < rows_valid) {
-        const __nv_bfloat16* rp = (SINGLE ? p.res : p.x) + (((size_t)n * p.H + h0 + a_) * p.W + c_) * p.C + col0;
-        xn0 = __ldg(reinterpret_cast<const uint4*>(rp));
-        xn1 = __ldg(reinterpret_cast<const uint4*>(rp + 8));
-      }
-    };
-    if (p.M1 == 0) fetch_residual(0, 0);
-    int t = 0, s = 0;
+    const int units = PH << p.cg_shift, cg_mask = (1 << p.cg_shift) - 1;   // (phase, 16 channels) pairs of a tile
+    const bool do_res = SINGLE ? p.residual != 0 : true;
+    if (tid < 2 * p.C) sBias[tid] = SINGLE ? (tid >= p.C && p.b2 ? p.b2[tid - p.C] : 0.0f) : (tid < p.C ? p.b1[tid] : p.b2[tid - p.C]);
     for (int seq = 0; seq < ntiles; ++seq) {
-      if (seq == p.M1) { t = 0; s = 0; }
-      const bool second = seq >= p.M1;
+      const bool second = seq >= p.T1;
       const int buf = seq & 1;
-      const int a = 4 * t + wq;                        // row of the intermediate / of the output inside the strip
-      // second convolution: lane j is output column 28 s + j
-      const int c = s * kSegCols + lane;
-      const bool valid = second && lane < kSegCols && c < p.W && a < rows_valid;
-      const size_t pix = ((size_t)n * p.H + h0 + a) * p.W + c;
-      const uint4 xr[2] = {xn0, xn1};
-      if (seq + 1 < ntiles && seq + 1 >= p.M1) {
-        if (seq + 1 == p.M1) fetch_residual(0, 0);
-        else if (s + 1 == p.NS) fetch_residual(t + 1, 0);
-        else fetch_residual(t, s + 1);
+      const int m = (second ? seq - p.T1 : seq) * kTile + wq * 32 + lane;
+      const int a = (int)fast_div((uint32_t)m, (uint32_t)p.Q, p.q_recip), q = m - a * p.Q;   // row of the intermediate / output in the strip
+      const size_t row0 = (((size_t)n * p.H + h0 + a) * p.W + PH * q) * p.C;                 // second: output column PH q of that row
+      uint4 xr[PH][2];                // the residual, fetched ahead of the accumulators
+#pragma unroll
+      for (int i = 0; i < PH; ++i) {
+        const int u = cg + 4 * i, o = u >> p.cg_shift, col0 = (u & cg_mask) * 16;
+        xr[i][0] = xr[i][1] = make_uint4(0u, 0u, 0u, 0u);
+        if (second && do_res && u < units && a < rows_valid && PH * q + o < p.W) {
+          const uint4* rp = reinterpret_cast<const uint4*>((SINGLE ? p.res : p.x) + row0 + o * p.C + col0);
+          xr[i][0] = __ldg(rp);
+          xr[i][1] = __ldg(rp + 1);
+        }
       }
-      mbar_wait(bar_acc + buf, (uint32_t)(seq >> 1) & 1u, abort_flag, p.status, 0x406);
+      // one warp polls, the others are parked: sixteen polling warps would take the issue slots of the MMA warp
+      if (warp == 0) mbar_wait(bar_acc + buf, (uint32_t)(seq >> 1) & 1u, abort_flag, p.status, 0x406);
+      named_barrier_sync(1u, kEpiThreads);
       tcgen05_fence_after_sync();
-      uint32_t v0[16], v1[16], v2[16];
-      const uint32_t tb = tmem_base + lane_base + (uint32_t)buf * nacc + (uint32_t)col0;
-      tmem_ld_x16(tb, v0);
-      tmem_ld_x16(tb + (uint32_t)p.C, v1);
-      tmem_ld_x16(tb + 2u * (uint32_t)p.C, v2);
-      tmem_ld_wait();
-      tcgen05_fence_before_sync();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar_accfree + buf);
-      float sum[16];
-      const float* bias = sBias + (second ? p.C : 0) + col0;
+      const uint32_t tb = tmem_base + lane_base + (uint32_t)buf * nacc;
+      const uint32_t bias0 = smem_u32(sBias) + (second ? (uint32_t)p.C * 4u : 0u);
 #pragma unroll
-      for (int j = 0; j < 16; j += 4) {
-        const float4 bj = *reinterpret_cast<const float4*>(bias + j);
-        sum[j] = __uint_as_float(v0[j]) + __uint_as_float(v1[j]) + __uint_as_float(v2[j]) + bj.x;
-        sum[j + 1] = __uint_as_float(v0[j + 1]) + __uint_as_float(v1[j + 1]) + __uint_as_float(v2[j + 1]) + bj.y;
-        sum[j + 2] = __uint_as_float(v0[j + 2]) + __uint_as_float(v1[j + 2]) + __uint_as_float(v2[j + 2]) + bj.z;
-        sum[j + 3] = __uint_as_float(v0[j + 3]) + __uint_as_float(v1[j + 3]) + __uint_as_float(v2[j + 3]) + bj.w;
-      }
-
-      if (!second) {
-        // P3: intermediate = ReLU(sum) inside the image, 0 outside -> the swizzled row of (segment, row a, pixel lane);
-        // lane j is column 28 s - 1 + j of the intermediate, lanes 30 and 31 have no complete sum
-        if (lane < 30 && a < p.R + 2) {
-          const int gh = h0 - 1 + a, cy = s * kSegCols - 1 + lane;
-          const bool inside = gh >= 0 && gh < p.H && cy >= 0 && cy < p.W;
+      for (int i = 0; i < PH; ++i) {
+        const int u = cg + 4 * i, o = u >> p.cg_shift, col0 = (u & cg_mask) * 16;
+        if (u < units) {
+          uint32_t v[16];
+          tmem_ld_x16(tb + (uint32_t)(o * p.C + col0), v);
+          tmem_ld_wait_on(v);
+          const uint32_t ba = bias0 + (uint32_t)col0 * 4u;
+          float s[16];
+#pragma unroll
+          for (int j = 0; j < 16; j += 4) {
+            float4 b4;
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(b4.x), "=f"(b4.y), "=f"(b4.z), "=f"(b4.w) : "r"(ba + 4u * j));
+            s[j] = __uint_as_float(v[j]) + b4.x; s[j + 1] = __uint_as_float(v[j + 1]) + b4.y;
+            s[j + 2] = __uint_as_float(v[j + 2]) + b4.z; s[j + 3] = __uint_as_float(v[j + 3]) + b4.w;
+          }
           uint32_t w[8];
+          if (!second) {
+            // P3: intermediate = ReLU(sum) inside the image, 0 outside; column PH q + o - 1 of the image
+            if (a < p.R + 2) {
+              if ((unsigned)(h0 - 1 + a) < (unsigned)p.H && (unsigned)(PH * q + o - 1) < (unsigned)p.W) {
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            w[j] = inside ? pack_bf16x2(fmaxf(sum[2 * j], 0.0f), fmaxf(sum[2 * j + 1], 0.0f)) : 0u;
-          // 16-byte chunk index XOR address bits [7, ..): the swizzle the MMA and TMA apply to absolute addresses
-          uint32_t a0 = x_addr + (uint32_t)s * seg_bytes + (uint32_t)(a * 32 + lane) * p.w_row_bytes + (uint32_t)col0 * 2u;
-          uint32_t a1 = a0 + 16u;
-          a0 ^= ((a0 >> 7) & swz_mask) << 4;
-          a1 ^= ((a1 >> 7) & swz_mask) << 4;
-          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a0), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
-          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a1), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
-        }
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_y + seq);
-      } else {
-        // P6: out = ReLU(sum + x)
-        uint32_t w[8];
-        const uint32_t xs[8] = {xr[0].x, xr[0].y, xr[0].z, xr[0].w, xr[1].x, xr[1].y, xr[1].z, xr[1].w};
+                for (int j = 0; j < 8; ++j) w[j] = pack_relu_bf16x2(s[2 * j], s[2 * j + 1]);
+              } else {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          float y0 = sum[2 * j] + bf16_lo(xs[j]);      // xs is zero without a residual
-          float y1 = sum[2 * j + 1] + bf16_hi(xs[j]);
-          if (do_relu) { y0 = fmaxf(y0, 0.0f); y1 = fmaxf(y1, 0.0f); }
-          w[j] = pack_bf16x2(y0, y1);
-        }
-        if (p.stage_mode != 0 || t > 0) {
-          uint8_t* stg_ptr = t > 0 ? sX + (size_t)s * seg_bytes + (size_t)(a - 4) * qbytes : stg0_ptr;
-          const uint32_t stg = smem_u32(stg_ptr);
-          if (t == 0 && s > 0) {
-            if (storer) bulk_wait_group_read_all();        // the first tile row's segments share one set of staging blocks
-            named_barrier_sync(2u + (uint32_t)wq, row_threads);
+                for (int j = 0; j < 8; ++j) w[j] = 0u;
+              }
+              // 16-byte chunk index XOR address bits [7, ..): the swizzle the MMA and TMA apply to absolute addresses
+              uint32_t a0 = x_addr + (uint32_t)(o * p.plane_bytes + m * p.w_row_bytes + col0 * 2);
+              a0 ^= ((a0 >> 7) & swz_mask) << 4;
+              const uint32_t a1 = a0 ^ 16u;     // the neighbouring chunk (col0 is a multiple of two chunks)
+              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a0), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
+              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a1), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
+            }
+          } else if (a < rows_valid && PH * q + o < p.W) {
+            // P6: out = [ReLU](sum + x); xr is zero without a residual
+            const uint32_t xs[8] = {xr[i][0].x, xr[i][0].y, xr[i][0].z, xr[i][0].w, xr[i][1].x, xr[i][1].y, xr[i][1].z, xr[i][1].w};
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              add_bf16x2(s[2 * j], s[2 * j + 1], xs[j]);
+              w[j] = !SINGLE || p.relu ? pack_relu_bf16x2(s[2 * j], s[2 * j + 1]) : pack_bf16x2(s[2 * j], s[2 * j + 1]);
+            }
+            __nv_bfloat16* dst = p.out + row0 + o * p.C + col0;
+            if (p.wide_store) {
+              store_global_32(dst, w);
+            } else {
+              *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
+              *reinterpret_cast<uint4*>(dst + 8) = make_uint4(w[4], w[5], w[6], w[7]);
+            }
           }
-          uint32_t a0 = stg + (uint32_t)lane * p.w_row_bytes + (uint32_t)col0 * 2u;
-          uint32_t a1 = a0 + 16u;
-          a0 ^= ((a0 >> 7) & swz_mask) << 4;
-          a1 ^= ((a1 >> 7) & swz_mask) << 4;
-          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a0), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
-          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a1), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
-          fence_proxy_async_smem();
-          named_barrier_sync(2u + (uint32_t)wq, row_threads);
-          if (storer && a < rows_valid) {
-            tma_store_3d(&tmap_out, stg_ptr, 0, s * kSegCols, n * p.H + h0 + a);
-            bulk_commit_group();
-          }
-        } else if (valid) {
-          *reinterpret_cast<uint4*>(p.out + pix * p.C + col0) = make_uint4(w[0], w[1], w[2], w[3]);
-          *reinterpret_cast<uint4*>(p.out + pix * p.C + col0 + 8) = make_uint4(w[4], w[5], w[6], w[7]);
         }
       }
-      if (++s == p.NS) { s = 0; ++t; }
+      tcgen05_fence_before_sync();
+      if (!second) fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(bar_accfree + buf);
+        if (!second) mbar_arrive(bar_y + seq);
+      }
     }
-    if (storer) bulk_wait_group_all();
   }
   tcgen05_fence_before_sync();
   __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem_base, 512);
+  if (warp == kEpiWarps + 1) tmem_dealloc(tmem_base, 512);
 }
 
 struct ConvHost {
@@ -402,45 +363,57 @@ int round_up_i(int v, int m) { return (v + m - 1) / m * m; }
 
 // Shared-memory layout common to both variants (pair: IH = R + 4 rows and both convolutions; single: IH = R + 2).
 bool conv_layout_common(ConvParams& q, bool pair, int* smem_bytes) {
-  q.NS = (q.W + kSegCols - 1) / kSegCols;
-  q.T1 = pair ? (q.R + 2 + 3) / 4 : 0;
-  q.T2 = (q.R + 3) / 4;
-  q.M1 = q.NS * q.T1;
-  q.M2 = q.NS * q.T2;
-  q.nact = 4 * std::min(4, q.C / 16);
-  if (q.IH > 256 || q.M1 > kMaxTiles1) return false;
-  q.CH = 4;
-  while (((q.IH + q.CH - 1) / q.CH) * q.NS > kMaxChunks) q.CH += 4;
-  q.NCH = (q.IH + q.CH - 1) / q.CH;
-  const int seg_bytes = q.IH * 32 * q.w_row_bytes;
+  const int PH = q.PH;
+  q.Q = (q.W + (pair ? 4 : 2) + PH - 1) / PH;
+  q.split_rows = PH * (q.Q - 1) + 1 > kMaxBoxCols;
+  if (q.split_rows) q.Q = round_up_i(q.Q, 32);      // rows are then brought by boxes of 32 positions
+  q.q_recip = fast_div_recip(q.Q);
+  q.T1 = pair ? ((q.R + 2) * q.Q + kTile - 1) / kTile : 0;
+  q.T2 = (q.R * q.Q + kTile - 1) / kTile;
+  q.cg_shift = q.C == 64 ? 2 : (q.C == 32 ? 1 : 0);
+  q.NCH = (q.IH + kChunkRows - 1) / kChunkRows;
+  if (q.IH > kMaxChunks * kChunkRows || q.T1 > kMaxTiles1 || (q.R + 2) * q.Q > 65535 - 2 * kTile) return false;
+  q.plane_bytes = round_up_i(q.IH * q.Q * q.w_row_bytes, 1024);
   int off = 0;
   q.off_x = off;
-  off = round_up_i(off + q.NS * seg_bytes, 1024);
+  off += q.PH * q.plane_bytes;
   q.off_w = off;
   off += round_up_i(9 * q.w_tap_bytes, 1024);
   q.off_bias = off;
   off += 1024;
   q.off_bar = off;
   off += 1024;
-  // Output staging: 32 pixels x C channels per image row of a tile (one KB per active epilogue warp). The pair has
-  // input rows that no valid output reads once the first convolution is complete (rows R + 2 and R + 3 of every
-  // segment: room for two image rows each); otherwise an area of its own if it fits.
-  q.off_stage = 0;
-  q.stage_mode = 0;
-  if (pair && (long)q.NS * 2 * 32 * q.w_row_bytes >= (long)q.nact * 1024) {
-    q.stage_mode = 1;
-  } else if (round_up_i(off, 1024) + q.nact * 1024 + 1024 <= 227 * 1024) {
-    q.stage_mode = 2;
-    off = round_up_i(off, 1024);   // staging rows are swizzled like operand rows: whole 1024-byte groups
-    q.off_stage = off;
-    off += q.nact * 1024;
-  }
   // The rows of the last tiles run past the strip (their results are dropped) but must stay inside the allocation:
-  // they then read filter rows or biases as activations, which is harmless.
-  const long reach = ((long)((q.NS - 1) * q.IH + 4 * (std::max(q.T1, q.T2) - 1) + 2) * 32 + 128) * q.w_row_bytes;
-  if (q.off_x + reach > (long)off) off = (int)round_up_i((int)(q.off_x + reach), 1024);
+  // they then read other phases, filter rows or biases as activations, which is harmless.
+  const long reach = q.off_x + (q.PH - 1l) * q.plane_bytes + ((long)std::max(q.T1, q.T2) * kTile + 2 * q.Q + 2) * q.w_row_bytes;
+  if (reach > off) off = round_up_i((int)reach, 1024);
   *smem_bytes = off + 1024;
   return *smem_bytes <= 227 * 1024;
+}
+
+// Phases and rows per strip: the least estimated time. Cycles of a CTA: start 5500; its tiles' products (37 + 0.33 N each; 58 at
+// N = 64, 100 at N = 192) or epilogues, whichever are longer; the last epilogue of either convolution. Among equals the
+// fewest CTAs (each loads all filters), rows evenly shared.
+template <class Layout>
+void choose_tiling(ConvParams& q, int* R, Layout&& layout) {
+  double best_cost = 0;
+  int best_ph = 4;
+  *R = 0;
+  for (int PH = 1; PH <= 4; PH *= 2) {
+    const double c = 0.33 * q.C, products = (PH + 2) * 37.0 + 3 * PH * c;
+    const double mma = products * 3 * (q.C / 16), epi = 400.0 + 350.0 * ((PH * q.C / 16 + 3) / 4);
+    for (int rows = 1; rows <= q.H; ++rows) {
+      const int strips = (q.H + rows - 1) / rows;
+      if ((q.H + strips - 1) / strips != rows) continue;
+      ConvParams t = q; int smem = 0;
+      t.PH = PH;
+      if (!layout(t, rows, &smem)) continue;
+      const long sms = device_sm_count(), waves = ((long)q.N * strips + sms - 1) / sms;
+      const double cost = (double)waves * (5500.0 + (t.T1 + t.T2) * std::max(mma, epi) + (t.T1 ? 2 : 1) * std::min(mma, epi));
+      if (*R == 0 || cost <= best_cost) { *R = rows; best_ph = PH; best_cost = cost; }
+    }
+  }
+  q.PH = best_ph;
 }
 
 bool conv_layout(ConvParams& q, int R, int* smem_bytes) {
@@ -448,6 +421,16 @@ bool conv_layout(ConvParams& q, int R, int* smem_bytes) {
   q.strips = (q.H + R - 1) / R;
   q.IH = R + 4;
   return conv_layout_common(q, true, smem_bytes);
+}
+
+// Every fourth column of a chunk of image rows (tail: of the last, shorter chunk), or of 32 positions of one row.
+bool encode_input(CUtensorMap* m, const void* x, const ConvParams& q, bool tail, std::string* err) {
+  const uint64_t dims[4] = {(uint64_t)q.C, (uint64_t)q.W, (uint64_t)q.H, (uint64_t)q.N};
+  const uint64_t strides[3] = {(uint64_t)q.C * 2, (uint64_t)q.W * q.C * 2, (uint64_t)q.H * q.W * q.C * 2};
+  const int rows = q.split_rows ? 1 : (tail ? q.IH - (q.NCH - 1) * kChunkRows : std::min(kChunkRows, q.IH));
+  const uint32_t box[4] = {(uint32_t)q.C, (uint32_t)(q.PH * ((q.split_rows ? 32 : q.Q) - 1) + 1), (uint32_t)rows, 1};
+  const uint32_t steps[4] = {1, (uint32_t)q.PH, 1, 1};
+  return encode_tmap_bf16(m, x, 4, dims, strides, box, q.w_row_bytes, err, steps);
 }
 
 }  // namespace
@@ -464,15 +447,9 @@ ago_status_t conv3x3_plan(Plan* plan, FusedState* st, std::string* err) {
   q.w_row_bytes = q.C * 2;
   q.w_swizzle = q.C == 16 ? tc::SW_32B : (q.C == 32 ? tc::SW_64B : tc::SW_128B);
   q.w_tap_bytes = q.C * q.w_row_bytes;   // taps lie back to back: the three of a filter row form one B operand of 3 C rows
-  int best_R = 0, best_smem = 0; double best_cost = 0;
-  for (int R = 1; R <= q.H; ++R) {
-    ConvParams t = q; int smem = 0;
-    if (!conv_layout(t, R, &smem)) continue;
-    const long ctas = (long)q.N * t.strips;
-    const long sms = device_sm_count(), waves = (ctas + sms - 1) / sms;
-    const double cost = (double)waves * (t.M1 + t.M2 + 1.0);
-    if (best_R == 0 || cost < best_cost) { best_R = R; best_cost = cost; best_smem = smem; }
-  }
+  int best_smem = 0;
+  int best_R = 0;
+  choose_tiling(q, &best_R, conv_layout);
   if (best_R == 0) return bad("no row-strip tiling fits shared memory / tensor memory");
   conv_layout(q, best_R, &best_smem);
   host->smem_bytes = best_smem;
@@ -494,22 +471,14 @@ ago_status_t conv3x3_run(const Plan& plan, FusedState* st, const void* const* in
   q.out = static_cast<__nv_bfloat16*>(output);
   q.status = status_word;
   q.res = q.x; q.residual = 1; q.relu = 1;
+  q.wide_store = reinterpret_cast<uintptr_t>(output) % 32 == 0;
   auto get_map = [&](const void* base, int which, CUtensorMap* out) -> bool {
     ConvHost::Key key{base, which};
     auto it = host->maps.find(key);
     if (it == host->maps.end()) {
       CUtensorMap m;
-      if (which == 0 || which == 4) {   // input rows: a chunk of CH rows, or the shorter last chunk
-        const int tail = q.IH - (q.NCH - 1) * q.CH;
-        const uint64_t dims[4] = {(uint64_t)q.C, (uint64_t)q.W, (uint64_t)q.H, (uint64_t)q.N};
-        const uint64_t strides[3] = {(uint64_t)q.C * 2, (uint64_t)q.W * q.C * 2, (uint64_t)q.H * q.W * q.C * 2};
-        const uint32_t box[4] = {(uint32_t)q.C, 32u, (uint32_t)(which == 0 ? std::min(q.CH, q.IH) : tail), 1};
-        if (!encode_tmap_bf16(&m, base, 4, dims, strides, box, q.w_row_bytes, err)) return false;
-      } else if (which == 3) {
-        const uint64_t dims[3] = {(uint64_t)q.C, (uint64_t)q.W, (uint64_t)q.N * q.H};
-        const uint64_t strides[2] = {(uint64_t)q.C * 2, (uint64_t)q.W * q.C * 2};
-        const uint32_t box[3] = {(uint32_t)q.C, (uint32_t)kSegCols, 1};
-        if (!encode_tmap_bf16(&m, base, 3, dims, strides, box, q.w_row_bytes, err)) return false;
+      if (which == 0 || which == 4) {   // input rows: a chunk of rows, or the shorter last chunk
+        if (!encode_input(&m, base, q, which == 4, err)) return false;
       } else {
         const uint64_t dims[3] = {(uint64_t)q.C, 9, (uint64_t)q.C};
         const uint64_t strides[2] = {(uint64_t)q.C * 2, (uint64_t)9 * q.C * 2};
@@ -522,15 +491,16 @@ ago_status_t conv3x3_run(const Plan& plan, FusedState* st, const void* const* in
     *out = it->second;
     return true;
   };
-  CUtensorMap mx, mxt, mw1, mw2, mo;
-  if (!get_map(inputs[0], 0, &mx) || !get_map(inputs[0], 4, &mxt) || !get_map(weights[0], 1, &mw1) || !get_map(weights[2], 2, &mw2) || !get_map(output, 3, &mo)) return AGO_ERR_CUDA;
+  CUtensorMap mx, mxt, mw1, mw2;
+  if (!get_map(inputs[0], 0, &mx) || !get_map(inputs[0], 4, &mxt) || !get_map(weights[0], 1, &mw1) || !get_map(weights[2], 2, &mw2)) return AGO_ERR_CUDA;
+  auto kernel = q.PH == 4 ? conv3x3_pair_kernel<false, 4> : q.PH == 2 ? conv3x3_pair_kernel<false, 2> : conv3x3_pair_kernel<false, 1>;
   {
-    static int smem_opt_in[64] = {};
-    cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(conv3x3_pair_kernel<false>), smem_opt_in);
+    static int smem_opt_in[3][64] = {};
+    cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(kernel), smem_opt_in[q.PH / 2]);
     if (e != cudaSuccess) { *err = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e); return AGO_ERR_CUDA; }
   }
   FusedLaunch launch(dim3((unsigned)(q.N * q.strips)), kThreads, (size_t)host->smem_bytes, stream);
-  cudaError_t e = cudaLaunchKernelEx(&launch.config, conv3x3_pair_kernel<false>, mx, mxt, mw1, mw2, mo, q);
+  cudaError_t e = cudaLaunchKernelEx(&launch.config, kernel, mx, mxt, mw1, mw2, q);
   if (e != cudaSuccess) { *err = std::string("fused conv3x3 pair launch: ") + cudaGetErrorString(e); return AGO_ERR_CUDA; }
   return AGO_OK;
 }
@@ -547,15 +517,15 @@ bool conv_layout_single(ConvParams& q, int R, int* smem_bytes) {
 }
 
 struct SingleKey {
-  const void *x, *w, *out; int N, H, W, C;
-  bool operator==(const SingleKey& o) const { return x == o.x && w == o.w && out == o.out && N == o.N && H == o.H && W == o.W && C == o.C; }
+  const void *x, *w; int N, H, W, C;
+  bool operator==(const SingleKey& o) const { return x == o.x && w == o.w && N == o.N && H == o.H && W == o.W && C == o.C; }
 };
 struct SingleKeyHash {
   size_t operator()(const SingleKey& k) const {
-    return std::hash<const void*>()(k.x) ^ (std::hash<const void*>()(k.w) * 31u) ^ (std::hash<const void*>()(k.out) * 131u) ^ ((size_t)k.N << 40) ^ ((size_t)k.H << 24) ^ ((size_t)k.W << 8) ^ (size_t)k.C;
+    return std::hash<const void*>()(k.x) ^ (std::hash<const void*>()(k.w) * 31u) ^ ((size_t)k.N << 40) ^ ((size_t)k.H << 24) ^ ((size_t)k.W << 8) ^ (size_t)k.C;
   }
 };
-struct SingleEntry { ConvParams prm; int smem_bytes; CUtensorMap mx, mxt, mw, mo; };
+struct SingleEntry { ConvParams prm; int smem_bytes; CUtensorMap mx, mxt, mw; };
 std::mutex g_single_mutex;
 std::unordered_map<SingleKey, SingleEntry, SingleKeyHash> g_single;
 
@@ -572,7 +542,7 @@ cudaError_t launch_conv3x3_tc(const void* x, const void* w, const float* bias, c
   SingleEntry entry;
   {
     std::lock_guard<std::mutex> lock(g_single_mutex);
-    const SingleKey key{x, w, out, N, H, W, C};
+    const SingleKey key{x, w, N, H, W, C};
     auto it = g_single.find(key);
     if (it == g_single.end()) {
       SingleEntry e{};
@@ -581,32 +551,18 @@ cudaError_t launch_conv3x3_tc(const void* x, const void* w, const float* bias, c
       q.w_row_bytes = C * 2;
       q.w_swizzle = C == 16 ? tc::SW_32B : (C == 32 ? tc::SW_64B : tc::SW_128B);
       q.w_tap_bytes = C * q.w_row_bytes;
-      int best_R = 0, best_smem = 0; double best_cost = 0;
-      for (int R = 1; R <= H; ++R) {
-        ConvParams t = q; int smem = 0;
-        if (!conv_layout_single(t, R, &smem)) continue;
-        const long sms = device_sm_count(), waves = ((long)N * t.strips + sms - 1) / sms;
-        const double cost = (double)waves * (t.M2 + 1.0);
-        if (best_R == 0 || cost < best_cost) { best_R = R; best_cost = cost; best_smem = smem; }
-      }
+      int best_smem = 0;
+      int best_R = 0;
+      choose_tiling(q, &best_R, conv_layout_single);
       if (best_R == 0) return cudaErrorInvalidConfiguration;
       conv_layout_single(q, best_R, &best_smem);
       e.smem_bytes = best_smem;
       std::string err;
-      const uint64_t xd[4] = {(uint64_t)C, (uint64_t)W, (uint64_t)H, (uint64_t)N};
-      const uint64_t xs[3] = {(uint64_t)C * 2, (uint64_t)W * C * 2, (uint64_t)H * W * C * 2};
-      const uint32_t xb[4] = {(uint32_t)C, 32u, (uint32_t)std::min(q.CH, q.IH), 1};
-      if (!encode_tmap_bf16(&e.mx, x, 4, xd, xs, xb, q.w_row_bytes, &err)) return cudaErrorInvalidValue;
-      const uint32_t xtb[4] = {(uint32_t)C, 32u, (uint32_t)(q.IH - (q.NCH - 1) * q.CH), 1};
-      if (!encode_tmap_bf16(&e.mxt, x, 4, xd, xs, xtb, q.w_row_bytes, &err)) return cudaErrorInvalidValue;
+      if (!encode_input(&e.mx, x, q, false, &err) || !encode_input(&e.mxt, x, q, true, &err)) return cudaErrorInvalidValue;
       const uint64_t wd[3] = {(uint64_t)C, 9, (uint64_t)C};
       const uint64_t ws[2] = {(uint64_t)C * 2, (uint64_t)9 * C * 2};
       const uint32_t wb[3] = {(uint32_t)C, 1, (uint32_t)C};
       if (!encode_tmap_bf16(&e.mw, w, 3, wd, ws, wb, q.w_row_bytes, &err)) return cudaErrorInvalidValue;
-      const uint64_t od[3] = {(uint64_t)C, (uint64_t)W, (uint64_t)N * H};
-      const uint64_t os[2] = {(uint64_t)C * 2, (uint64_t)W * C * 2};
-      const uint32_t ob[3] = {(uint32_t)C, (uint32_t)kSegCols, 1};
-      if (!encode_tmap_bf16(&e.mo, out, 3, od, os, ob, q.w_row_bytes, &err)) return cudaErrorInvalidValue;
       if (g_single.size() > 4096) g_single.clear();
       it = g_single.emplace(key, e).first;
     }
@@ -617,14 +573,16 @@ cudaError_t launch_conv3x3_tc(const void* x, const void* w, const float* bias, c
   q.b1 = nullptr; q.b2 = bias;
   q.res = static_cast<const __nv_bfloat16*>(res); q.residual = res != nullptr; q.relu = relu;
   q.out = static_cast<__nv_bfloat16*>(out);
+  q.wide_store = reinterpret_cast<uintptr_t>(out) % 32 == 0;
   q.status = status;
+  auto kernel = q.PH == 4 ? conv3x3_pair_kernel<true, 4> : q.PH == 2 ? conv3x3_pair_kernel<true, 2> : conv3x3_pair_kernel<true, 1>;
   {
-    static int smem_opt_in[64] = {};
-    cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(conv3x3_pair_kernel<true>), smem_opt_in);
+    static int smem_opt_in[3][64] = {};
+    cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(kernel), smem_opt_in[q.PH / 2]);
     if (e != cudaSuccess) return e;
   }
   FusedLaunch launch(dim3((unsigned)(q.N * q.strips)), kThreads, (size_t)entry.smem_bytes, stream);
-  return cudaLaunchKernelEx(&launch.config, conv3x3_pair_kernel<true>, entry.mx, entry.mxt, entry.mw, entry.mw, entry.mo, q);
+  return cudaLaunchKernelEx(&launch.config, kernel, entry.mx, entry.mxt, entry.mw, entry.mw, q);
 }
 
 }  // namespace ago

@@ -77,11 +77,6 @@ __device__ __forceinline__ uint32_t relu6_bf16x2(uint32_t w) {
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-__device__ __forceinline__ void store_global_32(void* dst, const uint32_t (&w)[8]) {   // 32-byte aligned: one sector
-  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" :: "l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]),
-               "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
-}
-
 // 16 fp32 sums + 16 bias values of shared memory
 __device__ __forceinline__ void add_bias16(uint32_t (&v)[16], const float* bias) {
 #pragma unroll

@@ -358,17 +358,6 @@ __device__ __forceinline__ void umma_commit_cluster_elected(uint32_t bar_cluster
       ::"r"(bar_cluster_addr), "r"(elected)
       : "memory");
 }
-// tcgen05.shift: every row of a 32-byte-wide (8 columns of 32 bits) block of tensor memory takes the value of the next
-// row (lane i <- lane i + 1), separately inside each block of 32 lanes: lanes 31, 63, 95 and 127 keep their values
-// (measured: ~10 cycles per instruction; asynchronous, in issue order with the MMAs of the same thread and tracked
-// by its commits). All lanes execute; one elected lane issues.
-__device__ __forceinline__ void tmem_shift_down_elected(uint32_t taddr, uint32_t elected) {
-  asm volatile(
-      "{\n\t.reg .pred q;\n\t"
-      "setp.ne.b32 q, %1, 0;\n\t"
-      "@q tcgen05.shift.cta_group::1.down [%0];\n\t}"
-      ::"r"(taddr), "r"(elected) : "memory");
-}
 __device__ __forceinline__ void umma_commit_elected(uint64_t* bar, uint32_t elected) {
   asm volatile(
       "{\n\t.reg .pred q;\n\t"
@@ -511,6 +500,11 @@ __device__ __forceinline__ void tmem_ld_wait_on(uint32_t (&v)[16]) {
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&h);
+}
+// Eight words to 32 bytes of device memory (32-byte aligned): one sector.
+__device__ __forceinline__ void store_global_32(void* dst, const uint32_t (&w)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" :: "l"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]),
+               "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7]) : "memory");
 }
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xffff0000u); }

@@ -13,7 +13,7 @@ std::once_flag g_once;
 }  // namespace
 
 bool encode_tmap_bf16(CUtensorMap* out, const void* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes,
-                      const uint32_t* box, int swizzle_bytes, std::string* err) {
+                      const uint32_t* box, int swizzle_bytes, std::string* err, const uint32_t* steps) {
   std::call_once(g_once, [] {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult qres;
@@ -23,7 +23,7 @@ bool encode_tmap_bf16(CUtensorMap* out, const void* base, int rank, const uint64
   });
   if (!g_encode) { *err = "cuTensorMapEncodeTiled is not available from the driver"; return false; }
   cuuint64_t gdims[5]; cuuint64_t gstrides[4]; cuuint32_t gbox[5]; cuuint32_t estr[5];
-  for (int i = 0; i < rank; ++i) { gdims[i] = dims[i]; gbox[i] = box[i]; estr[i] = 1; }
+  for (int i = 0; i < rank; ++i) { gdims[i] = dims[i]; gbox[i] = box[i]; estr[i] = steps ? steps[i] : 1; }
   for (int i = 0; i + 1 < rank; ++i) gstrides[i] = strides_bytes[i];
   CUtensorMapSwizzle sw = CU_TENSOR_MAP_SWIZZLE_NONE;
   if (swizzle_bytes == 32) sw = CU_TENSOR_MAP_SWIZZLE_32B;

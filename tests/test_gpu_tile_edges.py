@@ -169,3 +169,23 @@ def test_depthwise_strips_epilogues(ago, ops):
     wl = WL.Workload("dw_epilogues", [211], [(3, 22, 19, 40)], [("conv2d", dict(O=40, R=3, S=3, stride=1, pad=1, groups=40))] + ops,
                      samples=3, input_dist=["normal"])
     check(ago, wl, "auto")
+
+
+@pytest.mark.parametrize("shape", [
+    # n, h, w, c: one pixel, one row, one column; a tile and a position more; one, two and four column phases
+    (1, 1, 1, 16), (2, 1, 9, 32), (1, 9, 1, 64), (1, 3, 2, 16), (2, 15, 16, 64), (1, 7, 14, 64), (3, 8, 29, 32),
+    (14, 35, 33, 64), (4, 41, 42, 16), (33, 56, 54, 64), (13, 61, 59, 32), (20, 57, 75, 16), (5, 78, 76, 64),
+    # rows wider than one box: pieces of 32 positions
+    (1, 5, 253, 16), (1, 4, 300, 16), (1, 3, 560, 32), (2, 2, 896, 16),
+])
+def test_residual_block_phases_and_tiles(ago, shape):
+    n, h, w, c = shape
+    ops = WL.resnet_block("x", [0], 1, 8, c).ops
+    check(ago, WL.Workload("residual_edges", [212, *shape], [shape], ops, samples=n, input_dist=["relu_normal"]))
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 1, 16), (2, 9, 31, 64), (30, 56, 55, 64), (6, 40, 254, 16), (17, 33, 30, 32)])
+def test_single_convolution_phases_and_tiles(ago, shape):
+    n, h, w, c = shape
+    ops = [("conv2d", dict(O=c, R=3, S=3, stride=1, pad=1, groups=1)), ("bias_add", {}), ("relu", {})]
+    check(ago, WL.Workload("conv_edges", [213, *shape], [shape], ops, samples=n, input_dist=["relu_normal"]), "per_mini_subgraph")
