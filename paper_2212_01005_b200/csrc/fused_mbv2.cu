@@ -189,6 +189,7 @@ mbv2_fused_kernel(const Mbv2Params p) {
     auto stage = [&]() {
       const uint8_t* none = reinterpret_cast<const uint8_t*>(p.wd);      // never read: the copies from it have no bytes
       const uint32_t s0 = smem_u32(smem);
+      const float fold_b = FOLD && tid < p.Cexp ? __ldg(p.b1 + ch0 + tid) : 0.0f;     // on its way while the copies are issued
       if (EXPAND) {
         const int xblk = p.M1 * 128 * 128, wblk = p.Cexp * 128;
         auto place = [&](int row, int ch, int blk) -> uint32_t {
@@ -205,14 +206,7 @@ mbv2_fused_kernel(const Mbv2Params p) {
         });
         stage_region(p.Cexp, p.cpr, p.cpr_recip, [&](int row, int ch) {
           const uint32_t d = p.off_w1 + place(row, ch, wblk);
-          if (FOLD && ch == cin_chunks) {
-            // the bias as bf16 high and low parts (their sum carries 16 mantissa bits, and 1.0 * part is exact in the fp32 accumulator)
-            const float b = __ldg(p.b1 + ch0 + row);
-            const __nv_bfloat16 hi = __float2bfloat16_rn(b);
-            const __nv_bfloat16 lo = __float2bfloat16_rn(b - __bfloat162float(hi));
-            *reinterpret_cast<uint4*>(smem + d) = make_uint4((uint32_t)__bfloat16_as_ushort(hi) | ((uint32_t)__bfloat16_as_ushort(lo) << 16), 0, 0, 0);
-            return;
-          }
+          if (FOLD && ch == cin_chunks) return;     // the bias, below
           const bool in = ch < cin_chunks;
           cp_async_16(s0 + d, in ? w1p + (uint32_t)row * cin_bytes + ch * 16 : none, in ? 16u : 0u);
         });
@@ -237,6 +231,17 @@ mbv2_fused_kernel(const Mbv2Params p) {
       stage_bias(4, p.off_bd, p.bd + ch0, p.Cexp);
       if (PROJECT) stage_bias(8, p.off_b3, p.b3, p.Cout);
       if (EXPAND && !FOLD) stage_bias(12, p.off_b1, p.b1 + ch0, p.Cexp);
+      if (FOLD) {
+        for (int row = tid; row < p.Cexp; row += kThreads) {
+          // the bias as bf16 high and low parts (their sum carries 16 mantissa bits, and 1.0 * part is exact in the fp32 accumulator)
+          const float b = row == tid ? fold_b : __ldg(p.b1 + ch0 + row);
+          const __nv_bfloat16 hi = __float2bfloat16_rn(b);
+          const __nv_bfloat16 lo = __float2bfloat16_rn(b - __bfloat162float(hi));
+          const uint32_t i = ((uint32_t)row << cs) + (uint32_t)cin_chunks;
+          *reinterpret_cast<uint4*>(smem + p.off_w1 + ((i << 4) ^ (((i >> 3) & swz_mask) << 4))) =
+              make_uint4((uint32_t)__bfloat16_as_ushort(hi) | ((uint32_t)__bfloat16_as_ushort(lo) << 16), 0, 0, 0);
+        }
+      }
     };
     // ---- per-thread work mapping: needs no device memory, so it runs before the wait for the previous grid of the
     // stream (with back-to-back launches it overlaps that grid's tail) ----
