@@ -76,9 +76,10 @@ PyObject* call(PyObject* self, PyObject* const* args, size_t nargsf, PyObject* k
   try {
     PyObject* first = PySequence_GetItem(args[0], 0);
     if (!first) return nullptr;
-    Py_DECREF(first);                 // the sequence keeps it
-    if (!THPVariable_Check(first)) { PyErr_SetString(PyExc_TypeError, "inputs are torch tensors"); return nullptr; }
-    const at::Device dev = THPVariable_Unpack(first).device();
+    const bool is_tensor = THPVariable_Check(first);
+    const at::Device dev = is_tensor ? THPVariable_Unpack(first).device() : at::Device(at::kCPU);
+    Py_DECREF(first);
+    if (!is_tensor) { PyErr_SetString(PyExc_TypeError, "inputs are torch tensors"); return nullptr; }
     if (!dev.is_cuda()) return raise(r, kErrCuda, "inputs must be CUDA tensors: this library has no CPU path");
     if (r->workspace_bytes > 0) {
       if (args[4] == Py_None || !THPVariable_Check(args[4])) Py_RETURN_NONE;

@@ -1,0 +1,79 @@
+"""The native call behind `Subgraph.run`: what it returns, which stream it uses, when it attaches a workspace, how it fails."""
+import threading
+
+import pytest
+
+from paper_2212_01005_b200 import workloads as WL
+from helpers import to_device
+
+pytestmark = pytest.mark.gpu
+
+
+def handle(ago, wl, mode="fused"):
+    return ago.Subgraph(wl.ops, wl.input_shapes, mode=mode), to_device(wl, WL.generate(wl))
+
+
+def test_run_returns_the_given_output_and_allocates_its_own(ago):
+    import torch
+    sg, (ins, ws) = handle(ago, WL.pw_pw("call", [301], 2, 9, 64, 32, 64))
+    own = sg.run(ins, ws)
+    given = torch.empty_like(own)
+    assert sg.run(ins, ws, out=given) is given
+    assert sg.run(tuple(ins), tuple(ws)).shape == sg.output_shape
+    torch.cuda.synchronize()
+    assert torch.equal(own, given) and own.dtype == torch.bfloat16
+    sg.close()
+
+
+def test_run_attaches_a_workspace_and_uses_the_stream_it_is_given(ago):
+    import torch
+    sg, (ins, ws) = handle(ago, WL.ffn("call_ffn", [302], 512, 768, 3072, 1))
+    assert sg.workspace_bytes > 0
+    ref = sg.run(ins, ws)
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    a = sg.run(ins, ws, stream=side.cuda_stream)
+    with torch.cuda.stream(side):
+        b = sg.run(ins, ws)
+    torch.cuda.synchronize()
+    scale = float(ref.float().abs().max())
+    for o in (a, b):          # the additions arrive in any order: one bf16 step
+        assert float((o.float() - ref.float()).abs().max()) <= 2.0 ** -7 * scale
+    assert sg.status() == ago.AGO_OK
+    sg.close()
+
+
+def test_run_rejects_what_it_cannot_launch(ago):
+    sg, (ins, ws) = handle(ago, WL.pw_pw("call_bad", [303], 1, 8, 64, 32, 64))
+    with pytest.raises(ago.AgoError):
+        sg.run(ins, ws[:-1])                      # a weight short
+    with pytest.raises(ago.AgoError):
+        sg.run([t.cpu() for t in ins], ws)        # no CPU path
+    with pytest.raises((TypeError, IndexError)):
+        sg.run([], ws)
+    sg.close()
+
+
+def test_run_from_two_threads_on_streams_of_their_own(ago):
+    import torch
+    sg0, (ins0, ws0) = handle(ago, WL.pw_pw("call_t0", [304], 4, 20, 96, 24, 96))
+    sg1, (ins1, ws1) = handle(ago, WL.mbv2_block("call_t1", [305], 2, 14, 32, 192, 32, 1, True))
+    refs = [sg0.run(ins0, ws0), sg1.run(ins1, ws1)]
+    torch.cuda.synchronize()
+    outs = [[], []]
+
+    def work(k, sg, ins, ws):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for _ in range(50):
+                outs[k].append(sg.run(ins, ws))
+            torch.cuda.current_stream().synchronize()
+
+    threads = [threading.Thread(target=work, args=a) for a in ((0, sg0, ins0, ws0), (1, sg1, ins1, ws1))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert all(torch.equal(o, refs[0]) for o in outs[0])
+    scale = float(refs[1].float().abs().max())    # chunks are added in the order the groups finish: one bf16 step
+    assert all(float((o.float() - refs[1].float()).abs().max()) <= 2.0 ** -7 * scale for o in outs[1])
+    sg0.close(); sg1.close()
