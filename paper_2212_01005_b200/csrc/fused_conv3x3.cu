@@ -13,10 +13,12 @@
 // once for several taps: they are dealt out by column to PH phases, u = column + halo = PH q + phase, a phase's pixels one after
 // the other as rows [image row][q] of a swizzled K-major matrix (TMA loads of every PH-th column; zero outside the image).
 // Output column PH q + o needs the input columns PH q + j, j = o + dc, of three image rows, so the plane of phase j % PH, from
-// position j / PH on, serves the outputs o = j - 2, j - 1 and j of 128 positions at once: one MMA with N of up to 3 C that
-// multiplies it by [W(dr,2) | W(dr,1) | W(dr,0)] into neighbouring accumulators. PH + 2 products per filter row and 16
-// channels make 128 PH outputs; the taps meet in the accumulators, whatever the image's width.
-// PH = 4 or 2 for large images; with one phase a tile is 128 pixels and its chain the shortest, for small ones.
+// position j / PH on, serves those of the outputs j - 2, j - 1 and j that there are, of 128 positions at once: one MMA that
+// multiplies it by their part of [W(dr,2) | W(dr,1) | W(dr,0)] into neighbouring accumulators. PH + 2 products per filter
+// row and 16 channels make 128 PH outputs; the taps meet in the accumulators, whatever the image's width.
+// Two phases for large images (N = C, 2 C, 2 C, C: a fifth fewer operand bytes than tap by tap); with one a tile is 128
+// pixels and its chain the shortest, for small ones. Four phases (N up to 3 C) save another seventh of the bytes, but two
+// tiles then fill tensor memory and too little of their epilogues overlaps: 21.7 us at 32 x 56 x 56 x 64 where two take 20.6.
 //
 // A tile is 128 consecutive positions (row * Q + q) of all phases. The intermediate value of (row, PH q + o) is written over
 // the input at position (row, q) of phase o: every later tile reads from its own first position on, and the second
@@ -24,7 +26,7 @@
 //
 // Before, the taps of a filter row had an accumulator each (N = 3 C) that tcgen05.shift aligned, in segments of 28 columns, and
 // outputs were staged for TMA stores: the epilogue read three accumulators and took 2200 cycles per 112 pixels x 64
-// channels, twice the time of the products. 32 x 56 x 56 x 64 23.5 -> 21.6 us, 43 x 64 x 61 x 32 40.6 -> 17.3, 6 x 79 x 78 x 16
+// channels, twice the time of the products. 32 x 56 x 56 x 64 23.5 -> 20.6 us, 43 x 64 x 61 x 32 40.6 -> 17.3, 6 x 79 x 78 x 16
 // 11.4 -> 5.8, 14 x 14 x 64 (one image) 6.3 -> 5.3. Bound now by the products (13.8 us of the first, 8.9 at the dense rate), then by
 // the residual and the outputs, all of which move during the second convolution.
 //
@@ -72,7 +74,7 @@ struct ConvParams {
   unsigned int* status;
   int N, H, W, C;          // C = input = middle = output channels
   int R, strips, IH;       // output rows per strip, strips per image, input rows per strip (R + 4; R + 2 for one convolution)
-  int PH;                  // column phases: 4, 2 or 1
+  int PH;                  // column phases: 2 or 1
   int Q, T1, T2;           // positions per image row and phase; tiles of either convolution
   int NCH, split_rows;     // chunks of kChunkRows input rows; rows wider than one TMA box: boxes of 32 positions of one row
   int cg_shift;            // log2(C / 16)
@@ -149,9 +151,9 @@ conv3x3_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
   const uint32_t tmem_base = *tmem_slot;
   grid_dependency_wait();      // the previous grid of the stream has completed; device memory may be touched
   grid_launch_dependents();
-  // Filter rows are taken in an order that starts at another one in neighbouring CTAs: all of them read the same lines, and
-  // the L2 slice of a line serves them one after the other.
-  const int rot = (int)(blockIdx.x % 3u);
+  // Large images: filter rows are taken in an order that starts at another one in neighbouring CTAs: all of them read the same
+  // lines, and the L2 slice of a line serves them one after the other (2 to 5% of the time; fixed order on small ones, 2%).
+  const int rot = PH == 2 ? (int)(blockIdx.x % 3u) : 0;
   auto filter_row = [&](int i) { const int f = rot + i; return f >= 3 ? f - 3 : f; };
 
   if (warp == kEpiWarps) {
@@ -196,7 +198,7 @@ conv3x3_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     // The warp runs its loop converged; MMAs and commits are predicated on one elected lane and take ready 64-bit
     // descriptors (several times the issue rate of a lane-0 branch next to busy warps, see tc_common.cuh).
     const uint32_t elected = elect_one();
-    const uint32_t idesc[3] = {make_idesc_bf16(128, (uint32_t)p.C), make_idesc_bf16(128, (uint32_t)(2 * p.C)), make_idesc_bf16(128, (uint32_t)(3 * p.C))};
+    const uint32_t idesc1 = make_idesc_bf16(128, (uint32_t)p.C), idesc2 = make_idesc_bf16(128, (uint32_t)(2 * p.C));
     const uint32_t posu = (uint32_t)p.w_row_bytes >> 4;          // one position in 16-byte units
     const uint32_t planeu = (uint32_t)p.plane_bytes >> 4, tapu = (uint32_t)p.w_tap_bytes >> 4;
     const uint64_t wdesc0 = make_smem_desc(smem_u32(sW), 0, 8u * p.w_row_bytes, p.w_swizzle);
@@ -223,29 +225,34 @@ conv3x3_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
           mbar_wait(bar_wfull + frow, SINGLE ? 0u : (uint32_t)conv, abort_flag, p.status, 0x405);
           tcgen05_fence_after_sync();
         }
-        uint64_t a = a0 + (uint64_t)((uint32_t)(frow * p.Q) * posu), b = wdesc0 + (uint64_t)(3u * tapu * (uint32_t)frow);
-#pragma unroll 1
-        for (int ks = 0; ks < ksteps; ++ks, a += 2u, b += 2u) {
-          const uint32_t acc = (i | ks) != 0 ? 1u : 0u;
-          // input column j: outputs o = max(0, j - 2) .. min(PH - 1, j), from tap j - o of the first one on; the first
-          // products cover every output once and overwrite
-          if constexpr (PH == 4) {
-            umma_bf16_elected_acc(d, a + 2u * planeu, b, idesc[2], elected, acc);                       // j = 2
-            umma_bf16_elected_acc(d + 3u * p.C, a + planeu + posu, b, idesc[0], elected, acc);          // j = 5
-            umma_bf16_elected<true>(d, a, b + 2u * tapu, idesc[0], elected);                            // j = 0
-            umma_bf16_elected<true>(d, a + planeu, b + tapu, idesc[1], elected);                        // j = 1
-            umma_bf16_elected<true>(d + p.C, a + 3u * planeu, b, idesc[2], elected);                    // j = 3
-            umma_bf16_elected<true>(d + 2u * p.C, a + posu, b, idesc[1], elected);                      // j = 4
-          } else if constexpr (PH == 1) {
-            umma_bf16_elected_acc(d, a, b + 2u * tapu, idesc[0], elected, acc);                         // j = 0
-            umma_bf16_elected<true>(d, a + posu, b + tapu, idesc[0], elected);                          // j = 1
-            umma_bf16_elected<true>(d, a + 2u * posu, b, idesc[0], elected);                            // j = 2
+        const uint64_t a = a0 + (uint64_t)((uint32_t)(frow * p.Q) * posu), b = wdesc0 + (uint64_t)(3u * tapu * (uint32_t)frow);
+        // input column j: outputs o = max(0, j - 2) .. min(PH - 1, j), from tap j - o of the first one on; the first product
+        // covers every output and overwrites
+        auto kstep = [&](uint64_t a, uint64_t b, uint32_t acc) {
+          if constexpr (PH == 1) {
+            umma_bf16_elected_acc(d, a, b + 2u * tapu, idesc1, elected, acc);                         // j = 0
+            umma_bf16_elected<true>(d, a + posu, b + tapu, idesc1, elected);                          // j = 1
+            umma_bf16_elected<true>(d, a + 2u * posu, b, idesc1, elected);                            // j = 2
           } else {
-            umma_bf16_elected_acc(d, a + posu, b, idesc[1], elected, acc);                              // j = 2
-            umma_bf16_elected<true>(d, a, b + 2u * tapu, idesc[0], elected);                            // j = 0
-            umma_bf16_elected<true>(d, a + planeu, b + tapu, idesc[1], elected);                        // j = 1
-            umma_bf16_elected<true>(d + p.C, a + planeu + posu, b, idesc[0], elected);                  // j = 3
+            umma_bf16_elected_acc(d, a + posu, b, idesc2, elected, acc);                              // j = 2
+            umma_bf16_elected<true>(d, a, b + 2u * tapu, idesc1, elected);                            // j = 0
+            umma_bf16_elected<true>(d, a + planeu, b + tapu, idesc2, elected);                        // j = 1
+            umma_bf16_elected<true>(d + p.C, a + planeu + posu, b, idesc1, elected);                  // j = 3
           }
+        };
+        // straight-line for two phases (32 x 56 x 56 x 64 21.7 -> 20.6 us); a loop for one, whose few tiles are over before more
+        // code pays for its fetch (0.1 us of 4)
+        if (PH == 2 && ksteps == 4) {
+          kstep(a, b, i != 0 ? 1u : 0u);
+          kstep(a + 2u, b + 2u, 1u);
+          kstep(a + 4u, b + 4u, 1u);
+          kstep(a + 6u, b + 6u, 1u);
+        } else if (PH == 2) {
+          kstep(a, b, i != 0 ? 1u : 0u);
+          if (ksteps == 2) kstep(a + 2u, b + 2u, 1u);
+        } else {
+#pragma unroll 1
+          for (int ks = 0; ks < ksteps; ++ks) kstep(a + 2u * ks, b + 2u * ks, (i | ks) != 0 ? 1u : 0u);
         }
         if (!SINGLE && seq == p.T1 - 1) umma_commit_elected(bar_wfree + frow, elected);
       }
@@ -392,14 +399,14 @@ bool conv_layout_common(ConvParams& q, bool pair, int* smem_bytes) {
 }
 
 // Phases and rows per strip: the least estimated time. Cycles of a CTA: start 5500; its tiles' products (37 + 0.33 N each; 58 at
-// N = 64, 100 at N = 192) or epilogues, whichever are longer; the last epilogue of either convolution. Among equals the
+// N = 64) or epilogues, whichever are longer; the last epilogue of either convolution. Among equals the
 // fewest CTAs (each loads all filters), rows evenly shared.
 template <class Layout>
 void choose_tiling(ConvParams& q, int* R, Layout&& layout) {
   double best_cost = 0;
-  int best_ph = 4;
+  int best_ph = 2;
   *R = 0;
-  for (int PH = 1; PH <= 4; PH *= 2) {
+  for (int PH = 1; PH <= 2; ++PH) {
     const double c = 0.33 * q.C, products = (PH + 2) * 37.0 + 3 * PH * c;
     const double mma = products * 3 * (q.C / 16), epi = 400.0 + 350.0 * ((PH * q.C / 16 + 3) / 4);
     for (int rows = 1; rows <= q.H; ++rows) {
@@ -493,10 +500,10 @@ ago_status_t conv3x3_run(const Plan& plan, FusedState* st, const void* const* in
   };
   CUtensorMap mx, mxt, mw1, mw2;
   if (!get_map(inputs[0], 0, &mx) || !get_map(inputs[0], 4, &mxt) || !get_map(weights[0], 1, &mw1) || !get_map(weights[2], 2, &mw2)) return AGO_ERR_CUDA;
-  auto kernel = q.PH == 4 ? conv3x3_pair_kernel<false, 4> : q.PH == 2 ? conv3x3_pair_kernel<false, 2> : conv3x3_pair_kernel<false, 1>;
+  auto kernel = q.PH == 2 ? conv3x3_pair_kernel<false, 2> : conv3x3_pair_kernel<false, 1>;
   {
-    static int smem_opt_in[3][64] = {};
-    cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(kernel), smem_opt_in[q.PH / 2]);
+    static int smem_opt_in[2][64] = {};
+    cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(kernel), smem_opt_in[q.PH == 2]);
     if (e != cudaSuccess) { *err = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e); return AGO_ERR_CUDA; }
   }
   FusedLaunch launch(dim3((unsigned)(q.N * q.strips)), kThreads, (size_t)host->smem_bytes, stream);
@@ -575,10 +582,10 @@ cudaError_t launch_conv3x3_tc(const void* x, const void* w, const float* bias, c
   q.out = static_cast<__nv_bfloat16*>(out);
   q.wide_store = reinterpret_cast<uintptr_t>(out) % 32 == 0;
   q.status = status;
-  auto kernel = q.PH == 4 ? conv3x3_pair_kernel<true, 4> : q.PH == 2 ? conv3x3_pair_kernel<true, 2> : conv3x3_pair_kernel<true, 1>;
+  auto kernel = q.PH == 2 ? conv3x3_pair_kernel<true, 2> : conv3x3_pair_kernel<true, 1>;
   {
-    static int smem_opt_in[3][64] = {};
-    cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(kernel), smem_opt_in[q.PH / 2]);
+    static int smem_opt_in[2][64] = {};
+    cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(kernel), smem_opt_in[q.PH == 2]);
     if (e != cudaSuccess) return e;
   }
   FusedLaunch launch(dim3((unsigned)(q.N * q.strips)), kThreads, (size_t)entry.smem_bytes, stream);
