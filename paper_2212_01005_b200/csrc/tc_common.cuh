@@ -190,10 +190,6 @@ __device__ __forceinline__ void bulk_copy_to_cluster(uint32_t remote_dst, uint32
   asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                ::"r"(remote_dst), "r"(local_src), "r"(bytes), "r"(remote_bar) : "memory");
 }
-// tcgen05.commit onto an mbarrier given by its cluster address (this CTA's or a peer's).
-__device__ __forceinline__ void umma_commit_cluster(uint32_t bar_cluster_addr) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar_cluster_addr) : "memory");
-}
 
 // ---- per-thread asynchronous copies (global -> shared, 16 bytes, zero-filled beyond src_bytes) ----------
 
@@ -235,7 +231,6 @@ __device__ __forceinline__ void tma_store_3d(const void* tmap, const void* src, 
                : "memory");
 }
 __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait_group_read_all() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 // all of this thread's bulk groups but the most recent one have read their shared-memory source
 __device__ __forceinline__ void bulk_wait_group_read_but_one() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait_group_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
@@ -247,7 +242,6 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const void* tmap, uint64_
       "r"(c3)
       : "memory");
 }
-
 
 // ---- tensor memory ---------------------------------------------------------------------------
 
@@ -291,31 +285,6 @@ __host__ __device__ constexpr uint32_t make_idesc_bf16(uint32_t M, uint32_t N, u
          | (1u << 7)               // A format: bf16
          | (1u << 10)              // B format: bf16
          | (a_mn_major << 15) | (b_mn_major << 16) | ((N >> 3) << 17) | ((M >> 4) << 24);
-}
-
-// D[tmem] (+)= A[smem] * B[smem]; issued by ONE thread.
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                          uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-// Same, with the descriptors given as (low, high) 32-bit halves: the start address and LBO live in
-// the low word, so an issue loop can advance operands with one 32-bit add.
-__device__ __forceinline__ void umma_bf16_lohi(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
-                                               uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-      "mov.b64 da, {%1, %2};\n\t"
-      "mov.b64 db, {%3, %4};\n\t"
-      "setp.ne.b32 p, %6, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
-      : "memory");
 }
 
 // ---- MMA issue from a converged warp --------------------------------------------------------------
@@ -367,13 +336,6 @@ __device__ __forceinline__ void umma_commit_elected(uint64_t* bar, uint32_t elec
       : "memory");
 }
 
-// Arrive on `bar` once all MMAs issued so far by this thread have completed
-// (implies tcgen05.fence::before_thread_sync).
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
-}
-
 // ---- paired CTAs (cta_group::2): one MMA spans the two CTAs of a cluster of two -------------------------------
 // The CTA with the even cluster rank (the leader) issues every MMA; an M = 256 product takes rows 0..127 of A and of
 // the accumulator from the leader and rows 128..255 from its peer, and each CTA holds one half (N / 2 columns) of B
@@ -382,12 +344,6 @@ __device__ __forceinline__ void umma_commit(uint64_t* bar) {
 
 // TMA load whose completion is counted on a barrier that may live in the peer CTA (`bar_cluster_addr` is a
 // shared::cluster address, see cluster_map); the data lands in the issuing CTA.
-__device__ __forceinline__ void tma_load_4d_pair(void* dst, const void* tmap, uint32_t bar_cluster_addr, int c0, int c1, int c2, int c3) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar_cluster_addr), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
-      : "memory");
-}
 __device__ __forceinline__ void tma_load_2d_pair(void* dst, const void* tmap, uint32_t bar_cluster_addr, int c0, int c1) {
   asm volatile(
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
@@ -407,21 +363,8 @@ __device__ __forceinline__ void tmem_relinquish_pair() {
 __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
-// D[tmem of both CTAs] (+)= A * B across the pair; issued by ONE thread of the leader CTA.
-__device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// Arrive on the barrier at cluster address `bar_cluster_addr` once all MMAs issued so far by this thread have
-// completed in both CTAs.
-__device__ __forceinline__ void umma_commit_pair(uint32_t bar_cluster_addr) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar_cluster_addr) : "memory");
-}
-// The same two for a converged warp: every lane executes, the lane chosen once by elect_one() issues.
+// For a converged warp of the leader CTA: every lane executes, the lane chosen once by elect_one() issues.
+// D[tmem of both CTAs] (+)= A * B across the pair.
 __device__ __forceinline__ void umma_bf16_pair_elected(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t elected,
                                                        uint32_t accumulate) {
   asm volatile(
@@ -432,6 +375,7 @@ __device__ __forceinline__ void umma_bf16_pair_elected(uint32_t d_tmem, uint64_t
       ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(elected), "r"(accumulate)
       : "memory");
 }
+// Arrives on the barrier at that cluster address once all MMAs issued so far by this thread have completed in both CTAs.
 __device__ __forceinline__ void umma_commit_pair_elected(uint32_t bar_cluster_addr, uint32_t elected) {
   asm volatile(
       "{\n\t.reg .pred q;\n\t"
@@ -450,12 +394,6 @@ __device__ __forceinline__ void tma_store_2d(const void* tmap, const void* src, 
 // Warp w may touch TMEM lanes 32*(w%4) .. 32*(w%4)+31; thread t of the warp
 // reads lane 32*(w%4)+t, N consecutive 32-bit columns.
 
-__device__ __forceinline__ void tmem_ld_x8(uint32_t taddr, uint32_t* v) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-               : "r"(taddr)
-               : "memory");
-}
 __device__ __forceinline__ void tmem_ld_x16(uint32_t taddr, uint32_t* v) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
@@ -475,15 +413,6 @@ __device__ __forceinline__ void tmem_ld_x32(uint32_t taddr, uint32_t* v) {
       : "r"(taddr)
       : "memory");
 }
-// registers -> tensor memory (same lane / column mapping as the loads)
-__device__ __forceinline__ void tmem_st_x16(uint32_t taddr, const uint32_t* v) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
-      ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]),
-      "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
-      : "memory");
-}
-__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 // The same wait, naming the 16 registers of an outstanding load as in/out operands: no use of them can be moved above
 // the wait, and a later load into the same registers cannot be moved above their last use.
