@@ -316,3 +316,14 @@ def test_residual_block_relu_of_a_nan_is_zero(ago, shape, value, mode):
     assert np.array_equal(np.isfinite(out), np.isfinite(ref)) and not np.isnan(out).any()
     finite = np.isfinite(ref)
     assert_close(out[finite], ref[finite], what=f"residual with {value} {mode}")
+
+
+@pytest.mark.parametrize("mode", ["per_mini_subgraph", "per_op"])
+@pytest.mark.parametrize("shape", [
+    # rows, d, hidden, d_out on pairs of CTAs: last tiles of 8, 72, 104 and 232 columns and of 1, 44 and 196 rows; reductions that end
+    # inside a block; weights whose columns are whole blocks of 64 (one load for all) and not; one to three tiles per pair
+    (1100, 72, 2056, 136), (2500, 200, 1000, 968), (9473, 64, 264, 104), (5120, 128, 1024, 512), (8001, 40, 1088, 256),
+])
+def test_paired_gemm_edges(ago, shape, mode):
+    rows, d, hidden, d_out = shape
+    check(ago, WL.ffn("gemm_pair_edges", [230, *shape], rows, d, hidden, 1, d_out=d_out), mode)
