@@ -16,16 +16,22 @@
 // each B tile once for 256 rows: 131 flop per byte for the chain at BERT-base widths.
 //
 // Per CTA (pair P, half h; h == 0 leads its pair), steps g = (row block, own hidden tile):
-//   TMA     one thread: 24 KB stages -- X [128 x 64] + W1 [64 x 64] (this CTA's half of the tile) for the first
-//           GEMM, W2 [64 x N2 / 4] for the second. Both CTAs' loads complete on the leader's barrier.
+//   TMA     two warps, converged, an elected lane issuing: 24 KB stages in pairs -- X [128 x 64] + W1 [64 x 64] (this CTA's half of
+//           the tile) for the first GEMM, W2 [64 x N2 / 4] for the second. Both CTAs' loads complete on the leader's barrier, one
+//           per pair of stages; stages are handed back singly.
 //   MMA     one warp of the leader, converged, an elected lane issuing: G1(g + 1) into the H accumulator, then G2 over
-//           the two H tiles of step g
-//   epi     8 warps: H accumulator -> registers (accumulator handed back at once) -> + b1, GELU, bf16 -> own slot
+//           the two H tiles of step g, the pair's own one first
+//   epi     16 warps: H accumulator -> registers (accumulator handed back at once) -> + b1, GELU, bf16 -> own slot
 //           -> local "slot full" + bulk copy to the other pair; at the end of a row block: out -> + b2 -> bf16 -> Y
 //   helper  one thread: arms the barrier the other pair's copy completes on; in the non-leading CTA it also relays
-//           "accumulator drained" to the leader, and a thread of the idle MMA warp relays "slots full" and
-//           "output drained". (An arrival on another CTA's barrier is a release at cluster scope and costs about a
-//           thousand cycles: it is kept off the threads that feed the tensor pipe.)
+//           "accumulator drained" and "other pair's tile is here" to the leader, and a thread of the idle MMA warp relays "own
+//           tile is here" and "output drained". (An arrival on another CTA's barrier is a release at cluster scope and costs about
+//           a thousand cycles: it is kept off the threads that feed the tensor pipe.)
+// What bounds it: a step (768 inputs, 768 outputs) takes 6.1k cycles of products, and its tiles 7.75k of shared memory (384 KB
+// written by TMA, 510 KB read by the products, the H tiles, 128 bytes per cycle); measured 8.7k. It took 10.8k with one
+// thread issuing the loads from a lane-0 branch (38 bytes per cycle, see kernel_gemm_pair.cu), one wait per stage, eight epilogue
+// warps that waited for the slot and for the bias before they computed, and G2 waiting for both tiles. 12288 x 768 -> 3072 -> 768
+// 133 -> 119 us, 8448 rows 91 -> 79; the tensor pipe's load brings the clock down to 1.6 - 1.77 GHz meanwhile.
 // Rounds: the clusters the device keeps resident (33 of four CTAs on a B200) walk over the blocks of 256 rows. The blocks of
 // a last, partial round are split into J parts of S / J steps on J clusters; part j stores its fp32 output share in plane j
 // of the workspace (plain stores) and a second, elementwise launch adds the planes, + b2, -> bf16.
@@ -53,9 +59,9 @@ constexpr int kFK = 64;           // reduction elements per ring stage
 constexpr int kFStages = 6;
 constexpr int kFStageBytes = 24 * 1024;
 constexpr int kFSlotBytes = 32 * 1024;      // one H tile of this CTA's rows: 2 x [128 x 64] bf16, 128-byte swizzled
-constexpr int kFEpiWarps = 8;
+constexpr int kFEpiWarps = 16;
 constexpr int kFEpiThreads = kFEpiWarps * 32;
-constexpr int kFThreads = kFEpiThreads + 96;   // + TMA warp + MMA warp + helper warp
+constexpr int kFThreads = kFEpiThreads + 128;   // + MMA warp + helper warp + two TMA warps
 constexpr uint32_t kFOutCol = 128;          // tensor memory: [0, 128) first-GEMM accumulator, [128, 128 + NC) the output
 constexpr int kFSmemBytes = kFStages * kFStageBytes + 2 * kFSlotBytes + 512 + 1024;
 
@@ -78,11 +84,33 @@ struct FfnPairParams {
 };
 
 __device__ __forceinline__ float gelu_tanh_pair(float v) {
-  const float u = 0.7978845608028654f * (v + 0.044715f * v * v * v);
+  const float u = v * (0.7978845608028654f + 0.7978845608028654f * 0.044715f * v * v);
   float t;
   asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(u));
-  return 0.5f * v * (1.0f + t);
+  const float w = 0.5f * v;
+  return w + w * t;
 }
+
+// The steps of a cluster, one after the other. Work items: the whole blocks [0, units_whole), then J parts of S / J steps for
+// each of the other blocks; the cluster walks over the items blockIdx.y, + gridDim.y, ... (divisions only where an item ends).
+struct FfnSteps {
+  int item, unit, part, sb, sb0, sb_end;      // sb: index of the pair of hidden tiles inside the block
+  bool split;
+  __device__ __forceinline__ void start(const FfnPairParams& p, int it) {
+    const int q = (int)(blockIdx.y + (unsigned)it * gridDim.y);
+    item = it; part = 0; unit = q; sb0 = 0; sb_end = p.S;
+    split = q >= p.units_whole;
+    if (split) {
+      const int k = (q - p.units_whole) / p.J, steps = p.S / p.J;
+      part = q - p.units_whole - k * p.J; unit = p.units_whole + k;
+      sb0 = part * steps; sb_end = sb0 + steps;
+    }
+    sb = sb0;
+  }
+  __device__ __forceinline__ void next(const FfnPairParams& p) { if (++sb == sb_end) start(p, item + 1); }
+  __device__ __forceinline__ bool first() const { return sb == sb0; }
+  __device__ __forceinline__ bool last() const { return sb + 1 == sb_end; }
+};
 
 __global__ void __launch_bounds__(kFThreads, 1)
 ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_w1,
@@ -93,47 +121,32 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   uint8_t* sRing = smem;
   uint8_t* sH = smem + kFStages * kFStageBytes;          // slot k: the H tile made by pair k (these rows)
   uint64_t* bars = reinterpret_cast<uint64_t*>(sH + 2 * kFSlotBytes);
-  uint64_t* bar_full = bars;                    // [6] leader: ring stage landed in both CTAs
+  uint64_t* bar_full = bars;                    // [3] leader: both stages of a pair of ring stages landed in both CTAs (count 2)
   uint64_t* bar_empty = bars + 6;               // [6] ring stage consumed
   uint64_t* bar_hacc = bars + 12;               // first GEMM of a step complete (this CTA's rows)
   uint64_t* bar_hfree = bars + 13;              // this CTA's epilogue has read the H accumulator
   uint64_t* bar_phfree = bars + 14;             // leader: the same, relayed from the other CTA of the pair
   uint64_t* bar_slot = bars + 15;               // [2] the H tile of pair k is in slot k of this CTA
-  uint64_t* bar_pslots = bars + 17;             // leader: both slots of the other CTA of the pair are full (relayed)
+  uint64_t* bar_pslot = bars + 22;              // [2] leader: slot k of the other CTA of the pair is full (relayed)
   uint64_t* bar_hdone = bars + 18;              // the tile this CTA made has been multiplied by both pairs (count 2)
   uint64_t* bar_out = bars + 19;                // second GEMM of a row block complete
   uint64_t* bar_outfree = bars + 20;            // this CTA's epilogue has read the output accumulators
   uint64_t* bar_poutfree = bars + 21;           // leader: the same, relayed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 22);
-  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 23);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 24);
+  volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 25);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const uint32_t rank = cluster_ctarank();
   const int P = (int)(rank >> 1), h = (int)(rank & 1u);
   const bool leader = h == 0;
   const uint32_t lead_rank = rank & ~1u, mate_rank = rank ^ 1u, twin_rank = rank ^ 2u;   // pair leader, other CTA of the pair, same rows in the other pair
-  const int S = p.S;
-  // Work items: the whole blocks [0, units_whole), then J parts of S / J steps for each of the other blocks. A cluster
-  // walks over the items blockIdx.y, + gridDim.y, ... (whole blocks first); its steps form one sequence.
-  const int G = (int)gridDim.y, cidx = (int)blockIdx.y, Sp = S / p.J;
+  const int G = (int)gridDim.y, cidx = (int)blockIdx.y;
   const int n_all = p.units_whole + (p.units - p.units_whole) * p.J;
   const int n_items = cidx < n_all ? (n_all - 1 - cidx) / G + 1 : 0;
   const int n_w = cidx < p.units_whole ? (p.units_whole - 1 - cidx) / G + 1 : 0;
-  const int steps = n_w * S + (n_items - n_w) * Sp;
-  struct Step { int item, unit, sb, part; bool first, last, split; };   // sb: index of the pair of hidden tiles inside the block
-  auto step_of = [&](int g) {
-    Step r;
-    if (g < n_w * S) {
-      r.item = g / S; r.sb = g - r.item * S; r.unit = cidx + r.item * G;
-      r.first = r.sb == 0; r.last = r.sb == S - 1; r.split = false; r.part = 0;
-    } else {
-      const int g2 = g - n_w * S, k = g2 / Sp, sp = g2 - k * Sp, q = cidx + (n_w + k) * G - p.units_whole;
-      r.item = n_w + k; r.unit = p.units_whole + q / p.J; r.part = q % p.J; r.sb = r.part * Sp + sp;
-      r.first = sp == 0; r.last = sp == Sp - 1; r.split = true;
-    }
-    return r;
-  };
-  // output chunks of the pair's NC columns: one MMA each (N <= 256): 128 | 256 | 256 + 128
+  const int steps = n_w * p.S + (n_items - n_w) * (p.S / p.J);
+  // output chunks of the pair's NC columns: one MMA each (N <= 256): 128 | 256 | 256 + 128. CTA h of the pair holds B columns
+  // [h NC / 2, (h + 1) NC / 2), the first cn0 / 2 of them for the first chunk.
   const int cn0 = min(p.NC, 256), cn1 = p.NC - cn0;
   const uint32_t g2_tx = (uint32_t)(p.NC / 2) * kFK * 2u;            // W2 bytes per stage and CTA
   const uint32_t g1_tx = (uint32_t)(kFM * kFK * 2 + 64 * kFK * 2);   // X + W1 bytes per stage and CTA
@@ -142,78 +155,72 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
 
   if (tid == kFEpiThreads) {
     *abort_flag = 0u;
-    for (int i = 0; i < 6; ++i) { mbar_init(bar_full + i, 1); mbar_init(bar_empty + i, 1); }
+    for (int i = 0; i < 3; ++i) mbar_init(bar_full + i, 2);
+    for (int i = 0; i < 6; ++i) mbar_init(bar_empty + i, 1);
     mbar_init(bar_hacc, 1); mbar_init(bar_hfree, 1); mbar_init(bar_phfree, 1);
-    mbar_init(bar_slot, 1); mbar_init(bar_slot + 1, 1); mbar_init(bar_pslots, 1);
+    mbar_init(bar_slot, 1); mbar_init(bar_slot + 1, 1); mbar_init(bar_pslot, 1); mbar_init(bar_pslot + 1, 1);
     mbar_init(bar_hdone, 2);
     mbar_init(bar_out, 1); mbar_init(bar_outfree, 1); mbar_init(bar_poutfree, 1);
     fence_mbar_init();
     fence_proxy_async_smem();
   }
-  if (warp == kFEpiWarps + 1) {      // a pair-wide allocation is issued by a warp of either CTA
+  if (warp == kFEpiWarps) {      // a pair-wide allocation is issued by a warp of either CTA
     tmem_alloc_pair(tmem_slot, 512);
     tmem_relinquish_pair();
   }
   tcgen05_fence_before_sync();
   __syncthreads();
-  cluster_sync_all();
+  cluster_meet();
   tcgen05_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
 
-  if (warp == kFEpiWarps) {
-    // ================================ TMA producer (every CTA) ================================
-    if (lane == 0) {
-      tma_prefetch_desc(&tmap_x);
-      tma_prefetch_desc(&tmap_w1);
-      tma_prefetch_desc(&tmap_w2);
-      int s = 0, round = 0;
-      auto next_stage = [&](uint32_t tx_per_cta, uint32_t* full) -> uint8_t* {
-        if (round > 0) mbar_wait_poll(bar_empty + s, (uint32_t)(round - 1) & 1u, abort_flag, p.status, 0x801);
-        *full = cluster_map(smem_u32(bar_full + s), lead_rank);
-        if (leader) mbar_arrive_expect_tx(bar_full + s, 2u * tx_per_cta);   // the leader announces both CTAs' bytes
-        return sRing + s * kFStageBytes;
-      };
-      auto advance = [&]() { if (++s == kFStages) { s = 0; ++round; } };
-      auto load_g1 = [&](int g) {       // first GEMM of the pair's hidden tile of step g: this CTA's rows, its half of the tile
-        const Step st_ = step_of(g);
-        const int hid0 = (2 * st_.sb + P) * kFH + h * 64, row0 = st_.unit * 2 * kFM + h * kFM;
-        for (int kb = 0; kb < p.kblocks; ++kb) {
-          uint32_t full;
-          uint8_t* st = next_stage(g1_tx, &full);
-          tma_load_2d_pair(st, &tmap_x, full, kb * kFK, row0);                   // X [128 rows x 64 k]
-          tma_load_2d_pair(st + 16384, &tmap_w1, full, hid0, kb * kFK);          // W1 [64 k x 64 hidden]
-          advance();
-        }
-      };
-      if (steps > 0) load_g1(0);
-      for (int g = 0; g < steps; ++g) {
-        if (g + 1 < steps) load_g1(g + 1);
-        for (int k = 0; k < 2; ++k) {   // second GEMM over the H tile of pair k: two stages of 64 hidden units
-          const int hid0 = (2 * step_of(g).sb + k) * kFH;
-          for (int kk = 0; kk < 2; ++kk) {
-            uint32_t full;
-            uint8_t* st = next_stage(g2_tx, &full);
-            // this CTA's half of every output chunk, as blocks of [64 k x 64 n]
-            const int c_first = P * p.NC + h * (cn0 / 2);
-            for (int nb = 0; nb < cn0 / 2; nb += 64)
-              tma_load_2d_pair(st + (nb >> 6) * 8192, &tmap_w2, full, c_first + nb, hid0 + kk * 64);
-            if (cn1 > 0) tma_load_2d_pair(st + (cn0 / 128) * 8192, &tmap_w2, full, P * p.NC + cn0 + h * (cn1 / 2), hid0 + kk * 64);
-            advance();
-          }
-        }
+  if (warp >= kFEpiWarps + 2) {
+    // ================================ TMA producers (every CTA): one of the two stages of every pair each ================================
+    const uint32_t elected = elect_one();
+    const uint32_t announces = leader ? elected : 0u;      // the leader announces both CTAs' bytes
+    const int w = warp - kFEpiWarps - 2;
+    if (elected) { tma_prefetch_desc(&tmap_x); tma_prefetch_desc(&tmap_w1); tma_prefetch_desc(&tmap_w2); }
+    __syncwarp();
+    const uint32_t ring = smem_u32(sRing) + (uint32_t)(w * kFStageBytes), full0 = smem_u32(bar_full), lead_full0 = cluster_map(full0, lead_rank);
+    int s = 0, round = 0;                        // pair of stages
+    auto acquire = [&](uint32_t tx_per_cta) {
+      if (round > 0) mbar_wait_poll(bar_empty + 2 * s + w, (uint32_t)(round - 1) & 1u, abort_flag, p.status, 0x801);
+      mbar_arrive_expect_tx_elected(full0 + (uint32_t)(s * 8), 2u * tx_per_cta, announces);
+    };
+    auto advance = [&]() { if (++s == kFStages / 2) { s = 0; ++round; } };
+    auto load_g1 = [&](const FfnSteps& c) {       // first GEMM of the pair's hidden tile of a step: this CTA's rows, its half of the tile
+      const int hid0 = (2 * c.sb + P) * kFH + h * 64, row0 = c.unit * 2 * kFM + h * kFM;
+      for (int kb = w; kb < p.kblocks + w; kb += 2, advance()) {
+        if (kb >= p.kblocks) { acquire(0); continue; }      // an odd number of K blocks: nothing in the last stage
+        acquire(g1_tx);
+        const uint32_t st = ring + (uint32_t)(s * 2 * kFStageBytes), full = lead_full0 + (uint32_t)(s * 8);
+        tma_load_2d_pair_elected(st, &tmap_x, full, kb * kFK, row0, elected);                   // X [128 rows x 64 k]
+        tma_load_2d_pair_elected(st + 16384, &tmap_w1, full, hid0, kb * kFK, elected);          // W1 [64 k x 64 hidden]
+      }
+    };
+    FfnSteps cur, ahead;
+    if (steps > 0) { cur.start(p, 0); ahead = cur; load_g1(ahead); }
+    for (int g = 0; g < steps; ++g, cur.next(p)) {
+      if (g + 1 < steps) { ahead.next(p); load_g1(ahead); }
+      for (int t = 0; t < 2; ++t, advance()) {    // second GEMM over the H tile of pair k, the own one first: two stages of 64 hidden units
+        const int k = t ^ P;
+        acquire(g2_tx);
+        // this CTA's half of every output chunk, as blocks of [64 k x 64 n]
+        tma_load_3d_pair_elected(ring + (uint32_t)(s * 2 * kFStageBytes), &tmap_w2, lead_full0 + (uint32_t)(s * 8), 0,
+                                 (2 * cur.sb + k) * kFH + w * 64, (2 * P + h) * (p.NC >> 7), elected);
       }
     }
     __syncwarp();
   }
-  else if (warp == kFEpiWarps + 1) {
+  else if (warp == kFEpiWarps) {
     if (leader) {
       // ================================ MMA issuer (pair leader): whole warp, elected lane issues ================================
       const uint32_t elected = elect_one();
       const uint32_t idesc1 = make_idesc_bf16(256, kFH, 0, 1);               // A K-major, B N-major (weights as they lie in memory)
       const uint32_t idesc2a = make_idesc_bf16(256, (uint32_t)cn0, 0, 1);
       const uint32_t idesc2b = make_idesc_bf16(256, (uint32_t)max(cn1, 16), 0, 1);
-      int s = 0, round = 0;
-      auto advance = [&]() { if (++s == kFStages) { s = 0; ++round; } };
+      int s = 0, round = 0;                        // pair of stages
+      auto advance = [&]() { if (++s == kFStages / 2) { s = 0; ++round; } };
       auto commit_pair_bar = [&](uint64_t* bar) {      // onto the same barrier of both CTAs of this pair
         const uint32_t e = smem_u32(bar);
         umma_commit_pair_elected(cluster_map(e, rank), elected);
@@ -225,97 +232,113 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
           mbar_wait_poll(bar_phfree, (uint32_t)(g - 1) & 1u, abort_flag, p.status, 0x803);
           tcgen05_fence_after_sync();
         }
-        for (int kb = 0; kb < p.kblocks; ++kb) {
+        for (int kb = 0; kb < p.kblocks; kb += 2, advance()) {
           mbar_wait_poll(bar_full + s, (uint32_t)round & 1u, abort_flag, p.status, 0x804);
           tcgen05_fence_after_sync();
-          const uint32_t st = smem_u32(sRing + s * kFStageBytes);
+          const uint32_t st = smem_u32(sRing + s * 2 * kFStageBytes);
           const uint64_t ad = make_smem_desc(st, 0, 1024, SW_128B);
           const uint64_t bd = make_smem_desc(st + 16384, 8192, 1024, SW_128B);
 #pragma unroll
           for (int ks = 0; ks < kFK / 16; ++ks)
             umma_bf16_pair_elected(tmem_base, ad + 2u * ks, bd + (uint64_t)((ks * 2048) >> 4), idesc1, elected, (kb | ks) != 0);
-          commit_pair_bar(bar_empty + s);
-          advance();
+          commit_pair_bar(bar_empty + 2 * s);
+          if (kb + 1 < p.kblocks) {
+#pragma unroll
+            for (int ks = 0; ks < kFK / 16; ++ks)
+              umma_bf16_pair_elected(tmem_base, ad + (uint64_t)(kFStageBytes >> 4) + 2u * ks, bd + (uint64_t)((kFStageBytes + ks * 2048) >> 4), idesc1, elected, 1u);
+          }
+          commit_pair_bar(bar_empty + 2 * s + 1);
         }
         commit_pair_bar(bar_hacc);
       };
-      if (steps > 0) g1(0);
-      for (int g = 0; g < steps; ++g) {
+      FfnSteps cur;
+      if (steps > 0) { cur.start(p, 0); g1(0); }
+      for (int g = 0; g < steps; ++g, cur.next(p)) {
         if (g + 1 < steps) g1(g + 1);
-        const Step cur = step_of(g);
         const int bi = cur.item;
-        if (cur.first && bi >= 1) {   // the output accumulators of the previous row block have been read in both CTAs
+        const bool first = cur.first();
+        if (first && bi >= 1) {   // the output accumulators of the previous row block have been read in both CTAs
           mbar_wait_poll(bar_outfree, (uint32_t)(bi - 1) & 1u, abort_flag, p.status, 0x805);
           mbar_wait_poll(bar_poutfree, (uint32_t)(bi - 1) & 1u, abort_flag, p.status, 0x806);
           tcgen05_fence_after_sync();
         }
-        mbar_wait_poll(bar_pslots, (uint32_t)g & 1u, abort_flag, p.status, 0x807);     // both tiles of step g are in the other CTA
-        for (int k = 0; k < 2; ++k) {
-          mbar_wait_poll(bar_slot + k, (uint32_t)g & 1u, abort_flag, p.status, 0x808);  // ... and tile k is here
+        for (int t = 0; t < 2; ++t, advance()) {
+          const int k = t ^ P;       // the pair's own tile first: the other one has a copy to make before it is here
+          mbar_wait_poll(bar_slot + k, (uint32_t)g & 1u, abort_flag, p.status, 0x808);   // tile k of step g is here
+          mbar_wait_poll(bar_pslot + k, (uint32_t)g & 1u, abort_flag, p.status, 0x807);  // ... and in the other CTA
+          mbar_wait_poll(bar_full + s, (uint32_t)round & 1u, abort_flag, p.status, 0x809);
           tcgen05_fence_after_sync();
+#pragma unroll
           for (int kk = 0; kk < 2; ++kk) {
-            mbar_wait_poll(bar_full + s, (uint32_t)round & 1u, abort_flag, p.status, 0x809);
-            tcgen05_fence_after_sync();
-            const uint32_t st = smem_u32(sRing + s * kFStageBytes);
+            const uint32_t st = smem_u32(sRing + (2 * s + kk) * kFStageBytes);
             const uint64_t hd = make_smem_desc(smem_u32(sH + k * kFSlotBytes + kk * (kFM * 128)), 0, 1024, SW_128B);
             const uint64_t bd0 = make_smem_desc(st, 8192, 1024, SW_128B);
             const uint64_t bd1 = make_smem_desc(st + (uint32_t)(cn0 / 128) * 8192u, 8192, 1024, SW_128B);
+            const uint32_t acc0 = (uint32_t)(!first || (t | kk) != 0);
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-              const uint32_t acc = (uint32_t)(!cur.first || (k | kk | ks) != 0);
-              umma_bf16_pair_elected(tmem_base + kFOutCol, hd + 2u * ks, bd0 + (uint64_t)((ks * 2048) >> 4), idesc2a, elected, acc);
-              if (cn1 > 0) umma_bf16_pair_elected(tmem_base + kFOutCol + (uint32_t)cn0, hd + 2u * ks, bd1 + (uint64_t)((ks * 2048) >> 4), idesc2b, elected, acc);
+            for (int ks = 0; ks < 4; ++ks)
+              umma_bf16_pair_elected(tmem_base + kFOutCol, hd + 2u * ks, bd0 + (uint64_t)((ks * 2048) >> 4), idesc2a, elected, ks == 0 ? acc0 : 1u);
+            if (cn1 > 0) {
+#pragma unroll
+              for (int ks = 0; ks < 4; ++ks)
+                umma_bf16_pair_elected(tmem_base + kFOutCol + (uint32_t)cn0, hd + 2u * ks, bd1 + (uint64_t)((ks * 2048) >> 4), idesc2b, elected, ks == 0 ? acc0 : 1u);
             }
-            commit_pair_bar(bar_empty + s);
-            advance();
+            commit_pair_bar(bar_empty + 2 * s + kk);
           }
           // slot k has been read in both CTAs of this pair: tell the CTAs that made the tile (pair k)
           const uint32_t e = smem_u32(bar_hdone);
           umma_commit_pair_elected(cluster_map(e, (uint32_t)(2 * k)), elected);
           umma_commit_pair_elected(cluster_map(e, (uint32_t)(2 * k + 1)), elected);
         }
-        if (cur.last) commit_pair_bar(bar_out);
+        if (cur.last()) commit_pair_bar(bar_out);
       }
     } else if (lane == 0) {
-      // ============ relay (the CTA that does not lead): "both slots full", "output drained" -> leader ============
-      const uint32_t lead_pslots = cluster_map(smem_u32(bar_pslots), lead_rank);
+      // ============ relay (the CTA that does not lead): "own slot full", "output drained" -> leader ============
+      const uint32_t lead_pslot = cluster_map(smem_u32(bar_pslot + P), lead_rank);
       const uint32_t lead_poutfree = cluster_map(smem_u32(bar_poutfree), lead_rank);
-      for (int g = 0; g < steps; ++g) {
-        mbar_wait(bar_slot, (uint32_t)g & 1u, abort_flag, p.status, 0x80a);
-        mbar_wait(bar_slot + 1, (uint32_t)g & 1u, abort_flag, p.status, 0x80b);
-        mbar_remote_arrive(lead_pslots);
-        const Step cur = step_of(g);
-        if (cur.first && cur.item >= 1) {
+      FfnSteps cur;
+      if (steps > 0) cur.start(p, 0);
+      for (int g = 0; g < steps; ++g, cur.next(p)) {
+        mbar_wait(bar_slot + P, (uint32_t)g & 1u, abort_flag, p.status, 0x80a);
+        mbar_remote_arrive(lead_pslot);
+        if (cur.first() && cur.item >= 1) {
           mbar_wait(bar_outfree, (uint32_t)(cur.item - 1) & 1u, abort_flag, p.status, 0x80c);
           mbar_remote_arrive(lead_poutfree);
         }
       }
     }
     __syncwarp();
-  } else if (warp == kFEpiWarps + 2) {
-    // ============ helper: arms the barrier of the other pair's copy; relays "accumulator drained" ============
+  } else if (warp == kFEpiWarps + 1) {
+    // ============ helper: arms the barrier of the other pair's copy; relays "accumulator drained", "other slot full" ============
     if (lane == 0) {
+      const uint32_t lead_pslot = cluster_map(smem_u32(bar_pslot + 1 - P), lead_rank);
       const uint32_t lead_phfree = cluster_map(smem_u32(bar_phfree), lead_rank);
       for (int g = 0; g < steps; ++g) {
         mbar_arrive_expect_tx(bar_slot + (1 - P), (uint32_t)kFSlotBytes);
-        if (!leader) {
+        if (!leader && g + 1 < steps) {      // the last accumulator is not used again
           mbar_wait(bar_hfree, (uint32_t)g & 1u, abort_flag, p.status, 0x80d);
           mbar_remote_arrive(lead_phfree);
         }
         mbar_wait(bar_slot + (1 - P), (uint32_t)g & 1u, abort_flag, p.status, 0x80e);   // complete before the next phase is armed
+        if (!leader) mbar_remote_arrive(lead_pslot);
       }
     }
     __syncwarp();
   }
-  else if (warp < kFEpiWarps) {
-    // ================ epilogue warps: thread = (row, half of a tile's 128 hidden units / of the pair's output columns) ================
+  else {
+    // ================ epilogue warps: thread = (row, quarter of a tile's 128 hidden units / of the pair's output columns) ================
     const int row = (warp & 3) * 32 + lane;
-    const int half = warp >> 2;
+    const int quarter = warp >> 2;
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     uint8_t* slot = sH + P * kFSlotBytes;          // this pair's tiles live in slot P of every CTA
     const uint32_t twin_slot = cluster_map(smem_u32(slot), twin_rank);
     const uint32_t twin_bar = cluster_map(smem_u32(bar_slot + P), twin_rank);
-    const int hc = p.NC >> 1;                      // output columns per thread: 64, 128 or 192
+    const int hc = p.NC >> 2;                      // output columns per thread: 32, 64 or 96
+    // tensor-memory column of the pair's output column n (a multiple of 32): the halves of the chunks lie side by side
+    auto out_col = [&](int n) -> uint32_t {
+      const int side = n >= (p.NC >> 1) ? 1 : 0, i = n - side * (p.NC >> 1);
+      return kFOutCol + (uint32_t)(i < (cn0 >> 1) ? side * (cn0 >> 1) + i : cn0 + side * (cn1 >> 1) + i - (cn0 >> 1));
+    };
 
     auto drain_output = [&](int bi, int unit, bool split, int part) {
       // ---- output of work item bi: out (TMEM) -> + b2 -> bf16 -> device memory; the share of a part of a split block goes
@@ -324,12 +347,12 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       const bool row_ok = row0 + row < p.M;
       mbar_wait(bar_out, (uint32_t)bi & 1u, abort_flag, p.status, 0x80f);
       tcgen05_fence_after_sync();
-      const int n0 = P * p.NC + half * hc;
+      const int n0 = P * p.NC + quarter * hc;
       if (split) {
         float* arow = p.acc + ((size_t)part * p.split_rows + (size_t)(row0 + row - p.units_whole * 2 * kFM)) * p.N2 + n0;
         for (int c0 = 0; c0 < hc; c0 += 32) {
           uint32_t v[32];
-          tmem_ld_x32(tmem_base + lane_base + kFOutCol + (uint32_t)(half * hc + c0), v);
+          tmem_ld_x32(tmem_base + lane_base + out_col(quarter * hc + c0), v);
           tmem_ld_wait();
           if (row_ok) {
 #pragma unroll
@@ -346,7 +369,7 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       const float* b2 = p.b2 + n0;
       for (int c0 = 0; c0 < hc; c0 += 32) {
         uint32_t v[32];
-        tmem_ld_x32(tmem_base + lane_base + kFOutCol + (uint32_t)(half * hc + c0), v);
+        tmem_ld_x32(tmem_base + lane_base + out_col(quarter * hc + c0), v);
         tmem_ld_wait();
         if (row_ok) {
 #pragma unroll
@@ -367,36 +390,30 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
     };
 
     int prev_item = 0, prev_unit = 0, prev_part = 0; bool prev_split = false;     // the item whose last step has been seen
-    for (int g = 0; g < steps; ++g) {
-      const Step cur = step_of(g);
-      const int sb = cur.sb;
+    FfnSteps cur;
+    if (steps > 0) cur.start(p, 0);
+    for (int g = 0; g < steps; ++g, cur.next(p)) {
+      const float b1 = __ldg(p.b1 + (size_t)(2 * cur.sb + P) * kFH + quarter * 32 + lane);      // lane j: the bias of the warp's column j
       mbar_wait(bar_hacc, (uint32_t)g & 1u, abort_flag, p.status, 0x810);
       tcgen05_fence_after_sync();
       // the whole share of this thread goes to registers first, so that the accumulator is free for the next first GEMM
-      uint32_t v[64];
-      tmem_ld_x32(tmem_base + lane_base + (uint32_t)(half * 64), v);
-      tmem_ld_x32(tmem_base + lane_base + (uint32_t)(half * 64 + 32), v + 32);
+      uint32_t v[32];
+      tmem_ld_x32(tmem_base + lane_base + (uint32_t)(quarter * 32), v);
       tmem_ld_wait();
       tcgen05_fence_before_sync();
       named_barrier_sync(1, kFEpiThreads);
       if (tid == 0) mbar_arrive(bar_hfree);
+      uint32_t w[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+        w[j] = pack_bf16x2(gelu_tanh_pair(__uint_as_float(v[2 * j]) + __shfl_sync(0xffffffffu, b1, 2 * j)),
+                           gelu_tanh_pair(__uint_as_float(v[2 * j + 1]) + __shfl_sync(0xffffffffu, b1, 2 * j + 1)));
       // both pairs have multiplied the previous content of this slot (and the copy that delivered it is complete)
       if (g >= 1) mbar_wait(bar_hdone, (uint32_t)(g - 1) & 1u, abort_flag, p.status, 0x811);
-      uint8_t* tile = slot + half * (kFM * 128);
-      const float* bb = p.b1 + (size_t)(2 * sb + P) * kFH + half * 64;
+      const uint32_t tile = smem_u32(slot) + (uint32_t)((quarter >> 1) * (kFM * 128));
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const float4 b0 = __ldg(reinterpret_cast<const float4*>(bb + q * 8));
-        const float4 b1v = __ldg(reinterpret_cast<const float4*>(bb + q * 8 + 4));
-        const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1v.x, b1v.y, b1v.z, b1v.w};
-        uint32_t w[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int e = q * 8 + j * 2;
-          w[j] = pack_bf16x2(gelu_tanh_pair(__uint_as_float(v[e]) + bv[2 * j]), gelu_tanh_pair(__uint_as_float(v[e + 1]) + bv[2 * j + 1]));
-        }
-        *reinterpret_cast<uint4*>(tile + swz_offset((uint32_t)row, (uint32_t)q, 128)) = make_uint4(w[0], w[1], w[2], w[3]);
-      }
+      for (int q = 0; q < 4; ++q)
+        sts128(tile + swz_offset((uint32_t)row, (uint32_t)((quarter & 1) * 4 + q), 128), w[4 * q], w[4 * q + 1], w[4 * q + 2], w[4 * q + 3]);
       fence_proxy_async_smem();      // the MMA and the bulk copy read the tile through the async proxy
       named_barrier_sync(1, kFEpiThreads);
       if (tid == 0) {
@@ -404,15 +421,15 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         bulk_copy_to_cluster(twin_slot, smem_u32(slot), kFSlotBytes, twin_bar);   // ... and on its way to the other pair
       }
       // the output of the previous row block is complete once the first GEMM of this block's first step is
-      if (cur.first && cur.item >= 1) drain_output(prev_item, prev_unit, prev_split, prev_part);
-      if (cur.last) { prev_item = cur.item; prev_unit = cur.unit; prev_split = cur.split; prev_part = cur.part; }
+      if (cur.first() && cur.item >= 1) drain_output(prev_item, prev_unit, prev_split, prev_part);
+      if (cur.last()) { prev_item = cur.item; prev_unit = cur.unit; prev_split = cur.split; prev_part = cur.part; }
     }
     if (steps > 0) drain_output(prev_item, prev_unit, prev_split, prev_part);
   }
   tcgen05_fence_before_sync();
   __syncthreads();
-  cluster_sync_all();          // no CTA leaves while another may still copy into it, signal its barriers or multiply into its tensor memory
-  if (warp == kFEpiWarps + 1) tmem_dealloc_pair(tmem_base, 512);
+  cluster_meet();              // no CTA leaves while another may still copy into it, signal its barriers or multiply into its tensor memory
+  if (warp == kFEpiWarps) tmem_dealloc_pair(tmem_base, 512);
 }
 
 // Second launch of a run with split blocks: out = bf16(sum of the J planes + b2) over the rows of the split blocks.
@@ -548,11 +565,14 @@ ago_status_t ffn_pair_run(const Plan& plan, FusedState* st, const void* const* i
     auto it = host->maps.find(key);
     if (it == host->maps.end()) {
       CUtensorMap m;
-      uint64_t dims[2]; uint64_t strides[1]; uint32_t box[2];
+      uint64_t dims[3] = {}; uint64_t strides[2] = {}; uint32_t box[3] = {};
       if (which == 0) { dims[0] = q.K; dims[1] = q.M; strides[0] = (uint64_t)q.K * 2; box[0] = kFK; box[1] = kFM; }
       else if (which == 1) { dims[0] = q.Hid; dims[1] = q.K; strides[0] = (uint64_t)q.Hid * 2; box[0] = 64; box[1] = kFK; }
-      else { dims[0] = q.N2; dims[1] = q.Hid; strides[0] = (uint64_t)q.N2 * 2; box[0] = 64; box[1] = 64; }
-      if (!encode_tmap_bf16(&m, base, 2, dims, strides, box, 128, err)) return false;
+      else {      // blocks of 64 columns: one box brings a CTA's half of all output chunks
+        dims[0] = 64; dims[1] = q.Hid; dims[2] = q.N2 / 64; strides[0] = (uint64_t)q.N2 * 2; strides[1] = 128;
+        box[0] = 64; box[1] = 64; box[2] = q.NC / 128;
+      }
+      if (!encode_tmap_bf16(&m, base, which == 2 ? 3 : 2, dims, strides, box, 128, err)) return false;
       if (host->maps.size() > 4096) host->maps.clear();
       it = host->maps.emplace(key, m).first;
     }

@@ -327,3 +327,13 @@ def test_residual_block_relu_of_a_nan_is_zero(ago, shape, value, mode):
 def test_paired_gemm_edges(ago, shape, mode):
     rows, d, hidden, d_out = shape
     check(ago, WL.ffn("gemm_pair_edges", [230, *shape], rows, d, hidden, 1, d_out=d_out), mode)
+
+
+@pytest.mark.parametrize("shape", [
+    # 256-row blocks on paired clusters: one, three and five K blocks (an odd one leaves half a pair of stages empty), 256 to 768
+    # outputs (the halves of the chunks side by side), whole blocks before split ones, several blocks per cluster
+    (7200, 64, 256, 256), (7000, 192, 512, 768), (8700, 320, 512, 512), (17000, 64, 256, 768), (9000, 128, 768, 768),
+])
+def test_feed_forward_paired_clusters(ago, shape):
+    rows, d, hidden, d_out = shape
+    check(ago, WL.ffn("ffn_pair_edges", [231, *shape], rows, d, hidden, 1, d_out=d_out))
