@@ -31,7 +31,8 @@
 // written by TMA, 510 KB read by the products, the H tiles, 128 bytes per cycle); measured 8.7k. It took 10.8k with one
 // thread issuing the loads from a lane-0 branch (38 bytes per cycle, see kernel_gemm_pair.cu), one wait per stage, eight epilogue
 // warps that waited for the slot and for the bias before they computed, and G2 waiting for both tiles. 12288 x 768 -> 3072 -> 768
-// 133 -> 119 us, 8448 rows 91 -> 79; the tensor pipe's load brings the clock down to 1.6 - 1.77 GHz meanwhile.
+// 133 -> 119 us, 8448 rows 91 -> 79; the tensor pipe's load brings the clock down to 1.6 - 1.77 GHz meanwhile. With the last
+// item's outputs turned in the ring 119 -> 108, 3001 rows 52 -> 44.6, 1815 rows 40 -> 30.
 // Rounds: the clusters the device keeps resident (33 of four CTAs on a B200) walk over the blocks of 256 rows. The blocks of
 // a last, partial round are split into J parts of S / J steps on J clusters; part j stores its fp32 output share in plane j
 // of the workspace (plain stores) and a second, elementwise launch adds the planes, + b2, -> bf16.
@@ -81,6 +82,7 @@ struct FfnPairParams {
   int units_whole, J;
   float* acc;              // [J][split_rows][N2] fp32
   int split_rows;          // rows of the split blocks that exist: M - units_whole * 256
+  int wide_out, wide_acc;  // out / acc start on a 32-byte boundary (their rows then do too)
 };
 
 __device__ __forceinline__ float gelu_tanh_pair(float v) {
@@ -340,47 +342,70 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       return kFOutCol + (uint32_t)(i < (cn0 >> 1) ? side * (cn0 >> 1) + i : cn0 + side * (cn1 >> 1) + i - (cn0 >> 1));
     };
 
-    auto drain_output = [&](int bi, int unit, bool split, int part) {
+    auto drain_output = [&](int bi, int unit, bool split, int part, bool ring_free) {
       // ---- output of work item bi: out (TMEM) -> + b2 -> bf16 -> device memory; the share of a part of a split block goes
       // to its plane of the fp32 buffer instead (a second, small kernel adds the planes and writes the output) ----
+      // The cluster's last item goes through the ring, which nothing uses any more: a warp's 32 x 32 block is turned so that a store
+      // covers whole rows of it (a row per lane takes 32 lines per store: 16-byte stores took 6 us per 128 columns of
+      // fp32 sums, 768 columns 18 of a run's 23 us). The others are stored a sector at a time, beside the next item's products.
       const int row0 = unit * 2 * kFM + h * kFM;
-      const bool row_ok = row0 + row < p.M;
       mbar_wait(bar_out, (uint32_t)bi & 1u, abort_flag, p.status, 0x80f);
       tcgen05_fence_after_sync();
-      const int n0 = P * p.NC + quarter * hc;
-      if (split) {
-        float* arow = p.acc + ((size_t)part * p.split_rows + (size_t)(row0 + row - p.units_whole * 2 * kFM)) * p.N2 + n0;
-        for (int c0 = 0; c0 < hc; c0 += 32) {
-          uint32_t v[32];
-          tmem_ld_x32(tmem_base + lane_base + out_col(quarter * hc + c0), v);
-          tmem_ld_wait();
-          if (row_ok) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-              *reinterpret_cast<uint4*>(arow + c0 + q * 4) = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-          }
-        }
-        tcgen05_fence_before_sync();
-        named_barrier_sync(1, kFEpiThreads);
-        if (tid == 0) mbar_arrive(bar_outfree);
-        return;
-      }
-      __nv_bfloat16* orow = p.out + (size_t)(row0 + row) * p.N2 + n0;
-      const float* b2 = p.b2 + n0;
+      const int n0 = P * p.NC + quarter * hc, esz = split ? 4 : 2;
+      uint8_t* dst = split ? reinterpret_cast<uint8_t*>(p.acc + ((size_t)part * p.split_rows + (size_t)(row0 - p.units_whole * 2 * kFM)) * p.N2 + n0)
+                           : reinterpret_cast<uint8_t*>(p.out + (size_t)row0 * p.N2 + n0);        // the CTA's first row, this warp's first column
+      const size_t pitch = (size_t)p.N2 * esz;
+      const bool wide = split ? p.wide_acc : p.wide_out;
+      const uint32_t buf = smem_u32(sRing) + (uint32_t)(warp * 4096);
+      const int rows_left = p.M - row0 - (warp & 3) * 32;      // rows of this warp's quarter that exist
+      uint8_t* wdst = dst + (size_t)((warp & 3) * 32) * pitch;
       for (int c0 = 0; c0 < hc; c0 += 32) {
         uint32_t v[32];
         tmem_ld_x32(tmem_base + lane_base + out_col(quarter * hc + c0), v);
         tmem_ld_wait();
-        if (row_ok) {
+        if (!split) {
+          const float b = __ldg(p.b2 + n0 + c0 + lane);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const float4 b0 = __ldg(reinterpret_cast<const float4*>(b2 + c0 + q * 8));
-            const float4 b1v = __ldg(reinterpret_cast<const float4*>(b2 + c0 + q * 8 + 4));
-            *reinterpret_cast<uint4*>(orow + c0 + q * 8) =
-                make_uint4(pack_bf16x2(__uint_as_float(v[q * 8]) + b0.x, __uint_as_float(v[q * 8 + 1]) + b0.y),
-                           pack_bf16x2(__uint_as_float(v[q * 8 + 2]) + b0.z, __uint_as_float(v[q * 8 + 3]) + b0.w),
-                           pack_bf16x2(__uint_as_float(v[q * 8 + 4]) + b1v.x, __uint_as_float(v[q * 8 + 5]) + b1v.y),
-                           pack_bf16x2(__uint_as_float(v[q * 8 + 6]) + b1v.z, __uint_as_float(v[q * 8 + 7]) + b1v.w));
+          for (int j = 0; j < 16; ++j)
+            v[j] = pack_bf16x2(__uint_as_float(v[2 * j]) + __shfl_sync(0xffffffffu, b, 2 * j), __uint_as_float(v[2 * j + 1]) + __shfl_sync(0xffffffffu, b, 2 * j + 1));
+        }
+        uint8_t* cdst = wdst + (size_t)c0 * esz;
+        if (ring_free) {
+          __syncwarp();
+          if (split) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) sts128(buf + (uint32_t)(lane * 128 + ((k ^ (lane & 7)) << 4)), v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const int r = k * 4 + (lane >> 3), c = lane & 7;
+              const float4 f = lds128f(buf + (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4)));
+              if (r < rows_left) *reinterpret_cast<float4*>(cdst + (size_t)r * pitch + c * 16) = f;
+            }
+          } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) sts128(buf + swz_offset((uint32_t)lane, (uint32_t)k, 64), v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const int r = k * 8 + (lane >> 2), c = lane & 3;
+              const float4 f = lds128f(buf + swz_offset((uint32_t)r, (uint32_t)c, 64));
+              if (r < rows_left) *reinterpret_cast<float4*>(cdst + (size_t)r * pitch + c * 16) = f;
+            }
+          }
+        } else if (lane < rows_left) {
+          uint8_t* o = cdst + (size_t)lane * pitch;
+          const int words = split ? 32 : 16;
+#pragma unroll
+          for (int k = 0; k < 32; k += 8) {
+            if (k >= words) break;
+            if (wide) {
+              const uint32_t w[8] = {v[k], v[k + 1], v[k + 2], v[k + 3], v[k + 4], v[k + 5], v[k + 6], v[k + 7]};
+              store_global_32(o + k * 4, w);
+            } else {
+              *reinterpret_cast<uint4*>(o + k * 4) = make_uint4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+              *reinterpret_cast<uint4*>(o + k * 4 + 16) = make_uint4(v[k + 4], v[k + 5], v[k + 6], v[k + 7]);
+            }
           }
         }
       }
@@ -421,10 +446,10 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         bulk_copy_to_cluster(twin_slot, smem_u32(slot), kFSlotBytes, twin_bar);   // ... and on its way to the other pair
       }
       // the output of the previous row block is complete once the first GEMM of this block's first step is
-      if (cur.first() && cur.item >= 1) drain_output(prev_item, prev_unit, prev_split, prev_part);
+      if (cur.first() && cur.item >= 1) drain_output(prev_item, prev_unit, prev_split, prev_part, false);
       if (cur.last()) { prev_item = cur.item; prev_unit = cur.unit; prev_split = cur.split; prev_part = cur.part; }
     }
-    if (steps > 0) drain_output(prev_item, prev_unit, prev_split, prev_part);
+    if (steps > 0) drain_output(prev_item, prev_unit, prev_split, prev_part, true);
   }
   tcgen05_fence_before_sync();
   __syncthreads();
@@ -556,6 +581,8 @@ ago_status_t ffn_pair_run(const Plan& plan, FusedState* st, const void* const* i
   q.out = static_cast<__nv_bfloat16*>(output);
   q.status = status_word;
   q.acc = nullptr;
+  q.wide_out = reinterpret_cast<uintptr_t>(output) % 32 == 0;
+  q.wide_acc = reinterpret_cast<uintptr_t>(workspace) % 32 == 0;
   if (q.J > 1) {
     if (!workspace) { *err = "fused feed-forward (paired cluster, split last round): no workspace attached"; return AGO_ERR_INVALID_ARG; }
     q.acc = static_cast<float*>(workspace);   // every element of it is written before it is read: nothing to zero

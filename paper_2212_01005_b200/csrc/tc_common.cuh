@@ -228,6 +228,23 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const void* tmap, uint64_
       ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2)
       : "memory");
 }
+// The same from a converged warp, on its elected lane (see "MMA issue from a converged warp").
+__device__ __forceinline__ void tma_load_2d_elected(uint32_t dst_saddr, const void* tmap, uint32_t bar_saddr, int c0, int c1, uint32_t elected) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
+      "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n\t}"
+      ::"r"(dst_saddr), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar_saddr), "r"(c0), "r"(c1), "r"(elected)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_3d_elected(uint32_t dst_saddr, const void* tmap, uint32_t bar_saddr, int c0, int c1, int c2, uint32_t elected) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %6, 0;\n\t"
+      "@q cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];\n\t}"
+      ::"r"(dst_saddr), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar_saddr), "r"(c0), "r"(c1), "r"(c2), "r"(elected)
+      : "memory");
+}
 // Store of a shared-memory tile into a 3-D tensor (the part of the box outside the tensor is clipped). The copy belongs to
 // the issuing thread's bulk group: that thread commits the group and waits for it (for its reads of shared memory before the
 // tile is overwritten, for all of it before the CTA exits).
