@@ -16,7 +16,11 @@
 // into all N2 output columns without recomputation and without reductions outside the SM.
 //
 // Per CTA (rank r), T = hidden tiles / CS steps:
-//   ring   TMA producer warp: stages of X [RP x 64] + W1 [64 x BH] for the first GEMM, W2 [64 x N2/CS] for the second
+//   ring   two TMA warps, every second stage each (three stages or more, so a stage's previous use is over when its next is waited
+//          for): X [RP x 64] + W1 [64 x BH] for the first GEMM, W2 [64 x N2/CS] for the second; a third one for W2 tiles with
+//          memory of their own. Converged, an elected lane issuing, one load per operand: a thread in a lane-0 branch that loaded
+//          every 64 columns by themselves took 350 cycles per stage, 4.5k of a one-step run's 34k (512 rows 17.4 -> 15.7 us,
+//          64 rows 11.2 -> 9.5, 1815 rows 40 -> 36)
 //   MMA    one warp: G1(t+1): Hacc[(t+1) & 1] = X W1[:, tile (t+1) CS + r]; then for k = 0..CS-1
 //          G2(k): out += H slot k * W2[tile t CS + k, own columns]; its completion is committed onto CTA k's
 //          "slot consumed" barrier
@@ -46,7 +50,7 @@ using namespace ffn_cluster;
 // Epilogue warps: four per tensor-memory lane quarter, each with a quarter of a tile's columns; two where the epilogue hides
 // behind the next step's products (whole row blocks in several steps).
 constexpr int epi_warps_of(int bh, bool full) { return full && bh == 128 ? 8 : 16; }
-constexpr int threads_of(int bh, bool full) { return epi_warps_of(bh, full) * 32 + 64; }   // + TMA warp + MMA warp
+constexpr int threads_of(int bh, bool full) { return epi_warps_of(bh, full) * 32 + 128; }   // + MMA warp + three TMA warps
 constexpr uint32_t kOutCol = 256;            // tensor memory: [0, 256) two first-GEMM accumulators, [256, 256 + NC) the output
 
 struct FfnClusterParams : FfnClusterShape {
@@ -55,13 +59,15 @@ struct FfnClusterParams : FfnClusterShape {
   __nv_bfloat16* out;
   unsigned int* status;
   float* acc;              // J > 1: fp32 [M x N2] partial sums, zero between launches
+  int wide_out;            // out starts on a 32-byte boundary (its rows then do too)
 };
 
 __device__ __forceinline__ float gelu_tanh_fast(float v) {
-  const float u = 0.7978845608028654f * (v + 0.044715f * v * v * v);
+  const float u = v * (0.7978845608028654f + 0.7978845608028654f * 0.044715f * v * v);
   float t;
   asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(u));
-  return 0.5f * v * (1.0f + t);
+  const float w = 0.5f * v;
+  return w + w * t;
 }
 
 __device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float c, float d) {
@@ -115,9 +121,6 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
   auto unit_of = [&](int step) { return (int)blockIdx.y + (step / T) * (int)gridDim.y; };
   auto row0_of = [&](int step) { return (unit_of(step) / J) * kBM; };
   auto tile0_of = [&](int step) { return ((unit_of(step) % J) * T + step % T) * CS; };   // first of the step's CS hidden tiles
-  grid_dependency_wait();      // the previous grid of the stream has completed; device memory may be touched
-  grid_launch_dependents();
-
   if (tid == kEpiThreads) {
     *abort_flag = 0u;
     for (int i = 0; i < kMaxStages; ++i) { mbar_init(bar_full + i, 1); mbar_init(bar_empty + i, 1); }
@@ -145,63 +148,64 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
   auto cluster_started = [] { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); };
   tcgen05_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
+  // The set-up above overlaps the previous grid's tail (the second launch of the previous run leaves the SM room for this CTA).
+  grid_dependency_wait();      // the previous grid of the stream has completed; device memory may be touched
+  grid_launch_dependents();
   const int n0 = r * p.NC;     // first output column of this CTA
 
-  if (warp == kEpiWarps) {
-    // ================================ TMA producer ================================
-    if (lane == 0) {
-      tma_prefetch_desc(&tmap_x);
-      tma_prefetch_desc(&tmap_w1);
-      tma_prefetch_desc(&tmap_w2);
-      int s = 0, round = 0;
-      auto next_stage = [&](uint32_t bytes) -> uint8_t* {
-        if (round > 0) mbar_wait(bar_empty + s, (uint32_t)(round - 1) & 1u, abort_flag, p.status, 0x701);
-        mbar_arrive_expect_tx(bar_full + s, bytes);
-        return sRing + s * stage_bytes;
-      };
-      auto advance = [&]() { if (++s == stages) { s = 0; ++round; } };
-      auto load_g1 = [&](int step, int from, int to) {       // first GEMM of this CTA's hidden tile of that step
-        const int hid0 = (tile0_of(step) + r) * BH, row0 = row0_of(step);
-        for (int kb = from; kb < to; ++kb) {
-          uint8_t* st = next_stage((uint32_t)(RP * 128 + BH * 128));
-          tma_load_2d(st, &tmap_x, bar_full + s, kb * kBK, row0);                          // X [RP rows x 64 k]
-          for (int h = 0; h < halves; ++h)                                                 // W1 [64 k x 64 n] blocks
-            tma_load_2d(st + RP * 128 + h * 8192, &tmap_w1, bar_full + s, hid0 + h * 64, kb * kBK);
-          advance();
-        }
-      };
-      const int ahead = min(stages, p.kblocks);
-      if (steps > 0) load_g1(0, 0, ahead);
-      if (own_w2 && steps > 0) {             // the whole second GEMM's operand is on its way before the ring comes round
+  if (warp > kEpiWarps) {
+    // ================================ TMA producers: two for every second ring stage each, one for W2 tiles with memory of their own ================================
+    const int w = warp - kEpiWarps - 1;
+    const uint32_t elected = elect_one();
+    if (elected) { tma_prefetch_desc(&tmap_x); tma_prefetch_desc(&tmap_w1); tma_prefetch_desc(&tmap_w2); }
+    __syncwarp();
+    if (w == 2) {
+      if (own_w2 && steps > 0) {             // the whole second GEMM's operand
         for (int i = 0; i < CS; ++i) {
           const int hid0 = (tile0_of(0) + (int)((r + CS - i) % CS)) * BH;
           for (int h = 0; h < halves; ++h) {
-            uint64_t* bar = bar_w2 + i * halves + h;
-            uint8_t* st = smem + p.w2_off + (i * halves + h) * p.NC * 128;
-            mbar_arrive_expect_tx(bar, (uint32_t)(p.NC * 128));
-            for (int nb = 0; nb < p.NC; nb += 64) tma_load_2d(st + nb * 128, &tmap_w2, bar, n0 + nb, hid0 + h * 64);
+            const uint32_t bar = smem_u32(bar_w2 + i * halves + h), st = smem_u32(smem) + (uint32_t)(p.w2_off + (i * halves + h) * p.NC * 128);
+            mbar_arrive_expect_tx_elected(bar, (uint32_t)(p.NC * 128), elected);
+            tma_load_3d_elected(st, &tmap_w2, bar, 0, hid0 + h * 64, n0 >> 6, elected);
           }
         }
       }
-      if (steps > 0) load_g1(0, ahead, p.kblocks);
+    } else {
+      const uint32_t ring = smem_u32(sRing), full0 = smem_u32(bar_full);
+      int s = 0, round = 0;
+      bool mine = w == 0;                    // stages go to the two warps in turn
+      auto acquire = [&](uint32_t bytes) -> uint32_t {
+        if (round > 0) mbar_wait_poll(bar_empty + s, (uint32_t)(round - 1) & 1u, abort_flag, p.status, 0x701);
+        mbar_arrive_expect_tx_elected(full0 + (uint32_t)(s * 8), bytes, elected);
+        return ring + (uint32_t)(s * stage_bytes);
+      };
+      auto advance = [&]() { mine = !mine; if (++s == stages) { s = 0; ++round; } };
+      auto load_g1 = [&](int step) {         // first GEMM of this CTA's hidden tile of that step
+        const int hid0 = (tile0_of(step) + r) * BH, row0 = row0_of(step);
+        for (int kb = 0; kb < p.kblocks; ++kb, advance()) {
+          if (!mine) continue;
+          const uint32_t st = acquire((uint32_t)(RP * 128 + BH * 128)), full = full0 + (uint32_t)(s * 8);
+          tma_load_2d_elected(st, &tmap_x, full, kb * kBK, row0, elected);                                              // X [RP rows x 64 k]
+          tma_load_3d_elected(st + (uint32_t)(RP * 128), &tmap_w1, full, 0, kb * kBK, hid0 >> 6, elected);              // W1 [64 k x 64 n] blocks
+        }
+      };
+      if (steps > 0) load_g1(0);
       for (int step = 0; step < steps && !own_w2; ++step) {
-        if (step + 1 < steps) load_g1(step + 1, 0, p.kblocks);
+        if (step + 1 < steps) load_g1(step + 1);
         for (int i = 0; i < CS; ++i) {      // second GEMM over hidden tile t CS + k: two stages of 64 hidden units
           const int k = (int)((r + CS - i) % CS);   // in the order the MMA warp consumes the slots: own tile first
           const int hid0 = (tile0_of(step) + k) * BH;
-          for (int h = 0; h < halves; ++h) {
-            uint8_t* st = next_stage((uint32_t)(p.NC * 128));
-#pragma unroll
-            for (int nb = 0; nb < 4; ++nb)          // W2 [64 k x 64 n] per block
-              if (nb * 64 < p.NC) tma_load_2d(st + nb * 8192, &tmap_w2, bar_full + s, n0 + nb * 64, hid0 + h * 64);
-            advance();
+          for (int h = 0; h < halves; ++h, advance()) {
+            if (!mine) continue;
+            const uint32_t st = acquire((uint32_t)(p.NC * 128));
+            tma_load_3d_elected(st, &tmap_w2, full0 + (uint32_t)(s * 8), 0, hid0 + h * 64, n0 >> 6, elected);           // W2 [64 k x 64 n] blocks
           }
         }
       }
     }
     __syncwarp();
     cluster_started();
-  } else if (warp == kEpiWarps + 1) {
+  } else if (warp == kEpiWarps) {
     // ================================ MMA issuer ================================
     // the whole warp, converged; MMAs and commits predicated on one elected lane (see tc_common.cuh)
     {
@@ -398,15 +402,17 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
             tmem_ld_x16(tmem_base + lane_base + kOutCol + part * hc + c0, v);
             tmem_ld_wait();
             if (row_ok) {
+              uint32_t w[8];
 #pragma unroll
-              for (int q = 0; q < 2; ++q) {
-                const float4 b0 = __ldg(reinterpret_cast<const float4*>(b2 + c0 + q * 8));
-                const float4 b1v = __ldg(reinterpret_cast<const float4*>(b2 + c0 + q * 8 + 4));
-                *reinterpret_cast<uint4*>(orow + c0 + q * 8) =
-                    make_uint4(pack_bf16x2(__uint_as_float(v[q * 8]) + b0.x, __uint_as_float(v[q * 8 + 1]) + b0.y),
-                               pack_bf16x2(__uint_as_float(v[q * 8 + 2]) + b0.z, __uint_as_float(v[q * 8 + 3]) + b0.w),
-                               pack_bf16x2(__uint_as_float(v[q * 8 + 4]) + b1v.x, __uint_as_float(v[q * 8 + 5]) + b1v.y),
-                               pack_bf16x2(__uint_as_float(v[q * 8 + 6]) + b1v.z, __uint_as_float(v[q * 8 + 7]) + b1v.w));
+              for (int q = 0; q < 4; ++q) {
+                const float4 b = __ldg(reinterpret_cast<const float4*>(b2 + c0 + q * 4));
+                w[2 * q] = pack_bf16x2(__uint_as_float(v[q * 4]) + b.x, __uint_as_float(v[q * 4 + 1]) + b.y);
+                w[2 * q + 1] = pack_bf16x2(__uint_as_float(v[q * 4 + 2]) + b.z, __uint_as_float(v[q * 4 + 3]) + b.w);
+              }
+              if (p.wide_out) store_global_32(orow + c0, w);      // a whole sector
+              else {
+                *reinterpret_cast<uint4*>(orow + c0) = make_uint4(w[0], w[1], w[2], w[3]);
+                *reinterpret_cast<uint4*>(orow + c0 + 8) = make_uint4(w[4], w[5], w[6], w[7]);
               }
             }
           }
@@ -419,7 +425,7 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
   }
   tcgen05_fence_before_sync();
   __syncthreads();
-  cluster_sync_all();          // no CTA leaves while a peer may still copy into it or signal its barriers
+  cluster_meet();              // no CTA leaves while a peer may still copy into it or signal its barriers
   if (warp == 0) tmem_dealloc(tmem_base, 512);
 }
 
@@ -486,9 +492,10 @@ bool cluster_shape(const Plan& plan, FfnClusterParams* q) {
 }
 }  // namespace
 
-// Set-up + steps of the longest cluster x (the first product's operands, W2's, a constant, what a W2 stage costs besides its bytes);
+// Set-up + steps of the longest cluster x (the first product's operands, W2's, a constant, what a W2 stage costs besides its bytes, the
+// chain of hand-offs where an input of one K block does not hide it);
 // split row blocks: the additions (3 T bytes/s). One step with W2 stages of its own: everything is on its way at once, which is
-// a chain of latencies. 507 measured chains of 1 to 12288 rows and widths of 64 to 4096: 6.7 % and 5.5 % rms.
+// a chain of latencies. 232 measured chains of 1 to 12288 rows and widths of 64 to 4096: 6 % and 3 % rms.
 double ffn_cluster_estimate(const Plan& plan) {
   FfnClusterParams q{};
   if (!cluster_shape(plan, &q)) return -1.0;
@@ -496,8 +503,8 @@ double ffn_cluster_estimate(const Plan& plan) {
   const double units = (double)((q.M + kBM - 1) / kBM) * q.J, steps = std::ceil(units / kResident[q.CS]) * q.Tp;
   const double w2_stages = q.CS * (q.BH / 64), g1 = q.kblocks * (q.RP + q.BH) / 256.0, w2 = w2_stages * q.NC / 256.0;      // in 32 KB
   const double additions = q.J > 1 ? (double)q.J * q.M * q.N2 * 4 / 3.0e6 : 0.0;
-  if (q.w2_off > 0) return 5.25 + 0.136 * g1 + 0.48 * w2 + 0.111 * q.kblocks + 1.56 * q.RP / kBM + 1.07 * additions;
-  return 5.27 + steps * (0.202 * g1 + 0.445 * w2 + 0.53 + 0.5 * w2_stages) + 0.92 * additions;
+  if (q.w2_off > 0) return 5.05 + 0.096 * g1 + 0.477 * w2 + 0.089 * q.kblocks + 2.02 * q.RP / kBM + 0.72 * additions;
+  return 4.53 + steps * (0.18 * g1 + 0.216 * w2 + 0.339 + 0.584 * w2_stages + (q.kblocks == 1 ? 0.38 : 0.0)) + 1.04 * additions;
 }
 
 // AGO_ERR_UNSUPPORTED (without touching *err) when the shape has no cluster split: the caller falls back to the
@@ -541,6 +548,7 @@ ago_status_t ffn_cluster_run(const Plan& plan, FusedState* st, const void* const
   q.b2 = static_cast<const float*>(weights[3]);
   q.out = static_cast<__nv_bfloat16*>(output);
   q.status = status_word;
+  q.wide_out = reinterpret_cast<uintptr_t>(output) % 32 == 0;
   if (q.J > 1) {
     if (!workspace) { *err = "fused feed-forward (cluster, split row blocks): no workspace attached"; return AGO_ERR_INVALID_ARG; }
     q.acc = static_cast<float*>(workspace);
@@ -558,11 +566,14 @@ ago_status_t ffn_cluster_run(const Plan& plan, FusedState* st, const void* const
     auto it = host->maps.find(key);
     if (it == host->maps.end()) {
       CUtensorMap m;
-      uint64_t dims[2]; uint64_t strides[1]; uint32_t box[2];
+      uint64_t dims[3] = {}; uint64_t strides[2] = {}; uint32_t box[3] = {};
       if (which == 0) { dims[0] = q.K; dims[1] = q.M; strides[0] = (uint64_t)q.K * 2; box[0] = kBK; box[1] = (uint32_t)q.RP; }
-      else if (which == 1) { dims[0] = q.Hid; dims[1] = q.K; strides[0] = (uint64_t)q.Hid * 2; box[0] = 64; box[1] = kBK; }
-      else { dims[0] = q.N2; dims[1] = q.Hid; strides[0] = (uint64_t)q.N2 * 2; box[0] = 64; box[1] = 64; }
-      if (!encode_tmap_bf16(&m, base, 2, dims, strides, box, 128, err)) return false;
+      else {      // a weight matrix in blocks of 64 columns: one box brings a tile's
+        const int cols = which == 1 ? q.Hid : q.N2;
+        dims[0] = 64; dims[1] = which == 1 ? q.K : q.Hid; dims[2] = cols / 64; strides[0] = (uint64_t)cols * 2; strides[1] = 128;
+        box[0] = 64; box[1] = 64; box[2] = (uint32_t)((which == 1 ? q.BH : q.NC) / 64);
+      }
+      if (!encode_tmap_bf16(&m, base, which == 0 ? 2 : 3, dims, strides, box, 128, err)) return false;
       if (host->maps.size() > 4096) host->maps.clear();
       it = host->maps.emplace(key, m).first;
     }
