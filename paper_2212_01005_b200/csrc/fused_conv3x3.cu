@@ -28,7 +28,9 @@
 // outputs were staged for TMA stores: the epilogue read three accumulators and took 2200 cycles per 112 pixels x 64
 // channels, twice the time of the products. 32 x 56 x 56 x 64 23.5 -> 20.6 us, 43 x 64 x 61 x 32 40.6 -> 17.3, 6 x 79 x 78 x 16
 // 11.4 -> 5.8, 14 x 14 x 64 (one image) 6.3 -> 5.3. Bound now by the products (13.8 us of the first, 8.9 at the dense rate), then by
-// the residual and the outputs, all of which move during the second convolution.
+// the residual and the outputs, all of which move during the second convolution: 32 lines per request, so a tile's epilogue took
+// up to 4.4k cycles where its products take 3.6k, 2.6k with whole sectors of the residual per request. (Issuing the loads converged, on an
+// elected lane, as the other kernels do, makes the MMA loop spill: 22.4 us.)
 //
 // All nine taps of one convolution stay resident (three slots of one filter row
 // each); the second convolution's rows replace the first's slot by slot as the
@@ -104,7 +106,9 @@ __device__ __forceinline__ void add_bf16x2(float& a, float& b, uint32_t x) {
 
 // SINGLE = false: the fused pair. SINGLE = true: one convolution with its simple operators (second-convolution
 // tiles only, reading the input rows directly), the tensor-core stage kernel of the unfused mode.
-template <bool SINGLE, int PH>
+// WIDE: the residual is read a sector per request (a second instance: the loads' register groups cost the narrower shapes' loops more
+// than they save, 43 x 64 x 61 x 32 17.7 -> 19.4 us)
+template <bool SINGLE, int PH, bool WIDE>
 __global__ void __launch_bounds__(kThreads, 1)
 conv3x3_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_xtail,
                     const __grid_constant__ CUtensorMap tmap_w1, const __grid_constant__ CUtensorMap tmap_w2, const ConvParams p) {
@@ -276,15 +280,19 @@ conv3x3_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
       const int m = (second ? seq - p.T1 : seq) * kTile + wq * 32 + lane;
       const int a = (int)fast_div((uint32_t)m, (uint32_t)p.Q, p.q_recip), q = m - a * p.Q;   // row of the intermediate / output in the strip
       const size_t row0 = (((size_t)n * p.H + h0 + a) * p.W + PH * q) * p.C;                 // second: output column PH q of that row
-      uint4 xr[PH][2];                // the residual, fetched ahead of the accumulators
+      uint32_t xr[PH][8];             // the residual, fetched ahead of the accumulators
 #pragma unroll
       for (int i = 0; i < PH; ++i) {
         const int u = cg + 4 * i, o = u >> p.cg_shift, col0 = (u & cg_mask) * 16;
-        xr[i][0] = xr[i][1] = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) xr[i][j] = 0u;
         if (second && do_res && u < units && a < rows_valid && PH * q + o < p.W) {
-          const uint4* rp = reinterpret_cast<const uint4*>((SINGLE ? p.res : p.x) + row0 + o * p.C + col0);
-          xr[i][0] = __ldg(rp);
-          xr[i][1] = __ldg(rp + 1);
+          const __nv_bfloat16* rp = (SINGLE ? p.res : p.x) + row0 + o * p.C + col0;
+          if constexpr (WIDE) load_global_32(rp, xr[i]);      // 32 lines per request, as many as for 16 bytes
+          else {
+            const uint4 lo = __ldg(reinterpret_cast<const uint4*>(rp)), hi = __ldg(reinterpret_cast<const uint4*>(rp) + 1);
+            xr[i][0] = lo.x; xr[i][1] = lo.y; xr[i][2] = lo.z; xr[i][3] = lo.w; xr[i][4] = hi.x; xr[i][5] = hi.y; xr[i][6] = hi.z; xr[i][7] = hi.w;
+          }
         }
       }
       // one warp polls, the others are parked: sixteen polling warps would take the issue slots of the MMA warp
@@ -329,10 +337,9 @@ conv3x3_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             }
           } else if (a < rows_valid && PH * q + o < p.W) {
             // P6: out = [ReLU](sum + x); xr is zero without a residual
-            const uint32_t xs[8] = {xr[i][0].x, xr[i][0].y, xr[i][0].z, xr[i][0].w, xr[i][1].x, xr[i][1].y, xr[i][1].z, xr[i][1].w};
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-              add_bf16x2(s[2 * j], s[2 * j + 1], xs[j]);
+              add_bf16x2(s[2 * j], s[2 * j + 1], xr[i][j]);
               w[j] = !SINGLE || p.relu ? pack_relu_bf16x2(s[2 * j], s[2 * j + 1]) : pack_bf16x2(s[2 * j], s[2 * j + 1]);
             }
             __nv_bfloat16* dst = p.out + row0 + o * p.C + col0;
@@ -357,6 +364,13 @@ conv3x3_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
   tcgen05_fence_before_sync();
   __syncthreads();
   if (warp == kEpiWarps + 1) tmem_dealloc(tmem_base, 512);
+}
+
+// Kernel of a tiling: 0 one phase, 1 two phases, 2 two phases with whole sectors of the residual per request, which pays where a
+// pixel is a whole line of 64 channels (32 x 56 x 56 x 64 21.9 -> 21.3 us; one phase: no difference).
+int which_kernel(const ConvParams& q) {
+  if (q.PH != 2) return 0;
+  return q.C == 64 && q.residual && reinterpret_cast<uintptr_t>(q.res) % 32 == 0 ? 2 : 1;
 }
 
 struct ConvHost {
@@ -501,10 +515,11 @@ ago_status_t conv3x3_run(const Plan& plan, FusedState* st, const void* const* in
   };
   CUtensorMap mx, mxt, mw1, mw2;
   if (!get_map(inputs[0], 0, &mx) || !get_map(inputs[0], 4, &mxt) || !get_map(weights[0], 1, &mw1) || !get_map(weights[2], 2, &mw2)) return AGO_ERR_CUDA;
-  auto kernel = q.PH == 2 ? conv3x3_pair_kernel<false, 2> : conv3x3_pair_kernel<false, 1>;
+  const int which = which_kernel(q);
+  auto kernel = which == 2 ? conv3x3_pair_kernel<false, 2, true> : which == 1 ? conv3x3_pair_kernel<false, 2, false> : conv3x3_pair_kernel<false, 1, false>;
   {
-    static int smem_opt_in[2][64] = {};
-    cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(kernel), smem_opt_in[q.PH == 2]);
+    static int smem_opt_in[3][64] = {};
+    cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(kernel), smem_opt_in[which]);
     if (e != cudaSuccess) { *err = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e); return AGO_ERR_CUDA; }
   }
   FusedLaunch launch(dim3((unsigned)(q.N * q.strips)), kThreads, (size_t)host->smem_bytes, stream);
@@ -583,10 +598,11 @@ cudaError_t launch_conv3x3_tc(const void* x, const void* w, const float* bias, c
   q.out = static_cast<__nv_bfloat16*>(out);
   q.wide_store = reinterpret_cast<uintptr_t>(out) % 32 == 0;
   q.status = status;
-  auto kernel = q.PH == 2 ? conv3x3_pair_kernel<true, 2> : conv3x3_pair_kernel<true, 1>;
+  const int which = which_kernel(q);
+  auto kernel = which == 2 ? conv3x3_pair_kernel<true, 2, true> : which == 1 ? conv3x3_pair_kernel<true, 2, false> : conv3x3_pair_kernel<true, 1, false>;
   {
-    static int smem_opt_in[2][64] = {};
-    cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(kernel), smem_opt_in[q.PH == 2]);
+    static int smem_opt_in[3][64] = {};
+    cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(kernel), smem_opt_in[which]);
     if (e != cudaSuccess) return e;
   }
   FusedLaunch launch(dim3((unsigned)(q.N * q.strips)), kThreads, (size_t)entry.smem_bytes, stream);
