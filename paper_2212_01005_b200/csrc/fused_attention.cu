@@ -207,9 +207,6 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
   const int n = (int)((long long)(blockIdx.x + 1) * p.total / gridDim.x) - g0;
   const int u0 = g0 / p.tiles, t0 = g0 - u0 * p.tiles;
   const int b0 = u0 / p.heads, h0 = u0 - b0 * p.heads;
-  grid_dependency_wait();      // the previous grid of the stream has completed; device memory may be touched
-  grid_launch_dependents();
-
   if (tid == kTmaWarp * 32) {
     *abort_flag = 0u;
     for (int i = 0; i < 22; ++i) mbar_init(bars + i, ((i >= 6 && i <= 9) || i == 12 || i == 13) ? kGroupWarps : 1);
@@ -219,16 +216,21 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
     tma_prefetch_desc(&tmap_k);
     tma_prefetch_desc(&tmap_v);
     tma_prefetch_desc(&tmap_o);
+  }
+  if (warp == 0) {
+    tmem_alloc(tmem_slot, 512);
+    tmem_relinquish();
+  }
+  // The set-up above overlaps the previous grid's tail where an SM has room or nothing to do.
+  grid_dependency_wait();      // the previous grid of the stream has completed; device memory may be touched
+  grid_launch_dependents();
+  if (tid == kTmaWarp * 32) {
     mbar_arrive_expect_tx(bar_k, (uint32_t)(p.nkb * kKeyBlock * kD * 2));
     for (int kb = 0; kb < p.nkb; ++kb) tma_load_3d(sK + kb * kKeyBlock * kD * 2, &tmap_k, bar_k, h0 * kD, kb * kKeyBlock, b0);
     mbar_arrive_expect_tx(bar_q, (uint32_t)(kBlockM * kD * 2));
     tma_load_3d(sQ, &tmap_q, bar_q, h0 * kD, t0 * kBlockM, b0);
     mbar_arrive_expect_tx(bar_v, (uint32_t)(p.nkb * kKeyBlock * kD * 2));
     for (int kb = 0; kb < p.nkb; ++kb) tma_load_3d(sV + kb * kKeyBlock * kD * 2, &tmap_v, bar_v, h0 * kD, kb * kKeyBlock, b0);
-  }
-  if (warp == 0) {
-    tmem_alloc(tmem_slot, 512);
-    tmem_relinquish();
   }
   tcgen05_fence_before_sync();
   __syncthreads();
