@@ -152,9 +152,6 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   const int cn0 = min(p.NC, 256), cn1 = p.NC - cn0;
   const uint32_t g2_tx = (uint32_t)(p.NC / 2) * kFK * 2u;            // W2 bytes per stage and CTA
   const uint32_t g1_tx = (uint32_t)(kFM * kFK * 2 + 64 * kFK * 2);   // X + W1 bytes per stage and CTA
-  grid_dependency_wait();
-  grid_launch_dependents();
-
   if (tid == kFEpiThreads) {
     *abort_flag = 0u;
     for (int i = 0; i < 3; ++i) mbar_init(bar_full + i, 2);
@@ -175,6 +172,9 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   cluster_meet();
   tcgen05_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
+  // The set-up above overlaps the previous grid's tail.
+  grid_dependency_wait();
+  grid_launch_dependents();
 
   if (warp >= kFEpiWarps + 2) {
     // ================================ TMA producers (every CTA): one of the two stages of every pair each ================================
@@ -349,9 +349,12 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       // covers whole rows of it (a row per lane takes 32 lines per store: 16-byte stores took 6 us per 128 columns of
       // fp32 sums, 768 columns 18 of a run's 23 us). The others are stored a sector at a time, beside the next item's products.
       const int row0 = unit * 2 * kFM + h * kFM;
+      const int n0 = P * p.NC + quarter * hc, esz = split ? 4 : 2;
+      float b2[3];             // lane j: the biases of the warp's columns j, 32 + j, 64 + j
+#pragma unroll
+      for (int k = 0; k < 3; ++k) b2[k] = !split && 32 * k < hc ? __ldg(p.b2 + n0 + 32 * k + lane) : 0.0f;
       mbar_wait(bar_out, (uint32_t)bi & 1u, abort_flag, p.status, 0x80f);
       tcgen05_fence_after_sync();
-      const int n0 = P * p.NC + quarter * hc, esz = split ? 4 : 2;
       uint8_t* dst = split ? reinterpret_cast<uint8_t*>(p.acc + ((size_t)part * p.split_rows + (size_t)(row0 - p.units_whole * 2 * kFM)) * p.N2 + n0)
                            : reinterpret_cast<uint8_t*>(p.out + (size_t)row0 * p.N2 + n0);        // the CTA's first row, this warp's first column
       const size_t pitch = (size_t)p.N2 * esz;
@@ -364,7 +367,7 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
         tmem_ld_x32(tmem_base + lane_base + out_col(quarter * hc + c0), v);
         tmem_ld_wait();
         if (!split) {
-          const float b = __ldg(p.b2 + n0 + c0 + lane);
+          const float b = c0 == 0 ? b2[0] : c0 == 32 ? b2[1] : b2[2];
 #pragma unroll
           for (int j = 0; j < 16; ++j)
             v[j] = pack_bf16x2(__uint_as_float(v[2 * j]) + __shfl_sync(0xffffffffu, b, 2 * j), __uint_as_float(v[2 * j + 1]) + __shfl_sync(0xffffffffu, b, 2 * j + 1));
