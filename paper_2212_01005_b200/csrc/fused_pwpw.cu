@@ -13,7 +13,9 @@
 //                  first product of the next tile runs while this tile's outputs are stored.
 //   epilogue warps P3: TMEM -> registers: + b1 [ReLU6], bf16 -> shared memory as the swizzled A operand of the second
 //                  product; P5: TMEM -> registers: + b2 [ReLU6], bf16 -> device memory, a 32-byte sector per store.
-// Both weight matrices are fetched once per CTA into the same layout by asynchronous copies.
+// Both weight matrices are fetched once per CTA into the same layout: by the copy warp's TMA loads where few CTAs ask for them,
+// else by the epilogue threads' asynchronous copies through L1 (weights_by_tma). 1200 pixels x 64 -> 16 -> 64 3.15 -> 2.65 us,
+// 1936 x 192 -> 40 -> 192 5.50 -> 4.93, the chain below on 1568 rows x 120 -> 240 5.79 -> 5.22, 17248 x 64 -> 128 4.53 -> 4.14.
 // What bounds it: the stores and loads on large tensors, the chain weights -> product -> epilogue -> product -> epilogue
 // of one tile on small ones. With block-wide barriers between the steps, the outputs staged in shared memory and the X
 // tile's buffer busy until they had left it, a tile took 4.0-4.8 us with every unit idle most of that time; now 2.2-2.7.
@@ -68,6 +70,8 @@ struct PwPwParams {
   int tmem_cols, acc2_col;   // tensor-memory columns; first column of the second product (0: both share their columns)
   int wide_store;            // output rows start at multiples of 32 bytes
   int off_x, off_a, off_w1, off_w2, off_b, off_bar;
+  int tma_weights;           // the weights come by TMA (the kernel template's TMA)
+  int w1_rows, w2_rows, w1_box, w2_box, w1_tx, w2_tx;     // rows of a block of the weight tiles and of one load, bytes of all blocks
 };
 
 // ReLU6 of two bf16 values: rounding is monotone and both bounds are bf16 numbers, so it may follow the rounding.
@@ -89,11 +93,17 @@ __device__ __forceinline__ void add_bias16(uint32_t (&v)[16], const float* bias)
   }
 }
 
+template <bool TMA> struct WeightMaps { CUtensorMap w1, w2; };
+template <> struct WeightMaps<false> {};
+
 // CHAIN: the GEMM -> + tensor -> row permutation -> GEMM chain: [K][N] weights, no biases, no activations.
 // Otherwise two 1x1 convolutions: [N][K] weights, biases and optional activations.
-template <bool CHAIN>
+// TMA: the copy warp fetches the weights too, and nothing but the barriers' set-up is ahead of the roles; otherwise the epilogue
+// threads copy them through L1 (weights_by_tma).
+template <bool CHAIN, bool TMA>
 __global__ void __launch_bounds__(kThreads, 2)
-pwpw_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_r, const PwPwParams p) {
+pwpw_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_r,
+                  const __grid_constant__ WeightMaps<TMA> tmap_w, const PwPwParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sX = smem + p.off_x;
@@ -111,6 +121,7 @@ pwpw_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
   uint64_t* bar_d = bars + 5;    // columns of the second product drained (used where both products share their columns)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 6);
   volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 7);
+  uint64_t* bar_w = bars + 8;    // TMA: [2] W1, W2 landed
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int kMmaWarp = kEpiThreads / 32, kCopyWarp = kMmaWarp + 1;
@@ -122,10 +133,12 @@ pwpw_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     for (int i = 0; i < 4; ++i) mbar_init(bars + i, 1);
     mbar_init(bar_a, kEpiThreads / 32);
     mbar_init(bar_d, kEpiThreads / 32);
+    if (TMA) { mbar_init(bar_w, 1); mbar_init(bar_w + 1, 1); }
     fence_mbar_init();
     fence_proxy_async_smem();
     tma_prefetch_desc(&tmap_x);
     if (CHAIN) tma_prefetch_desc(&tmap_r);
+    if constexpr (TMA) { tma_prefetch_desc(&tmap_w.w1); tma_prefetch_desc(&tmap_w.w2); }
   }
   if (warp == kMmaWarp) {
     tmem_alloc(tmem_slot, (uint32_t)p.tmem_cols);
@@ -139,18 +152,36 @@ pwpw_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     mbar_arrive_expect_tx(bar_r, (uint32_t)p.r_tx);
     for (int kb = 0; kb < p.nkb1; ++kb) tma_load_2d(sA + kb * kXBlock, &tmap_r, bar_r, kb * kBK, tile * p.BR);
   };
+  // the blocks of 64 columns of a weight matrix as it lies in memory; rows and columns that the padding adds read as zeros
+  auto load_w = [&](const CUtensorMap* map, uint64_t* bar, uint8_t* dst, int rows, int box, int tx) {   // one thread
+    mbar_arrive_expect_tx(bar, (uint32_t)tx);
+    for (int at = 0, n0 = 0; at < tx; at += rows * 128, n0 += kBK)
+      for (int r0 = 0; r0 < rows; r0 += box) tma_load_2d(dst + at + r0 * 128, map, bar, n0, r0);
+  };
+  auto meet = [&]() {
+    tcgen05_fence_before_sync();
+    __syncthreads();
+    tcgen05_fence_after_sync();
+  };
+  if (TMA) meet();
   grid_dependency_wait();
   grid_launch_dependents();
   if (tid == kCopyWarp * 32 && (int)blockIdx.x < ntiles) {
     load_x(blockIdx.x);
+    if constexpr (TMA) load_w(&tmap_w.w1, bar_w, sW1, p.w1_rows, p.w1_box, p.w1_tx);
     if (CHAIN) load_r(blockIdx.x);
+    if constexpr (TMA) load_w(&tmap_w.w2, bar_w + 1, sW2, p.w2_rows, p.w2_box, p.w2_tx);
   }
+  auto stage_biases = [&]() {       // by the epilogue threads
+    for (int i = tid; i < p.C1p + p.C2p; i += kEpiThreads)
+      sB1[i] = i < p.C1p ? (i < p.C1 && p.b1 ? __ldg(p.b1 + i) : 0.0f) : (i - p.C1p < p.C2 && p.b2 ? __ldg(p.b2 + i - p.C1p) : 0.0f);
+  };
   // Weights: 16-byte asynchronous copies into the swizzled blocks, W1 as one group and W2 as a second one that is
   // only waited for before the first tile's second product; rows and reduction channels added by the padding are
   // zero-filled. All CTAs read the same few lines at the same moment, which the lines' L2 slices serve one after the
   // other: the copies go through L1, so that a line is requested once per SM (27783 pixels x 112/24 channels: 5.1 us,
   // 7.5 us past L1, from sector to sector).
-  if (tid < kEpiThreads) {
+  if (!TMA && tid < kEpiThreads) {
     // [N][K] weights: a piece is (row n, 16-byte chunk of k) -> K-major block k / 64, row n;
     // [K][N] weights: a piece is (row k, 16-byte chunk of n) -> N-major block n / 64, row k
     // The valid pieces lie one after the other in memory.
@@ -174,15 +205,12 @@ pwpw_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     } else {
       stage(p.w1, sW1, p.w1_block, p.C1p, p.C0p, p.C1, p.C0, p.c0_recip);
       stage(p.w2, sW2, p.w2_block, p.C2p, p.C1p, p.C2, p.C1, p.c1_recip);
-      for (int i = tid; i < p.C1p + p.C2p; i += kEpiThreads)
-        sB1[i] = i < p.C1p ? (i < p.C1 && p.b1 ? __ldg(p.b1 + i) : 0.0f) : (i - p.C1p < p.C2 && p.b2 ? __ldg(p.b2 + i - p.C1p) : 0.0f);
+      stage_biases();
     }
     cp_async_wait_but_one();
     fence_proxy_async_smem();
   }
-  tcgen05_fence_before_sync();
-  __syncthreads();
-  tcgen05_fence_after_sync();
+  if (!TMA) meet();
   const uint32_t tmem_base = *tmem_slot;
 
   if (warp == kCopyWarp) {
@@ -216,11 +244,13 @@ pwpw_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
       if (shared_cols && it) mbar_wait(bar_d, par ^ 1u, abort_flag, p.status, 0x606);
       // ---- P2: first product ----
       mbar_wait(bar_x, par, abort_flag, p.status, 0x600);
+      if (TMA && it == 0) mbar_wait(bar_w, 0, abort_flag, p.status, 0x608);
       tcgen05_fence_after_sync();
       product(tmem_base, sX, sW1, p.w1_block, p.nkb0, p.C0p, idesc1);
       umma_commit_elected(bar_m1, elected);
       // ---- P4: second product ----
       mbar_wait(bar_a, par, abort_flag, p.status, 0x607);
+      if (TMA && it == 0) mbar_wait(bar_w + 1, 0, abort_flag, p.status, 0x609);
       tcgen05_fence_after_sync();
       product(tmem_base + (uint32_t)p.acc2_col, sA, sW2, p.w2_block, p.nkb1, p.C1p, idesc2);
       umma_commit_elected(bar_m2, elected);
@@ -230,6 +260,10 @@ pwpw_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     const int quarter_rows = (warp & 3) * 32;   // first row of this warp's tensor-memory lane quarter
     const int half = warp >> 2;                 // the warps of a lane quarter take the 16-column groups of an epilogue round-robin
     const int r = quarter_rows + lane;          // this thread's row of the tile = its tensor-memory lane
+    if (TMA && !CHAIN) {                        // while the first tile and the weights travel
+      stage_biases();
+      named_barrier_sync(1, kEpiThreads);
+    }
     for (int tile = blockIdx.x, it = 0; tile < ntiles; tile += gridDim.x, ++it) {
       const uint32_t par = (uint32_t)it & 1u;
       const int row0 = tile * p.BR, rows = min(p.BR, p.M - row0);
@@ -270,7 +304,7 @@ pwpw_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
           *d0 = make_uint4(w[0], w[1], w[2], w[3]);
           *d1 = make_uint4(w[4], w[5], w[6], w[7]);
         }
-      if (it == 0) cp_async_wait_all();   // W2 (this thread's pieces; the arrivals below cover everybody's)
+      if (!TMA && it == 0) cp_async_wait_all();   // W2 (this thread's pieces; the arrivals below cover everybody's)
       fence_proxy_async_smem();
       tcgen05_fence_before_sync();
       __syncwarp();
@@ -314,12 +348,23 @@ pwpw_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
 
 int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
+// Whether the weights come by TMA. That takes one thread and starts at once, where the copies take every thread 1.5k to 3.7k
+// cycles; but each row of a block is a request to L2 past L1, and all CTAs make them for the same lines at the same moment.
+// Against the copies, 176 pairs and 35 chains of 81 to 17248 rows: up to 40 CTAs 1.06 to 1.23x; with 12 KB of weights up to 72 CTAs
+// 1.0 to 1.2x; rows of whole 64 bytes and tiles of up to 64 rows 1.03 to 1.1x up to one CTA per SM (pairs of larger tiles 0.96x);
+// 98 to 148 CTAs with rows of 48 or 80 bytes 0.7 to 0.95x.
+bool weights_by_tma(const PwPwParams& q, bool chain, int grid, int sms) {
+  if (grid <= 40) return true;
+  const bool whole = q.C0 % 32 == 0 && q.C1 % 32 == 0 && q.C2 % 32 == 0 && (chain || q.BR <= 64);
+  return 2 * q.C1 * (q.C0 + q.C2) >= 12 * 1024 && grid <= (whole ? sms : 72);
+}
+
 struct PwPwHost {
   PwPwParams prm;
   int smem_bytes = 0;
   int grid = 0;   // persistent CTAs: two per SM
   bool chain = false;   // the GEMM -> + input -> row transpose -> GEMM chain instead of two 1x1 convolutions
-  std::unordered_map<const void*, CUtensorMap> maps, maps_r;   // tensor maps of X / of the added tensor by base address
+  std::unordered_map<const void*, CUtensorMap> maps, maps_r, maps_w1, maps_w2;   // tensor maps of X / the added tensor / the weights by base address
 };
 
 }  // namespace
@@ -355,15 +400,19 @@ ago_status_t pwpw_plan(Plan* plan, FusedState* st, std::string* err) {
   const int w1_rows = host->chain ? q.C0p : q.C1p, w2_rows = host->chain ? q.C1p : q.C2p;
   q.c0_recip = fast_div_recip((host->chain ? q.C1 : q.C0) / 8); q.c1_recip = fast_div_recip((host->chain ? q.C2 : q.C1) / 8);
   q.w1_block = w1_rows * 128; q.w2_block = w2_rows * 128;
-  const int w1_bytes = (w1_chunks + 7) / 8 * q.w1_block, w2_bytes = (w2_chunks + 7) / 8 * q.w2_block;
+  q.w1_rows = w1_rows; q.w2_rows = w2_rows;
+  q.w1_tx = (w1_chunks + 7) / 8 * q.w1_block; q.w2_tx = (w2_chunks + 7) / 8 * q.w2_block;
+  // a load brings up to 256 rows: the fewest equal pieces of whole swizzle patterns
+  auto box_rows = [](int rows) { int n = (rows + 255) / 256; while (rows % (8 * n) != 0) ++n; return rows / n; };
+  q.w1_box = box_rows(w1_rows); q.w2_box = box_rows(w2_rows);
   int off = 0;
   auto take = [&](int bytes) { int o = off; off = round_up(off + bytes, 1024); return o; };
   q.off_x = take(q.nkb0 * kXBlock);
   q.off_a = take(q.nkb1 * kXBlock);
-  q.off_w1 = take(w1_bytes);
-  q.off_w2 = take(w2_bytes);
+  q.off_w1 = take(q.w1_tx);
+  q.off_w2 = take(q.w2_tx);
   q.off_b = take((q.C1p + q.C2p) * 4);
-  q.off_bar = take(64);
+  q.off_bar = take(128);
   host->smem_bytes = off + 1024;
   if (host->smem_bytes > 227 * 1024) return bad("the operands of one row tile do not fit shared memory");
   if ((long)w1_rows * w1_chunks > 65535 || (long)w2_rows * w2_chunks > 65535)
@@ -384,12 +433,24 @@ ago_status_t pwpw_plan(Plan* plan, FusedState* st, std::string* err) {
   q.x_tx = q.nkb0 * q.BR * 128;
   q.r_tx = q.nkb1 * q.BR * 128;
   host->grid = (int)std::min<long>((q.M + q.BR - 1) / q.BR, slots);
+  q.tma_weights = weights_by_tma(q, host->chain, host->grid, (int)sms) ? 1 : 0;
   st->impl = host;
   st->impl_free = [](void* p) { delete static_cast<PwPwHost*>(p); };
   st->tile_rows = q.BR; st->grid = host->grid; st->smem_bytes = host->smem_bytes;
   plan->tile_rows = q.BR; plan->smem_bytes = host->smem_bytes;
   return AGO_OK;
 }
+
+namespace {
+template <bool CHAIN, bool TMA>
+cudaError_t launch_pwpw(const PwPwHost& host, const PwPwParams& q, const CUtensorMap& mx, const CUtensorMap& mr, const WeightMaps<TMA>& mw, cudaStream_t stream) {
+  static int smem_opt_in[64] = {};
+  const cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(pwpw_fused_kernel<CHAIN, TMA>), smem_opt_in);
+  if (e != cudaSuccess) return e;
+  FusedLaunch launch(dim3((unsigned)host.grid), kThreads, (size_t)host.smem_bytes, stream);
+  return cudaLaunchKernelEx(&launch.config, pwpw_fused_kernel<CHAIN, TMA>, mx, mr, mw, q);
+}
+}  // namespace
 
 ago_status_t pwpw_run(const Plan& plan, FusedState* st, const void* const* inputs, const void* const* weights,
                       void* output, unsigned int* status_word, cudaStream_t stream, std::string* err) {
@@ -406,14 +467,14 @@ ago_status_t pwpw_run(const Plan& plan, FusedState* st, const void* const* input
   q.out = static_cast<__nv_bfloat16*>(output);
   q.status = status_word;
   q.wide_store = q.C2 % 16 == 0 && reinterpret_cast<uintptr_t>(output) % 32 == 0;
-  // [M][C] bf16 matrices as K-major tiles of 128 rows x 64 channels
-  auto get_map = [&](std::unordered_map<const void*, CUtensorMap>& cache, const void* base, int C, CUtensorMap* out) -> bool {
+  // [M][C] bf16 matrices as tiles of 64 columns: BR rows of X and of the added tensor, blocks of the weights
+  auto get_map = [&](std::unordered_map<const void*, CUtensorMap>& cache, const void* base, int M, int C, int box_rows, CUtensorMap* out) -> bool {
     auto it = cache.find(base);
     if (it == cache.end()) {
       CUtensorMap m;
-      const uint64_t dims[2] = {(uint64_t)C, (uint64_t)q.M};
+      const uint64_t dims[2] = {(uint64_t)C, (uint64_t)M};
       const uint64_t strides[1] = {(uint64_t)C * 2};
-      const uint32_t box[2] = {(uint32_t)kBK, (uint32_t)q.BR};
+      const uint32_t box[2] = {(uint32_t)kBK, (uint32_t)box_rows};
       if (!encode_tmap_bf16(&m, base, 2, dims, strides, box, 128, err)) return false;
       if (cache.size() > 4096) cache.clear();
       it = cache.emplace(base, m).first;
@@ -422,17 +483,16 @@ ago_status_t pwpw_run(const Plan& plan, FusedState* st, const void* const* input
     return true;
   };
   CUtensorMap mx, mr;
-  if (!get_map(host->maps, inputs[0], q.C0, &mx)) return AGO_ERR_CUDA;
+  WeightMaps<true> mw;
+  if (!get_map(host->maps, inputs[0], q.M, q.C0, q.BR, &mx)) return AGO_ERR_CUDA;
   mr = mx;
-  if (host->chain && !get_map(host->maps_r, inputs[1], q.C1, &mr)) return AGO_ERR_CUDA;
-  auto kernel = host->chain ? pwpw_fused_kernel<true> : pwpw_fused_kernel<false>;
-  {
-    static int smem_opt_in[2][64] = {};
-    cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(kernel), smem_opt_in[host->chain]);
-    if (e != cudaSuccess) { *err = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e); return AGO_ERR_CUDA; }
+  if (host->chain && !get_map(host->maps_r, inputs[1], q.M, q.C1, q.BR, &mr)) return AGO_ERR_CUDA;
+  if (q.tma_weights) {      // 1x1 convolutions: [N][K]; the chain's operands: [K][N]
+    if (!get_map(host->maps_w1, q.w1, host->chain ? q.C0 : q.C1, host->chain ? q.C1 : q.C0, q.w1_box, &mw.w1)) return AGO_ERR_CUDA;
+    if (!get_map(host->maps_w2, q.w2, host->chain ? q.C1 : q.C2, host->chain ? q.C2 : q.C1, q.w2_box, &mw.w2)) return AGO_ERR_CUDA;
   }
-  FusedLaunch launch(dim3((unsigned)host->grid), kThreads, (size_t)host->smem_bytes, stream);
-  cudaError_t e = cudaLaunchKernelEx(&launch.config, kernel, mx, mr, q);
+  cudaError_t e = host->chain ? (q.tma_weights ? launch_pwpw<true, true>(*host, q, mx, mr, mw, stream) : launch_pwpw<true, false>(*host, q, mx, mr, {}, stream))
+                              : (q.tma_weights ? launch_pwpw<false, true>(*host, q, mx, mr, mw, stream) : launch_pwpw<false, false>(*host, q, mx, mr, {}, stream));
   if (e != cudaSuccess) { *err = std::string("fused pointwise pair launch: ") + cudaGetErrorString(e); return AGO_ERR_CUDA; }
   return AGO_OK;
 }
