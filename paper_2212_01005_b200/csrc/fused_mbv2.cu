@@ -19,7 +19,7 @@
 // Per CTA (one image, R output rows, full width, its share of the channels):
 //   P1  16-byte asynchronous copies bring the NHWC input strip (with its row
 //       halo; rows outside the image -> 0, channels padded to the MMA K
-//       granularity), W1 and W3 into swizzled K-major tiles; descriptors and work
+//       granularity), W1 and W3 into swizzled K-major tiles (X and W1 by TMA for wide pixels); descriptors and work
 //       mapping are computed while they travel. (A pixel is Cin * 2 bytes there,
 //       e.g. 48: one TMA box row per pixel was several times slower.)
 //   for each 16-channel chunk c of the expanded tensor:
@@ -38,10 +38,13 @@
 
 #include <algorithm>
 #include <cmath>
+#include <mutex>
+#include <unordered_map>
 
 #include "dw_common.cuh"
 #include "fused.h"
 #include "tc_common.cuh"
+#include "tmap.h"
 
 namespace ago {
 
@@ -93,15 +96,21 @@ struct Mbv2Params {
   int e_plane, d_plane;         // byte distance between the two 8-channel planes of an E / D chunk
   // shared-memory byte offsets (from the 1024-aligned base)
   int off_x, off_w1, off_e, off_d, off_w3, off_wd, off_b1, off_bd, off_b3, off_bar;
+  int tma, w1_box;              // X and W1 by TMA, rows of W1 per load
 };
 
 // FOLD: the expand bias rides in the expand GEMM (see the prologue). EXPAND / PROJECT select the pairs of the
 // block: <true, true> the whole block, <true, false> pointwise -> depthwise
 // (the depthwise result of every chunk goes to device memory), <false, true> depthwise -> pointwise (every chunk of
 // the input is copied into the E buffers instead of being computed).
-template <bool EXPAND, bool PROJECT, bool FOLD, int NG>
+// TMA: the input strip and W1 come by TMA (not with FOLD, where channels of their K blocks belong to a bias). An instance of its own: with
+// both ways in one kernel either ran 3 % slower.
+template <bool MAPS> struct Mbv2Maps { CUtensorMap x, w1; };
+template <> struct Mbv2Maps<false> {};
+
+template <bool EXPAND, bool PROJECT, bool FOLD, int NG, bool TMA>
 __global__ void __launch_bounds__(kThreads, 1)
-mbv2_fused_kernel(const Mbv2Params p) {
+mbv2_fused_kernel(const Mbv2Params p, const __grid_constant__ Mbv2Maps<TMA> maps) {
   constexpr int kGroupWarps = kWarps / NG;
   constexpr int kGroupThreads = kGroupWarps * 32;
   extern __shared__ uint8_t smem_raw[];
@@ -123,6 +132,7 @@ mbv2_fused_kernel(const Mbv2Params p) {
   uint64_t* bar_chain = bars + 18;  // two groups: group 0's first expand GEMM complete. One phase only: a waiter on bar_e could
                                     // fall behind its next phase and then wait for a parity that has come and gone
   uint64_t* bar_red = bars + 12;    // [kMaxPieces] a piece of the partial sums of the other CTAs of the cluster has arrived
+  uint64_t* bar_x = bars + 19;      // input strip and W1 landed (TMA)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 20);
   volatile uint32_t* abort_flag = reinterpret_cast<volatile uint32_t*>(bars + 21);
 
@@ -146,8 +156,10 @@ mbv2_fused_kernel(const Mbv2Params p) {
     mbar_init(bar_chain, kExpandIssuers);
     for (int k = 0; k < kMaxPieces; ++k) mbar_init(bar_red + k, 1);
     mbar_init(bar_done, (uint32_t)(p.M2 * min(p.NC, NG)));
+    if (TMA) mbar_init(bar_x, 1);
     fence_mbar_init();
     fence_proxy_async_smem();
+    if constexpr (TMA) { tma_prefetch_desc(&maps.x); tma_prefetch_desc(&maps.w1); }
   }
     // ---- P1: stage the input strip, the weights and the biases by asynchronous 16-byte copies, region by region; row and
     // column of a thread's chunks advance by fixed steps. X and W1 rows go to their swizzled K-major tiles (one tile of 16, 32
@@ -174,7 +186,7 @@ mbv2_fused_kernel(const Mbv2Params p) {
       const uint8_t* none = reinterpret_cast<const uint8_t*>(p.wd);      // never read: the copies from it have no bytes
       const uint32_t s0 = smem_u32(smem);
       const float fold_b = FOLD && tid < p.Cexp ? __ldg(p.b1 + ch0 + tid) : 0.0f;     // on its way while the copies are issued
-      if (EXPAND) {
+      if (EXPAND && !TMA) {
         const int xblk = p.M1 * 128 * 128, wblk = p.Cexp * 128;
         auto place = [&](int row, int ch, int blk) -> uint32_t {
           if (wide) return (uint32_t)((ch >> 3) * blk + row * 128 + (((ch ^ row) & 7) << 4));
@@ -315,6 +327,19 @@ mbv2_fused_kernel(const Mbv2Params p) {
     }
     grid_dependency_wait();      // first access to device memory below
     grid_launch_dependents();
+    if constexpr (TMA) {
+      if (warp == kWarps - 1) {      // the warp that set the barrier up
+        __syncwarp();
+        const uint32_t one = elect_one(), bar = smem_u32(bar_x), s0 = smem_u32(smem), rb = (uint32_t)p.row_bytes;
+        mbar_arrive_expect_tx_elected(bar, (uint32_t)(p.kblocks * (p.M1 * 128 + p.Cexp)) * rb, one);
+        for (int kb = 0; kb < p.kblocks; ++kb) {
+          for (int t = 0; t < p.M1; ++t)
+            tma_load_3d_elected(s0 + (uint32_t)p.off_x + (uint32_t)(kb * p.M1 + t) * 128u * rb, &maps.x, bar, kb * 64, gh0 * p.W + t * 128, n, one);
+          for (int r0 = 0; r0 < p.Cexp; r0 += p.w1_box)
+            tma_load_2d_elected(s0 + (uint32_t)p.off_w1 + (uint32_t)(kb * p.Cexp + r0) * rb, &maps.w1, bar, kb * 64, ch0 + r0, one);
+        }
+      }
+    }
     if (!EXPAND) { load_chunk(g, 0); load_chunk(g + NG, 1); }   // the first two chunks travel while the weights are staged
     stage();
     // the zero padding columns of the two E chunk buffers (written once: every chunk reuses them)
@@ -445,6 +470,7 @@ mbv2_fused_kernel(const Mbv2Params p) {
 #pragma unroll
     for (int k = 0; k < kTilesPerWarp; ++k) if (e_tm[k] != kNone) e_tm[k] += tmem_base;
     if (EXPAND && xi >= 0) {
+      if (TMA) mbar_wait(bar_x, 0, abort_flag, p.status, 0x109);
       if (NG == 2) {
         // group 1 issues its first expand GEMM once group 0's is through the tensor pipe: group 0 has the longer chain
         // of chunks, and its first epilogue would otherwise wait for both groups' MMAs
@@ -658,7 +684,8 @@ mbv2_fused_kernel(const Mbv2Params p) {
           }
         }
         cluster_wait();                           // the copies out of this CTA have arrived: it may leave
-      } else
+      } else {
+      if (TMA && p.residual) mbar_wait(bar_x, 0, abort_flag, p.status, 0x109);      // complete since the first product: the strip is read below
       for (int t = warp >> 2; t < p.M2; t += kWarps / 4) {
         const int po = t * 128 + (warp & 3) * 32 + lane;
         for (int j0 = 0; j0 < p.Coutp; j0 += 16) {
@@ -688,6 +715,7 @@ mbv2_fused_kernel(const Mbv2Params p) {
           }
         }
       }
+      }
     }
   tcgen05_fence_before_sync();
   __syncthreads();
@@ -704,6 +732,8 @@ struct Mbv2Host {
   Mbv2Params prm;
   int smem_bytes = 0;
   bool expand = true, project = true;
+  std::mutex guard;                                               // of the maps: runs of one handle may come from several threads
+  std::unordered_map<const void*, CUtensorMap> maps_x, maps_w1;   // by base address
 };
 
 bool layout(Mbv2Params& q, int R, bool expand, bool project, int* smem_bytes) {
@@ -873,6 +903,13 @@ ago_status_t mbv2_plan(Plan* plan, FusedState* st, std::string* err) {
   set_split(q, best_cs);
   layout(q, best_R, expand, project, &best_smem);
   if ((long)q.N * q.strips > 65535) return bad("more than 65535 row strips in the batch");
+  // Input strip and W1 by TMA where a pixel is 64 bytes or more and the strip is a large part of what a CTA waits for: the threads'
+  // 16-byte copies bring 27 bytes per cycle. 25 images of 15 x 15 x 96 15.5 -> 14.6 us, 40 of 20 x 20 x 64 18.6 -> 17.7, 32 of
+  // 28 x 28 x 32 at stride 2 9.7 -> 9.2; strips of fewer than 96 pixels 1 % slower (one image 14 x 14 x 32: 42 pixels, 5.8 -> 5.9), pixels
+  // of 32 bytes up to 7 % (8 images of 56 x 56 x 16: 7.6 -> 8.1).
+  q.tma = expand && !q.fold_b1 && q.Cin >= 32 && q.P_x >= 96 ? 1 : 0;
+  q.w1_box = std::min(q.Cexp, 256);
+  while (q.Cexp % q.w1_box != 0) q.w1_box -= kChunk;
   host->smem_bytes = best_smem;
   st->impl = host;
   st->impl_free = [](void* p) { delete static_cast<Mbv2Host*>(p); };
@@ -885,10 +922,10 @@ ago_status_t mbv2_plan(Plan* plan, FusedState* st, std::string* err) {
 
 namespace {
 
-template <bool EXPAND, bool PROJECT, bool FOLD, int NG>
-ago_status_t launch_groups(const Mbv2Params& q, int smem_bytes, cudaStream_t stream, std::string* err) {
+template <bool EXPAND, bool PROJECT, bool FOLD, int NG, bool TMA>
+ago_status_t launch_groups(const Mbv2Params& q, const Mbv2Maps<TMA>& maps, int smem_bytes, cudaStream_t stream, std::string* err) {
   static int smem_opt_in[64] = {};
-  cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(mbv2_fused_kernel<EXPAND, PROJECT, FOLD, NG>), smem_opt_in);
+  cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(mbv2_fused_kernel<EXPAND, PROJECT, FOLD, NG, TMA>), smem_opt_in);
   if (e != cudaSuccess) { *err = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e); return AGO_ERR_CUDA; }
   FusedLaunch launch(dim3((unsigned)(q.N * q.strips * q.CS)), kThreads, (size_t)smem_bytes, stream);
   cudaLaunchAttribute attr[2] = {launch.attr[0], {}};
@@ -898,14 +935,33 @@ ago_status_t launch_groups(const Mbv2Params& q, int smem_bytes, cudaStream_t str
     launch.config.attrs = attr;
     launch.config.numAttrs = 2;
   }
-  e = cudaLaunchKernelEx(&launch.config, mbv2_fused_kernel<EXPAND, PROJECT, FOLD, NG>, q);
+  e = cudaLaunchKernelEx(&launch.config, mbv2_fused_kernel<EXPAND, PROJECT, FOLD, NG, TMA>, q, maps);
   if (e != cudaSuccess) { *err = std::string("fused inverted-residual launch: ") + cudaGetErrorString(e); return AGO_ERR_CUDA; }
   return AGO_OK;
 }
-template <bool EXPAND, bool PROJECT, bool FOLD>
-ago_status_t launch_variant(const Mbv2Params& q, int smem_bytes, cudaStream_t stream, std::string* err) {
-  return q.groups == 4 ? launch_groups<EXPAND, PROJECT, FOLD, 4>(q, smem_bytes, stream, err)
-                       : launch_groups<EXPAND, PROJECT, FOLD, 2>(q, smem_bytes, stream, err);
+template <bool EXPAND, bool PROJECT, bool FOLD, bool TMA = false>
+ago_status_t launch_variant(const Mbv2Params& q, Mbv2Host* host, cudaStream_t stream, std::string* err) {
+  Mbv2Maps<TMA> maps;
+  if constexpr (TMA) {
+    auto get = [&](std::unordered_map<const void*, CUtensorMap>& cache, const void* base, bool weights, CUtensorMap* out) -> bool {
+      auto it = cache.find(base);
+      if (it == cache.end()) {
+        CUtensorMap m;
+        const uint64_t wdims[2] = {(uint64_t)q.Cin, (uint64_t)q.Cfull}, xdims[3] = {(uint64_t)q.Cin, (uint64_t)q.H * q.W, (uint64_t)q.N};
+        const uint64_t strides[2] = {(uint64_t)q.Cin * 2, (uint64_t)q.H * q.W * q.Cin * 2};
+        const uint32_t wbox[2] = {(uint32_t)q.Kp, (uint32_t)q.w1_box}, xbox[3] = {(uint32_t)q.Kp, 128, 1};
+        if (!encode_tmap_bf16(&m, base, weights ? 2 : 3, weights ? wdims : xdims, strides, weights ? wbox : xbox, q.row_bytes, err)) return false;
+        if (cache.size() > 4096) cache.clear();
+        it = cache.emplace(base, m).first;
+      }
+      *out = it->second;
+      return true;
+    };
+    std::lock_guard<std::mutex> lock(host->guard);
+    if (!get(host->maps_x, q.x, false, &maps.x) || !get(host->maps_w1, q.w1, true, &maps.w1)) return AGO_ERR_CUDA;
+  }
+  return q.groups == 4 ? launch_groups<EXPAND, PROJECT, FOLD, 4, TMA>(q, maps, host->smem_bytes, stream, err)
+                       : launch_groups<EXPAND, PROJECT, FOLD, 2, TMA>(q, maps, host->smem_bytes, stream, err);
 }
 
 }  // namespace
@@ -921,12 +977,14 @@ ago_status_t mbv2_run(const Plan& plan, FusedState* st, const void* const* input
   if (host->project) { q.w3 = static_cast<const __nv_bfloat16*>(weights[w]); q.b3 = static_cast<const float*>(weights[w + 1]); }
   q.out = static_cast<__nv_bfloat16*>(output);
   q.status = status_word;
-  if (!host->expand) return launch_variant<false, true, false>(q, host->smem_bytes, stream, err);
+  if (!host->expand) return launch_variant<false, true, false>(q, host, stream, err);
   if (!host->project)
-    return q.fold_b1 ? launch_variant<true, false, true>(q, host->smem_bytes, stream, err)
-                     : launch_variant<true, false, false>(q, host->smem_bytes, stream, err);
-  return q.fold_b1 ? launch_variant<true, true, true>(q, host->smem_bytes, stream, err)
-                   : launch_variant<true, true, false>(q, host->smem_bytes, stream, err);
+    return q.fold_b1 ? launch_variant<true, false, true>(q, host, stream, err)
+         : q.tma    ? launch_variant<true, false, false, true>(q, host, stream, err)
+                    : launch_variant<true, false, false>(q, host, stream, err);
+  return q.fold_b1 ? launch_variant<true, true, true>(q, host, stream, err)
+       : q.tma    ? launch_variant<true, true, false, true>(q, host, stream, err)
+                  : launch_variant<true, true, false>(q, host, stream, err);
 }
 
 }  // namespace ago
