@@ -308,8 +308,8 @@ namespace {
 // costs less than about a third of the contractions' tensor-core time: both modes are then bound by the contractions
 // (Section VI-B reports the same for pointwise -> pointwise chains). Data-sheet-class constants; only the ratio matters.
 bool fusion_pays(const Plan& p) {
-  // Feed-forward chains: both ways are estimated, with the kernel that fused_plan chose (768 -> 3072: fused 17.4 against 26 us at 512
-  // rows, 26 against 30 at 1000, but 40 against 32 at 1500 and 137 against 102 at 12288; the reduction-tiling kernel 8 against 19 us
+  // Feed-forward chains: both ways are estimated, with the kernel that fused_plan chose (768 -> 3072: fused 15.7 against 26 us at 512
+  // rows, but 45 against 26 at 3001 and 109 against 91 at 12288; the reduction-tiling kernel 8 against 19 us
   // at 7 rows of 192 -> 1920 -> 256, 77 against 22 at 2215 rows of 64 -> 1920 -> 1024).
   if (p.fused_kernel == AGO_KERNEL_FFN) {
     const double fused = p.fused_variant == 3 ? ffn_pair_estimate(p) : p.fused_variant == 0 ? ffn_estimate(p) : ffn_cluster_estimate(p);

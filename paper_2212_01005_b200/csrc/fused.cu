@@ -58,7 +58,7 @@ ago_status_t fused_plan(Plan* plan, FusedState* st, std::string* err) {
       // kernel of the least estimate: the pairs (768 -> 3072: 2500 rows 35 against 56 us), the cluster kernel, or the one that tiles
       // the reduction, which needs no row block to be shared out evenly (646 rows of 64 -> 3328 -> 384: 24 against 37 us). The pairs
       // have to win by more than the estimates' error (4157 rows of 128 -> 2048 -> 256: 27.4 against 28.5). Over 173 chains that both
-      // serve, 1 to 12288 rows, the choice costs 0.2 % on average.
+      // serve, 1 to 12288 rows, the choice costs 0.4 % on average.
       const double pair = ffn_pair_estimate(*plan) * 1.04, cluster = ffn_cluster_estimate(*plan), reduction = ffn_estimate(*plan);
       const int64_t rows = plan->inputs[0].numel() / plan->inputs[0].last();
       const bool fills = pair >= 0 && (rows + 255) / 256 * 4 >= (int64_t)device_sm_count() * 3 / 4;

@@ -3,8 +3,8 @@
 // with few row blocks each row block's hidden tiles are split over J clusters, whose output shares meet in an fp32 buffer
 // (J additions per element), and a second, small launch turns the buffer into the output. There the run is a chain of
 // latencies, so a cluster of one step requests everything it needs at once, keeps only the rows that exist and takes hidden
-// tiles of 64 where they put more clusters to work: 768 -> 3072 -> 768 with 1 row 14.6 -> 8.1 us, 128 rows 18.1 -> 11.9,
-// 256 rows 18.7 -> 12.6, 512 rows 19.9 -> 17.4 (of which 3.8 us are the 9.4 MB of additions at the rate of the L2).
+// tiles of 64 where they put more clusters to work: 768 -> 3072 -> 768 with 1 row 14.6 -> 7.9 us, 128 rows 18.1 -> 10.8,
+// 256 rows 18.7 -> 11.6, 512 rows 19.9 -> 15.7 (of which 3.8 us are the 9.4 MB of additions at the rate of the L2).
 //
 // Tile choice (Section III-B, "downstream pointwise / matmul"): the second GEMM reuses H only along its output
 // columns, so the downstream tile keeps ALL output columns of a block of 128 rows. Those (768 fp32 columns for

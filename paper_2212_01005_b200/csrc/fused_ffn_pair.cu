@@ -11,9 +11,8 @@
 // multicast), to the CTA of the other pair that holds the same rows; both pairs then multiply it into their own
 // output columns.
 //
-// Why pairs: with unpaired CTAs every SM streams a whole 128-wide B tile per 128 rows (64 - 128 flop per byte that
-// crosses L2 -> SM, and that link, about 9 TB/s in all, is what bounds the unpaired cluster kernel). A pair streams
-// each B tile once for 256 rows: 131 flop per byte for the chain at BERT-base widths.
+// Why pairs: with unpaired CTAs every SM writes and reads a whole 128-wide B tile in shared memory per 128 rows; a pair's CTA
+// holds half of each B tile, 131 flop per byte that enters the SM for the chain at BERT-base widths against 64 - 128.
 //
 // Per CTA (pair P, half h; h == 0 leads its pair), steps g = (row block, own hidden tile):
 //   TMA     two warps, converged, an elected lane issuing: 24 KB stages in pairs -- X [128 x 64] + W1 [64 x 64] (this CTA's half of

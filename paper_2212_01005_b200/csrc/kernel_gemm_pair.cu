@@ -371,7 +371,7 @@ bool pair_epilogue(const EpiProgram& e, GemmPairParams* p) {
 }  // namespace
 
 static long pair_tiles(const GemmArgs& a, int bn) { return (long)((a.M + 255) / 256) * ((a.N + bn - 1) / bn); }
-// Columns per tile: 256 (128 flop per byte that crosses L2 -> SM), or 128 where tiles of 256 would leave half of the pairs idle or
+// Columns per tile: 256 (128 flop per byte that enters the SM), or 128 where tiles of 256 would leave half of the pairs idle or
 // fill a last round by less than a third (rounds x bytes per K block: 64 against 48 KB).
 static int pair_columns(const GemmArgs& a) {
   if (a.N <= 128) return 128;
