@@ -903,11 +903,11 @@ ago_status_t mbv2_plan(Plan* plan, FusedState* st, std::string* err) {
   set_split(q, best_cs);
   layout(q, best_R, expand, project, &best_smem);
   if ((long)q.N * q.strips > 65535) return bad("more than 65535 row strips in the batch");
-  // Input strip and W1 by TMA where a pixel is 64 bytes or more and the strip is a large part of what a CTA waits for: the threads'
-  // 16-byte copies bring 27 bytes per cycle. 25 images of 15 x 15 x 96 15.5 -> 14.6 us, 40 of 20 x 20 x 64 18.6 -> 17.7, 32 of
-  // 28 x 28 x 32 at stride 2 9.7 -> 9.2; strips of fewer than 96 pixels 1 % slower (one image 14 x 14 x 32: 42 pixels, 5.8 -> 5.9), pixels
-  // of 32 bytes up to 7 % (8 images of 56 x 56 x 16: 7.6 -> 8.1).
-  q.tma = expand && !q.fold_b1 && q.Cin >= 32 && q.P_x >= 96 ? 1 : 0;
+  // Input strip and W1 by TMA where a pixel is 64 bytes or more and the strip 12.5 KB or more: the threads' 16-byte copies bring 27
+  // bytes per cycle. 25 images of 15 x 15 x 96 15.5 -> 14.6 us, 40 of 20 x 20 x 64 18.6 -> 17.7, 32 of 28 x 28 x 32 at stride 2 9.7 -> 9.2, 26 of
+  // 8 x 8 x 160 14.8 -> 13.2; 32 shapes on this side of the line 1.01 to 1.1x. Short strips were 1 to 1.5 % slower (one image 14 x 14 x 32:
+  // 2.7 KB, 5.8 -> 5.9; two of 9 x 9 x 96 at stride 2: 5.2 KB), pixels of 32 bytes up to 7 % (8 images of 56 x 56 x 16: 7.6 -> 8.1).
+  q.tma = expand && !q.fold_b1 && q.Cin >= 32 && q.P_x >= 64 && q.P_x * q.Cin * 2 >= 12800 ? 1 : 0;
   q.w1_box = std::min(q.Cexp, 256);
   while (q.Cexp % q.w1_box != 0) q.w1_box -= kChunk;
   host->smem_bytes = best_smem;
