@@ -10,6 +10,7 @@
 #include <ATen/ATen.h>
 #include <ATen/EmptyTensor.h>
 #include <ATen/ops/empty.h>
+#include <ATen/record_function.h>
 #include <c10/core/impl/LocalDispatchKeySet.h>
 #include <c10/cuda/CUDACachingAllocator.h>
 #include <c10/cuda/CUDAFunctions.h>
@@ -81,14 +82,18 @@ bool stream_of(PyObject* o, void** stream) {
 }
 
 // The output tensor, as at::empty makes it. Where nothing takes part in a factory call (no dispatch mode, transform, tracer or
-// autocast on this thread, no deterministic fill) and the device is the current one, without the dispatcher's way there: 0.3 us of a
-// call's host time, which is what a small subgraph takes (fp32 depthwise stage 2 x 9 x 9 x 64 3.95 -> 3.6 us, depthwise pair 3.25 -> 2.95).
+// autocast on this thread, no deterministic fill, no profiler that records operators) and the device is the current one, without the
+// dispatcher's way there: 0.3 us of a call's host time, which is what a small subgraph takes (fp32 depthwise stage 2 x 9 x 9 x 64
+// 3.95 -> 3.6 us, depthwise pair 3.25 -> 2.95). The allocator needs torch's CUDA state, which nothing but this call may have asked
+// for where all inputs are another library's arrays: initialised here as at::empty does it (a flag once that is done).
 at::Tensor make_output(const Runner* r, at::Device dev) {
   const auto tls = c10::impl::tls_local_dispatch_key_set();
-  if ((tls.included_ - c10::default_included_set).empty() && !at::globalContext().deterministicAlgorithms() &&
-      dev.index() == c10::cuda::current_device())
+  if ((tls.included_ - c10::default_included_set).empty() && !at::globalContext().deterministicAlgorithms() && !at::hasCallbacks() &&
+      dev.index() == c10::cuda::current_device()) {
+    at::globalContext().lazyInitDevice(c10::DeviceType::CUDA);
     return at::Tensor(at::detail::empty_generic(*r->shape, c10::cuda::CUDACachingAllocator::get(), c10::DispatchKeySet(c10::DispatchKey::CUDA),
                                                 r->dtype, std::nullopt));
+  }
   return at::empty(*r->shape, at::TensorOptions().dtype(r->dtype).device(dev));
 }
 

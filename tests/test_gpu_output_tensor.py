@@ -30,7 +30,8 @@ def deterministic():
 
 
 CONTEXTS = {"plain": contextlib.nullcontext, "inference": torch.inference_mode, "no_grad": torch.no_grad, "dispatch": Factories,
-            "autocast": lambda: torch.autocast("cuda"), "deterministic": deterministic, "stream": lambda: torch.cuda.stream(torch.cuda.Stream())}
+            "autocast": lambda: torch.autocast("cuda"), "deterministic": deterministic, "stream": lambda: torch.cuda.stream(torch.cuda.Stream()),
+            "profiler": lambda: torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CPU])}
 
 
 @pytest.mark.parametrize("fp32", [False, True])
@@ -57,6 +58,8 @@ def test_output_tensor(ago, name, fp32):
         if name == "dispatch":
             assert any("empty" in f for f in active.seen)
         torch.cuda.current_stream().synchronize()
+    if name == "profiler":
+        assert any(e.key == "aten::empty" for e in active.key_averages())
     assert out.shape == given.shape and out.dtype == dtype and out.device == given.device and out.is_contiguous() and not out.requires_grad
     assert out.data_ptr() != given.data_ptr() and torch.equal(out, given)
     sg.close()

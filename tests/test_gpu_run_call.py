@@ -1,4 +1,7 @@
 """The native call behind `Subgraph.run`: what it returns, which stream it uses, when it attaches a workspace, how it fails."""
+import os
+import subprocess
+import sys
 import threading
 
 import pytest
@@ -106,3 +109,44 @@ def test_run_takes_whatever_has_a_device_and_an_address(ago):
     with pytest.raises(ago.AgoError):
         sg2, (ins, ws) = handle(ago, wl)
         sg2.run([Array(t.cpu(), torch.device("cpu")) for t in ins], ws)
+
+
+FOREIGN = """
+import ctypes
+import numpy as np
+import torch
+from oracle import oracle as O
+from paper_2212_01005_b200 import binding as B, workloads as WL
+
+rt = ctypes.CDLL("libcudart.so.12")      # the one torch has loaded
+
+class Array:
+    device = "cuda:0"
+    def __init__(self, a):
+        a = np.ascontiguousarray(a)
+        p = ctypes.c_void_p()
+        assert rt.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(a.nbytes)) == 0
+        assert rt.cudaMemcpy(p, a.ctypes.data_as(ctypes.c_void_p), ctypes.c_size_t(a.nbytes), 1) == 0
+        self.address = p.value
+    def data_ptr(self):
+        return self.address
+
+wl = WL.pw_pw("call_foreign", [308], 1, 8, 64, 32, 64)
+data = WL.generate(wl)
+bf16 = lambda a: (np.ascontiguousarray(a, np.float32).view(np.uint32) >> 16).astype(np.uint16)      # the values are bf16 numbers
+ins = [Array(bf16(a)) for a in data["inputs"]]
+ws = [Array(a.astype(np.float32) if k == "bias" else bf16(a)) for a, k in zip(data["weights"], wl.weight_kinds)]
+sg = B.Subgraph(wl.ops, wl.input_shapes, mode="fused")
+out = sg.run(ins, ws)
+ref = O.run_chain(wl.ops, data["inputs"], data["weights"])
+got = out.double().cpu().numpy()
+assert sg.status() == B.AGO_OK and tuple(out.shape) == sg.output_shape
+assert abs(got - ref).max() <= 1e-2 * abs(ref).max() + 1e-3
+"""
+
+
+def test_run_is_the_first_that_asks_torch_for_the_device():
+    # a process whose arrays are all another library's: nothing has initialised torch's CUDA state when the output is made
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", FOREIGN], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
