@@ -43,6 +43,7 @@
 #include <mutex>
 #include <unordered_map>
 
+#include "ffn_pair_ring.h"
 #include "fused.h"
 #include "tc_common.cuh"
 #include "tmap.h"
@@ -52,12 +53,9 @@ namespace ago {
 namespace {
 
 using namespace tc;
+using namespace ffn_pair;
 
-constexpr int kFM = 128;          // rows per CTA (256 per pair and per cluster)
 constexpr int kFH = 128;          // hidden units per tile
-constexpr int kFK = 64;           // reduction elements per ring stage
-constexpr int kFStages = 6;
-constexpr int kFStageBytes = 24 * 1024;
 constexpr int kFSlotBytes = 32 * 1024;      // one H tile of this CTA's rows: 2 x [128 x 64] bf16, 128-byte swizzled
 constexpr int kFEpiWarps = 16;
 constexpr int kFEpiThreads = kFEpiWarps * 32;
@@ -150,7 +148,6 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
   // [h NC / 2, (h + 1) NC / 2), the first cn0 / 2 of them for the first chunk.
   const int cn0 = min(p.NC, 256), cn1 = p.NC - cn0;
   const uint32_t g2_tx = (uint32_t)(p.NC / 2) * kFK * 2u;            // W2 bytes per stage and CTA
-  const uint32_t g1_tx = (uint32_t)(kFM * kFK * 2 + 64 * kFK * 2);   // X + W1 bytes per stage and CTA
   if (tid == kFEpiThreads) {
     *abort_flag = 0u;
     for (int i = 0; i < 3; ++i) mbar_init(bar_full + i, 2);
@@ -184,19 +181,19 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
     __syncwarp();
     const uint32_t ring = smem_u32(sRing) + (uint32_t)(w * kFStageBytes), full0 = smem_u32(bar_full), lead_full0 = cluster_map(full0, lead_rank);
     int s = 0, round = 0;                        // pair of stages
-    auto acquire = [&](uint32_t tx_per_cta) {
+    auto acquire = [&](uint32_t tx_of_pair) {
       if (round > 0) mbar_wait_poll(bar_empty + 2 * s + w, (uint32_t)(round - 1) & 1u, abort_flag, p.status, 0x801);
-      mbar_arrive_expect_tx_elected(full0 + (uint32_t)(s * 8), 2u * tx_per_cta, announces);
+      mbar_arrive_expect_tx_elected(full0 + (uint32_t)(s * 8), tx_of_pair, announces);
     };
     auto advance = [&]() { if (++s == kFStages / 2) { s = 0; ++round; } };
     auto load_g1 = [&](const FfnSteps& c) {       // first GEMM of the pair's hidden tile of a step: this CTA's rows, its half of the tile
       const int hid0 = (2 * c.sb + P) * kFH + h * 64, row0 = c.unit * 2 * kFM + h * kFM;
-      for (int kb = w; kb < p.kblocks + w; kb += 2, advance()) {
-        if (kb >= p.kblocks) { acquire(0); continue; }      // an odd number of K blocks: nothing in the last stage
-        acquire(g1_tx);
+      for (int kb = w; kb < g1_stages(p.kblocks); kb += 2, advance()) {
+        acquire((uint32_t)(g1_stage_bytes(kb, p.kblocks, true) + g1_stage_bytes(kb, p.kblocks, false)));
         const uint32_t st = ring + (uint32_t)(s * 2 * kFStageBytes), full = lead_full0 + (uint32_t)(s * 8);
-        tma_load_2d_pair_elected(st, &tmap_x, full, kb * kFK, row0, elected);                   // X [128 rows x 64 k]
-        tma_load_2d_pair_elected(st + 16384, &tmap_w1, full, hid0, kb * kFK, elected);          // W1 [64 k x 64 hidden]
+        const int bytes = g1_stage_bytes(kb, p.kblocks, leader);
+        if (bytes > kW1Bytes) tma_load_2d_pair_elected(st, &tmap_x, full, kb * kFK, row0, elected);                 // X [128 rows x 64 k]
+        if (bytes > 0) tma_load_2d_pair_elected(st + kXBytes, &tmap_w1, full, hid0, kb * kFK, elected);             // W1 [64 k x 64 hidden]
       }
     };
     FfnSteps cur, ahead;
@@ -205,7 +202,7 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       if (g + 1 < steps) { ahead.next(p); load_g1(ahead); }
       for (int t = 0; t < 2; ++t, advance()) {    // second GEMM over the H tile of pair k, the own one first: two stages of 64 hidden units
         const int k = t ^ P;
-        acquire(g2_tx);
+        acquire(2u * g2_tx);
         // this CTA's half of every output chunk, as blocks of [64 k x 64 n]
         tma_load_3d_pair_elected(ring + (uint32_t)(s * 2 * kFStageBytes), &tmap_w2, lead_full0 + (uint32_t)(s * 8), 0,
                                  (2 * cur.sb + k) * kFH + w * 64, (2 * P + h) * (p.NC >> 7), elected);
