@@ -223,7 +223,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
   }
   // The set-up above overlaps the previous grid's tail where an SM has room or nothing to do.
   grid_dependency_wait();      // the previous grid of the stream has completed; device memory may be touched
-  grid_launch_dependents();
+  grid_launch_dependents_if(warp == 0);
   if (tid == kTmaWarp * 32) {
     mbar_arrive_expect_tx(bar_k, (uint32_t)(p.nkb * kKeyBlock * kD * 2));
     for (int kb = 0; kb < p.nkb; ++kb) tma_load_3d(sK + kb * kKeyBlock * kD * 2, &tmap_k, bar_k, h0 * kD, kb * kKeyBlock, b0);
@@ -675,7 +675,7 @@ ago_status_t attention_run(const Plan& plan, FusedState* st, const void* const* 
     cudaError_t e = ensure_max_dynamic_smem(reinterpret_cast<const void*>(attention_fused_kernel), smem_opt_in);
     if (e != cudaSuccess) { *err = std::string("cudaFuncSetAttribute: ") + cudaGetErrorString(e); return AGO_ERR_CUDA; }
   }
-  dim3 grid((unsigned)std::min(q.total, device_sm_count()));     // one persistent CTA per SM (the shared memory admits no second one)
+  dim3 grid((unsigned)std::min(q.total, device_sm_count()));     // one persistent CTA per SM (it takes all of the tensor memory)
   FusedLaunch launch(grid, kThreads, (size_t)host->smem_bytes, stream);
   cudaError_t e = cudaLaunchKernelEx(&launch.config, attention_fused_kernel, *maps[0], *maps[1], *maps[2], *maps[3], q);
   if (e != cudaSuccess) { *err = std::string("fused attention launch: ") + cudaGetErrorString(e); return AGO_ERR_CUDA; }

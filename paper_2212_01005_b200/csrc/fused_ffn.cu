@@ -99,7 +99,6 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   const int row0 = rb * kBM;
   const int G = p.G, stages = p.stages;
   grid_dependency_wait();      // the previous grid of the stream has completed; device memory may be touched
-  grid_launch_dependents();
   // tensor memory: columns [0, 256) two first-GEMM accumulators, [256, 512) two output-slice accumulators
   constexpr uint32_t kOutCol = 256;
 
@@ -114,6 +113,7 @@ ffn_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_consta
   if (warp == 0) {
     tmem_alloc(tmem_slot, 512);
     tmem_relinquish();
+    grid_launch_dependents();
   }
   tcgen05_fence_before_sync();
   __syncthreads();

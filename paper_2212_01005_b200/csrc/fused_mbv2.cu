@@ -326,7 +326,7 @@ mbv2_fused_kernel(const Mbv2Params p, const __grid_constant__ Mbv2Maps<TMA> maps
       tmem_relinquish();
     }
     grid_dependency_wait();      // first access to device memory below
-    grid_launch_dependents();
+    grid_launch_dependents_if(warp == kWarps - 2);
     if constexpr (TMA) {
       if (warp == kWarps - 1) {      // the warp that set the barrier up
         __syncwarp();

@@ -165,7 +165,7 @@ pwpw_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
   };
   if (TMA) meet();
   grid_dependency_wait();
-  grid_launch_dependents();
+  grid_launch_dependents_if(warp == kMmaWarp);
   if (tid == kCopyWarp * 32 && (int)blockIdx.x < ntiles) {
     load_x(blockIdx.x);
     if constexpr (TMA) load_w(&tmap_w.w1, bar_w, sW1, p.w1_rows, p.w1_box, p.w1_tx);

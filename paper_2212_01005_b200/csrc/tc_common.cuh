@@ -142,8 +142,16 @@ __device__ __forceinline__ void named_barrier_sync(uint32_t id, uint32_t threads
 // memory, index arithmetic) overlap that grid's tail. grid_dependency_wait() returns once the previous grid has
 // completed and its memory is visible -- every thread calls it before its first access to device memory.
 // (Without the launch attribute both are no-ops.)
+// One thread's grid_launch_dependents() counts for its CTA. A CTA that takes tensor memory calls it only once it has its columns:
+// from the warp that allocated them, or behind a __syncthreads() after the allocation. The allocation blocks until columns are
+// free, without a limit; a CTA of the next grid that shares the SM could otherwise take them first and then wait for this grid.
+// (The allocating warp alone, predicated: up to 1 % of a small kernel's time, the first of sixteen warps is earlier by that. Behind a
+// barrier of its own 3 % and behind the staging's 5 %, the inverted-residual block of 14 x 14 pixels.)
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_dependents_if(bool yes) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %0, 0;\n\t@q griddepcontrol.launch_dependents;\n\t}" ::"r"((uint32_t)yes) : "memory");
+}
 
 // ---- proxies and fences ---------------------------------------------------------------
 
