@@ -197,6 +197,9 @@ ago_subgraph_t ago_subgraph_create(const ago_subgraph_desc_t* desc);
  * of two convolutions": the upstream tile is produced inside the downstream
  * operator's outer tile loops); the unfused modes launch one kernel per
  * operator / per mini-subgraph and need a workspace (ago_subgraph_set_workspace).
+ * Runs of one handle may come from several threads: the handle's host state has
+ * a lock of its own. Runs that use a workspace share it, so the caller orders
+ * those on the GPU (one stream, or events).
  * Errors: AGO_ERR_INVALID_ARG (NULL), AGO_ERR_ALIGNMENT, AGO_ERR_WORKSPACE,
  * AGO_ERR_CUDA (launch failure). */
 ago_status_t ago_subgraph_run(ago_subgraph_t h, const void* const* inputs,

@@ -4,6 +4,7 @@
 
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 
@@ -22,6 +23,7 @@ struct ago_subgraph_s {
   unsigned int wait_budget_us = 0;      // 0: the kernels' default
   unsigned int skip_signal_code = 0;    // test hook, 0: none
   FusedState fused;                     // per-kernel host state (tensor maps, launch geometry)
+  std::mutex guard;                     // of everything above that a run changes: runs of one handle may come from several threads
 };
 
 namespace {
@@ -364,6 +366,7 @@ ago_status_t ago_subgraph_set_workspace(ago_subgraph_t h, void* dev_ptr, size_t 
   if (!h) return fail(AGO_ERR_INVALID_ARG, "handle is NULL");
   if (dev_ptr && (reinterpret_cast<uintptr_t>(dev_ptr) & 255u)) return fail(AGO_ERR_ALIGNMENT, "workspace is not 256-byte aligned");
   if (bytes < needed_workspace(h->plan)) return fail(AGO_ERR_WORKSPACE, "workspace smaller than ago_subgraph_workspace_bytes()");
+  std::lock_guard<std::mutex> lock(h->guard);
   h->workspace = dev_ptr;
   h->workspace_bytes = bytes;
   ++h->fused.workspace_epoch;   // nothing remembered about the old contents survives an attach
@@ -375,6 +378,7 @@ ago_status_t ago_subgraph_run(ago_subgraph_t h, const void* const* inputs, const
   ago_status_t s = check_run_args(h, inputs, weights, outputs);
   if (s != AGO_OK) return s;
   cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+  std::lock_guard<std::mutex> lock(h->guard);
   s = ensure_status_word(h);
   if (s != AGO_OK) return s;
   const Plan& p = h->plan;
@@ -454,6 +458,7 @@ ago_status_t ago_subgraph_query(ago_subgraph_t h, int32_t what, int64_t* out) {
 ago_status_t ago_subgraph_debug(ago_subgraph_t h, int32_t what, int64_t value) {
   if (!h) return fail(AGO_ERR_INVALID_ARG, "handle is NULL");
   if (value < 0 || value > 0xffffffffll) return fail(AGO_ERR_INVALID_ARG, "ago_subgraph_debug: value out of range");
+  std::lock_guard<std::mutex> lock(h->guard);
   if (what == AGO_DEBUG_WAIT_BUDGET_US) h->wait_budget_us = (unsigned int)value;
   else if (what == AGO_DEBUG_SKIP_SIGNAL) h->skip_signal_code = (unsigned int)value;
   else return fail(AGO_ERR_INVALID_ARG, "ago_subgraph_debug: unknown selector");
@@ -471,6 +476,7 @@ ago_status_t ago_subgraph_status(ago_subgraph_t h) {
   if (!h) return fail(AGO_ERR_INVALID_ARG, "handle is NULL");
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceSynchronize");
+  std::lock_guard<std::mutex> lock(h->guard);
   if (!h->status_word) return AGO_OK;
   unsigned int w = 0;
   e = cudaMemcpy(&w, h->status_word, sizeof(w), cudaMemcpyDeviceToHost);

@@ -16,7 +16,7 @@ struct FusedState {
   int variant = 0;         // kernel variant within the family (feed-forward chain: 1 = thread-block cluster, 3 = cluster of two CTA pairs)
   unsigned workspace_epoch = 0;   // bumped by every ago_subgraph_set_workspace: whatever a kernel family remembers about
                                   // the workspace contents (e.g. "already zeroed") is void after a new attach
-  void* impl = nullptr;                  // kernel-family host state (parameters, tensor-map cache)
+  void* impl = nullptr;                  // kernel-family host state (parameters, tensor-map cache); the handle's lock is held while it runs
   void (*impl_free)(void*) = nullptr;
   ~FusedState() { if (impl && impl_free) impl_free(impl); }
 };

@@ -38,7 +38,6 @@
 
 #include <algorithm>
 #include <cmath>
-#include <mutex>
 #include <unordered_map>
 
 #include "dw_common.cuh"
@@ -732,7 +731,6 @@ struct Mbv2Host {
   Mbv2Params prm;
   int smem_bytes = 0;
   bool expand = true, project = true;
-  std::mutex guard;                                               // of the maps: runs of one handle may come from several threads
   std::unordered_map<const void*, CUtensorMap> maps_x, maps_w1;   // by base address
 };
 
@@ -957,7 +955,6 @@ ago_status_t launch_variant(const Mbv2Params& q, Mbv2Host* host, cudaStream_t st
       *out = it->second;
       return true;
     };
-    std::lock_guard<std::mutex> lock(host->guard);
     if (!get(host->maps_x, q.x, false, &maps.x) || !get(host->maps_w1, q.w1, true, &maps.w1)) return AGO_ERR_CUDA;
   }
   return q.groups == 4 ? launch_groups<EXPAND, PROJECT, FOLD, 4, TMA>(q, maps, host->smem_bytes, stream, err)

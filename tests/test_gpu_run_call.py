@@ -82,6 +82,47 @@ def test_run_from_two_threads_on_streams_of_their_own(ago):
     sg0.close(); sg1.close()
 
 
+@pytest.mark.parametrize("wl", [
+    WL.pw_pw("call_many", [309], 1, 6, 64, 32, 64), WL.mbv2_block("call_many", [310], 1, 12, 64, 96, 64, 1, True), WL.attention("call_many", [311], 1, 32, 1, 64),
+    WL.Workload("call_many", [312], [(1, 5, 6, 16)], WL.resnet_block("x", [0], 1, 8, 16).ops, samples=1), WL.unfold_chain("call_many", [313], 1, 4, 9, 32, 64),
+], ids=["pw_pw", "block", "attention", "residual", "unfold"])
+def test_one_handle_from_two_threads_on_new_addresses(ago, wl):
+    # every run meets addresses that the handle has not seen: the two threads' runs change what it remembers about them at once
+    import torch
+    runs = 300
+    sg, (ins, ws) = handle(ago, wl)
+    ref = sg.run(ins, ws)
+
+    def copies(t):      # the tensor at `runs` places, 256 bytes apart or more
+        step = -(-t.numel() * t.element_size() // 256) * 256 // t.element_size()
+        flat = torch.zeros(runs * step, dtype=t.dtype, device=t.device).view(runs, step)
+        flat[:, :t.numel()] = t.flatten()
+        return [flat[i, :t.numel()].view(t.shape) for i in range(runs)]
+
+    places = [[copies(t) for t in ins + ws] for _ in range(2)]
+    torch.cuda.synchronize()
+    outs, start = [[], []], threading.Barrier(2)
+
+    def work(k):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            start.wait()
+            for i in range(runs):
+                args = [p[i] for p in places[k]]
+                outs[k].append(sg.run(args[:len(ins)], args[len(ins):]))
+            torch.cuda.current_stream().synchronize()
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert sg.status() == ago.AGO_OK and [len(o) for o in outs] == [runs, runs]
+    scale = float(ref.float().abs().max())
+    for o in outs[0] + outs[1]:
+        assert float((o.float() - ref.float()).abs().max()) <= 2.0 ** -7 * scale      # the block's chunks: one bf16 step
+    sg.close()
+
+
 def test_run_takes_whatever_has_a_device_and_an_address(ago):
     # arrays of another library, more weights than the handle reads, a stream as a ctypes pointer
     import ctypes
