@@ -136,9 +136,14 @@ typedef enum {
   AGO_Q_TILE_ROWS = 14,        /* fused kernel: downstream tile extent along the tiled dimension   */
   AGO_Q_SMEM_BYTES = 15,       /* fused kernel: dynamic shared memory per CTA                      */
   AGO_Q_MODE = 16,             /* the mode the handle runs in (what AGO_MODE_AUTO resolved to)     */
-  AGO_Q_WORKSPACE_TRAFFIC = 17 /* fused kernel: bytes per run stored or added into / read back from */
+  AGO_Q_WORKSPACE_TRAFFIC = 17,/* fused kernel: bytes per run stored or added into / read back from */
                                /* its device-memory workspace (partial sums of a split reduction); not */
                                /* part of AGO_Q_IO_BYTES; 0 when all intermediates stay on chip     */
+  AGO_Q_FUSED_VARIANT = 18     /* fused kernel: variant chosen for the shape. Feed-forward chain: 0 tiles the     */
+                               /* reduction, 1 cluster, 2 cluster with split row blocks, 3 paired clusters.       */
+                               /* Inverted-residual block, CONV1x1 -> DW3x3, pointwise pair and projection chain: */
+                               /* 1 when TMA brings input strip and first weights / the weights, 0 when the       */
+                               /* threads copy them. Other kernels and unfused modes: 0                           */
 } ago_query_t;
 #define AGO_Q_INDEXED(what, i) ((int32_t)(what) | ((int32_t)(i) << 16))
 

@@ -914,7 +914,7 @@ ago_status_t mbv2_plan(Plan* plan, FusedState* st, std::string* err) {
   // cycles -> us, the constant factor of each chain over 976 measured shapes (rms 7 % blocks, 10 to 11 % pairs)
   plan->fused_us = best_cost / (project ? 1820.0 : 2170.0);
   st->tile_rows = best_R; st->grid = q.N * q.strips * q.CS; st->smem_bytes = best_smem;
-  plan->tile_rows = best_R; plan->smem_bytes = best_smem;
+  plan->tile_rows = best_R; plan->smem_bytes = best_smem; plan->fused_variant = q.tma;
   return AGO_OK;
 }
 

@@ -437,7 +437,7 @@ ago_status_t pwpw_plan(Plan* plan, FusedState* st, std::string* err) {
   st->impl = host;
   st->impl_free = [](void* p) { delete static_cast<PwPwHost*>(p); };
   st->tile_rows = q.BR; st->grid = host->grid; st->smem_bytes = host->smem_bytes;
-  plan->tile_rows = q.BR; plan->smem_bytes = host->smem_bytes;
+  plan->tile_rows = q.BR; plan->smem_bytes = host->smem_bytes; plan->fused_variant = q.tma_weights;
   return AGO_OK;
 }
 

@@ -1,6 +1,6 @@
-"""Pointwise pairs and unfolded projection chains whose weights come by TMA, at the edges of that rule (few CTAs, small and large
-weights, rows of whole 64 bytes) and of its loads (padded channels, several blocks, blocks of more than 256 rows), against the
-oracle. Tolerance: the one of the parity tests (bf16 in and out, fp32 accumulate: max|gpu - ref| <= 1e-2 max|ref| + 1e-3)."""
+"""Pointwise pairs and unfolded projection chains whose weights come by TMA, on both sides of that rule (which shape takes which is
+checked on the host, test_tilings.py) and at the edges of its loads (padded channels, several blocks, blocks of more than 256 rows),
+against the oracle. Tolerance: the one of the parity tests (bf16 in and out, fp32 accumulate: max|gpu - ref| <= 1e-2 max|ref| + 1e-3)."""
 import pytest
 
 from paper_2212_01005_b200 import workloads as WL
@@ -9,14 +9,27 @@ from test_gpu_tile_edges import check
 pytestmark = pytest.mark.gpu
 
 
+def pair(shape):
+    n, h, c0, c1, c2 = shape
+    return WL.pw_pw("pw_pw_weights", [230, *shape], n, h, c0, c1, c2)
+
+
+def chain(shape):
+    b, p, n, c0, c1, c2 = shape
+    m = b * p * n
+    ops = [("gemm", dict(N=c1)), ("reshape", dict(shape=(b * p, n, c1))), ("add_input", dict(input=1)),
+           ("reshape", dict(shape=(b, p, n, c1))), ("transpose", dict(a=1, b=2)), ("reshape", dict(shape=(m, c1))),
+           ("gemm", dict(N=c2)), ("reshape", dict(shape=(b, n, p, c2)))]
+    return WL.Workload("unfold_weights", [231, *shape], [(m, c0), (b * p, n, c1)], ops, samples=b, input_dist=["normal", "normal"])
+
+
 @pytest.mark.parametrize("shape", [
     # n, h, c0, c1, c2: one pixel; one CTA; 40 and 41 CTAs of 32 rows; 72 and 73; 148 with rows of 64 bytes
     (1, 1, 8, 8, 8), (1, 5, 24, 8, 40), (1, 7, 200, 120, 104), (5, 16, 48, 24, 48), (1, 36, 48, 24, 48),
     (9, 16, 192, 40, 192), (1, 48, 192, 40, 192), (1, 97, 192, 32, 192), (2, 70, 96, 32, 96), (1, 20, 264, 72, 136),
 ])
 def test_pointwise_pair(ago, shape):
-    n, h, c0, c1, c2 = shape
-    check(ago, WL.pw_pw("pw_pw_weights", [230, *shape], n, h, c0, c1, c2))
+    check(ago, pair(shape))
 
 
 @pytest.mark.parametrize("shape", [
@@ -25,9 +38,4 @@ def test_pointwise_pair(ago, shape):
     (1, 4, 324, 32, 32, 64), (6, 4, 196, 64, 64, 128), (9, 9, 256, 96, 96, 192), (3, 4, 196, 120, 120, 240),
 ])
 def test_unfold_chain(ago, shape):
-    b, p, n, c0, c1, c2 = shape
-    m = b * p * n
-    ops = [("gemm", dict(N=c1)), ("reshape", dict(shape=(b * p, n, c1))), ("add_input", dict(input=1)),
-           ("reshape", dict(shape=(b, p, n, c1))), ("transpose", dict(a=1, b=2)), ("reshape", dict(shape=(m, c1))),
-           ("gemm", dict(N=c2)), ("reshape", dict(shape=(b, n, p, c2)))]
-    check(ago, WL.Workload("unfold_weights", [231, *shape], [(m, c0), (b * p, n, c1)], ops, samples=b, input_dist=["normal", "normal"]))
+    check(ago, chain(shape))

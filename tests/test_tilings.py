@@ -2,6 +2,8 @@
 import ctypes
 
 import test_ffn_cluster_shape as FS
+import test_gpu_block_strip_loads as S
+import test_gpu_pointwise_weights as P
 import test_gpu_tile_edges as E
 from paper_2212_01005_b200 import binding as B
 from paper_2212_01005_b200 import workloads as WL
@@ -80,3 +82,55 @@ def test_feed_forward_chains_take_the_kernel_of_the_least_estimate():
         sg = B.Subgraph(wl.ops, wl.input_shapes, mode="fused")
         assert (sg.query(B.AGO_Q_TILE_ROWS), sg.query(B.AGO_Q_SMEM_BYTES)) == (tile_rows, smem), shape
         sg.close()
+
+
+def variant(wl):
+    sg = B.Subgraph(wl.ops, wl.input_shapes, mode="fused")
+    v = sg.query(B.AGO_Q_FUSED_VARIANT)
+    sg.close()
+    return v
+
+
+# Shapes whose strip and first weights the threads copy: the others of the two tests take them by TMA. (bytes of the strip, its pixels)
+COPIED_STRIPS = {
+    (40, 7, 7, 32, 192, 32, 1, True), (1, 33, 31, 32, 96, 16, 1, False), (1, 32, 32, 32, 96, 16, 1, False),      # 4032 to 6144 bytes
+    (9, 12, 10, 256, 512, 64, 1, False),      # 30720 bytes, 60 pixels (68 and 75 go by TMA)
+    (8, 28, 28, 16, 96, 24, 1, False),      # 17920 bytes, pixels of 32
+    (4, 20, 32, 128, 1), (3, 31, 64, 96, 2),      # 6400 and 11904 bytes (13056 go by TMA)
+}
+
+
+def test_inverted_residual_strips_come_as_their_rule_says():
+    blocks, pairs = cases(S.test_block), cases(S.test_pointwise_depthwise)
+    assert COPIED_STRIPS <= set(blocks) | set(pairs)
+    for s in blocks:
+        assert variant(S.block(s)) == (s not in COPIED_STRIPS), s
+    for s in pairs:
+        assert variant(WL.pw_dw("x", [0], *s)) == (s not in COPIED_STRIPS), s
+    assert variant(WL.dw_pw("x", [0], 32, 28, 96, 32, 1)) == 0
+
+
+# Shapes whose weights the threads copy. (CTAs, bytes of weights)
+COPIED_WEIGHTS = {
+    (1, 36, 48, 24, 48), (1, 4, 324, 32, 32, 64),      # 41 CTAs, 4608 and 6144 bytes (40 CTAs take them by TMA)
+    (2, 70, 96, 32, 96),      # 148 CTAs, 12288 bytes in whole rows, tiles of 67 rows (of 64 go by TMA)
+    (3, 4, 196, 120, 120, 240),      # 74 CTAs, 86400 bytes, rows that end inside 64 bytes
+}
+
+
+def test_pointwise_weights_come_as_their_rule_says():
+    pairs, chains = cases(P.test_pointwise_pair), cases(P.test_unfold_chain)
+    assert COPIED_WEIGHTS <= set(pairs) | set(chains)
+    for s in pairs:
+        assert variant(P.pair(s)) == (s not in COPIED_WEIGHTS), s
+    for s in chains:
+        assert variant(P.chain(s)) == (s not in COPIED_WEIGHTS), s
+
+
+def test_feed_forward_variants_are_named():
+    for (rows, d, hidden, d_out), v in {(646, 64, 3328, 384): 0, (12288, 64, 256, 128): 1, (512, 768, 3072, 768): 2, (12288, 768, 3072, 768): 3}.items():
+        assert variant(WL.ffn("x", [0], rows, d, hidden, 1, d_out=d_out)) == v
+    wl = WL.get("ffn_512")
+    sg = B.Subgraph(wl.ops, wl.input_shapes, mode="per_mini_subgraph")
+    assert sg.query(B.AGO_Q_FUSED_VARIANT) == 0
+    sg.close()
