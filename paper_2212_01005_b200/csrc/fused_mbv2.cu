@@ -905,7 +905,12 @@ ago_status_t mbv2_plan(Plan* plan, FusedState* st, std::string* err) {
   // bytes per cycle. 25 images of 15 x 15 x 96 15.5 -> 14.6 us, 40 of 20 x 20 x 64 18.6 -> 17.7, 32 of 28 x 28 x 32 at stride 2 9.7 -> 9.2, 26 of
   // 8 x 8 x 160 14.8 -> 13.2; 32 shapes on this side of the line 1.01 to 1.1x. Short strips were 1 to 1.5 % slower (one image 14 x 14 x 32:
   // 2.7 KB, 5.8 -> 5.9; two of 9 x 9 x 96 at stride 2: 5.2 KB), pixels of 32 bytes up to 7 % (8 images of 56 x 56 x 16: 7.6 -> 8.1).
-  q.tma = expand && !q.fold_b1 && q.Cin >= 32 && q.P_x >= 64 && q.P_x * q.Cin * 2 >= 12800 ? 1 : 0;
+  // Pixels that end inside a 32-byte sector cost their neighbours' bytes too, and boxes of 64 channels that are mostly padding bring zeros:
+  // over 36 shapes each the mean of TMA over copies is 1.04 at 72 channels, 1.03 at 88, 1.01 at 104, 0.99 and 1.00 at 136 and 152 with single
+  // shapes up to 1.2 (30 images of 17 x 20 x 72 10.3 -> 11.4 us, 40 of 18 x 18 x 72 expanded to 32 4.3 -> 5.1), but 0.96 to 0.98 at 120
+  // and 184, in whole blocks also at 168 and 200 (pairs 1.0), and 0.93 to 0.99 for whole sectors.
+  const bool whole_sectors = q.Cin % 16 == 0 || q.Cin % 64 == 56 || (project && q.Cin >= 168);
+  q.tma = expand && !q.fold_b1 && whole_sectors && q.Cin >= 32 && q.P_x >= 64 && q.P_x * q.Cin * 2 >= 12800 ? 1 : 0;
   q.w1_box = std::min(q.Cexp, 256);
   while (q.Cexp % q.w1_box != 0) q.w1_box -= kChunk;
   host->smem_bytes = best_smem;

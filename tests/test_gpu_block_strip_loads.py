@@ -20,12 +20,12 @@ def block(shape):
     (30, 13, 9, 72, 144, 24, 2, False), (25, 15, 15, 96, 576, 96, 1, True), (12, 14, 14, 136, 768, 136, 1, True), (3, 29, 27, 64, 384, 64, 1, True),
     (160, 14, 14, 32, 512, 32, 1, True), (32, 28, 28, 32, 192, 64, 2, False), (2, 57, 58, 32, 192, 40, 2, False), (6, 20, 20, 64, 384, 160, 1, False),
     (9, 12, 10, 256, 512, 64, 1, False), (26, 8, 8, 160, 960, 96, 1, False), (4, 15, 15, 96, 576, 96, 2, False),
-    (8, 28, 28, 16, 96, 24, 1, False),
+    (8, 28, 28, 16, 96, 24, 1, False), (4, 16, 15, 112, 160, 112, 1, True), (5, 14, 17, 120, 192, 48, 2, False), (2, 9, 23, 168, 64, 24, 1, False),
 ])
 def test_block(ago, shape):
     check(ago, block(shape))
 
 
-@pytest.mark.parametrize("shape", [(4, 20, 32, 128, 1), (3, 31, 64, 96, 2), (2, 17, 96, 192, 1)])      # n, h, c_in, c_exp, stride
+@pytest.mark.parametrize("shape", [(4, 20, 32, 128, 1), (3, 31, 64, 96, 2), (2, 17, 96, 192, 1), (2, 24, 168, 64, 1), (1, 26, 120, 48, 1)])      # n, h, c_in, c_exp, stride
 def test_pointwise_depthwise(ago, shape):
     check(ago, WL.pw_dw("pw_dw_strips", [241, *shape], *shape))

@@ -96,6 +96,7 @@ COPIED_STRIPS = {
     (40, 7, 7, 32, 192, 32, 1, True), (1, 33, 31, 32, 96, 16, 1, False), (1, 32, 32, 32, 96, 16, 1, False),      # 4032 to 6144 bytes
     (9, 12, 10, 256, 512, 64, 1, False),      # 30720 bytes, 60 pixels (68 and 75 go by TMA)
     (8, 28, 28, 16, 96, 24, 1, False),      # 17920 bytes, pixels of 32
+    (30, 13, 9, 72, 144, 24, 2, False), (12, 14, 14, 136, 768, 136, 1, True), (2, 24, 168, 64, 1),      # pixels that end inside a sector
     (4, 20, 32, 128, 1), (3, 31, 64, 96, 2),      # 6400 and 11904 bytes (13056 go by TMA)
 }
 
