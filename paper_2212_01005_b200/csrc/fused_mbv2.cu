@@ -907,7 +907,7 @@ ago_status_t mbv2_plan(Plan* plan, FusedState* st, std::string* err) {
   // 2.7 KB, 5.8 -> 5.9; two of 9 x 9 x 96 at stride 2: 5.2 KB), pixels of 32 bytes up to 7 % (8 images of 56 x 56 x 16: 7.6 -> 8.1).
   // Pixels that end inside a 32-byte sector cost their neighbours' bytes too, and boxes of 64 channels that are mostly padding bring zeros:
   // over 36 shapes each the mean of TMA over copies is 1.04 at 72 channels, 1.03 at 88, 1.01 at 104, 0.99 and 1.00 at 136 and 152 with single
-  // shapes up to 1.2 (30 images of 17 x 20 x 72 10.3 -> 11.4 us, 40 of 18 x 18 x 72 expanded to 32 4.3 -> 5.1), but 0.96 to 0.98 at 120
+  // shapes up to 1.2 (30 images of 17 x 20 x 72 10.3 -> 11.4 us, 40 of 18 x 18 x 72 expanded to 32 5.1 -> 6.1), but 0.96 to 0.98 at 120
   // and 184, in whole blocks also at 168 and 200 (pairs 1.0), and 0.93 to 0.99 for whole sectors.
   const bool whole_sectors = q.Cin % 16 == 0 || q.Cin % 64 == 56 || (project && q.Cin >= 168);
   q.tma = expand && !q.fold_b1 && whole_sectors && q.Cin >= 32 && q.P_x >= 64 && q.P_x * q.Cin * 2 >= 12800 ? 1 : 0;
