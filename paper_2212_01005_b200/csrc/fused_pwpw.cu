@@ -350,13 +350,20 @@ int round_up(int v, int m) { return (v + m - 1) / m * m; }
 
 // Whether the weights come by TMA. That takes one thread and starts at once, where the copies take every thread 1.5k to 3.7k
 // cycles; but each row of a block is a request to L2 past L1, and all CTAs make them for the same lines at the same moment.
-// Against the copies, 176 pairs and 35 chains of 81 to 17248 rows: up to 40 CTAs 1.06 to 1.23x; with 12 KB of weights up to 72 CTAs
-// 1.0 to 1.2x; rows of whole 64 bytes and tiles of up to 64 rows 1.03 to 1.1x up to one CTA per SM (pairs of larger tiles 0.96x);
-// 98 to 148 CTAs with rows of 48 or 80 bytes 0.7 to 0.95x.
+// Against the copies, 134 pairs and 123 chains of 1 to 60000 rows, time by TMA over time by copies:
+//   pairs    up to 40 CTAs 0.78 to 0.96; with 12 KB of weights up to 64 CTAs (16 KB: 72) 0.83 to 0.95, but 1.10 at 72 with 13.8 KB;
+//            rows of whole 64 bytes and tiles of up to 64 rows 0.9 to 0.97 up to one CTA per SM; else 1.0 to 1.26 from 86 CTAs on
+//   chains   up to 24 CTAs 0.84 to 0.97; with less than 20 KB of weights 1.01 to 1.10 from 31 CTAs on, with more 0.82 to 1.0 up to 72;
+//            rows of whole 64 bytes 0.89 to 1.02 up to one CTA per SM, 1.01 to 1.02 with tiles of more than 120 rows; else up to 1.2;
+//            weights in rows of 16 bytes (8 columns) 1.02 to 1.12 whatever the CTAs
+// and 1.0 to 1.4 with two CTAs per SM.
 bool weights_by_tma(const PwPwParams& q, bool chain, int grid, int sms) {
-  if (grid <= 40) return true;
-  const bool whole = q.C0 % 32 == 0 && q.C1 % 32 == 0 && q.C2 % 32 == 0 && (chain || q.BR <= 64);
-  return 2 * q.C1 * (q.C0 + q.C2) >= 12 * 1024 && grid <= (whole ? sms : 72);
+  const int bytes = 2 * q.C1 * (q.C0 + q.C2);
+  const bool whole = q.C0 % 32 == 0 && q.C1 % 32 == 0 && q.C2 % 32 == 0 && q.BR <= (chain ? 120 : 64);
+  if (chain && std::min(q.C1, q.C2) < 16) return false;
+  if (grid <= (chain ? 24 : 40)) return true;
+  if (bytes < (chain ? 20 : 12) * 1024) return false;
+  return grid <= (whole ? sms : bytes >= 16 * 1024 ? 72 : 64);
 }
 
 struct PwPwHost {

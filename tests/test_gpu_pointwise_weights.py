@@ -24,18 +24,21 @@ def chain(shape):
 
 
 @pytest.mark.parametrize("shape", [
-    # n, h, c0, c1, c2: one pixel; one CTA; 40 and 41 CTAs of 32 rows; 72 and 73; 148 with rows of 64 bytes
+    # n, h, c0, c1, c2: one pixel; one CTA; 40 and 41 CTAs of 32 rows; 72 with 30 KB of weights, 64 and 67 with 13.8 KB; 148 with rows of 64 bytes
     (1, 1, 8, 8, 8), (1, 5, 24, 8, 40), (1, 7, 200, 120, 104), (5, 16, 48, 24, 48), (1, 36, 48, 24, 48),
     (9, 16, 192, 40, 192), (1, 48, 192, 40, 192), (1, 97, 192, 32, 192), (2, 70, 96, 32, 96), (1, 20, 264, 72, 136),
+    (2, 32, 144, 24, 144), (1, 46, 144, 24, 144),
 ])
 def test_pointwise_pair(ago, shape):
     check(ago, pair(shape))
 
 
 @pytest.mark.parametrize("shape", [
-    # images, pixels per patch, patches, C0, C1, C2: one row per image; blocks of 264, 320 and 512 rows; 40 and 41 CTAs; 148 with whole rows
-    (1, 1, 1, 8, 8, 8), (1, 4, 9, 264, 40, 64), (2, 4, 16, 320, 64, 128), (1, 4, 25, 512, 24, 72), (1, 4, 320, 32, 32, 64),
+    # images, pixels per patch, patches, C0, C1, C2: one row per image; blocks of 264, 320 and 512 rows; 40 and 41 CTAs; 148 with whole rows;
+    # 24 and 25 CTAs with 13.8 KB of weights, 72 and 73 with 86 KB; tiles of 111 and 123 rows
+    (1, 1, 1, 8, 8, 8), (1, 1, 1, 16, 16, 16), (1, 4, 9, 264, 40, 64), (2, 4, 16, 320, 64, 128), (1, 4, 25, 512, 24, 72), (1, 4, 320, 32, 32, 64),
     (1, 4, 324, 32, 32, 64), (6, 4, 196, 64, 64, 128), (9, 9, 256, 96, 96, 192), (3, 4, 196, 120, 120, 240),
+    (1, 4, 192, 48, 48, 96), (1, 4, 196, 48, 48, 96), (1, 4, 576, 120, 120, 240), (1, 4, 584, 120, 120, 240), (32, 4, 256, 96, 96, 192), (32, 4, 284, 96, 96, 192),
 ])
 def test_unfold_chain(ago, shape):
     check(ago, chain(shape))

@@ -113,9 +113,12 @@ def test_inverted_residual_strips_come_as_their_rule_says():
 
 # Shapes whose weights the threads copy. (CTAs, bytes of weights)
 COPIED_WEIGHTS = {
-    (1, 36, 48, 24, 48), (1, 4, 324, 32, 32, 64),      # 41 CTAs, 4608 and 6144 bytes (40 CTAs take them by TMA)
+    (1, 36, 48, 24, 48), (1, 46, 144, 24, 144),      # pairs: 41 CTAs (40 take them by TMA); 67 CTAs, 13824 bytes (64 by TMA, and 72 with 30720 bytes)
     (2, 70, 96, 32, 96),      # 148 CTAs, 12288 bytes in whole rows, tiles of 67 rows (of 64 go by TMA)
-    (3, 4, 196, 120, 120, 240),      # 74 CTAs, 86400 bytes, rows that end inside 64 bytes
+    (1, 4, 320, 32, 32, 64), (1, 4, 324, 32, 32, 64), (1, 4, 196, 48, 48, 96),      # chains: 25 to 41 CTAs, 6144 and 13824 bytes (24 CTAs by TMA)
+    (1, 4, 584, 120, 120, 240), (3, 4, 196, 120, 120, 240),      # 73 and 74 CTAs, rows that end inside 64 bytes (72 by TMA)
+    (1, 1, 1, 8, 8, 8),      # a chain's weights in rows of 16 bytes
+    (32, 4, 284, 96, 96, 192),      # one CTA per SM, whole rows, tiles of 123 rows (of 111 by TMA)
 }
 
 
