@@ -28,6 +28,11 @@ struct FfnClusterShape {
   int w2_off;              // > 0: one step per cluster and everything fits: the step's W2 tiles have stages of their own there
 };
 
+// Two warps fill the ring in turn. With two stages or more, the load two before a stage's next one has seen the use before its last one
+// over, so that the wait's one bit of parity suffices whichever warp filled it. A single stage holds this many loads: the second
+// waits for the first, a third could pass before the second.
+constexpr int kLoadsOfOneStage = 2;
+
 // A part's partial sums (64 rows or more) are staged as blocks of 64 columns in two buffers from the start of the ring on. The ring
 // itself is free by then. Where the buffers are larger they run into the hidden tiles' slots, which the other CTAs of the cluster may
 // still be copying this CTA's tile out of: the kernel then waits until they have used it.

@@ -16,9 +16,8 @@
 // into all N2 output columns without recomputation and without reductions outside the SM.
 //
 // Per CTA (rank r), T = hidden tiles / CS steps:
-//   ring   two TMA warps, every second stage each (three stages or more, so a stage's previous use is over when its next is waited
-//          for): X [RP x 64] + W1 [64 x BH] for the first GEMM, W2 [64 x N2/CS] for the second; a third one for W2 tiles with
-//          memory of their own. Converged, an elected lane issuing, one load per operand: a thread in a lane-0 branch that loaded
+//   ring   two TMA warps, every second load each (ffn_cluster_shape.h, kLoadsOfOneStage): X [RP x 64] + W1 [64 x BH] for the first
+//          GEMM, W2 [64 x N2/CS] for the second; a third one for W2 tiles with memory of their own. Converged, an elected lane issuing, one load per operand: a thread in a lane-0 branch that loaded
 //          every 64 columns by themselves took 350 cycles per stage, 4.5k of a one-step run's 34k (512 rows 17.4 -> 15.7 us,
 //          64 rows 11.2 -> 9.5, 1815 rows 40 -> 36)
 //   MMA    one warp: G1(t+1): Hacc[(t+1) & 1] = X W1[:, tile (t+1) CS + r]; then for k = 0..CS-1
@@ -144,8 +143,7 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
   __syncthreads();
   // Every CTA's barriers exist before a peer signals them: the arrival is here (relaxed: fence_mbar_init published them), each
   // role waits before it first touches another CTA.
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-  auto cluster_started = [] { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); };
+  cluster_arrive();
   tcgen05_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
   // The set-up above overlaps the previous grid's tail (the second launch of the previous run leaves the SM room for this CTA).
@@ -173,7 +171,7 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     } else {
       const uint32_t ring = smem_u32(sRing), full0 = smem_u32(bar_full);
       int s = 0, round = 0;
-      bool mine = w == 0;                    // stages go to the two warps in turn
+      bool mine = w == 0;                    // loads go to the two warps in turn
       auto acquire = [&](uint32_t bytes) -> uint32_t {
         if (round > 0) mbar_wait_poll(bar_empty + s, (uint32_t)(round - 1) & 1u, abort_flag, p.status, 0x701);
         mbar_arrive_expect_tx_elected(full0 + (uint32_t)(s * 8), bytes, elected);
@@ -204,7 +202,7 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
       }
     }
     __syncwarp();
-    cluster_started();
+    cluster_wait();
   } else if (warp == kEpiWarps) {
     // ================================ MMA issuer ================================
     // the whole warp, converged; MMAs and commits predicated on one elected lane (see tc_common.cuh)
@@ -235,7 +233,7 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
         umma_commit_elected(bar_hacc + b, elected);
       };
       if (steps > 0) g1(0);
-      cluster_started();
+      cluster_wait();
       for (int step = 0; step < steps; ++step) {
         if (step + 1 < steps) g1(step + 1);
         const int t = step % T, bi = step / T;
@@ -279,7 +277,7 @@ ffn_cluster_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_cons
     uint8_t* slot = sH + r * slot_bytes;           // this CTA produces into slot r everywhere
     constexpr int kParts = kEpiWarps / 4;
     constexpr int pc = BH / kParts;                        // columns per thread: 16 or 32
-    cluster_started();
+    cluster_wait();
 
     for (int step = 0; step < steps; ++step) {
       const int b = step & 1, t = step % T;

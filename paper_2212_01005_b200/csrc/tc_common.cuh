@@ -184,10 +184,6 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-// Every thread of every CTA of the cluster arrives; returns when all have (release / acquire at cluster scope).
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 // The two halves of a cluster barrier (all threads) that publishes nothing: where barriers are made visible by fence_mbar_init and
 // data by the copies' own completion, the arrival can be relaxed. A release at cluster scope takes 1200 cycles, more behind
 // outstanding stores.
@@ -375,14 +371,8 @@ __device__ __forceinline__ void umma_commit_elected(uint64_t* bar, uint32_t elec
 // loads of both CTAs complete on the leader's barrier.
 
 // TMA load whose completion is counted on a barrier that may live in the peer CTA (`bar_cluster_addr` is a
-// shared::cluster address, see cluster_map); the data lands in the issuing CTA.
-__device__ __forceinline__ void tma_load_2d_pair(void* dst, const void* tmap, uint32_t bar_cluster_addr, int c0, int c1) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(tmap)), "r"(bar_cluster_addr), "r"(c0), "r"(c1)
-      : "memory");
-}
-// The same from a converged warp, on its elected lane (see "MMA issue from a converged warp"), and a box of a 3-D tensor.
+// shared::cluster address, see cluster_map); the data lands in the issuing CTA. From a converged warp, on its elected lane (see
+// "MMA issue from a converged warp"), and a box of a 3-D tensor.
 __device__ __forceinline__ void tma_load_2d_pair_elected(uint32_t dst_saddr, const void* tmap, uint32_t bar_cluster_addr, int c0, int c1, uint32_t elected) {
   asm volatile(
       "{\n\t.reg .pred q;\n\t"

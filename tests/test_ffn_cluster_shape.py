@@ -18,6 +18,7 @@ extern "C" int plan(FfnClusterShape* q) {      // M, K, Hid, N2 given -> bytes o
   if (!choose_split(q, (q->M + kBM - 1) / kBM, kResident)) return 0;
   return layout(q);
 }
+extern "C" int loads_of_one_stage() { return kLoadsOfOneStage; }
 extern "C" int clusters(int row_blocks, int J, int resident) { return launched_clusters(row_blocks, J, resident); }
 """
 
@@ -70,6 +71,15 @@ def test_staged_sums_stay_off_what_is_still_copied(lib):
         waits[(q.M, q.K, q.Hid, q.N2)] = past
     assert waits[(300, 64, 2048, 256)] and waits[(1000, 128, 512, 384)]
     assert not waits[(511, 768, 3072, 768)]
+
+
+def test_ring_has_the_stages_that_two_producers_need(lib):
+    short = 0
+    for q, _ in shapes(lib):
+        loads = q.kblocks if q.w2_off else q.Tp * (q.kblocks + q.CS * (q.BH // 64))      # of a part or row block
+        assert q.stages >= 2 or q.stages == 1 and q.w2_off and loads <= lib.loads_of_one_stage(), list(getattr(q, n) for n in FIELDS)
+        short += q.stages < 3
+    assert short > 0
 
 
 def test_layout_and_kernel_agree_on_whole_row_blocks(lib):
