@@ -315,7 +315,7 @@ attention_fused_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_
         if (i + 1 < n) {
           mbar_wait(bar_d + 0, ph, abort_flag, p.status, 0x20a);
           mbar_wait(bar_q, ph ^ 1u, abort_flag, p.status, 0x207);
-          if (last_of_head) mbar_wait(bar_k, head_ph ^ 1u, abort_flag, p.status, 0x202);
+          if (last_of_head) mbar_wait(bar_k, head_ph ^ 1u, abort_flag, p.status, 0x20c);
           tcgen05_fence_after_sync();
           issue_scores(0);
         }

@@ -579,7 +579,7 @@ mbv2_fused_kernel(const Mbv2Params p, const __grid_constant__ Mbv2Maps<TMA> maps
       }
       fence_proxy_async_smem();
       // the expand GEMM of the group's next chunk (issued after the previous barrier) is complete
-      if (EXPAND && waiter && c + NG < p.NC) mbar_wait(bar_e + g, (uint32_t)(it + 1) & 1u, abort_flag, p.status, 0x102);
+      if (EXPAND && waiter && c + NG < p.NC) mbar_wait(bar_e + g, (uint32_t)(it + 1) & 1u, abort_flag, p.status, 0x105);
       named_barrier_sync(gbar, kGroupThreads);
       if (!EXPAND) load_chunk(c + 2 * NG, it & 1);   // the E buffer of chunk c is free
       if (!PROJECT) {
@@ -684,7 +684,7 @@ mbv2_fused_kernel(const Mbv2Params p, const __grid_constant__ Mbv2Maps<TMA> maps
         }
         cluster_wait();                           // the copies out of this CTA have arrived: it may leave
       } else {
-      if (TMA && p.residual) mbar_wait(bar_x, 0, abort_flag, p.status, 0x109);      // complete since the first product: the strip is read below
+      if (TMA && p.residual) mbar_wait(bar_x, 0, abort_flag, p.status, 0x10a);      // complete since the first product: the strip is read below
       for (int t = warp >> 2; t < p.M2; t += kWarps / 4) {
         const int po = t * 128 + (warp & 3) * 32 + lane;
         for (int j0 = 0; j0 < p.Coutp; j0 += 16) {

@@ -216,10 +216,10 @@ pwpw_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
   if (warp == kCopyWarp) {
     if (lane == 0)
       for (int tile = blockIdx.x + gridDim.x, it = 0; tile < ntiles; tile += gridDim.x, ++it) {
-        mbar_wait(bar_m1, (uint32_t)it & 1u, abort_flag, p.status, 0x603);   // the first product has read the X tile
+        mbar_wait(bar_m1, (uint32_t)it & 1u, abort_flag, p.status, 0x903);   // the first product has read the X tile
         load_x(tile);
         if (CHAIN) {
-          mbar_wait(bar_m2, (uint32_t)it & 1u, abort_flag, p.status, 0x605);   // the second product has read the buffer
+          mbar_wait(bar_m2, (uint32_t)it & 1u, abort_flag, p.status, 0x905);   // the second product has read the buffer
           load_r(tile);
         }
       }
@@ -241,16 +241,16 @@ pwpw_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
     };
     for (int tile = blockIdx.x, it = 0; tile < ntiles; tile += gridDim.x, ++it) {
       const uint32_t par = (uint32_t)it & 1u;
-      if (shared_cols && it) mbar_wait(bar_d, par ^ 1u, abort_flag, p.status, 0x606);
+      if (shared_cols && it) mbar_wait(bar_d, par ^ 1u, abort_flag, p.status, 0x906);
       // ---- P2: first product ----
-      mbar_wait(bar_x, par, abort_flag, p.status, 0x600);
-      if (TMA && it == 0) mbar_wait(bar_w, 0, abort_flag, p.status, 0x608);
+      mbar_wait(bar_x, par, abort_flag, p.status, 0x900);
+      if (TMA && it == 0) mbar_wait(bar_w, 0, abort_flag, p.status, 0x908);
       tcgen05_fence_after_sync();
       product(tmem_base, sX, sW1, p.w1_block, p.nkb0, p.C0p, idesc1);
       umma_commit_elected(bar_m1, elected);
       // ---- P4: second product ----
-      mbar_wait(bar_a, par, abort_flag, p.status, 0x607);
-      if (TMA && it == 0) mbar_wait(bar_w + 1, 0, abort_flag, p.status, 0x609);
+      mbar_wait(bar_a, par, abort_flag, p.status, 0x907);
+      if (TMA && it == 0) mbar_wait(bar_w + 1, 0, abort_flag, p.status, 0x909);
       tcgen05_fence_after_sync();
       product(tmem_base + (uint32_t)p.acc2_col, sA, sW2, p.w2_block, p.nkb1, p.C1p, idesc2);
       umma_commit_elected(bar_m2, elected);
@@ -273,8 +273,8 @@ pwpw_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
         const int g = m / ab, rem = m - g * ab, i = rem / p.perm_b, j = rem - i * p.perm_b;
         m = (g * p.perm_b + j) * p.perm_a + i;
       }
-      mbar_wait(bar_m1, par, abort_flag, p.status, 0x601);
-      if (CHAIN) mbar_wait(bar_r, par, abort_flag, p.status, 0x604);
+      mbar_wait(bar_m1, par, abort_flag, p.status, 0x901);
+      if (CHAIN) mbar_wait(bar_r, par, abort_flag, p.status, 0x904);
       tcgen05_fence_after_sync();
       // ---- P3: [+ b1, ReLU6 | + tensor] -> swizzled A operand of the second product (no rows past the tile) ----
       if (quarter_rows < rows)
@@ -309,7 +309,7 @@ pwpw_fused_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_const
       tcgen05_fence_before_sync();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_a);
-      mbar_wait(bar_m2, par, abort_flag, p.status, 0x602);
+      mbar_wait(bar_m2, par, abort_flag, p.status, 0x902);
       tcgen05_fence_after_sync();
       // ---- P5: [+ b2, ReLU6] -> device memory; every thread its row, 32 bytes at a time ----
       if (quarter_rows < rows) {
