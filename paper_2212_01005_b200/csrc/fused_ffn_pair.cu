@@ -79,7 +79,7 @@ struct FfnPairParams {
   int units_whole, J;
   float* acc;              // [J][split_rows][N2] fp32
   int split_rows;          // rows of the split blocks that exist: M - units_whole * 256
-  int wide_out, wide_acc;  // out / acc start on a 32-byte boundary (their rows then do too)
+  int wide_out;            // out starts on a 32-byte boundary (its rows then do too; a workspace starts on 256 bytes)
 };
 
 __device__ __forceinline__ float gelu_tanh_pair(float v) {
@@ -354,7 +354,7 @@ ffn_pair_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constan
       uint8_t* dst = split ? reinterpret_cast<uint8_t*>(p.acc + ((size_t)part * p.split_rows + (size_t)(row0 - p.units_whole * 2 * kFM)) * p.N2 + n0)
                            : reinterpret_cast<uint8_t*>(p.out + (size_t)row0 * p.N2 + n0);        // the CTA's first row, this warp's first column
       const size_t pitch = (size_t)p.N2 * esz;
-      const bool wide = split ? p.wide_acc : p.wide_out;
+      const bool wide = split || p.wide_out;
       const uint32_t buf = smem_u32(sRing) + (uint32_t)(warp * 4096);
       const int rows_left = p.M - row0 - (warp & 3) * 32;      // rows of this warp's quarter that exist
       uint8_t* wdst = dst + (size_t)((warp & 3) * 32) * pitch;
@@ -581,7 +581,6 @@ ago_status_t ffn_pair_run(const Plan& plan, FusedState* st, const void* const* i
   q.status = status_word;
   q.acc = nullptr;
   q.wide_out = reinterpret_cast<uintptr_t>(output) % 32 == 0;
-  q.wide_acc = reinterpret_cast<uintptr_t>(workspace) % 32 == 0;
   if (q.J > 1) {
     if (!workspace) { *err = "fused feed-forward (paired cluster, split last round): no workspace attached"; return AGO_ERR_INVALID_ARG; }
     q.acc = static_cast<float*>(workspace);   // every element of it is written before it is read: nothing to zero

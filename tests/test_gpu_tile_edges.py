@@ -210,6 +210,46 @@ def test_pointwise_pair_output_between_sectors(ago):
     sg.close()
 
 
+BETWEEN_SECTORS = [
+    # paired clusters, blocks in the middle of a cluster's run and its last one; a cluster with whole row blocks
+    (WL.ffn("ffn_offset", [242], 17000, 64, 256, 1, d_out=768), "fused", 3), (WL.ffn("ffn_offset", [243], 12300, 64, 256, 1, d_out=128), "fused", 1),
+    # 64 channels in two column phases, whose residual is read by whole sectors where it starts on one: the pair, and the single
+    # convolution of the unfused mode with the residual in its epilogue; one phase
+    (WL.Workload("conv_offset", [244], [(14, 35, 33, 64)], WL.resnet_block("x", [0], 1, 8, 64).ops, samples=14, input_dist=["relu_normal"]), "fused", 0),
+    (WL.Workload("conv_offset", [245], [(14, 35, 33, 64)], WL.resnet_block("x", [0], 1, 8, 64).ops, samples=14, input_dist=["relu_normal"]), "per_mini_subgraph", 0),
+    (WL.Workload("conv_offset", [246], [(2, 9, 9, 32)], WL.resnet_block("x", [0], 1, 8, 32).ops, samples=2, input_dist=["relu_normal"]), "fused", 0),
+]
+
+
+@pytest.mark.parametrize("wl, mode, variant", BETWEEN_SECTORS, ids=["ffn_pair", "ffn_cluster", "conv_pair", "conv_single", "conv_one_phase"])
+def test_tensors_between_sectors(ago, wl, mode, variant):
+    # inputs and output 16 but not 32 bytes aligned take other loads and stores than aligned ones, for the same values
+    import torch
+    from helpers import to_device
+    sg = ago.Subgraph(wl.ops, wl.input_shapes, mode=mode)
+    assert sg.query(ago.AGO_Q_FUSED_VARIANT) == variant
+    ins, ws = to_device(wl, WL.generate(wl))
+
+    def shifted(t):      # the tensor 16 bytes into a buffer with a guard on either side
+        flat = torch.zeros(t.numel() + 16, dtype=t.dtype, device=t.device)
+        flat[8:8 + t.numel()] = t.flatten()
+        return flat, flat[8:8 + t.numel()].view(t.shape)
+
+    ref = sg.run(ins, ws)
+    flat, out = shifted(torch.full_like(ref, float("nan")))
+    moved = [shifted(t)[1] for t in ins]
+    assert all(t.data_ptr() % 32 == 16 for t in moved + [out])
+    sg.run(moved, ws, out=out)
+    only_out = torch.empty_like(ref)
+    sg.run(moved, ws, out=only_out)
+    torch.cuda.synchronize()
+    assert sg.status() == ago.AGO_OK and torch.equal(out, ref) and torch.equal(only_out, ref)
+    assert not flat[:8].any() and not flat[-8:].any()
+    sg.close()
+    if ref.numel() < 2000000:
+        check(ago, wl, mode)
+
+
 @pytest.mark.parametrize("fp32", [True, False])
 @pytest.mark.parametrize("shape", [
     # n, h, w, c, stride: one pixel, one row, one column, fewer pixels than a piece; even and odd sizes at stride 2
