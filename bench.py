@@ -9,7 +9,9 @@ durations behind `roofline` are measured inside the timed region.
 
 The default workload is the largest configuration, `bert_layer_384`: the attention chain (`attn_384`) and then the
 feed-forward chain (`ffn_12288`) on the same 32 sequences of 384 tokens. `--workload NAME` times one chain alone.
-Prints ONE JSON line (rank 0); `workloads` in it holds the full record of every other configuration.
+Prints ONE JSON line of about 2 KB (rank 0): the headline with its roofline, and per configuration the microseconds of a launch set
+fused and per mini-subgraph with their roofline fractions. The whole record (every chain's roofline, end-to-end and CPU figures of
+every configuration; about 17 KB) goes to standard error, or to the file named by --record.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--workload NAME] [--mode fused|per_mini_subgraph|per_op|auto]
     python bench.py --impl reference ...      # the CPU oracle on the host cores, same metric
@@ -231,6 +233,24 @@ def run_reference(args):
     }))
 
 
+def headline(record):
+    """The line that is printed: what the record says about the timed run, the rest in one short entry per configuration."""
+    line = {k: v for k, v in record.items() if k not in ("chains", "context", "per_mini_subgraph", "workloads")}
+    line["roofline"] = {k: record["roofline"][k] for k in ("bound", "achieved", "peak", "unit", "frac", "traffic", "peak_source", "us_per_launch", "kernel_of")}
+    line["clocks"] = {k: record["clocks"][k] for k in ("sm_mhz", "sm_max_mhz", "reasons")} if record["clocks"] else None
+
+    def brief(r):      # microseconds and roofline fraction (of the longest chain) fused, then per mini-subgraph
+        out = []
+        for part in (r, r.get("per_mini_subgraph", {})):
+            if part.get("chains"):
+                longest = max(part["chains"], key=lambda c: c["us_per_launch_set"])
+                out += [round(part["us_per_launch_set"], 2), round(longest["roofline"]["frac"], 3)]
+        return out
+
+    line["workloads"] = {name: brief(r) for name, r in record["workloads"].items()}
+    return line
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -243,6 +263,7 @@ def main():
     ap.add_argument("--sets", type=int, default=0, help="rotating buffer sets per step (0 = enough to exceed 4x L2)")
     ap.add_argument("--skip-cpu-baseline", action="store_true")
     ap.add_argument("--skip-unfused", action="store_true")
+    ap.add_argument("--record", default="", metavar="FILE", help="write the whole record there instead of to standard error")
     ap.add_argument("--headline-only", action="store_true", help="skip the records of the other configurations")
     args = ap.parse_args()
 
@@ -494,7 +515,7 @@ def main():
         return
 
     dominant = max(head["chains"], key=lambda c: c["us_per_launch_set"])
-    line = {
+    record = {
         "metric": "fused-subgraph samples/s", "value": head["value"], "unit": "samples/s", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": head["ms_per_step"], "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": "bf16", "data": "synthetic",
@@ -502,7 +523,7 @@ def main():
             "workload": args.workload, "chains": parts_of(args.workload), "mode": args.mode,
             "samples_per_launch_set": WL.get(parts_of(args.workload)[0]).samples,
             "launches_per_step": head["launches_per_step"], "buffer_sets": head["buffer_sets"],
-            "l2_policy": f"inputs larger than L2: {head['buffer_sets']} rotating buffer sets x {head['bytes_per_set'] / 1e6:.2f} MB >= 4 x L2 ({l2 / 1e6:.0f} MB)",
+            "l2_policy": f"{head['buffer_sets']} rotating buffer sets x {head['bytes_per_set'] / 1e6:.2f} MB >= 4 x L2 ({l2 / 1e6:.0f} MB)",
             "cuda_graph": not args.no_graph, "parallelism": f"replicas x{world}",
             "us_per_launch_set": head["us_per_launch_set"],
         },
@@ -514,9 +535,14 @@ def main():
     }
     for k in ("per_mini_subgraph", "fused_speedup_vs_per_mini_subgraph", "auto_mode_picks", "cpu_baseline"):
         if k in head:
-            line[k] = head[k]
-    line["workloads"] = others
-    print(json.dumps(line))
+            record[k] = head[k]
+    record["workloads"] = others
+    if args.record:
+        with open(args.record, "w") as f:
+            json.dump(record, f)
+    else:
+        print(json.dumps(record), file=sys.stderr, flush=True)
+    print(json.dumps(headline(record)), flush=True)
     if dist is not None:
         dist.destroy_process_group()
 
