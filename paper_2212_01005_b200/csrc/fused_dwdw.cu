@@ -13,7 +13,8 @@
 // neighbouring channel pairs, so a pixel is one 128-byte request of a warp; the SEG + 4 columns that neighbouring
 // segments share come from L1.
 //
-// What bounds it: issue slots (about 0.65 of them used). Per output pair 18 FMAs of the second and
+// What bounds it: issue slots (0.69 of them used: 10.5 of 16.2 M warp instructions are the FMAs, 4.4 M go to the integer pipe, which takes
+// two cycles each: conversions of the results, clamps, edges, addresses). Per output pair 18 FMAs of the second and
 // 18 (SEG + 2) / SEG (R + 2) / R of the first convolution, about 55 instructions in all at 7 columns x 14 rows. The previous
 // kernel (input, intermediate and output tiles in shared memory, three barriers per CTA, two CTAs per SM) needed as many
 // and ran at half the issue rate: 32 x 56 x 56 x 144 31.7 -> 22.5 us (2.6 TB/s), 3 x 14 x 14 x 128 5.9 -> 2.1 us.
